@@ -189,10 +189,10 @@ int snn_row_lengths(snn_net* net, int64_t j0, int64_t n, int32_t* counts);
 
 /*
  * snn_debug_offset_count -- testing aid with no counterpart in the paper: adds
- * delta to the number of delivery items the library has counted for `column`
- * (0 <= column < grid_w * grid_h) and to the count of its group of 32
- * columns, or to the group count only when group_only is nonzero, as a
- * bookkeeping fault would.  The spike lists are left as they are, so the next
+ * delta to the number of delivery items the library has counted for the group
+ * of columns (delivery tile) that holds `column` (0 <= column < grid_w *
+ * grid_h) and to the count of all groups, or to the latter only when
+ * group_only is nonzero, as a bookkeeping fault would.  The spike lists are left as they are, so the next
  * delivery finds counts that disagree with them and must set the net's status
  * word (see snn_step).  Synchronises the net's stream.  SNN_EINVAL for a
  * column out of range.
@@ -202,7 +202,7 @@ int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t 
 /*
  * snn_info -- sizes of the net: info[0] = N neurons, [1] = synapses,
  * [2] = device bytes held, [3] = bytes of the synapse table, [4] = row
- * capacity in synapse slots, [5] = precision, [6] = side of the delivery
+ * capacity in synapse slots, [5] = precision, [6] = width of the delivery
  * tiles in columns, [7] = delivery blocks, [8] = update blocks.  n = entries
  * available (at most 9 are written).
  */

@@ -19,12 +19,13 @@ struct snn_net {
   int precision = 0, rowcap = 0, rec_size = 0, num_sms = 0, update_grid = 0;
   bool agg = true;
   int deliver_grid = 0;
-  int tile = 1, ring = 0, win_cap = 0, desc_words = 8;  // delivery tiles and windows
-  int part_cols = kMaxTileCols;
-  size_t window_budget = 0;  // bytes of shared memory a delivery window may take
+  int npc4 = 0, unit = kSlotUnit;     // words of a column in acc; slots of a bucket unit
+  int planes = 1;                     // planes of a spike descriptor
+  int tw = 1, th = 1, ntile = 1;      // delivery tiles
+  bool batch_member = false;          // windows sized for the batch kernel's blocks
   unsigned min_items = 256;  // fewest items a delivery block takes
-  unsigned win_items = kWinMinItems;  // fewest items of a windowed tile part
-  unsigned cost_win = kCostWin, cost_part = kCostPart;  // range split's fixed costs
+  unsigned win_items = 0;  // fewest items of a windowed tile part
+  unsigned cost_win = 0, cost_part = kCostPart;  // range split's fixed costs
   long long N = 0, Npad = 0, ncol = 0;
   uint64_t seed = 0;
   snn_neuron_params neuron{};
@@ -37,12 +38,16 @@ struct snn_net {
   float* C = nullptr;
   uint8_t* R = nullptr;
   int32_t* acc = nullptr;
-  uint32_t* desc = nullptr;               // spike descriptors
-  uint32_t* vcol = nullptr;               // delivery order of the columns
+  uint4* list = nullptr;                  // spike lists
+  uint32_t* ctile = nullptr;              // geometry tables (see snn_internal.h)
   uint32_t* colv = nullptr;
+  uint2* tinfo = nullptr;
+  uint32_t* nbg = nullptr;
+  std::vector<uint32_t> h_ctile;
+  unsigned* icnt = nullptr;
+  BuildParams bp{};                       // the construction's draws, for readback
   unsigned* hstatus = nullptr;            // status word (pinned, mapped)
   unsigned* hstatus_dev = nullptr;
-  unsigned* cnt = nullptr;
   unsigned* ccnt = nullptr;
   uint32_t* deg = nullptr;                 // out-degree per neuron (paper law)
   unsigned long long* syn_part = nullptr;  // synaptic events per update block
@@ -167,9 +172,10 @@ void release(snn_net* net) {
   if (net->ingest) cudaFree(net->ingest);
   if (net->hingest) cudaFreeHost(net->hingest);
   if (net->ingest_ev) cudaEventDestroy(net->ingest_ev);
-  void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc,
-                  net->desc, net->vcol, net->colv, net->cnt, net->ccnt, net->deg, net->syn_part, net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage, net->dhdr, net->colcnt,
-                  net->ext_part, net->spk_part};
+  void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->ctile,
+                  net->colv, net->tinfo, net->nbg, net->icnt, net->ccnt, net->deg, net->syn_part,
+                  net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage, net->dhdr,
+                  net->colcnt, net->ext_part, net->spk_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (net->own_stream && net->stream) cudaStreamDestroy(net->stream);
@@ -215,65 +221,94 @@ int validate(int gw, int gh, const snn_neuron_params* n, const snn_synapse_param
   return SNN_OK;
 }
 
-// min(floor(2^32 / d), 2^32 - 1): the multiplier of the kernels' divisions.
-uint32_t recip32(uint32_t d) {
-  const unsigned long long m = (1ull << 32) / (unsigned long long)d;
-  return m > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)m;
-}
-
-// Delivery tiles: the largest square tile (side <= kMaxTile) whose window --
-// the tile plus a ring of kWindowRing columns, clipped to the grid -- fits the
-// shared memory budget of a delivery block: one block per SM for a net of its
-// own, two per SM in the batch kernel.  Measured at 96x96 (FP16, Down, middle
-// and Up states): a 6x6 tile without ring (80 % of the synapses land in the
-// window, each column is flushed once per part) beats a 4x4 tile with a ring
-// of one (88 %, but 36 window columns flushed per 16 columns of spikes) by
-// 13 %, 17 % and 3 %; 5x5 and 4x4 tiles without ring and 3x3 with a ring are
-// slower still.
+// Delivery tiles: the largest square tile (side <= kMaxTile) whose window,
+// neighbour table and the warps' sector lists fit the shared memory of a
+// delivery block -- one block per SM for a net of its own, two per SM in the
+// batch kernel -- then evened out over the grid's sides (24 columns make four
+// tiles of 6, 8 make two of 4).  Measured at 96x96 (FP16, Down, middle and Up
+// states): a 6x6 tile without ring (80 % of the synapses land in the window,
+// each column is flushed once per part) beats a 4x4 tile with a ring of one
+// (88 %, but 36 window columns flushed per 16 columns of spikes) by 13 %, 17 %
+// and 3 %; 5x5 and 4x4 tiles without ring and 3x3 with a ring are slower still.
+constexpr size_t kSmemBudget = 224 * 1024;
+constexpr size_t kBatchSmemBudget = 110 * 1024;
 constexpr size_t kWindowBudget = 196 * 1024;
-constexpr size_t kBatchWindowBudget = 96 * 1024;
 // Fewest items a delivery block takes (fewer blocks run when a step has few
-// items).  Measured on the 64-net batch: 256 per block beat 512, 2048 and
-// 8192, so members use the same value as nets of their own.
-constexpr unsigned kMinItems = 256;
+// items).
+constexpr unsigned kMinItems = 64;
 constexpr unsigned kBatchMinItems = 256;
-// Most columns of a delivery part without window (runs of sparse tiles): its
-// (column, bucket) and neighbour tables take part_cols * (d_max + 64) words
-// of shared memory beside the window.
-constexpr int kPartCols = kMaxTileCols;
-constexpr int kBatchPartCols = 16;
-constexpr int kWindowRing = 0;
 
 void choose_tiles(snn_net* net) {
-  net->ring = kWindowRing;
+  net->npc4 = (net->npc + 3) / 4 * 4;
+  const size_t budget = net->batch_member ? kBatchSmemBudget : kSmemBudget;
   int t = std::min(kMaxTile, std::max(net->W, net->H));
   for (; t > 1; --t) {
-    const size_t ww = (size_t)std::min(t + 2 * net->ring, net->W);
-    const size_t wh = (size_t)std::min(t + 2 * net->ring, net->H);
-    if (ww * wh * (size_t)net->npc * 4 <= net->window_budget) break;
+    const int cols = std::min(t, net->W) * std::min(t, net->H);
+    if (deliver_smem(cols, net->npc4, net->batch_member) <= budget &&
+        (size_t)cols * net->npc4 * 4 <= kWindowBudget)
+      break;
   }
-  net->tile = t;
-  net->part_cols = std::max(net->part_cols, t * t);
-  const long long ww = std::min(t + 2 * net->ring, net->W);
-  const long long wh = std::min(t + 2 * net->ring, net->H);
-  net->win_cap = (int)((ww * wh * net->npc + 3) / 4 * 4);
+  auto even = [](int side, int t) {
+    const int n = (side + t - 1) / t;
+    return (side + n - 1) / n;
+  };
+  net->tw = even(net->W, std::min(t, net->W));
+  net->th = even(net->H, std::min(t, net->H));
+  const int words = net->tw * net->th * net->npc4;
+  net->win_items = (unsigned)std::max(32, words / kWinWordsPerItem);
+  net->cost_win = (unsigned)std::max(32, words / kCostWordsPerItem);
+  net->ntile = ((net->W + net->tw - 1) / net->tw) * ((net->H + net->th - 1) / net->th);
 }
 
-// Virtual (delivery) order of the columns: tile by tile, tiles and the
-// columns inside a tile in row-major order.  vcol[v] = real column.
-void column_order(int W, int H, int T, std::vector<uint32_t>* vcol, std::vector<uint32_t>* colv) {
-  vcol->assign((size_t)W * H, 0u);
-  colv->assign((size_t)W * H, 0u);
+// Geometry tables (see snn_internal.h): the tile, place and virtual index of
+// every column, every tile's first virtual column and columns, and the first
+// word in acc of the column at each stencil offset of each virtual column.
+struct Geometry {
+  std::vector<uint32_t> ctile, colv, nbg;
+  std::vector<uint2> tinfo;
+};
+
+void geometry_tables(const snn_net* net, Geometry* g) {
+  const int W = net->W, H = net->H;
+  g->ctile.assign((size_t)net->ncol, 0u);
+  g->colv.assign((size_t)net->ncol, 0u);
+  g->nbg.assign((size_t)net->ncol * 64, 0u);
+  uint32_t v = 0u;
+  for (int y0 = 0; y0 < H; y0 += net->th)
+    for (int x0 = 0; x0 < W; x0 += net->tw) {
+      const int w = std::min(net->tw, W - x0), h = std::min(net->th, H - y0);
+      uint2 ti;
+      ti.x = v;
+      ti.y = (unsigned)(w * h);
+      for (int y = y0; y < y0 + h; ++y)
+        for (int x = x0; x < x0 + w; ++x, ++v) {
+          const size_t c = (size_t)y * W + x;
+          g->ctile[c] = (uint32_t)g->tinfo.size() << 6 | (v - ti.x);
+          g->colv[c] = v;
+        }
+      g->tinfo.push_back(ti);
+    }
   for (int y = 0; y < H; ++y)
     for (int x = 0; x < W; ++x) {
-      const int tr = y / T, tc = x / T;
-      const int th = std::min(T, H - tr * T), tw = std::min(T, W - tc * T);
-      const long long v = (long long)tr * T * W + (long long)tc * th * T +
-                          (long long)(y - tr * T) * tw + (x - tc * T);
-      const uint32_t c = (uint32_t)(y * W + x);
-      (*vcol)[(size_t)v] = c;
-      (*colv)[c] = (uint32_t)v;
+      uint32_t* row = g->nbg.data() + (size_t)g->colv[(size_t)y * W + x] * 64;
+      for (int dy = -3; dy <= 3; ++dy)
+        for (int dx = -3; dx <= 3; ++dx) {
+          const int tx = ((x + dx) % W + W) % W, ty = ((y + dy) % H + H) % H;
+          row[(dy + 3) << 3 | (dx + 3)] = g->colv[(size_t)ty * W + tx] * (uint32_t)net->npc4;
+        }
     }
+}
+
+// Slots of a bucket unit and of a row for rows of at most K synapses in
+// `parts` bucket parts: units of 8 slots, or of 16 where a row could exceed
+// the 255 units that its bucket ends count.
+void choose_unit(snn_net* net, int K) {
+  const int parts = 2 * net->ndel;
+  for (net->unit = kSlotUnit;; net->unit *= 2) {
+    const int n = std::min(K, parts);  // parts that hold a synapse
+    net->rowcap = (K + (net->unit - 1) * n + net->unit - 1) / net->unit * net->unit;
+    if (net->rowcap / net->unit <= 255 || net->unit == 2 * kSlotUnit) break;
+  }
 }
 
 // A kernel found inconsistent counts: the net's stepping is no longer exact.
@@ -322,20 +357,19 @@ void fill_step_params(snn_net* net) {
   p.dmin = net->dmin;
   p.ndel = net->ndel;
   p.nslot = net->nslot;
-  p.rowcap = net->rowcap;
+  p.row_sec = net->rowcap * net->rec_size / 32;
+  p.unit_sec = net->unit * net->rec_size / 32;
   p.ncol = (int)net->ncol;
   p.agg = net->agg ? 1 : 0;
-  p.tile = net->tile;
-  p.part_cols = net->part_cols;
-  p.ring = net->ring;
-  p.win_cap = net->win_cap;
-  p.desc_words = net->desc_words;
+  p.npc4 = net->npc4;
+  p.ntile = net->ntile;
+  p.tcols = net->tw * net->th;
+  p.tcap = p.tcols * net->npc;
   p.min_items = net->min_items;
   p.win_items = net->win_items;
   p.cost_win = net->cost_win;
   p.cost_part = net->cost_part;
   p.npc_m = recip32((uint32_t)net->npc);
-  p.w_m = recip32((uint32_t)net->W);
   p.seed_lo = (uint32_t)(net->seed & 0xFFFFFFFFu);
   p.seed_hi = (uint32_t)(net->seed >> 32);
   p.pvv = t.pvv;
@@ -352,11 +386,15 @@ void fill_step_params(snn_net* net) {
   p.R = net->R;
   p.acc = net->acc;
   p.ids = nullptr;
-  p.desc = net->desc;
-  p.vcol = net->vcol;
+  p.list = net->list;
+  p.planes = net->planes;
+  p.ctile = net->ctile;
   p.colv = net->colv;
+  p.tinfo = net->tinfo;
+  p.nbg = net->nbg;
+  p.icnt = net->icnt;
   p.hstatus = net->hstatus_dev;
-  p.cnt = net->cnt;
+  p.cnt = nullptr;
   p.ccnt = net->ccnt;
   // a shard keeps the out-degree of its rows (synapses into its own columns)
   // for snn_row_lengths; its spikes count the full k_out synaptic events
@@ -365,7 +403,7 @@ void fill_step_params(snn_net* net) {
   p.sg = net->sg;
   p.isum = net->isum;
   p.gsum = net->gsum;
-  p.bend = net->bend;
+  p.bend = reinterpret_cast<const uint4*>(net->bend);
   p.syn = net->syn;
   p.ctl = net->ctl;
   p.rec = net->rec;
@@ -396,7 +434,8 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   net->N = net->ncol * np->n_per_col;
   net->Npad = (net->N + 3) / 4 * 4;
   net->rec_size = precision == SNN_EXACT_F16W ? 4 : 8;
-  net->rowcap = (sp->k_out + (kSlotUnit - 1) * net->ndel + kSlotUnit - 1) / kSlotUnit * kSlotUnit;
+  net->planes = (net->ndel + kPlaneBuckets - 1) / kPlaneBuckets;
+  choose_unit(net, sp->k_out);
   net->rec_cap = 1LL << 24;
   rc = make_host_tables(*np, *sp, precision, &net->tables, &why);
   if (rc != SNN_OK) return fail(net, rc, why);
@@ -409,14 +448,13 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   SNN_CUDA(net, cudaDeviceGetAttribute(&net->num_sms, cudaDevAttrMultiProcessorCount, dev));
   net->update_grid = update_grid(net->N, net->num_sms);
   choose_tiles(net);
-  net->desc_words = net->ndel <= 28 ? 8 : 16;
   fill_step_params(net);
   net->deliver_grid = deliver_grid(net->sp, precision, net->num_sms);
   if (net->deliver_grid < 1) return fail(net, SNN_ECUDA, "delivery kernel does not fit on the device");
   net->rec_region = (net->rec_cap + net->update_grid - 1) / net->update_grid;
 
   net->connectivity = sp->connectivity;
-  BuildParams bp{};
+  BuildParams& bp = net->bp;
   bp.N = net->N;
   bp.npc = net->npc;
   bp.nexc = net->nexc;
@@ -439,7 +477,27 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   std::memcpy(bp.poff_dx, net->tables.poff_dx, sizeof(bp.poff_dx));
   std::memcpy(bp.poff_dy, net->tables.poff_dy, sizeof(bp.poff_dy));
   bp.sg = net->sg;
-  if ((rc = dalloc(net, &net->bend, (size_t)net->N * kBendStride))) return rc;
+  bp.npc4 = net->npc4;
+  bp.tw = net->tw;
+  bp.th = net->th;
+  bp.unit = net->unit;
+  bp.planes = net->planes;
+  Geometry geo;
+  geometry_tables(net, &geo);
+  net->h_ctile = geo.ctile;
+  auto upload = [&](auto** dst, const auto& src) -> int {
+    const size_t bytes = src.size() * sizeof(src[0]);
+    if (int arc = dalloc(net, dst, bytes)) return arc;
+    SNN_CUDA(net, cudaMemcpyAsync(*dst, src.data(), bytes, cudaMemcpyHostToDevice, net->stream));
+    return SNN_OK;
+  };
+  if ((rc = upload(&net->ctile, geo.ctile))) return rc;
+  if ((rc = upload(&net->colv, geo.colv))) return rc;
+  if ((rc = upload(&net->tinfo, geo.tinfo))) return rc;
+  if ((rc = upload(&net->nbg, geo.nbg))) return rc;
+  SNN_CUDA(net, cudaStreamSynchronize(net->stream));
+  bp.colv = net->colv;
+  if ((rc = dalloc(net, &net->bend, (size_t)net->N * net->planes * 16))) return rc;
   net->total_syn = net->N * (long long)net->K;
   if (net->sg.on && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
   if (net->connectivity == SNN_CONN_PAPER) {
@@ -447,22 +505,27 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
     // the row stride of the table
     unsigned* dmax = nullptr;
     if ((rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
-    if ((rc = dalloc(net, &dmax, 4))) return rc;
-    net->device_bytes -= 4;
-    unsigned max_units = 0u;
+    if ((rc = dalloc(net, &dmax, 8))) return rc;
+    net->device_bytes -= 8;
+    unsigned max_units[2] = {0u, 0u};
     bp.bend = net->bend;
     bp.deg = net->deg;
     bp.max_units = dmax;
-    cudaError_t ce = cudaMemsetAsync(dmax, 0, 4, net->stream);
-    if (ce == cudaSuccess) ce = launch_paper_count(bp, net->num_sms, net->stream);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(&max_units, dmax, 4, cudaMemcpyDeviceToHost, net->stream);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(net->stream);
+    cudaError_t ce = cudaSuccess;
+    for (net->unit = kSlotUnit; ce == cudaSuccess; net->unit *= 2) {
+      bp.unit = net->unit;
+      ce = cudaMemsetAsync(dmax, 0, 8, net->stream);
+      if (ce == cudaSuccess) ce = launch_paper_count(bp, net->num_sms, net->stream);
+      if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(max_units, dmax, 8, cudaMemcpyDeviceToHost, net->stream);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(net->stream);
+      if (max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
+    }
     cudaFree(dmax);
     if (ce != cudaSuccess) return cuda_fail(net, ce, "connectivity count pass");
-    if (max_units > 255u)
+    if (max_units[1] > 255u || max_units[0] > 255u)
       return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
-    net->rowcap = (int)std::max(1u, max_units) * kSlotUnit;
+    net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
     std::vector<uint32_t> deg((size_t)net->N);
     SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
                                   net->stream));
@@ -476,14 +539,17 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->V, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->C, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->R, (size_t)net->Npad))) return rc;
-  if ((rc = dalloc(net, &net->acc, (size_t)net->Npad * 4))) return rc;
-  if ((rc = dalloc(net, &net->desc, (size_t)net->nslot * net->N * net->desc_words * 4))) return rc;
-  if ((rc = dalloc(net, &net->vcol, (size_t)net->ncol * 4))) return rc;
-  if ((rc = dalloc(net, &net->colv, (size_t)net->ncol * 4))) return rc;
-  if ((rc = dalloc(net, &net->cnt, (size_t)net->nslot * 4))) return rc;
-  if ((rc = dalloc(net, &net->ccnt, (size_t)net->nslot * net->ncol * 4))) return rc;
-  if ((rc = dalloc(net, &net->isum, (size_t)net->ncol * 4))) return rc;
-  if ((rc = dalloc(net, &net->gsum, (size_t)(net->ncol + 31) / 32 * 4))) return rc;
+  const size_t acc_bytes = (size_t)net->ncol * net->npc4 * 4;
+  const size_t ccnt_bytes = (size_t)net->nslot * net->ntile * kCntStride * 4;
+  const size_t isum_bytes = (size_t)net->ntile * kCntStride * 4;
+  if ((rc = dalloc(net, &net->acc, acc_bytes))) return rc;
+  const size_t tcap = (size_t)net->tw * net->th * net->npc;
+  if ((rc = dalloc(net, &net->list, (size_t)net->nslot * net->planes * net->ntile * tcap * 16)))
+    return rc;
+  if ((rc = dalloc(net, &net->ccnt, ccnt_bytes))) return rc;
+  if ((rc = dalloc(net, &net->isum, isum_bytes))) return rc;
+  if ((rc = dalloc(net, &net->gsum, 4))) return rc;
+  if (net->sg.on && (rc = dalloc(net, &net->icnt, (size_t)net->ncol * 4))) return rc;
   if ((rc = dalloc(net, &net->ctl, sizeof(Ctl)))) return rc;
   if ((rc = dalloc(net, &net->rec, (size_t)net->rec_region * net->update_grid * 8))) return rc;
   if ((rc = dalloc(net, &net->rcnt, (size_t)net->update_grid * 8))) return rc;
@@ -505,22 +571,15 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &wtab, net->tables.wtab.size() * 4))) return rc;
   net->device_bytes -= net->tables.wtab.size() * 4;
 
-  std::vector<uint32_t> vcol, colv;
-  column_order(net->W, net->H, net->tile, &vcol, &colv);
   cudaError_t e = cudaMemcpyAsync(wtab, net->tables.wtab.data(), net->tables.wtab.size() * 4,
                                   cudaMemcpyHostToDevice, net->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(net->vcol, vcol.data(), vcol.size() * 4, cudaMemcpyHostToDevice, net->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(net->colv, colv.data(), colv.size() * 4, cudaMemcpyHostToDevice, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->ctl, 0, sizeof(Ctl), net->stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(net->cnt, 0, (size_t)net->nslot * 4, net->stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(net->ccnt, 0, (size_t)net->nslot * net->ncol * 4, net->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(net->isum, 0, (size_t)net->ncol * 4, net->stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(net->gsum, 0, (size_t)(net->ncol + 31) / 32 * 4, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(net->acc, 0, acc_bytes, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(net->ccnt, 0, ccnt_bytes, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(net->isum, 0, isum_bytes, net->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(net->gsum, 0, 4, net->stream);
+  if (e == cudaSuccess && net->icnt)
+    e = cudaMemsetAsync(net->icnt, 0, (size_t)net->ncol * 4, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->colcnt, 0, (size_t)net->ncol * 16, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->ext_part, 0, (size_t)net->update_grid * 8, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->spk_part, 0, (size_t)net->update_grid * 8, net->stream);
@@ -573,7 +632,14 @@ int net_view(snn_net* net, NetView* v) {
   v->syn = net->syn;
   v->bend = net->bend;
   v->N = net->N;
+  v->acc_words = net->ncol * (long long)net->npc4;
   v->npc = net->npc;
+  v->npc4 = net->npc4;
+  v->unit = net->unit;
+  v->planes = net->planes;
+  v->ctile = net->ctile;
+  v->colv = net->colv;
+  v->nbg = net->nbg;
   v->nexc = net->nexc;
   v->dmin = net->dmin;
   v->ndel = net->ndel;
@@ -596,8 +662,8 @@ namespace {
 
 int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
               const snn_synapse_params* synapse, uint64_t seed, int precision,
-              void* cuda_stream, size_t window_budget, unsigned min_items, int part_cols,
-              snn_net** out, const ShardGeo* shard = nullptr) {
+              void* cuda_stream, bool batch_member, snn_net** out,
+              const ShardGeo* shard = nullptr) {
   if (!out) return fail(nullptr, SNN_EINVAL, "out is NULL");
   *out = nullptr;
   std::string why;
@@ -605,9 +671,8 @@ int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
   if (vrc != SNN_OK) return fail(nullptr, vrc, why);
   snn_net* net = new (std::nothrow) snn_net();
   if (!net) return fail(nullptr, SNN_ENOMEM, "host allocation failed");
-  net->window_budget = window_budget;
-  net->min_items = min_items;
-  net->part_cols = part_cols;
+  net->batch_member = batch_member;
+  net->min_items = batch_member ? kBatchMinItems : kMinItems;
   if (shard) net->sg = *shard;
   if (cuda_stream) {
     net->stream = static_cast<cudaStream_t>(cuda_stream);
@@ -637,8 +702,7 @@ extern "C" {
 int snn_build(int grid_w, int grid_h, const snn_neuron_params* neuron,
               const snn_synapse_params* synapse, uint64_t seed, int precision,
               void* cuda_stream, snn_net** out) {
-  return build_net(grid_w, grid_h, neuron, synapse, seed, precision, cuda_stream, kWindowBudget,
-                   kMinItems, kPartCols, out);
+  return build_net(grid_w, grid_h, neuron, synapse, seed, precision, cuda_stream, false, out);
 }
 
 }  // extern "C"
@@ -718,8 +782,7 @@ int snn_build_shard(int grid_w, int grid_h, int x0, int y0, int w, int h,
   int ew = 0, eh = 0;
   const int grc = shard_geometry(grid_w, grid_h, x0, y0, w, h, synapse->stencil_radius, &g, &ew, &eh);
   if (grc != SNN_OK) return grc;
-  return build_net(ew, eh, neuron, synapse, seed, precision, cuda_stream, kWindowBudget, kMinItems,
-                   kPartCols, out, &g);
+  return build_net(ew, eh, neuron, synapse, seed, precision, cuda_stream, false, out, &g);
 }
 
 int snn_shard_update(snn_net* net) {
@@ -1062,65 +1125,60 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   if (!net || j0 < 0 || n < 0 || j0 + n > net->N || (n > 0 && (!target || !delay || !wfx)))
     return fail(net, SNN_EINVAL, "bad argument");
   if (n == 0) return SNN_OK;
-  const size_t row_bytes = (size_t)net->rowcap * net->rec_size;
-  std::vector<uint8_t> rows((size_t)n * row_bytes);
-  std::vector<uint8_t> ends((size_t)n * kBendStride);
-  SNN_CUDA(net, cudaMemcpyAsync(rows.data(), (const char*)net->syn + (size_t)j0 * row_bytes,
-                                rows.size(), cudaMemcpyDeviceToHost, net->stream));
-  SNN_CUDA(net, cudaMemcpyAsync(ends.data(), net->bend + (size_t)j0 * kBendStride, ends.size(),
-                                cudaMemcpyDeviceToHost, net->stream));
-  int rc = sync(net);
-  if (rc) return rc;
   std::vector<int32_t> len((size_t)n);
-  rc = snn_row_lengths(net, j0, n, len.data());
+  int rc = snn_row_lengths(net, j0, n, len.data());
   if (rc) return rc;
-  long long total = 0;
-  for (int32_t v : len) total += v;
-  long long o = 0;
-  for (int64_t r = 0; r < n; ++r) {
-    const long long j = j0 + r;
-    const long long col = j / net->npc;
-    const int cy = (int)(col / net->W), cx = (int)(col % net->W);
-    const bool exc = (int)(j % net->npc) < net->nexc;
-    int beg = 0;
-    for (int b = 0; b < net->ndel; ++b) {
-      const int end = ends[(size_t)r * kBendStride + b] * kSlotUnit;
-      for (int s = beg; s < end; ++s) {
-        uint32_t code, wbits;
-        const uint8_t* rp = rows.data() + (size_t)r * row_bytes + (size_t)s * net->rec_size;
-        int32_t w;
-        if (net->precision == SNN_EXACT_F16W) {
-          uint32_t rec;
-          std::memcpy(&rec, rp, 4);
-          if (is_pad_f16(rec)) continue;
-          code = rec & 0x1FFFFu;
-          __half_raw hr;
-          hr.x = (unsigned short)(rec >> 17);
-          const float f = __half2float(__half(hr));
-          w = (int32_t)std::rint((exc ? f : -f) * 65536.0f);
-        } else {
-          std::memcpy(&code, rp, 4);
-          std::memcpy(&wbits, rp + 4, 4);
-          if (code == kPad) continue;
-          w = (int32_t)wbits;
-        }
-        if (o >= total) return fail(net, SNN_ESTATE, "row holds too many synapses");
-        if (net->precision == SNN_EXACT_F16W) {
-          const int dy = (int)((code >> 14) & 7u) - 3, dx = (int)((code >> 11) & 7u) - 3;
-          const int ty = ((cy + dy) % net->H + net->H) % net->H;
-          const int tx = ((cx + dx) % net->W + net->W) % net->W;
-          target[o] = ((long long)ty * net->W + tx) * net->npc + (code & 0x7FFu);
-        } else {
-          target[o] = (long long)code;
-        }
-        delay[o] = net->dmin + b;
-        wfx[o] = w;
-        ++o;
-      }
-      beg = end;
-    }
+  // the device walks each row's draws again and decodes the records in that
+  // order, a bounded number of rows at a time
+  constexpr int64_t kRows = 4096;
+  const int64_t m = std::min(n, kRows);
+  size_t most = 0;
+  std::vector<long long> off;
+  for (int64_t r0 = 0; r0 < n; r0 += m) {
+    size_t k = 0;
+    for (int64_t r = r0; r < std::min(n, r0 + m); ++r) k += (size_t)len[r];
+    most = std::max(most, k);
   }
-  if (o != total) return fail(net, SNN_ESTATE, "row holds too few synapses");
+  unsigned char* buf = nullptr;  // offsets, targets, delays, weights
+  const size_t off_bytes = (size_t)m * 8, b8 = most * 8, b4 = most * 4;
+  rc = dalloc(net, &buf, off_bytes + b8 + 2 * b4);
+  if (rc) return rc;
+  net->device_bytes -= off_bytes + b8 + 2 * b4;
+  BuildParams bp = net->bp;
+  bp.syn = net->syn;
+  bp.bend = net->bend;
+  bp.unit = net->unit;
+  bp.rowcap = net->rowcap;
+  bp.rd_off = reinterpret_cast<long long*>(buf);
+  bp.rd_target = reinterpret_cast<long long*>(buf + off_bytes);
+  bp.rd_delay = reinterpret_cast<int32_t*>(buf + off_bytes + b8);
+  bp.rd_wfx = reinterpret_cast<int32_t*>(buf + off_bytes + b8 + b4);
+  cudaError_t e = cudaSuccess;
+  size_t at = 0;
+  for (int64_t r0 = 0; r0 < n && e == cudaSuccess; r0 += m) {
+    bp.j0 = j0 + r0;
+    bp.n_rows = std::min(n - r0, m);
+    off.assign((size_t)bp.n_rows, 0);
+    size_t k = 0;
+    for (int64_t r = 0; r < bp.n_rows; ++r) {
+      off[(size_t)r] = (long long)k;
+      k += (size_t)len[r0 + r];
+    }
+    e = cudaMemcpyAsync(buf, off.data(), off.size() * 8, cudaMemcpyHostToDevice, net->stream);
+    if (e == cudaSuccess)
+      e = launch_read_rows(bp, net->precision, net->connectivity == SNN_CONN_PAPER, net->stream);
+    if (e == cudaSuccess && k > 0) {
+      e = cudaMemcpyAsync(target + at, bp.rd_target, k * 8, cudaMemcpyDeviceToHost, net->stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(delay + at, bp.rd_delay, k * 4, cudaMemcpyDeviceToHost, net->stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(wfx + at, bp.rd_wfx, k * 4, cudaMemcpyDeviceToHost, net->stream);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
+    at += k;
+  }
+  cudaFree(buf);
+  if (e != cudaSuccess) return cuda_fail(net, e, "synapse readback");
   return SNN_OK;
 }
 
@@ -1141,7 +1199,7 @@ int snn_info(snn_net* net, int64_t* info, int n) {
   if (!net || !info) return fail(net, SNN_EINVAL, "null argument");
   const int64_t v[9] = {net->N, (int64_t)net->total_syn, (int64_t)net->device_bytes,
                         net->N * (int64_t)net->rowcap * net->rec_size, net->rowcap,
-                        net->precision, net->tile, net->deliver_grid, net->update_grid};
+                        net->precision, net->tw, net->deliver_grid, net->update_grid};
   for (int i = 0; i < n && i < 9; ++i) info[i] = v[i];
   return SNN_OK;
 }
@@ -1155,17 +1213,16 @@ int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t 
   if (column < 0 || column >= net->ncol) return fail(net, SNN_EINVAL, "column out of range");
   int rc = sync(net);
   if (rc) return rc;
-  uint32_t v = 0u;
-  SNN_CUDA(net, cudaMemcpy(&v, net->colv + column, 4, cudaMemcpyDeviceToHost));
+  unsigned* const tile = net->isum + (size_t)(net->h_ctile[(size_t)column] >> 6) * kCntStride;
   unsigned word = 0u;
   if (!group_only) {
-    SNN_CUDA(net, cudaMemcpy(&word, net->isum + v, 4, cudaMemcpyDeviceToHost));
+    SNN_CUDA(net, cudaMemcpy(&word, tile, 4, cudaMemcpyDeviceToHost));
     word += (unsigned)delta;
-    SNN_CUDA(net, cudaMemcpy(net->isum + v, &word, 4, cudaMemcpyHostToDevice));
+    SNN_CUDA(net, cudaMemcpy(tile, &word, 4, cudaMemcpyHostToDevice));
   }
-  SNN_CUDA(net, cudaMemcpy(&word, net->gsum + (v >> 5), 4, cudaMemcpyDeviceToHost));
+  SNN_CUDA(net, cudaMemcpy(&word, net->gsum, 4, cudaMemcpyDeviceToHost));
   word += (unsigned)delta;
-  SNN_CUDA(net, cudaMemcpy(net->gsum + (v >> 5), &word, 4, cudaMemcpyHostToDevice));
+  SNN_CUDA(net, cudaMemcpy(net->gsum, &word, 4, cudaMemcpyHostToDevice));
   return SNN_OK;
 }
 
@@ -1278,7 +1335,7 @@ int batch_run(snn_batch* b, long long n_steps) {
   bp.spin_limit = b->spin_limit;
   bp.extra_arrivals = b->extra_arrivals;
   size_t dsm = 0;
-  for (const snn_net* net : b->nets) dsm = std::max(dsm, deliver_smem(net->sp, b->precision));
+  for (const snn_net* net : b->nets) dsm = std::max(dsm, deliver_smem(net->sp.tcols, net->sp.npc4, true));
   const size_t smem = batch_smem(dsm);
   const int grid = batch_grid(b->precision, b->infl, b->num_sms, smem);
   if (grid < 1) return bfail(b, SNN_ECUDA, "batch kernel does not fit on the device");
@@ -1327,7 +1384,7 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
   for (int k = 0; k < n_nets && rc == SNN_OK; ++k) {
     snn_net* net = nullptr;
     rc = build_net(grid_w[k], grid_h[k], neuron + k, synapse + k, seeds[k], precision, b->stream,
-                   kBatchWindowBudget, kBatchMinItems, kBatchPartCols, &net);
+                   true, &net);
     if (rc != SNN_OK) break;
     net->in_batch = true;
     b->nets.push_back(net);

@@ -7,17 +7,20 @@
 //   k >= k_local : stencil offset = first m with x1 < thr[m] (P ~ exp(-r/lambda)),
 //                  target l = u_n(x0) in column ((x+dx) mod W, (y+dy) mod H);
 //   delay d = d_min + u_ndel(x2);  weight = table[population][x3 >> 16].
-// F16W records keep the target as a stencil code and the weight's magnitude as
-// a half; F32W records keep the target's neuron index and the FP32 weight
-// already scaled to the input's fixed-point units, round(w * 2^16).
-// One warp owns one row: a first pass counts the synapses of every delay
-// bucket, a second pass regenerates them and stores each into its bucket in
-// k order (warp match + popc rank), then the bucket tails are padded.
+// A delay bucket has two parts (see snn_internal.h): the synapses that end in
+// the source's own delivery tile, stored as words of the tile's window, and
+// the others, stored as a stencil offset and an index.
+// One warp owns one row: a first pass counts the synapses of every bucket
+// part, a second pass regenerates them and stores each into its part in k
+// order (warp match + popc rank), then the parts' tails are padded.  Rows are
+// stored, and walked, in virtual column order.  The same walk reads rows back
+// in the order in which they were drawn.
 // A shard (see ShardGeo) draws every synapse with the neuron's global index
-// and keeps only those whose target column is one of its own; an F32W record
-// then holds the target's local index (local and global stencil arithmetic
-// agree for such targets: the halo is as wide as the stencil, or the local
-// grid spans the whole global side).
+// and keeps only those whose target column is one of its own (local and
+// global stencil arithmetic agree for such targets: the halo is as wide as
+// the stencil, or the local grid spans the whole global side).
+#include <cuda_fp16.h>
+
 #include "snn_device.cuh"
 #include "snn_internal.h"
 
@@ -25,130 +28,280 @@ namespace snn {
 namespace {
 
 constexpr int kBuildWarps = 8;
+constexpr int kDropped = 0xFE;  // offset class: not kept by the shard
+constexpr int kOut = 0xFF;      // offset class: another tile
+constexpr int kModeCount = 0, kModeFill = 1, kModeRead = 2;
 
-template <int PREC>
-__global__ void __launch_bounds__(kBuildWarps * 32)
-    build_rows_kernel(const BuildParams P) {
-  __shared__ unsigned s_cnt[kBuildWarps][32];
-  __shared__ unsigned s_cur[kBuildWarps][32];
-  __shared__ uint32_t s_thr[kMaxOff];
-  __shared__ int s_code[kMaxOff];
-  __shared__ int s_dx[kMaxOff], s_dy[kMaxOff];
-  for (int m = threadIdx.x; m < kMaxOff; m += blockDim.x) {
-    s_thr[m] = P.stencil_thr[m];
-    s_code[m] = m < P.n_off ? ((P.off_dy[m] + 3) << 3) | (P.off_dx[m] + 3) : kCenterCode;
-    s_dx[m] = m < P.n_off ? P.off_dx[m] : 0;
-    s_dy[m] = m < P.n_off ? P.off_dy[m] : 0;
+// Shared tables of a block and its warps' rows.
+struct RowSmem {
+  unsigned cnt[kBuildWarps][64];       // synapses per bucket part (2 b, 2 b + 1)
+  unsigned cur[kBuildWarps][64];       // next slot of each part
+  unsigned rd[kBuildWarps][32];        // readback: next entry of each delay
+  uint8_t cls[kBuildWarps][kMaxOff + 1];  // target's place in the tile per offset
+  uint32_t thr[kMaxOff];
+  uint8_t guide[256];                  // offsets whose threshold is <= (b << 24)
+  int8_t dx[kMaxOff + 1], dy[kMaxOff + 1];  // the last entry is (0, 0)
+};
+
+// The row a warp works on.
+struct Row {
+  long long j;        // its neuron (real, local index)
+  uint32_t jj;        // the index its draws are keyed on
+  int lj, cx, cy;
+  int x0, y0, tw;     // first column and width of its tile
+  size_t at;          // its place in syn and bend
+};
+
+template <bool PAPER>
+__device__ __forceinline__ void load_offsets(const BuildParams& P, RowSmem& S) {
+  const int n = PAPER ? P.n_poff : P.n_off;
+  for (int m = threadIdx.x; m <= kMaxOff; m += blockDim.x) {
+    S.dx[m] = m < n ? (PAPER ? P.poff_dx[m] : P.off_dx[m]) : (int8_t)0;
+    S.dy[m] = m < n ? (PAPER ? P.poff_dy[m] : P.off_dy[m]) : (int8_t)0;
+    if (m < kMaxOff) S.thr[m] = P.stencil_thr[m];
   }
   __syncthreads();
+  for (int b = threadIdx.x; b < 256; b += blockDim.x) {
+    int g = 0;
+    while (g + 1 < P.n_off && S.thr[g] <= (uint32_t)b << 24) ++g;
+    S.guide[b] = (uint8_t)g;
+  }
+  __syncthreads();
+}
+
+// Row of neuron l of column c, and the class of every stencil offset of it:
+// the target column's place in the tile, kOut, or kDropped.
+template <bool PAPER>
+__device__ __forceinline__ Row open_row(const BuildParams& P, RowSmem& S, int c, int l) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  Row r;
+  r.j = (long long)c * P.npc + l;
+  r.lj = l;
+  r.cy = c / P.W;
+  r.cx = c - r.cy * P.W;
+  int gx, gy;
+  shard_global_col(P.sg, r.cx, r.cy, &gx, &gy);
+  r.jj = P.sg.on ? ((uint32_t)gy * (uint32_t)P.sg.GW + (uint32_t)gx) * (uint32_t)P.npc + (uint32_t)l
+                 : (uint32_t)r.j;
+  r.x0 = r.cx / P.tw * P.tw;
+  r.y0 = r.cy / P.th * P.th;
+  r.tw = min(P.tw, P.W - r.x0);
+  const int th = min(P.th, P.H - r.y0);
+  r.at = (size_t)P.colv[c] * P.npc + l;
+  const int n = PAPER ? P.n_poff : P.n_off;
+  __syncwarp();
+  for (int m = lane; m <= kMaxOff; m += 32) {
+    const int dx = S.dx[m], dy = S.dy[m];
+    const int ox = wrap(r.cx + dx, P.W) - r.x0, oy = wrap(r.cy + dy, P.H) - r.y0;
+    int v = (unsigned)ox < (unsigned)r.tw && (unsigned)oy < (unsigned)th ? oy * r.tw + ox : kOut;
+    if (P.sg.on && (m < n || m == kMaxOff) &&
+        !shard_owns_global(P.sg, P.W, P.H, wrap(gx + dx, P.sg.GW), wrap(gy + dy, P.sg.GH)))
+      v = kDropped;
+    S.cls[w][m] = (uint8_t)v;
+  }
+  __syncwarp();
+  return r;
+}
+
+// Stencil offset of word x: the first m with x < thr[m] (the last catches all).
+__device__ __forceinline__ int offset_of(const BuildParams& P, const RowSmem& S, uint32_t x) {
+  int m = S.guide[x >> 24];
+  while (m + 1 < P.n_off && x >= S.thr[m]) ++m;
+  return m;
+}
+
+// Parts' sizes (S.cnt) to bucket ends and first slots; lane b holds bucket b.
+// Returns the row's units.
+template <int MODE>
+__device__ __forceinline__ unsigned open_parts(const BuildParams& P, RowSmem& S, const Row& r) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned unit = (unsigned)P.unit;
+  const unsigned ci = lane < P.ndel ? S.cnt[w][2 * lane] : 0u;
+  const unsigned co = lane < P.ndel ? S.cnt[w][2 * lane + 1] : 0u;
+  const unsigned ui = (ci + unit - 1u) / unit, uo = (co + unit - 1u) / unit;
+  unsigned incl = ui + uo, icnt = ci + co;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const unsigned c = __shfl_up_sync(0xFFFFFFFFu, icnt, o);
+    if (lane >= o) {
+      incl += v;
+      icnt += c;
+    }
+  }
+  const unsigned excl = incl - ui - uo;
+  S.cur[w][2 * lane] = excl * unit;
+  S.cur[w][2 * lane + 1] = (excl + ui) * unit;
+  if (MODE == kModeRead) {
+    S.rd[w][lane] = icnt - ci - co;
+  } else {
+    uint8_t* d = P.bend + r.at * P.planes * 16;
+    if (lane < P.planes * kPlaneBuckets)
+      *reinterpret_cast<uint16_t*>(d + desc_end(lane)) =
+          (uint16_t)(min(excl + ui, 255u) | min(incl, 255u) << 8);
+    if (lane < P.planes * kPlaneBuckets && lane % kPlaneBuckets == 0) {
+      const uint32_t row = (uint32_t)((r.cy - r.y0) * r.tw + (r.cx - r.x0)) * (uint32_t)P.npc + (uint32_t)r.lj;
+      *reinterpret_cast<uint32_t*>(d + desc_start(lane) - 2) = row | min(excl, 255u) << 16;
+    }
+  }
+  __syncwarp();
+  return __shfl_sync(0xFFFFFFFFu, incl, 31);
+}
+
+// Places (or reads back) one synapse per lane: part bb = 2 bucket + (0 in,
+// 1 out) or 64 for none.
+template <int PREC, int MODE>
+__device__ __forceinline__ void place(const BuildParams& P, RowSmem& S, const Row& r, int bb, int m,
+                                      uint32_t l, uint32_t wbits, long long out0) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const bool valid = bb < 64;
+  const unsigned peers = __match_any_sync(0xFFFFFFFFu, bb);
+  const unsigned rank = __popc(peers & lt);
+  const unsigned pos = S.cur[w][bb & 63] + rank;
+  unsigned dpeers = 0u, dpos = 0u;
+  if (MODE == kModeRead) {
+    dpeers = __match_any_sync(0xFFFFFFFFu, bb >> 1);
+    dpos = S.rd[w][(bb >> 1) & 31] + __popc(dpeers & lt);
+  }
+  __syncwarp();
+  if (valid) {
+    const size_t s = r.at * (size_t)P.rowcap + pos;
+    const bool out = bb & 1;
+    if (MODE == kModeFill) {
+      const uint32_t code = out ? (uint32_t)((S.dy[m] + 3) << 3 | (S.dx[m] + 3)) << 11 | l
+                                : (uint32_t)S.cls[w][m] * (uint32_t)P.npc4 + l;
+      if (PREC == SNN_EXACT_F16W) {
+        const uint32_t mag = wbits & 0x7FFFu;
+        const uint32_t half = (mag == kPadHalf ? 0u : mag) | (r.lj < P.nexc ? 0u : 0x8000u);
+        static_cast<uint32_t*>(P.syn)[s] = out ? mag << 17 | code : half << 16 | code;
+      } else {
+        // the FP32 weight, delivered as round(w * 2^16) in the input's units
+        const int32_t wfx = __float2int_rn(__fmul_rn(__uint_as_float(wbits), 65536.0f));
+        static_cast<uint2*>(P.syn)[s] = make_uint2(code, (uint32_t)wfx);
+      }
+    } else {
+      uint32_t code;
+      int32_t wfx;
+      if (PREC == SNN_EXACT_F16W) {
+        const uint32_t rec = static_cast<const uint32_t*>(P.syn)[s];
+        code = out ? rec & 0x1FFFFu : rec & 0xFFFFu;
+        const uint32_t mag = out ? rec >> 17 : rec >> 16 & 0x7FFFu;
+        const float f = __half2float(__ushort_as_half((unsigned short)mag));
+        wfx = __float2int_rn(__fmul_rn(r.lj < P.nexc ? f : -f, 65536.0f));
+      } else {
+        const uint2 rec = static_cast<const uint2*>(P.syn)[s];
+        code = rec.x;
+        wfx = (int32_t)rec.y;
+      }
+      int tx, ty;
+      uint32_t tl;
+      if (out) {
+        tx = wrap(r.cx + (int)(code >> 11 & 7u) - 3, P.W);
+        ty = wrap(r.cy + (int)(code >> 14 & 7u) - 3, P.H);
+        tl = code & 2047u;
+      } else {
+        const int k = (int)(code / (uint32_t)P.npc4);
+        ty = r.y0 + k / r.tw;
+        tx = r.x0 + k % r.tw;
+        tl = code - (uint32_t)k * (uint32_t)P.npc4;
+      }
+      const long long o = out0 + dpos;
+      P.rd_target[o] = ((long long)ty * P.W + tx) * P.npc + tl;
+      P.rd_delay[o] = P.dmin + (bb >> 1);
+      P.rd_wfx[o] = wfx;
+    }
+    if (rank == 0) S.cur[w][bb] += __popc(peers);
+    if (MODE == kModeRead && (dpeers & lt) == 0u) S.rd[w][bb >> 1] += __popc(dpeers);
+  }
+  __syncwarp();
+}
+
+// Pads every part of the row up to its end (lane b: bucket b).  An in pad
+// names the source's own word, so that pads of different rows fall on
+// different words.
+template <int PREC>
+__device__ __forceinline__ void pad_parts(const BuildParams& P, RowSmem& S, const Row& r) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t own = (uint32_t)((r.cy - r.y0) * r.tw + (r.cx - r.x0)) * (uint32_t)P.npc4 + (uint32_t)r.lj;
+  if (lane < P.ndel) {
+    const unsigned unit = (unsigned)P.unit;
+    for (int part = 0; part < 2; ++part) {
+      const unsigned at = S.cur[w][2 * lane + part];
+      const unsigned end = (at + unit - 1u) / unit * unit;
+      for (unsigned s = at; s < end; ++s) {
+        const size_t o = r.at * (size_t)P.rowcap + s;
+        if (PREC == SNN_EXACT_F16W)
+          static_cast<uint32_t*>(P.syn)[o] = part ? kPadF16 : kPadHalf << 16 | own;
+        else
+          static_cast<uint2*>(P.syn)[o] = make_uint2(part ? kPad : kPad | own, 0u);
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// Rows of the fixed law, one warp per row; MODE fill builds them, read writes
+// rows j0 .. j0 + n_rows - 1 to the rd_* arrays.
+template <int PREC, int MODE>
+__global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const BuildParams P) {
+  __shared__ RowSmem S;
+  load_offsets<false>(P, S);
   const int w = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const long long nwarps = (long long)gridDim.x * kBuildWarps;
   const uint32_t ndel = (uint32_t)P.ndel;
+  const long long rows = MODE == kModeRead ? P.n_rows : P.N;
 
-  for (long long j = (long long)blockIdx.x * kBuildWarps + w; j < P.N; j += nwarps) {
-    const int col = (int)((uint32_t)j / (uint32_t)P.npc);
-    const int lj = (int)(j - (long long)col * P.npc);
-    const int cy = col / P.W, cx = col - cy * P.W;
-    int gx, gy;
-    shard_global_col(P.sg, cx, cy, &gx, &gy);
-    const uint32_t jj = P.sg.on ? ((uint32_t)gy * (uint32_t)P.sg.GW + (uint32_t)gx) * (uint32_t)P.npc + (uint32_t)lj
-                                : (uint32_t)j;
-    const bool src_own = shard_owns_global(P.sg, P.W, P.H, gx, gy);
-    // whether synapse k (Philox block x) ends in one of the shard's columns
-    auto kept = [&](int k, const uint4& x) -> bool {
-      if (!P.sg.on) return true;
-      if (k < P.k_local) return src_own;
-      int m = 0;
-      for (int i = 0; i + 1 < P.n_off; ++i) m += (x.y >= s_thr[i]) ? 1 : 0;
-      return shard_owns_global(P.sg, P.W, P.H, wrap(gx + s_dx[m], P.sg.GW), wrap(gy + s_dy[m], P.sg.GH));
-    };
-    s_cnt[w][lane] = 0u;
+  for (long long i = (long long)blockIdx.x * kBuildWarps + w; i < rows; i += nwarps) {
+    const uint32_t j = (uint32_t)(MODE == kModeRead ? P.j0 + i : i);
+    const int c = (int)(j / (uint32_t)P.npc);
+    const Row r = open_row<false>(P, S, c, (int)(j - (uint32_t)c * (uint32_t)P.npc));
+    S.cnt[w][lane] = 0u;
+    S.cnt[w][lane + 32] = 0u;
     __syncwarp();
-    // pass 1: synapses per delay bucket
+    // pass 1: synapses per bucket part
     unsigned nkept = 0u;
     for (int k = lane; k < P.K; k += 32) {
-      const uint4 x = philox4x32_10(make_uint4(jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
-      if (kept(k, x)) {
-        atomicAdd(&s_cnt[w][below(x.z, ndel)], 1u);
+      const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
+      const int cl = S.cls[w][k < P.k_local ? kMaxOff : offset_of(P, S, x.y)];
+      if (cl != kDropped) {
+        atomicAdd(&S.cnt[w][2 * below(x.z, ndel) + (cl == kOut ? 1 : 0)], 1u);
         ++nkept;
       }
     }
-    if (P.deg != nullptr) {
+    if (MODE == kModeFill && P.deg != nullptr) {
       nkept = __reduce_add_sync(0xFFFFFFFFu, nkept);
       if (lane == 0) P.deg[j] = nkept;
     }
     __syncwarp();
-    const unsigned units = lane < P.ndel ? (s_cnt[w][lane] + (kSlotUnit - 1)) / kSlotUnit : 0u;
-    unsigned incl = units;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    P.bend[j * kBendStride + lane] = (uint8_t)(lane < P.ndel ? incl : 0u);
-    s_cur[w][lane] = (incl - units) * kSlotUnit;
-    __syncwarp();
+    open_parts<MODE>(P, S, r);
 
-    const long long row = j * (long long)P.rowcap;
-    const uint32_t* wt = P.wtab + (lj < P.nexc ? 0 : 65536);
+    const uint32_t* wt = P.wtab + (r.lj < P.nexc ? 0 : 65536);
+    const long long out0 = MODE == kModeRead ? P.rd_off[i] : 0;
     // pass 2: regenerate and place every synapse
     for (int k0 = 0; k0 < P.K; k0 += 32) {
       const int k = k0 + lane;
-      const uint4 x = philox4x32_10(make_uint4(jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
-      const bool valid = k < P.K && kept(k, x);
-      const int b = valid ? (int)below(x.z, ndel) : 63;
-      uint32_t code;  // F16W: stencil code; F32W: target neuron index
+      const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
+      int m = kMaxOff;
+      uint32_t l;
       if (k < P.k_local) {
-        uint32_t l = below(x.x, (uint32_t)(P.npc - 1));
-        l += (l >= (uint32_t)lj) ? 1u : 0u;
-        code = PREC == SNN_EXACT_F16W ? ((uint32_t)kCenterCode << 11) | l
-                                      : (uint32_t)col * (uint32_t)P.npc + l;
+        l = below(x.x, (uint32_t)(P.npc - 1));
+        l += (l >= (uint32_t)r.lj) ? 1u : 0u;
       } else {
-        int m = 0;
-        for (int i = 0; i + 1 < P.n_off; ++i) m += (x.y >= s_thr[i]) ? 1 : 0;
-        const uint32_t l = below(x.x, (uint32_t)P.npc);
-        if (PREC == SNN_EXACT_F16W) {
-          code = ((uint32_t)s_code[m] << 11) | l;
-        } else {
-          const int ty = wrap(cy + s_dy[m], P.H);
-          const int tx = wrap(cx + s_dx[m], P.W);
-          code = ((uint32_t)ty * (uint32_t)P.W + (uint32_t)tx) * (uint32_t)P.npc + l;
-        }
+        m = offset_of(P, S, x.y);
+        l = below(x.x, (uint32_t)P.npc);
       }
-      const uint32_t wbits = wt[x.w >> 16];
-      const unsigned peers = __match_any_sync(0xFFFFFFFFu, b);
-      const unsigned rank = __popc(peers & ((1u << lane) - 1u));
-      const unsigned pos = s_cur[w][b & 31] + rank;
-      __syncwarp();
-      if (valid) {
-        if (PREC == SNN_EXACT_F16W) {
-          static_cast<uint32_t*>(P.syn)[row + pos] = ((wbits & 0x7FFFu) << 17) | code;
-        } else {
-          // the FP32 weight, delivered as round(w * 2^16) in the input's units
-          const int32_t wfx = __float2int_rn(__fmul_rn(__uint_as_float(wbits), 65536.0f));
-          static_cast<uint2*>(P.syn)[row + pos] = make_uint2(code, (uint32_t)wfx);
-        }
-        if (rank == 0) s_cur[w][b] += __popc(peers);
-      }
-      __syncwarp();
+      const int cl = S.cls[w][m];
+      const int bb = k < P.K && cl != kDropped ? 2 * (int)below(x.z, ndel) + (cl == kOut ? 1 : 0) : 64;
+      place<PREC, MODE>(P, S, r, bb, m, l, MODE == kModeFill ? wt[x.w >> 16] : 0u, out0);
     }
-    // pad every bucket up to its 8-slot boundary
-    if (lane < P.ndel) {
-      const unsigned end = incl * kSlotUnit;
-      for (unsigned s = s_cur[w][lane]; s < end; ++s) {
-        if (PREC == SNN_EXACT_F16W)
-          static_cast<uint32_t*>(P.syn)[row + s] = kPadF16;
-        else
-          static_cast<uint2*>(P.syn)[row + s] = make_uint2(kPad, 0u);
-      }
-    }
-    __syncwarp();
+    if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
   }
 }
 
 // Initial state: V_i uniform in [0, theta) at 24-bit resolution from word
-// i mod 4 of Philox(i / 4, 0, INIT); calcium, refractoriness and input zero.
+// i mod 4 of Philox(i / 4, 0, INIT); calcium and refractoriness zero.
 // A shard draws with the global index i (n_per_col is a multiple of 4 there,
 // so a quad of local neurons is a quad of global ones).
 __global__ void __launch_bounds__(256) init_state_kernel(const StepParams P) {
@@ -173,7 +326,6 @@ __global__ void __launch_bounds__(256) init_state_kernel(const StepParams P) {
   v.w = __fmul_rn(P.theta, __fmul_rn(__uint2float_rn(u.w >> 8), s));
   reinterpret_cast<float4*>(P.V)[q] = v;
   reinterpret_cast<float4*>(P.C)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-  reinterpret_cast<int4*>(P.acc)[q] = make_int4(0, 0, 0, 0);
   reinterpret_cast<uchar4*>(P.R)[q] = make_uchar4(0, 0, 0, 0);
 }
 
@@ -183,153 +335,126 @@ __global__ void __launch_bounds__(256) init_state_kernel(const StepParams P) {
 // below its threshold.  The k-th kept candidate is synapse k, whose delay and
 // weight come from Philox(j, k, CONN) as under the fixed law.  One warp per
 // row; in pass it, lane e takes candidates 128 it + 4 e .. + 3, so a warp
-// scan of the lanes' kept counts ranks them.  The count pass (FILL false)
-// writes the bucket ends, the out-degree and the largest row; the fill pass
-// makes the same draws and places every synapse (warp match + popc rank, as
-// in build_rows_kernel), then pads the buckets.
-template <int PREC, bool FILL>
+// scan of the lanes' kept counts ranks them.  The count pass writes the
+// bucket ends, the out-degree and the largest row; the fill pass makes the
+// same draws and places every synapse, then pads the parts; the read pass
+// counts and then reads back.
+template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const BuildParams P) {
-  __shared__ unsigned s_cnt[kBuildWarps][32];
-  __shared__ unsigned s_cur[kBuildWarps][32];
-  __shared__ unsigned long long s_thr[kMaxOff];
-  __shared__ int s_dx[kMaxOff], s_dy[kMaxOff];
-  for (int m = threadIdx.x; m < kMaxOff; m += blockDim.x) {
-    s_thr[m] = m < P.n_poff ? P.poff_thr[m] : 0ull;
-    s_dx[m] = m < P.n_poff ? P.poff_dx[m] : 0;
-    s_dy[m] = m < P.n_poff ? P.poff_dy[m] : 0;
-  }
-  __syncthreads();
+  __shared__ RowSmem S;
+  __shared__ unsigned long long s_pthr[kMaxOff];
+  for (int m = threadIdx.x; m < kMaxOff; m += blockDim.x) s_pthr[m] = m < P.n_poff ? P.poff_thr[m] : 0ull;
+  load_offsets<true>(P, S);
   const int w = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const long long nwarps = (long long)gridDim.x * kBuildWarps;
   const uint32_t ndel = (uint32_t)P.ndel;
-  const unsigned lt_mask = (1u << lane) - 1u;
+  const long long rows = MODE == kModeRead ? P.n_rows : P.N;
 
-  for (long long j = (long long)blockIdx.x * kBuildWarps + w; j < P.N; j += nwarps) {
-    const uint32_t jj = (uint32_t)j;
-    const int col = (int)((uint32_t)j / (uint32_t)P.npc);
-    const int lj = (int)(j - (long long)col * P.npc);
-    const int cy = col / P.W, cx = col - cy * P.W;
-    const uint32_t* wt = P.wtab + (lj < P.nexc ? 0 : 65536);
-    const long long row = j * (long long)P.rowcap;
-    if (FILL)
-      s_cur[w][lane] = lane < P.ndel ? (lane ? (unsigned)P.bend[j * kBendStride + lane - 1] : 0u) * kSlotUnit : 0u;
-    else
-      s_cnt[w][lane] = 0u;
+  for (long long i = (long long)blockIdx.x * kBuildWarps + w; i < rows; i += nwarps) {
+    const uint32_t j = (uint32_t)(MODE == kModeRead ? P.j0 + i : i);
+    const int col = (int)(j / (uint32_t)P.npc);
+    const Row r = open_row<true>(P, S, col, (int)(j - (uint32_t)col * (uint32_t)P.npc));
+    const uint32_t* wt = P.wtab + (r.lj < P.nexc ? 0 : 65536);
+    const long long out0 = MODE == kModeRead ? P.rd_off[i] : 0;
+    S.cnt[w][lane] = 0u;
+    S.cnt[w][lane + 32] = 0u;
+    if (MODE == kModeFill && lane < P.ndel) {
+      const uint8_t* d = P.bend + r.at * P.planes * 16;
+      const int at = lane % kPlaneBuckets ? desc_end(lane) - 1 : desc_start(lane);
+      S.cur[w][2 * lane] = (unsigned)d[at] * (unsigned)P.unit;
+      S.cur[w][2 * lane + 1] = (unsigned)d[desc_end(lane)] * (unsigned)P.unit;
+    }
     __syncwarp();
-    unsigned k_run = 0u;
-    for (long long c0 = 0; c0 < P.n_cand; c0 += 128) {
-      const long long cb = c0 + 4 * lane;
-      const uint4 x = philox4x32_10(make_uint4(jj, (uint32_t)(cb >> 2), kTagPConn, 0u), P.seed_lo,
-                                    P.seed_hi);
-      const uint32_t words[4] = {x.x, x.y, x.z, x.w};
-      unsigned bits = 0u;
-      int lq[4], mq[4];
+    // one walk over the candidates; `placing`: place them, else count them
+    auto walk = [&](bool placing) -> unsigned {
+      unsigned k_run = 0u;
+      for (long long c0 = 0; c0 < P.n_cand; c0 += 128) {
+        const long long cb = c0 + 4 * lane;
+        const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)(cb >> 2), kTagPConn, 0u), P.seed_lo,
+                                      P.seed_hi);
+        const uint32_t words[4] = {x.x, x.y, x.z, x.w};
+        unsigned bits = 0u;
+        int lq[4], mq[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const long long c = cb + q;
-        lq[q] = 0;
-        mq[q] = -1;
-        if (c >= P.n_cand) continue;
-        unsigned long long thr;
-        if (c < P.npc - 1) {
-          thr = P.plocal_thr;
-          lq[q] = (int)c + ((int)c >= lj ? 1 : 0);
-        } else {
-          const long long r = c - (P.npc - 1);
-          const int m = (int)((uint32_t)r / (uint32_t)P.npc);
-          thr = s_thr[m];
-          mq[q] = m;
-          lq[q] = (int)(r - (long long)m * P.npc);
-        }
-        if ((unsigned long long)words[q] < thr) bits |= 1u << q;
-      }
-      const unsigned nb = (unsigned)__popc(bits);
-      unsigned incl = nb;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const unsigned kb = k_run + incl - nb;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const bool keep = (bits >> q) & 1u;
-        int b = 63;
-        uint32_t code = 0u, wbits = 0u;
-        if (keep) {
-          const unsigned k = kb + (unsigned)__popc(bits & ((1u << q) - 1u));
-          const uint4 y = philox4x32_10(make_uint4(jj, k, kTagConn, 0u), P.seed_lo, P.seed_hi);
-          b = (int)below(y.z, ndel);
-          if (FILL) wbits = wt[y.w >> 16];
-          const int m = mq[q];
-          const int dx = m < 0 ? 0 : s_dx[m], dy = m < 0 ? 0 : s_dy[m];
-          if (PREC == SNN_EXACT_F16W) {
-            code = ((uint32_t)(((dy + 3) << 3) | (dx + 3)) << 11) | (uint32_t)lq[q];
+        for (int q = 0; q < 4; ++q) {
+          const long long c = cb + q;
+          lq[q] = 0;
+          mq[q] = kMaxOff;
+          if (c >= P.n_cand) continue;
+          unsigned long long thr;
+          if (c < P.npc - 1) {
+            thr = P.plocal_thr;
+            lq[q] = (int)c + ((int)c >= r.lj ? 1 : 0);
           } else {
-            const int ty = wrap(cy + dy, P.H), tx = wrap(cx + dx, P.W);
-            code = ((uint32_t)ty * (uint32_t)P.W + (uint32_t)tx) * (uint32_t)P.npc + (uint32_t)lq[q];
+            const long long rr = c - (P.npc - 1);
+            const int m = (int)((uint32_t)rr / (uint32_t)P.npc);
+            thr = s_pthr[m];
+            mq[q] = m;
+            lq[q] = (int)(rr - (long long)m * P.npc);
           }
+          if ((unsigned long long)words[q] < thr) bits |= 1u << q;
         }
-        if (!FILL) {
-          if (keep) atomicAdd(&s_cnt[w][b], 1u);
-        } else {
-          const unsigned peers = __match_any_sync(0xFFFFFFFFu, b);
-          const unsigned rank = __popc(peers & lt_mask);
-          const unsigned pos = s_cur[w][b & 31] + rank;
-          __syncwarp();
-          if (keep) {
-            if (PREC == SNN_EXACT_F16W) {
-              static_cast<uint32_t*>(P.syn)[row + pos] = ((wbits & 0x7FFFu) << 17) | code;
-            } else {
-              const int32_t wfx = __float2int_rn(__fmul_rn(__uint_as_float(wbits), 65536.0f));
-              static_cast<uint2*>(P.syn)[row + pos] = make_uint2(code, (uint32_t)wfx);
-            }
-            if (rank == 0) s_cur[w][b] += __popc(peers);
-          }
-          __syncwarp();
-        }
-      }
-      k_run += __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-    __syncwarp();
-    if (!FILL) {
-      const unsigned units = lane < P.ndel ? (s_cnt[w][lane] + (kSlotUnit - 1)) / kSlotUnit : 0u;
-      unsigned incl = units;
+        const unsigned nb = (unsigned)__popc(bits);
+        unsigned incl = nb;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= o) incl += v;
+        }
+        const unsigned kb = k_run + incl - nb;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          int bb = 64;
+          uint32_t wbits = 0u;
+          if ((bits >> q) & 1u) {
+            const unsigned k = kb + (unsigned)__popc(bits & ((1u << q) - 1u));
+            const uint4 y = philox4x32_10(make_uint4(r.jj, k, kTagConn, 0u), P.seed_lo, P.seed_hi);
+            bb = 2 * (int)below(y.z, ndel) + (S.cls[w][mq[q]] == kOut ? 1 : 0);
+            if (MODE == kModeFill) wbits = wt[y.w >> 16];
+          }
+          if (!placing) {
+            if (bb < 64) atomicAdd(&S.cnt[w][bb], 1u);
+          } else {
+            place<PREC, MODE>(P, S, r, bb, mq[q], (uint32_t)lq[q], wbits, out0);
+          }
+        }
+        k_run += __shfl_sync(0xFFFFFFFFu, incl, 31);
       }
-      P.bend[j * kBendStride + lane] = (uint8_t)(lane < P.ndel ? (incl < 255u ? incl : 255u) : 0u);
-      if (lane == 31) atomicMax(P.max_units, incl);
-      if (lane == 0) P.deg[j] = k_run;
-    } else if (lane < P.ndel) {
-      const unsigned end = (unsigned)P.bend[j * kBendStride + lane] * kSlotUnit;
-      for (unsigned s = s_cur[w][lane]; s < end; ++s) {
-        if (PREC == SNN_EXACT_F16W)
-          static_cast<uint32_t*>(P.syn)[row + s] = kPadF16;
-        else
-          static_cast<uint2*>(P.syn)[row + s] = make_uint2(kPad, 0u);
+      __syncwarp();
+      return k_run;
+    };
+    if (MODE != kModeFill) {
+      const unsigned deg = walk(false);
+      const unsigned units = open_parts<MODE>(P, S, r);
+      if (MODE == kModeCount) {
+        unsigned u8 = lane < P.ndel ? (S.cnt[w][2 * lane] + S.cnt[w][2 * lane + 1] + 7u) / 8u : 0u;
+        u8 = __reduce_add_sync(0xFFFFFFFFu, u8);
+        if (lane == 0) {
+          atomicMax(P.max_units, units);
+          atomicMax(P.max_units + 1, u8);
+          P.deg[j] = deg;
+        }
       }
     }
-    __syncwarp();
+    if (MODE != kModeCount) walk(true);
+    if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
   }
 }
 
 }  // namespace
 
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st) {
-  paper_rows_kernel<SNN_EXACT_F32W, false><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
+  paper_rows_kernel<SNN_EXACT_F32W, kModeCount><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
   return cudaGetLastError();
 }
 
 cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
                               cudaStream_t st) {
   if (precision == SNN_EXACT_F16W)
-    paper_rows_kernel<SNN_EXACT_F16W, true><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
+    paper_rows_kernel<SNN_EXACT_F16W, kModeFill><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
   else
-    paper_rows_kernel<SNN_EXACT_F32W, true><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
+    paper_rows_kernel<SNN_EXACT_F32W, kModeFill><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
   return cudaGetLastError();
 }
 
@@ -337,9 +462,23 @@ cudaError_t launch_build(const BuildParams& bp, int precision, int num_sms,
                          cudaStream_t st) {
   const int grid = num_sms * 8;
   if (precision == SNN_EXACT_F16W)
-    build_rows_kernel<SNN_EXACT_F16W><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+    build_rows_kernel<SNN_EXACT_F16W, kModeFill><<<grid, kBuildWarps * 32, 0, st>>>(bp);
   else
-    build_rows_kernel<SNN_EXACT_F32W><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+    build_rows_kernel<SNN_EXACT_F32W, kModeFill><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_read_rows(const BuildParams& bp, int precision, bool paper, cudaStream_t st) {
+  const unsigned grid = (unsigned)((bp.n_rows + kBuildWarps - 1) / kBuildWarps);
+  const bool f16 = precision == SNN_EXACT_F16W;
+  if (paper && f16)
+    paper_rows_kernel<SNN_EXACT_F16W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+  else if (paper)
+    paper_rows_kernel<SNN_EXACT_F32W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+  else if (f16)
+    build_rows_kernel<SNN_EXACT_F16W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+  else
+    build_rows_kernel<SNN_EXACT_F32W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
   return cudaGetLastError();
 }
 

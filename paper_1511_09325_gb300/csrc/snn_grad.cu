@@ -3,7 +3,7 @@
 //
 // The paper simulates the spiking network only.  This file adds the standard
 // surrogate-gradient treatment of the same recursion, on the same synapse
-// table (F32W records: target index, fixed-point weight):
+// table (F32W records: target code, fixed-point weight):
 //
 //   X_E,i(t), X_I,i(t): sums of w s_j(t - d) over excitatory / inhibitory sources
 //   I_i = a[E][p_i] X_E,i + a[I][p_i] X_I,i + J (lam + sqrt(lam) xi_i(t))
@@ -56,8 +56,11 @@ constexpr float kTwoM16 = 1.52587890625e-05f;       // 2^-16
 constexpr float kTwoM24 = 5.9604644775390625e-08f;  // 2^-24
 
 struct GradParams {
-  long long N;
-  int npc, nexc, dmin, ndel, nslot, rowcap, hard, T;
+  long long N, accw;          // neurons; words of an array in acc order
+  int npc, npc4, nexc, dmin, ndel, nslot, rowcap, unit, planes, hard, T;
+  const uint32_t* ctile;      // geometry of the net (see snn_internal.h)
+  const uint32_t* colv;
+  const uint32_t* nbg;
   uint32_t seed_lo, seed_hi;
   float beta, theta, vr, dc, pvv, pcc, pvc_e, pvc_i, kappa, J, lam, sqlam;
   float a[4];  // a_EE, a_EI, a_IE, a_II
@@ -68,14 +71,14 @@ struct GradParams {
   float* V;
   float* C;
   float* shist;               // [nslot][N] s of the last nslot steps
-  unsigned long long* xe;     // [N] input sums from E sources, 2^-32 mV
-  unsigned long long* xin;    // [N] the same from I sources
+  unsigned long long* xe;     // [accw] input sums from E sources, 2^-32 mV, acc order
+  unsigned long long* xin;    // [accw] the same from I sources
   float* tape;                // [ckpt][kTape][N]
   double* rate_part;          // [update blocks][2]
   float* vbar;
   float* cbar;
-  float* ibe;                 // [nslot][N] a[E][p_i] * adjoint of I_i(t)
-  float* ibi;                 // [nslot][N] a[I][p_i] * adjoint of I_i(t)
+  float* ibe;                 // [nslot][accw] a[E][p_i] * adjoint of I_i(t), acc order
+  float* ibi;                 // [nslot][accw] a[I][p_i] * adjoint of I_i(t)
   float* gb;                  // [3][N] -adjoint of g_i(t) where the gate is open
   float* sg;                  // [N] gathered adjoint of s_j(t) through its synapses
   double* gacc;               // [6][N] parameter partials per neuron
@@ -103,6 +106,39 @@ __global__ void __launch_bounds__(kThreads) grad_init_kernel(const GradParams P)
   const uint32_t u = (i & 3) == 0 ? x.x : (i & 3) == 1 ? x.y : (i & 3) == 2 ? x.z : x.w;
   P.V[i] = __fmul_rn(P.theta, __fmul_rn(__uint2float_rn(u >> 8), kTwoM24));
   P.C[i] = 0.f;
+}
+
+// Word of neuron i in arrays in acc order.
+__device__ __forceinline__ long long acc_word(const GradParams& P, long long i) {
+  const uint32_t c = (uint32_t)i / (uint32_t)P.npc;
+  return (long long)P.colv[c] * P.npc4 + ((uint32_t)i - c * (uint32_t)P.npc);
+}
+
+// A source row: its records, and where its records' targets lie: in parts
+// from word `tile` on, out parts through the row `nb` of the neighbour table.
+struct GradRow {
+  const uint2* rec;
+  const uint8_t* ends;
+  const uint32_t* nb;
+  uint32_t tile;
+  bool exc;
+};
+__device__ __forceinline__ GradRow grad_row(const GradParams& P, long long j) {
+  const uint32_t c = (uint32_t)j / (uint32_t)P.npc;
+  const uint32_t l = (uint32_t)j - c * (uint32_t)P.npc;
+  const uint32_t v = P.colv[c];
+  const size_t at = (size_t)v * P.npc + l;
+  GradRow r;
+  r.rec = P.syn + at * (size_t)P.rowcap;
+  r.ends = P.bend + at * (size_t)(P.planes * 16);
+  r.nb = P.nbg + (size_t)v * 64;
+  r.tile = (v - (P.ctile[c] & 63u)) * (uint32_t)P.npc4;
+  r.exc = (int)l < P.nexc;
+  return r;
+}
+// Word of the target of a record with code `code` of an in or out part.
+__device__ __forceinline__ uint32_t target_word(const GradRow& r, bool in, uint32_t code) {
+  return in ? r.tile + code : __ldg(r.nb + ((code >> 11) & 63u)) + (code & 2047u);
 }
 
 // Bucket ends (slots) in lanes 0..ndel-1 of the warp; the bucket holding
@@ -133,21 +169,26 @@ __global__ void __launch_bounds__(kThreads) grad_deliver_kernel(const GradParams
   const int lane = threadIdx.x & 31;
   if (j >= P.N) return;
   float s_lane = 0.f;
-  int end_lane = 0x7FFFFFFF;
+  int end_lane = 0x7FFFFFFF, mid_lane = 0;
   if (lane < P.ndel) {
     const long long src = t - (P.dmin + lane);
     s_lane = src >= 0 ? P.shist[ring(src, P.nslot) * P.N + j] : 0.f;
-    end_lane = (int)P.bend[j * kBendStride + lane] * kSlotUnit;
   }
   if (__ballot_sync(0xFFFFFFFFu, s_lane != 0.f) == 0u) return;
-  const bool exc = (int)((uint32_t)j % (uint32_t)P.npc) < P.nexc;
-  unsigned long long* acc = exc ? P.xe : P.xin;
+  const GradRow R = grad_row(P, j);
+  if (lane < P.ndel) {
+    const uint32_t e = *reinterpret_cast<const uint16_t*>(R.ends + desc_end(lane));
+    mid_lane = (int)(e & 0xFFu) * P.unit;
+    end_lane = (int)(e >> 8) * P.unit;
+  }
+  unsigned long long* acc = R.exc ? P.xe : P.xin;
   const int row_end = __shfl_sync(0xFFFFFFFFu, end_lane, P.ndel - 1);
-  const uint2* row = P.syn + j * (long long)P.rowcap;
+  const uint2* row = R.rec;
   for (int k0 = 0; k0 < row_end; k0 += 128) {
     const int k = k0 + 4 * lane;
     const int b = bucket_of(k, end_lane, P.ndel);
     const float s = __shfl_sync(0xFFFFFFFFu, s_lane, b);
+    const bool in = k < __shfl_sync(0xFFFFFFFFu, mid_lane, b);
     if (k < row_end && s != 0.f) {
       const uint4 r01 = __ldcs(reinterpret_cast<const uint4*>(row + k));
       const uint4 r23 = __ldcs(reinterpret_cast<const uint4*>(row + k + 2));
@@ -155,11 +196,11 @@ __global__ void __launch_bounds__(kThreads) grad_deliver_kernel(const GradParams
       const uint32_t wf[4] = {r01.y, r01.w, r23.y, r23.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        if (tg[q] == kPad) continue;
+        if (tg[q] & kPad) continue;
         const int32_t wfx = (int32_t)wf[q];
         const long long v = P.hard ? (long long)wfx * 65536ll
                                    : __float2ll_rn(__fmul_rn(__fmul_rn(s, (float)wfx), 65536.f));
-        atomicAdd(acc + tg[q], (unsigned long long)v);
+        atomicAdd(acc + target_word(R, in, tg[q]), (unsigned long long)v);
       }
     }
   }
@@ -175,10 +216,11 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
   float s = 0.f;
   bool exc = false;
   if (i < P.N) {
-    const float XE = __fmul_rn(__ll2float_rn((long long)P.xe[i]), kTwoM32);
-    const float XI = __fmul_rn(__ll2float_rn((long long)P.xin[i]), kTwoM32);
-    P.xe[i] = 0ull;
-    P.xin[i] = 0ull;
+    const long long iw = acc_word(P, i);
+    const float XE = __fmul_rn(__ll2float_rn((long long)P.xe[iw]), kTwoM32);
+    const float XI = __fmul_rn(__ll2float_rn((long long)P.xin[iw]), kTwoM32);
+    P.xe[iw] = 0ull;
+    P.xin[iw] = 0ull;
     exc = (int)((uint32_t)i % (uint32_t)P.npc) < P.nexc;
     const float xi = normal_draw(P, i, t);
     const float e = __fmul_rn(P.J, __fadd_rn(P.lam, __fmul_rn(P.sqlam, xi)));
@@ -247,23 +289,26 @@ __global__ void __launch_bounds__(kThreads) grad_gather_kernel(const GradParams 
   const long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (j >= P.N) return;
-  const bool exc = (int)((uint32_t)j % (uint32_t)P.npc) < P.nexc;
-  const float* ib = exc ? P.ibe : P.ibi;
+  const GradRow R = grad_row(P, j);
+  const float* ib = R.exc ? P.ibe : P.ibi;
   long long off_lane = -1;  // ring offset of bucket `lane`'s step, -1 beyond T
-  int end_lane = 0x7FFFFFFF;
+  int end_lane = 0x7FFFFFFF, mid_lane = 0;
   if (lane < P.ndel) {
     const long long dst = tau + P.dmin + lane;
-    off_lane = dst < P.T ? ring(dst, P.nslot) * P.N : -1;
-    end_lane = (int)P.bend[j * kBendStride + lane] * kSlotUnit;
+    off_lane = dst < P.T ? ring(dst, P.nslot) * P.accw : -1;
+    const uint32_t e = *reinterpret_cast<const uint16_t*>(R.ends + desc_end(lane));
+    mid_lane = (int)(e & 0xFFu) * P.unit;
+    end_lane = (int)(e >> 8) * P.unit;
   }
   const int row_end = __shfl_sync(0xFFFFFFFFu, end_lane, P.ndel - 1);
-  const uint2* row = P.syn + j * (long long)P.rowcap;
+  const uint2* row = R.rec;
   float acc = 0.f;
 #pragma unroll 2
   for (int k0 = 0; k0 < row_end; k0 += 128) {
     const int k = k0 + 4 * lane;
     const int b = bucket_of(k, end_lane, P.ndel);
     const long long off = __shfl_sync(0xFFFFFFFFu, off_lane, b);
+    const bool in = k < __shfl_sync(0xFFFFFFFFu, mid_lane, b);
     if (k < row_end && off >= 0) {
       const uint4 r01 = __ldcs(reinterpret_cast<const uint4*>(row + k));
       const uint4 r23 = __ldcs(reinterpret_cast<const uint4*>(row + k + 2));
@@ -272,7 +317,7 @@ __global__ void __launch_bounds__(kThreads) grad_gather_kernel(const GradParams 
       const uint32_t wf[4] = {r01.y, r01.w, r23.y, r23.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (tg[q] != kPad) acc = __fmaf_rn((float)(int32_t)wf[q], ibs[tg[q]], acc);
+        if (!(tg[q] & kPad)) acc = __fmaf_rn((float)(int32_t)wf[q], ibs[target_word(R, in, tg[q])], acc);
     }
   }
 #pragma unroll
@@ -318,8 +363,9 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   P.gb[ring(tau, 3) * P.N + i] = g > 0.f ? -ubar * (V + I - P.vr) : 0.f;
   const float aE = exc ? P.a[0] : P.a[1];
   const float aI = exc ? P.a[2] : P.a[3];
-  P.ibe[ring(tau, P.nslot) * P.N + i] = aE * ib;
-  P.ibi[ring(tau, P.nslot) * P.N + i] = aI * ib;
+  const long long iw = ring(tau, P.nslot) * P.accw + acc_word(P, i);
+  P.ibe[iw] = aE * ib;
+  P.ibi[iw] = aI * ib;
   // I = a[E][p] X_E + a[I][p] X_I + J (lam + sqrt(lam) xi),  h = 1 ms
   ga[(exc ? 0 : 1) * P.N] += (double)ib * (double)XE;
   ga[(exc ? 2 : 3) * P.N] += (double)ib * (double)XI;
@@ -428,7 +474,14 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
 
   GradParams& P = g->P;
   P.N = N;
+  P.accw = v.acc_words;
   P.npc = v.npc;
+  P.npc4 = v.npc4;
+  P.unit = v.unit;
+  P.planes = v.planes;
+  P.ctile = v.ctile;
+  P.colv = v.colv;
+  P.nbg = v.nbg;
   P.nexc = v.nexc;
   P.dmin = v.dmin;
   P.ndel = v.ndel;
@@ -450,19 +503,19 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   P.bend = v.bend;
 
   int rc = SNN_OK;
-  const size_t n = (size_t)N;
+  const size_t n = (size_t)N, accw = (size_t)v.acc_words;
   if (!rc) rc = galloc(g, &g->q, 65536);
   if (!rc) rc = galloc(g, &P.V, n);
   if (!rc) rc = galloc(g, &P.C, n);
   if (!rc) rc = galloc(g, &P.shist, n * g->nslot);
-  if (!rc) rc = galloc(g, &P.xe, n);
-  if (!rc) rc = galloc(g, &P.xin, n);
+  if (!rc) rc = galloc(g, &P.xe, accw);
+  if (!rc) rc = galloc(g, &P.xin, accw);
   if (!rc) rc = galloc(g, &P.tape, n * kTape * g->ckpt);
   if (!rc) rc = galloc(g, &P.rate_part, (size_t)g->ublocks * 2);
   if (!rc) rc = galloc(g, &P.vbar, n);
   if (!rc) rc = galloc(g, &P.cbar, n);
-  if (!rc) rc = galloc(g, &P.ibe, n * g->nslot);
-  if (!rc) rc = galloc(g, &P.ibi, n * g->nslot);
+  if (!rc) rc = galloc(g, &P.ibe, accw * g->nslot);
+  if (!rc) rc = galloc(g, &P.ibi, accw * g->nslot);
   if (!rc) rc = galloc(g, &P.gb, n * 3);
   if (!rc) rc = galloc(g, &P.sg, n);
   if (!rc) rc = galloc(g, &P.gacc, n * 6);
@@ -502,15 +555,15 @@ int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, 
   P.sqlam = (float)std::sqrt(lam);
   cudaStream_t st = g->v.stream;
   const long long N = g->v.N;
-  const size_t n = (size_t)N;
+  const size_t n = (size_t)N, accw = (size_t)g->v.acc_words;
   const size_t ckw = n * (2 + g->nslot);  // floats per checkpoint
 
   // forward, saving a checkpoint at the start of every segment
   grad_init_kernel<<<g->ublocks, kThreads, 0, st>>>(P);
   SNN_GCUDA(g, cudaGetLastError());
   SNN_GCUDA(g, cudaMemsetAsync(P.shist, 0, n * g->nslot * 4, st));
-  SNN_GCUDA(g, cudaMemsetAsync(P.xe, 0, n * 8, st));
-  SNN_GCUDA(g, cudaMemsetAsync(P.xin, 0, n * 8, st));
+  SNN_GCUDA(g, cudaMemsetAsync(P.xe, 0, accw * 8, st));
+  SNN_GCUDA(g, cudaMemsetAsync(P.xin, 0, accw * 8, st));
   SNN_GCUDA(g, cudaMemsetAsync(P.rate_part, 0, (size_t)g->ublocks * 16, st));
   for (long long t = 0; t < g->T; ++t) {
     if (t % g->ckpt == 0) {
@@ -546,8 +599,8 @@ int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, 
   P.dlds_i = NI > 0 ? (float)(2.0 * (rI - g->targets[1]) * 1000.0 / ((double)g->T * NI)) : 0.f;
   SNN_GCUDA(g, cudaMemsetAsync(P.vbar, 0, n * 4, st));
   SNN_GCUDA(g, cudaMemsetAsync(P.cbar, 0, n * 4, st));
-  SNN_GCUDA(g, cudaMemsetAsync(P.ibe, 0, n * g->nslot * 4, st));
-  SNN_GCUDA(g, cudaMemsetAsync(P.ibi, 0, n * g->nslot * 4, st));
+  SNN_GCUDA(g, cudaMemsetAsync(P.ibe, 0, accw * g->nslot * 4, st));
+  SNN_GCUDA(g, cudaMemsetAsync(P.ibi, 0, accw * g->nslot * 4, st));
   SNN_GCUDA(g, cudaMemsetAsync(P.gb, 0, n * 3 * 4, st));
   SNN_GCUDA(g, cudaMemsetAsync(P.gacc, 0, n * 6 * 8, st));
   for (int seg = g->nseg - 1; seg >= 0; --seg) {

@@ -1,41 +1,48 @@
 // snn_internal.h -- types shared by the translation units of the library.
 //
-// Device data layout of one net (all arrays are library-owned, 256 B aligned):
-//   syn    outgoing-synapse table, row j at j * rowcap slots.  A row holds the
-//          neuron's k_out synapses grouped by delay bucket b = d - d_min; every
-//          bucket starts on a multiple of 8 slots and is padded with PAD
-//          records up to the next multiple of 8 (so a bucket is a whole number
-//          of 32 B sectors in the F16W layout).
-//            F16W: u32 record  = half_magnitude(15) << 17 | code(17)
-//            F32W: u32x2 record = { target neuron index, int32 round(w * 2^16) }
-//          padding records have weight 0 (kPadF16 / {kPad, 0}).
-//          (w the FP32 weight in mV, so the record holds exactly what is added)
-//          code = ((dy + 3) << 3 | (dx + 3)) << 11 | l  (stencil offset of the
-//          target column and index l inside it; local synapses use dx=dy=0).
-//          The weight's sign is the source population's (Dale's principle),
-//          so the F16W record drops the half's sign bit without loss.
-//   bend   u8[N][32]: bend[j][b] = end of bucket b of row j in units of 8 slots.
+// Device data layout of one net (all arrays are library-owned, 256 B aligned).
+// The grid is covered by delivery tiles of tw x th columns; a column's
+// virtual index v counts the columns tile by tile (tiles in row-major order,
+// row-major inside a tile), so the columns of a tile are consecutive and the
+// k-th column of a tile is v = first + k.
+//   syn    outgoing-synapse table.  Row of neuron l of virtual column v at
+//          (v * npc + l) * rowcap slots.  A row holds the neuron's synapses
+//          grouped by delay bucket b = d - d_min; a bucket holds the synapses
+//          that end in the source's own tile ("in"), then the others ("out"),
+//          each part padded to whole units of 8 slots (16 where a row would
+//          exceed 255 units of 8).
+//            in, F16W:  u32 = half(16, signed) << 16 | code(16)
+//            in, F32W:  { code, int32 round(w * 2^16) }
+//              code = k * npc4 + l: word of the target in its tile's window
+//              (k the target column's place in the tile)
+//            out, F16W: u32 = half_magnitude(15) << 17 | off(6) << 11 | l(11)
+//            out, F32W: { off << 11 | l, int32 round(w * 2^16) }
+//              off = (dy + 3) << 3 | (dx + 3): stencil offset of the target
+//              column; F16W: the sign is the source population's (Dale)
+//          padding records deliver 0 (kPadHalf / kPadF16 / kPad).
+//   bend   [ncol * npc][planes] of 16 bytes, rows in the order of syn: a
+//          spiker's descriptor.  Plane p covers buckets 6p .. 6p + 5: bytes 0-1
+//          the neuron's row in its tile (k * npc + l), byte 2 the start of
+//          bucket 6p, bytes 4 + 2i and 5 + 2i the ends of the in and out parts
+//          of bucket 6p + i, in units.
 //   V, C   float[Npad] membrane potential (mV) and calcium.
 //   R      u8[Npad] remaining refractory steps.
-//   acc    int32[Npad] recurrent input of the next step, 2^-16 mV units.
-//   desc   spike descriptors of the last d_max + 1 steps (slot t % (d_max +
-//          1)), desc_words u32 each: the spiker's id, then its bucket ends
-//          (bend[j][0 .. ndel - 1], one byte each).  The spikes of column c
-//          at step t are entries [slot][c * n_per_col + r], r < ccnt[slot][c],
-//          in no fixed order.
-//   ccnt   u32[d_max + 1][ncol] spikes of each slot's step per column.
-//   vcol, colv  u32[ncol] delivery order of the columns: virtual column v is
-//          real column vcol[v]; colv is the inverse.  Columns are numbered
-//          tile by tile (tiles of `tile` x `tile` columns in row-major order,
-//          row-major inside a tile), so a run of virtual columns is a compact
-//          patch of the grid.
-//   isum   u32[ncol] (bucket, spiker) items of each virtual column over the
-//          steps that the next delivery reads (the sum of its d_max - d_min +
-//          1 slots).
-//   gsum   u32[ceil(ncol / 32)] isum summed over groups of 32 virtual columns.
-//   cnt    u32[d_max + 1] spikes of each slot's step.
-//   ctl    control block (step counter, completion counter, overflow flag,
-//          status).
+//   acc    int32[ncol * npc4] recurrent input of the next step, 2^-16 mV
+//          units; neuron l of virtual column v at v * npc4 + l (npc4 = npc
+//          rounded up to 4), so a tile's input is one run of words.
+//   list   [d_max + 1][planes][ntile][tcap] of 16 bytes: descriptors of the
+//          spikes of the last d_max + 1 steps (slot t % (d_max + 1)) per tile,
+//          in no fixed order; ccnt[slot][tile] of them (one counter per 32
+//          bytes).  The items of a bucket read one plane of one list in order.
+//   isum   u32[ntile] (bucket, spiker) items of each tile over the steps that
+//          the delivery of step t reads, less step t itself (one counter per 32
+//          bytes); gsum: their sum.
+//   ctile  u32[ncol] tile << 6 | k of each real column; colv: its virtual index.
+//   tinfo  {first virtual column, columns} of each tile.
+//   nbg    u32[ncol][64] first word in acc of the column at each stencil offset
+//          of each virtual column.
+//   cnt    u32 spikes of the step (compact-list form only).
+//   ctl    control block (step counters, overflow flag, status).
 //   rec    u64 spike records (step << 32 | id), one region per update block,
 //          rcnt[b] records in region b since the last drain.
 //   colcnt u64[ncol][2] spike counts per column and population.
@@ -59,25 +66,35 @@ constexpr uint32_t kTagInit = 3u;
 constexpr uint32_t kTagSurr = 4u;  // normal draws of the differentiable form
 constexpr uint32_t kTagPConn = 5u; // candidate draws of the paper connectivity law
 constexpr int kMaxDelays = 32;   // d_max <= 32
-constexpr int kBendStride = 32;  // bytes of bucket ends per neuron
-constexpr int kSlotUnit = 8;     // buckets are padded to 8 synapse slots
+constexpr int kPlaneBuckets = 6; // buckets that a 16-byte plane of a descriptor covers
+constexpr int kSlotUnit = 8;     // bucket parts are padded to 8 (or 16) synapse slots
 constexpr int kMaxPoisThr = 127; // Poisson thresholds below 2^32
 constexpr int kMaxOff = 48;      // remote stencil offsets (radius <= 3)
-constexpr uint32_t kPad = 0xFFFFFFFFu;  // target of an F32W padding record (weight 0)
-// F16W padding record: weight magnitude 0 and stencil field dx + 3 = 7, which
-// no synapse uses (|dx| <= 3).
+// Padding records.  F32W: bit 31 of the code set, weight 0.  F16W: an in
+// record of the half 2^-24, which rounds to 0 input units (a synapse of that
+// weight is stored as the half 0 instead), or an out record of weight 0 and
+// stencil field dx + 3 = 7, which no synapse uses (|dx| <= 3).
+constexpr uint32_t kPad = 0x80000000u;
+constexpr uint32_t kPadHalf = 1u;
 constexpr uint32_t kPadF16 = 7u << 11;
-__host__ __device__ constexpr bool is_pad_f16(uint32_t rec) { return ((rec >> 11) & 7u) == 7u; }
 constexpr int kCenterCode = (3 << 3) | 3;
 constexpr int kMaxGridSide = 16383;     // columns per grid side (14-bit coordinates)
 constexpr int kMaxTile = 8;             // delivery tile side, columns
 constexpr int kMaxTileCols = kMaxTile * kMaxTile;
-constexpr unsigned kWinMinItems = 512;  // default fewest items of a windowed tile part
-// Fixed costs, in items, that the delivery's range split adds to a group of
-// 32 columns with at least kWinMinItems items (window set-up and flush) and
-// to one with fewer but some items (table set-up).
-constexpr unsigned kCostWin = 1024;
-constexpr unsigned kCostPart = 256;
+constexpr int kCntStride = 8;           // words from one tile counter to the next
+// Words of a tile's window per item of the fewest that make a part use the
+// window, and per item of its fixed cost in the range split (set-up and
+// flush); the fixed cost, in items, of a tile with fewer but some items.
+// Without a window each of an item's ~62 synapses is an L2 reduction (about
+// 1.3 per ns and SM), with one the window's words are cleared and added once
+// (about 7.5 words per ns and SM).  Measured (us per delivery, mean state): a
+// window from 1 item per 87, 175 and 350 words on gives 18.9, 18.2 and 18.1 at
+// 8x8 FP16, 45.1, 43.4 and 43.5 at 24x24 FP16, the same at 96x96; a cost of 1
+// item per 30, 44 and 88 words gives 44.4, 43.4 and 43.2 at 24x24 FP16, and
+// 368, 365 and 372 at 96x96.
+constexpr int kWinWordsPerItem = 250;
+constexpr int kCostWordsPerItem = 60;
+constexpr unsigned kCostPart = 32;
 
 // Tables computed on the host in FP64 and rounded once.
 struct HostTables {
@@ -109,9 +126,9 @@ const std::vector<double>& quantile_table();
 
 // Device control block.
 struct Ctl {
-  long long t;                  // step index of the next update
+  long long t;                  // step index of the next update (set by the delivery)
+  long long td;                 // step index of the next delivery (set by the update)
   unsigned int drained;         // blocks done with the current record drain
-  unsigned int done;            // delivery blocks finished this step
   unsigned int rec_overflow;    // set when a record did not fit its region
   unsigned int status;          // nonzero: a delivery found inconsistent counts
 };
@@ -158,17 +175,17 @@ __host__ __device__ inline bool shard_owns_global(const ShardGeo& g, int W, int 
 // Everything a step kernel needs, passed by value (constant bank).
 struct StepParams {
   long long N;
-  int npc, nexc, W, H, K, dmin, ndel, nslot, rowcap;
-  int ncol;
-  int agg;  // shared-memory windows over each delivery tile and its ring
-  int tile, ring;          // delivery tile side and window ring, in columns
-  int part_cols;           // most columns of a delivery part without window (>= tile^2)
-  int win_cap;             // ints of the window (largest tile window)
-  int desc_words;          // u32 words per spike descriptor (8 or 16)
+  int npc, npc4, nexc, W, H, K, dmin, ndel, nslot;
+  int ncol, ntile;
+  int tcap;                // list entries per slot and tile
+  int tcols;               // columns of the largest tile
+  int planes;              // 16-byte planes of a spike descriptor
+  int row_sec, unit_sec;   // 32-byte sectors of a row and of a bucket unit
+  int agg;                 // shared-memory windows over the delivery tiles
   unsigned min_items;      // fewest items a delivery block takes (fewer blocks run)
-  unsigned win_items;      // fewest items of a tile part that uses the window
-  unsigned cost_win, cost_part;  // fixed cost (in items) of a windowed / other group
-  uint32_t npc_m, w_m;     // floor(2^32 / n_per_col), floor(2^32 / W) (capped)
+  unsigned win_items;      // fewest items of a part that uses the window
+  unsigned cost_win, cost_part;  // fixed cost (in items) of a windowed / other tile
+  uint32_t npc_m;          // floor(2^32 / n_per_col) (capped)
   uint32_t seed_lo, seed_hi;
   float theta, vr, dc, pvv, pcc, pvc_e, pvc_i;
   int32_t jx;
@@ -180,16 +197,19 @@ struct StepParams {
   float* C;
   uint8_t* R;
   int32_t* acc;
-  uint32_t* ids;   // compact spike-id list (no descriptors: noalloc form only)
-  uint32_t* desc;  // spike descriptors (see above); null: write ids instead
-  const uint32_t* vcol;
-  const uint32_t* colv;
+  uint32_t* ids;   // compact spike-id list (noalloc form only)
+  uint4* list;     // spike lists per slot, plane and tile (with ccnt)
+  const uint32_t* ctile;
+  const uint32_t* colv;   // null: acc is indexed by the real neuron index
+  const uint2* tinfo;
+  const uint32_t* nbg;
   unsigned* hstatus;  // mapped host copy of Ctl::status (may be null)
   unsigned* cnt;
-  unsigned* ccnt;  // per-column counts (column-indexed lists); null: one compact list
-  unsigned* isum;  // per-column items of the delivery window (with ccnt)
-  unsigned* gsum;  // isum per group of 32 columns
-  const uint8_t* bend;
+  unsigned* ccnt;  // list lengths per slot and tile; null: one compact list
+  unsigned* isum;  // items per tile of the delivery window (with ccnt)
+  unsigned* gsum;  // their sum
+  unsigned* icnt;  // shard: halo spikes of each column listed this step
+  const uint4* bend;
   const void* syn;
   Ctl* ctl;
   unsigned long long* rec;
@@ -218,11 +238,15 @@ struct BatchParams {
 
 struct BuildParams {
   long long N;
-  int npc, nexc, W, H, K, k_local, dmin, ndel, rowcap, n_off;
+  int npc, npc4, nexc, W, H, K, k_local, dmin, ndel, rowcap, n_off;
+  int tw, th;             // delivery tile, columns
+  int unit;               // slots per bucket unit (8 or 16)
+  int planes;
   uint32_t seed_lo, seed_hi;
   uint32_t stencil_thr[kMaxOff];
   int8_t off_dx[kMaxOff], off_dy[kMaxOff];
   const uint32_t* wtab;
+  const uint32_t* colv;
   void* syn;
   uint8_t* bend;
   // paper connectivity law
@@ -232,21 +256,45 @@ struct BuildParams {
   unsigned long long plocal_thr;
   int8_t poff_dx[kMaxOff], poff_dy[kMaxOff];
   uint32_t* deg;          // [N] out-degree of each neuron
-  unsigned* max_units;    // largest row, in units of 8 slots
+  // [0] the largest row, in units; [1] the largest row in units of 8 slots
+  // with one part per bucket (the size limit of the paper law)
+  unsigned* max_units;
   ShardGeo sg;            // shard geometry (sg.on = 0: a whole network)
+  // readback: rows j0 .. j0 + n_rows - 1, row r's synapses from entry rd_off[r]
+  long long j0, n_rows;
+  const long long* rd_off;
+  long long* rd_target;
+  int32_t* rd_delay;
+  int32_t* rd_wfx;
 };
+
+// Byte of a descriptor that holds the end of the in part of bucket b (the end
+// of its out part follows), and of the start of its plane's first bucket.
+__host__ __device__ constexpr int desc_end(int b) {
+  return b / kPlaneBuckets * 16 + 4 + 2 * (b % kPlaneBuckets);
+}
+__host__ __device__ constexpr int desc_start(int b) { return b / kPlaneBuckets * 16 + 2; }
 
 // What the differentiable form reads of a net (snn_api.cu fills it).
 struct NetView {
   const void* syn;
   const uint8_t* bend;
-  long long N;
-  int npc, nexc, dmin, ndel, rowcap, precision, num_sms;
+  long long N, acc_words;
+  int npc, npc4, nexc, dmin, ndel, rowcap, unit, planes, precision, num_sms;
+  const uint32_t* ctile;
+  const uint32_t* colv;
+  const uint32_t* nbg;
   uint64_t seed;
   snn_neuron_params neuron;
   cudaStream_t stream;
 };
 int net_view(snn_net* net, NetView* v);
+
+// min(floor(2^32 / d), 2^32 - 1): the multiplier of the kernels' divisions.
+inline uint32_t recip32(uint32_t d) {
+  const unsigned long long m = (1ull << 32) / (unsigned long long)d;
+  return m > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)m;
+}
 
 // Shared host helpers (snn_api.cu).
 int fail_global(int code, const std::string& msg);
@@ -260,13 +308,16 @@ cudaError_t launch_build(const BuildParams& bp, int precision, int num_sms,
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st);
 cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
                               cudaStream_t st);
+// Readback of rows in the order they were drawn, within a row by delay.
+cudaError_t launch_read_rows(const BuildParams& bp, int precision, bool paper, cudaStream_t st);
 cudaError_t launch_init_state(const StepParams& p, cudaStream_t st);
 cudaError_t launch_update(const StepParams& p, int grid, cudaStream_t st);
 int update_grid(long long N, int num_sms);
-// Delivery: dynamic shared memory of one block (table, F16W neighbour table,
-// window), its thread count, and the persistent grid (0 if it does not fit).
-size_t deliver_smem(const StepParams& p, int precision);
-int deliver_threads();
+// Delivery: dynamic shared memory of one block of a net's own kernel or of
+// the batch kernel (window, neighbour table, the warps' sector lists) for
+// tiles of `cols` columns of npc4 words, and the persistent grid (0 if it
+// does not fit).
+size_t deliver_smem(int cols, int npc4, bool batch);
 int deliver_grid(const StepParams& p, int precision, int num_sms);
 cudaError_t launch_deliver(const StepParams& p, int precision, int grid, cudaStream_t st);
 // Compact the per-block record regions into id and step arrays and reset

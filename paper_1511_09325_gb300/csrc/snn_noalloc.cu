@@ -104,6 +104,7 @@ extern "C" int snn_update_noalloc(int grid_w, int grid_h, const snn_neuron_param
   p.W = grid_w;
   p.H = grid_h;
   p.nslot = 1;
+  p.npc_m = recip32((uint32_t)neuron->n_per_col);
   p.ncol = (int)ncol;
   p.seed_lo = (uint32_t)(seed & 0xFFFFFFFFu);
   p.seed_hi = (uint32_t)(seed >> 32);

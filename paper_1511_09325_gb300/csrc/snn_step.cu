@@ -1,40 +1,35 @@
 // snn_step.cu -- the two kernels of one 1 ms step.
 //
 // update_kernel (neuron update, arxiv 1511.09325 Sec. 2 LIF + SFA):
-//   grid-stride over tiles of 1024 neurons; one thread owns 4 consecutive
-//   neurons and one Philox4x32-10 block (counter (i/4, t, EXT, 0)) whose 4
-//   words give their external Poisson counts.  It reads and clears their
-//   recurrent input, applies refractoriness, threshold, reset and the exact
-//   propagator with explicitly rounded FP32 operations.  A tile's spikes are
-//   counted per column in shared memory and written to their column's part of
-//   the step's spike list (one atomic per column and tile) as descriptors --
-//   the spiker's id and its bucket ends, so that a delivery finds a bucket
-//   with one load -- and to the block's record region.  The per-column item
+//   grid-stride over chunks of 128 neurons, one warp each; one lane owns 4
+//   consecutive neurons and one Philox4x32-10 block (counter (i/4, t, EXT, 0))
+//   whose 4 words give their external Poisson counts.  It reads and clears
+//   their recurrent input, applies refractoriness, threshold, reset and the
+//   exact propagator with explicitly rounded FP32 operations.  A chunk's
+//   spikes go to their delivery tile's list of the step (one atomic per column
+//   and chunk) as descriptors -- the spiker's row and its bucket ends, copied
+//   from the build's table -- and to the block's record region.  The item
 //   counts of the next delivery (isum, gsum) are kept up to date here; spike
 //   and external-event totals go to per-block partial sums.
 //
 // deliver_kernel (event-driven delivery, Sec. 1), "pull by delay": the input
 //   of step t+1 is the sum over delays d of bucket d of every neuron that
-//   spiked at step t+1-d, so only one N-entry accumulator (resident in L2)
-//   receives additions, not a d_max-slot ring.  The (delay bucket, spiker)
-//   items of the last d_max steps, ordered by (virtual column, bucket,
-//   spiker), form one virtual list split evenly over a persistent grid of one
-//   768-thread block per SM.  Virtual columns run tile by tile (tiles of
-//   tile x tile columns, 6 x 6 at n_per_col = 1240), so a block's items come
-//   from a compact patch of the grid.  For each tile part with enough items,
-//   a block keeps a shared-memory window over the tile's columns (and a ring
-//   of P.ring columns around them) -- where about four fifths of the tile's
-//   synapses land (the local half and most of the near stencil) -- sums
-//   those synapses there with shared-memory reductions and flushes the window
-//   once into the accumulator by bulk asynchronous reductions; the other
-//   synapses go to L2 as fire-and-forget int32 reductions.  A warp takes
-//   batches of 32 items: lane e resolves item e (a binary search in the tile
-//   part's table of (column, bucket) counts and one descriptor load); the
-//   batch's buckets are then streamed as one list of 32-byte sectors dealt to
-//   the lanes in balanced rounds, two rounds in flight, and the next batch is
-//   resolved before the current one is streamed.  Integer addition makes the
-//   result independent of the order.  The last block to finish advances the
-//   step counter.
+//   spiked at step t+1-d, so only one accumulator (resident in L2) receives
+//   additions, not a d_max-slot ring.  The (delay bucket, spiker) items of the
+//   last d_max steps, ordered by (tile, bucket, spiker), form one virtual list
+//   split by cost over a persistent grid of one block per SM.  A part of a
+//   tile with enough items keeps a shared-memory window over the tile's
+//   columns, where about four fifths of the tile's synapses land (the local
+//   half and most of the near stencil; a bucket's "in" part, whose records
+//   name the window's word directly); those are summed there with
+//   shared-memory reductions and the window is added once to the accumulator
+//   by bulk asynchronous reductions.  The "out" parts go to L2 as
+//   fire-and-forget int32 reductions through the tile's neighbour table.  A
+//   warp resolves 32 items at a time (one per lane: list entry, bucket ends)
+//   and deals their 32-byte sectors to its lanes through a list in shared
+//   memory, in parts and then out parts, so that a round of 32 sectors runs
+//   one code path; the next batch's entries and ends are loaded meanwhile.
+//   Integer addition makes the result independent of the order.
 #include <algorithm>
 
 #include "snn_device.cuh"
@@ -47,12 +42,15 @@ constexpr int kUpdateThreads = 256;
 constexpr int kDeliverThreads = 768;   // one delivery block per SM (24 warps, 2 rounds in flight)
 constexpr int kBatchThreads = 512;     // batch kernel: 2 update sub-blocks or one delivery block
 constexpr int kUpdateSubs = kBatchThreads / kUpdateThreads;
-constexpr int kDepthF32 = 2;     // rounds of 32-byte sectors in flight per lane, F32W
-constexpr int kDepthF16 = 2;     // the same, F16W
-constexpr int kTile = kUpdateThreads * 4;    // neurons per update tile
-constexpr int kStageSpikes = 128;            // spikers per tile whose bucket ends are staged
-constexpr int kTileCols = kTile / 2 + 2;     // columns a tile can touch (npc >= 2)
-constexpr int kBatchItems = 32;              // items per warp batch (one per lane)
+constexpr int kDepth = 2;        // rounds of 32-byte sectors in flight per lane
+constexpr int kUpdateWarps = kUpdateThreads / 32;
+constexpr int kChunk = 128;      // neurons of a warp's chunk (four per lane)
+// Sector list of a warp: kListCap entries (a multiple of 32) at places p +
+// p / 32, so that lanes that write runs of about 8 entries meet few bank
+// conflicts.  A batch of 32 items of the default networks has about 290
+// entries; a longer one is streamed in pieces.
+constexpr int kListCap = 320;
+constexpr int kListWords = kListCap + kListCap / 32 + 2;
 
 struct NeuronOut {
   float v, c;
@@ -84,27 +82,17 @@ __device__ __forceinline__ NeuronOut neuron_step(float v, float c, uint32_t r,
   return o;
 }
 
-// Poisson count by inversion: the guide table gives the number of
-// thresholds below the top byte of x, a short scan finishes the count.
-__device__ __forceinline__ int poisson_count(uint32_t x, const uint8_t* guide,
-                                             const uint32_t* thr, int n) {
-  int k = guide[x >> 24];
-  while (k < n && x >= thr[k]) ++k;
-  return k;
+// Fire-and-forget int32 reductions into the accumulator and into shared
+// memory.  No compiler memory barrier: nothing the streaming
+// loops read aliases the window or the accumulator.
+__device__ __forceinline__ void red_add_nz(const int32_t* p, int32_t v) {  // nothing for v = 0
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.s32 p, %1, 0;\n\t"
+      "@p red.global.add.s32 [%0], %1;\n\t}" ::"l"(p), "r"(v));
 }
-
-// L2 evict-last policy for the accumulator, which the next step's update
-// re-reads.
-__device__ __forceinline__ uint64_t evict_last_policy() {
-  uint64_t pol;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-
-// Fire-and-forget int32 reduction into the accumulator under policy `pol`.
-__device__ __forceinline__ void red_add(int32_t* p, int32_t v, uint64_t pol) {
-  asm volatile("red.global.add.L2::cache_hint.s32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol)
-               : "memory");
+__device__ __forceinline__ void red_shared(uint32_t a, int32_t v) {
+  asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(a), "r"(v));
 }
 
 // Loads of the neuron state, read once per step: no L1 allocation, so that
@@ -123,11 +111,23 @@ __device__ __forceinline__ int4 ld_stream(const int4* p) {
                : "l"(p));
   return v;
 }
-__device__ __forceinline__ uchar4 ld_stream(const uchar4* p) {
+__device__ __forceinline__ uint32_t ld_stream(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
-  return make_uchar4((unsigned char)v, (unsigned char)(v >> 8), (unsigned char)(v >> 16),
-                     (unsigned char)(v >> 24));
+  return v;
+}
+
+// Poisson count of word x by inversion.  Entry b of the table (one per top
+// byte of x) holds bits 0-6: the thresholds <= b << 24; bits 8-31: the low 24
+// bits of the one threshold inside the bin, less one (2^24 - 1: none inside);
+// bit 7: more than one inside, scan from the count.  So x << 8 > entry exactly
+// when x has reached the bin's threshold.
+__device__ __forceinline__ uint32_t poisson_entry(const StepParams& P, int b) {
+  const int k = P.pois_guide[b];
+  const uint32_t lo = (uint32_t)b << 24;
+  const bool in1 = k < P.n_pois_thr && (P.pois_thr[k] - lo) >> 24 == 0u;
+  const bool in2 = k + 1 < P.n_pois_thr && (P.pois_thr[k + 1] - lo) >> 24 == 0u;
+  return (in1 ? (P.pois_thr[k] - lo - 1u) << 8 : 0xFFFFFF00u) | (in2 ? 128u : 0u) | (uint32_t)k;
 }
 
 // Barrier of an update body: the whole block (bar 0) or one 256-thread
@@ -146,249 +146,267 @@ __device__ __forceinline__ void set_status(const StepParams& P, unsigned code) {
   if (P.hstatus != nullptr) *reinterpret_cast<volatile unsigned*>(P.hstatus) = code;
 }
 
+// Quotient of x by d from m = min(floor(2^32 / d), 2^32 - 1): the estimate
+// is at most one below the quotient, so one correction step finishes it.
+__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t m) {
+  uint32_t q = __umulhi(x, m);
+  if (x - q * d >= d) ++q;
+  return q;
+}
+
+// The next place at *count for each active lane: one atomic for the lanes of
+// the same `key` (mostly one; the lanes of a key have the same counter).
+__device__ __forceinline__ unsigned next_place(unsigned* count, uint32_t key) {
+  const unsigned lane = threadIdx.x & 31u;
+  const unsigned peers = __match_any_sync(__activemask(), key);
+  const int lead = __ffs(peers) - 1;
+  unsigned pos = 0u;
+  if ((int)lane == lead) pos = atomicAdd(count, (unsigned)__popc(peers));
+  return __shfl_sync(peers, pos, lead) + (unsigned)__popc(peers & ((1u << lane) - 1u));
+}
+
 // Shared memory of one update body.
 struct UpdateSmem {
-  uint32_t thr[kMaxPoisThr + 1];  // Poisson thresholds
-  uint8_t guide[256];            // Poisson guide table
-  unsigned tpop[kTileCols][2];   // E / I spikes per column of the tile
-  unsigned tpos[kTileCols];      // first record of each column's spikes in the tile
-  long long lbase[kTileCols];    // list position of each column's first spike
-  long long cbase;               // compact list: position of the tile's first spike
-  unsigned long long rbase;      // record position of the tile's first spike
-  unsigned long long rc, spk;
-  unsigned long long synw[kUpdateThreads / 32];  // synaptic events per warp
-  unsigned ksum[kUpdateThreads / 32];
-  // bucket ends of the tile's first kStageSpikes spikers, copied
-  // asynchronously as soon as the spike is known, so the load's latency
-  // overlaps the tile's count bookkeeping (later spikers load theirs when
-  // the descriptor is written)
-  unsigned nbst;
-  uint4 bst[kStageSpikes][2];
+  uint32_t pois[256];
+  unsigned rc;                   // records written in this step
+  unsigned items;                // change of gsum
+  uint32_t id[kUpdateWarps][kChunk];  // the spikes of a warp's chunk
+  unsigned long long syn[kUpdateWarps];  // synaptic events per warp
+  unsigned ksum[kUpdateWarps];
 };
 
 // Update body vb of vgrid for step t, run by kUpdateThreads threads (thread
-// index tid, barrier `bar`): tiles vb, vb + vgrid, ...  Body vb owns
-// ext_part[vb], spk_part[vb] and record region vb of the net, so the grid
-// size must be the same every step.  Each spike goes to the step's list
-// (column c's part when P.ccnt is set, else one compact list) -- as a
-// descriptor when P.desc is set, else as its id -- and to the body's record
-// region as (step << 32 | id).  A shard (SHARD, P.sg.on) updates its own
-// columns only, draws the external input with global neuron indices and
-// records global indices; the halo's columns take part in the count
-// bookkeeping.
+// index tid, barrier `bar`): every warp takes chunks of kChunk neurons, lane e
+// of a chunk the quad of neurons 4 e .. 4 e + 3, and works without the other
+// warps.  A chunk's spikes are then dealt to the lanes, one each: a lane finds
+// its spike's column and takes the next place of the column's tile's list; the
+// chunk takes its places in the body's record region by one atomic.  Body vb
+// owns ext_part[vb], spk_part[vb], syn_part[vb] and record region vb of the
+// net, so the grid size must be the same every step.  Each spike goes to its
+// tile's list of the step (or to one compact list of ids, without ccnt) and to
+// the body's record region as (step << 32 | id).  A shard (SHARD, P.sg.on)
+// updates its own columns only, draws the external input with global neuron
+// indices and records global indices; the halo's columns take part in the
+// count bookkeeping.
 template <bool SHARD>
 __device__ __forceinline__ void update_body(const StepParams& P, long long t, int vb, int vgrid,
                                             UpdateSmem& S, int tid, int bar) {
+  const int lane = tid & 31, warp = tid >> 5;
+  const uint32_t npc = (uint32_t)P.npc;
+  const uint32_t quads = (uint32_t)((P.N + 3) / 4);  // below 2^29
+  const uint32_t stride = (uint32_t)vgrid * (uint32_t)(kUpdateWarps * 32);  // quads
+  // whole: a quad lies in one column; else (in a net) its input is read word
+  // by word
+  const bool whole = (npc & 3u) == 0u;
+  const bool direct = P.colv == nullptr || whole;
+
+  // The state of the warp's next chunk is requested before the current chunk
+  // is processed, and the virtual index of the column of the one after it
+  // (which its input's address needs), so their latency overlaps the work.
+  // q0: quad of the current chunk's lane 0; a: quad of the input; l: place of
+  // the quad's first neuron in its column.
+  float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), pc = pv;
+  uint32_t pr = 0u;
+  int4 pa = make_int4(0, 0, 0, 0);
+  auto place = [&](uint32_t q, uint32_t* l, uint32_t* v) {
+    const uint32_t c = div_by(4u * q, npc, P.npc_m);
+    *l = 4u * q - c * npc;
+    *v = P.colv != nullptr && q < quads ? __ldg(P.colv + c) : 0u;
+  };
+  auto input_quad = [&](uint32_t q, uint32_t l, uint32_t v) -> uint32_t {
+    return P.colv == nullptr ? q : (uint32_t)(((unsigned long long)v * (uint32_t)P.npc4 + l) >> 2);
+  };
+  auto load = [&](uint32_t q, uint32_t a) {
+    if (q < quads) {
+      pv = ld_stream(reinterpret_cast<const float4*>(P.V) + q);
+      pc = ld_stream(reinterpret_cast<const float4*>(P.C) + q);
+      pr = ld_stream(reinterpret_cast<const uint32_t*>(P.R) + q);
+      if (direct) pa = ld_stream(reinterpret_cast<const int4*>(P.acc) + a);
+    }
+  };
+  uint32_t q = (uint32_t)vb * (uint32_t)(kUpdateWarps * 32) + (uint32_t)tid;
+  uint32_t l, l_nxt, v, v_nxt;
+  place(q, &l, &v);
+  place(q + stride, &l_nxt, &v_nxt);
+  uint32_t a = input_quad(q, l, v);
+  load(q, a);
+
   body_sync(bar);  // the shared memory may still be read by a previous body
   const int slot = (int)(t % P.nslot);
-  for (int m = tid; m < 256; m += kUpdateThreads) S.guide[m] = P.pois_guide[m];
-  for (int m = tid; m <= kMaxPoisThr; m += kUpdateThreads) S.thr[m] = P.pois_thr[m];
+  S.pois[tid] = poisson_entry(P, tid);
   if (tid == 0) {
-    S.rc = P.rcnt[vb];
-    S.spk = 0ull;
+    S.rc = 0u;
+    S.items = 0u;
+    if (vb == 0) P.ctl->td = t;  // the step's delivery
   }
+  const unsigned long long rc0 = P.rcnt[vb];
   unsigned ksum = 0u;
-  unsigned long long syn = 0ull;  // out-degrees of this thread's spikes
-  const long long quads = (P.N + 3) / 4;
-  const long long tiles = (quads + kUpdateThreads - 1) / kUpdateThreads;
-  uint32_t* list = P.ids + (long long)slot * P.N;
-  unsigned long long* region = P.rec + (long long)vb * P.rec_region;
+  unsigned long long syn = 0ull;  // out-degrees of this thread's spikes (with deg)
+  body_sync(bar);
 
-  // Each column's item count (isum, gsum) moves from the delivery window of
-  // step t - 1, steps t - d_max .. t - d_min, to that of step t: step
-  // t + 1 - d_min comes in (as its spikes are counted, when d_min = 1) and
-  // step t - d_max, whose slot is (t + 1) mod (d_max + 1), goes out.  The tile
-  // in which a column starts applies the change for that column.
-  const long long s_in = t + 1 - P.dmin;
-  const unsigned* cin_ = (P.ccnt != nullptr && P.dmin >= 2 && s_in >= 0)
-                             ? P.ccnt + (s_in % P.nslot) * P.ncol : nullptr;
-  const unsigned* cout_ = P.ccnt != nullptr ? P.ccnt + ((t + 1) % P.nslot) * P.ncol : nullptr;
-
-  // the state of the body's next tile is requested before the current tile
-  // is processed, so its latency overlaps the current tile's work
-  float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), pc = pv;
-  uchar4 pr = make_uchar4(0, 0, 0, 0);
-  int4 pa = make_int4(0, 0, 0, 0);
-  {
-    const long long q0 = (long long)vb * kUpdateThreads + tid;
-    if (vb < tiles && q0 * 4 < P.N) {
-      pv = ld_stream(reinterpret_cast<const float4*>(P.V) + q0);
-      pc = ld_stream(reinterpret_cast<const float4*>(P.C) + q0);
-      pr = ld_stream(reinterpret_cast<const uchar4*>(P.R) + q0);
-      pa = ld_stream(reinterpret_cast<const int4*>(P.acc) + q0);
-    }
-  }
-  for (long long tile = vb; tile < tiles; tile += vgrid) {
-    const float4 v4 = pv, c4 = pc;
-    const uchar4 r4 = pr;
-    const int4 a4 = pa;
-    {
-      const long long qn = (tile + vgrid) * kUpdateThreads + tid;
-      if (tile + vgrid < tiles && qn * 4 < P.N) {
-        pv = ld_stream(reinterpret_cast<const float4*>(P.V) + qn);
-        pc = ld_stream(reinterpret_cast<const float4*>(P.C) + qn);
-        pr = ld_stream(reinterpret_cast<const uchar4*>(P.R) + qn);
-        pa = ld_stream(reinterpret_cast<const int4*>(P.acc) + qn);
+  // Each tile's item count (isum, their sum gsum) moves on by one step: it
+  // covers the steps t - d_max + 1 .. t - d_min + 1 that this step's delivery
+  // reads, less step t itself (d_min = 1), whose spikes the delivery adds.
+  // Step t - d_max, whose slot is (t + 1) mod (d_max + 1), goes out.
+  if (P.ccnt != nullptr) {
+    const long long s_in = P.dmin == 1 ? t - 1 : t + 1 - P.dmin;
+    const unsigned* cin_ = s_in >= 0 ? P.ccnt + (s_in % P.nslot) * P.ntile * kCntStride : nullptr;
+    const unsigned* cout_ = P.ccnt + ((t + 1) % P.nslot) * P.ntile * kCntStride;
+    for (long long m = (long long)vb * kUpdateThreads + tid; m < P.ntile;
+         m += (long long)vgrid * kUpdateThreads) {
+      const unsigned d = (cin_ ? cin_[m * kCntStride] : 0u) - cout_[m * kCntStride];
+      if (d) {
+        atomicAdd(P.isum + m * kCntStride, d);
+        atomicAdd(&S.items, d);
       }
     }
-    const long long first = tile * kTile;
-    const long long last = (first + kTile < P.N ? first + kTile : P.N) - 1;
-    // neuron indices are below 2^31: 32-bit divisions are exact (and cheap)
-    const int col0 = (int)((uint32_t)first / (uint32_t)P.npc);
-    const int ncols = (int)((uint32_t)last / (uint32_t)P.npc) - col0 + 1;
-    for (int k = tid; k < ncols; k += kUpdateThreads) {
-      S.tpop[k][0] = 0u;
-      S.tpop[k][1] = 0u;
-    }
-    if (tid == 0) S.nbst = 0u;
-    body_sync(bar);
+  }
+  if (SHARD)  // halo spikes per column that the step's ingest will count
+    for (long long c = (long long)vb * kUpdateThreads + tid; c < P.ncol;
+         c += (long long)vgrid * kUpdateThreads)
+      P.icnt[c] = 0u;
 
-    const long long q = tile * kUpdateThreads + tid;
-    const long long i0 = q * 4;
-    unsigned rank[4] = {0u, 0u, 0u, 0u};
-    int scol[4] = {-1, -1, -1, -1};
-    uint32_t gq = (uint32_t)q;  // global quad of the four neurons
-    bool own = true;
-    if (SHARD && i0 < P.N) {
-      const int c = (int)((uint32_t)i0 / (uint32_t)P.npc);
-      const int l0 = (int)((uint32_t)i0 - (uint32_t)c * (uint32_t)P.npc);
-      const int cy = c / P.W, cx = c - cy * P.W;
+  for (; q - (uint32_t)lane < quads; q += stride) {
+    const float4 v4 = pv, c4 = pc;
+    const uint32_t r4 = pr;
+    int4 a4 = pa;
+    const uint32_t a_own = a, l_own = l;
+    l = l_nxt;
+    a = input_quad(q + stride, l, v_nxt);
+    load(q + stride, a);
+    place(q + 2u * stride, &l_nxt, &v_nxt);
+
+    uint32_t gq = q;  // global quad of the four neurons
+    bool own = q < quads;
+    if (SHARD && own) {
+      const int col = (int)((4u * q - l_own) / npc);
+      const int cy = col / P.W, cx = col - cy * P.W;
       own = cx >= P.sg.tx0 && cx < P.sg.tx0 + P.sg.tw && cy >= P.sg.ty0 && cy < P.sg.ty0 + P.sg.th;
       int gx, gy;
       shard_global_col(P.sg, cx, cy, &gx, &gy);
-      gq = (((uint32_t)gy * (uint32_t)P.sg.GW + (uint32_t)gx) * (uint32_t)P.npc + (uint32_t)l0) >> 2;
+      gq = (((uint32_t)gy * (uint32_t)P.sg.GW + (uint32_t)gx) * npc + l_own) >> 2;
     }
-    if (i0 < P.N && own) {
+    unsigned spk = 0u;  // bit e: neuron 4 q + e fired
+    if (own) {
       const uint4 x = philox4x32_10(make_uint4(gq, (uint32_t)t, kTagExt, 0u), P.seed_lo, P.seed_hi);
-      reinterpret_cast<int4*>(P.acc)[q] = make_int4(0, 0, 0, 0);
-      const float vin[4] = {v4.x, v4.y, v4.z, v4.w};
-      const float cin[4] = {c4.x, c4.y, c4.z, c4.w};
-      const uint32_t rin[4] = {r4.x, r4.y, r4.z, r4.w};
-      const int32_t ain[4] = {a4.x, a4.y, a4.z, a4.w};
-      const uint32_t xin[4] = {x.x, x.y, x.z, x.w};
-      float vout[4], cout[4];
-      uint32_t rout[4];
-      int col = (int)((uint32_t)i0 / (uint32_t)P.npc);
-      int l = (int)((uint32_t)i0 - (uint32_t)col * (uint32_t)P.npc);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int k = poisson_count(xin[e], S.guide, S.thr, P.n_pois_thr);
-        const int32_t I = ain[e] + k * P.jx;
-        const bool exc = l < P.nexc;
-        const NeuronOut o = neuron_step(vin[e], cin[e], rin[e], I, exc ? P.pvc_e : P.pvc_i, P);
-        vout[e] = o.v;
-        cout[e] = o.c;
-        rout[e] = o.r;
-        if (i0 + e < P.N) {
-          ksum += (unsigned)k;
-          if (o.spike) {
-            scol[e] = col - col0;
-            rank[e] = atomicAdd(&S.tpop[col - col0][exc ? 0 : 1], 1u);
-            if (!exc) rank[e] |= 0x80000000u;  // ranked among the column's I spikes
-          }
-        }
-        if (++l == P.npc) {
-          l = 0;
-          ++col;
-        }
-      }
-      if (P.desc != nullptr) {
-        // stage the bucket ends of the first kStageSpikes spikers (slot in
-        // bits 16..23 of the rank; 255: none)
+      if (direct) {
+        reinterpret_cast<int4*>(P.acc)[a_own] = make_int4(0, 0, 0, 0);
+      } else {
+        int32_t in[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          if (scol[e] >= 0) {
-            const unsigned bs = atomicAdd(&S.nbst, 1u);
-            if (bs < (unsigned)kStageSpikes) {
-              const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&S.bst[bs][0]);
-              const uint4* src = reinterpret_cast<const uint4*>(P.bend + (i0 + e) * kBendStride);
-              asm volatile(
-                  "cp.async.cg.shared.global [%0], [%1], 16;\n\t"
-                  "cp.async.cg.shared.global [%2], [%3], 16;" ::"r"(dst),
-                  "l"(src), "r"(dst + 16u), "l"(src + 1)
-                  : "memory");
-            }
-            rank[e] |= (bs < (unsigned)kStageSpikes ? bs : 255u) << 16;
+          const long long i = 4ll * q + e;
+          in[e] = 0;
+          if (i < P.N) {
+            const uint32_t c = div_by((uint32_t)i, npc, P.npc_m);
+            int32_t* w = P.acc + (size_t)P.colv[c] * P.npc4 + ((uint32_t)i - c * npc);
+            in[e] = *w;
+            *w = 0;
           }
+        }
+        a4 = make_int4(in[0], in[1], in[2], in[3]);
+      }
+      const float vin[4] = {v4.x, v4.y, v4.z, v4.w};
+      const float cin[4] = {c4.x, c4.y, c4.z, c4.w};
+      const int32_t ain[4] = {a4.x, a4.y, a4.z, a4.w};
+      const uint32_t xin[4] = {x.x, x.y, x.z, x.w};
+      int kp[4];
+      uint32_t ent[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) ent[e] = S.pois[xin[e] >> 24];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) kp[e] = (int)(ent[e] & 127u) + ((xin[e] << 8) > ent[e] ? 1 : 0);
+      if ((ent[0] | ent[1] | ent[2] | ent[3]) & 128u) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (ent[e] & 128u) {
+            int k = (int)(ent[e] & 127u);
+            while (k < P.n_pois_thr && xin[e] >= P.pois_thr[k]) ++k;
+            kp[e] = k;
+          }
+      }
+      const bool tail = 4ll * q + 4 > P.N;  // the last quad may end early
+      float vout[4], cout[4];
+      uint32_t rout = 0u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t le = l_own + (uint32_t)e;
+        if (!whole) {  // n_per_col may be 2
+          le -= le >= npc ? npc : 0u;
+          le -= le >= npc ? npc : 0u;
+        }
+        const int32_t I = ain[e] + kp[e] * P.jx;
+        const NeuronOut o = neuron_step(vin[e], cin[e], r4 >> (8 * e) & 0xFFu, I,
+                                        le < (uint32_t)P.nexc ? P.pvc_e : P.pvc_i, P);
+        vout[e] = o.v;
+        cout[e] = o.c;
+        rout |= (o.r & 0xFFu) << (8 * e);
+        if (!tail || 4ll * q + e < P.N) {
+          ksum += (unsigned)kp[e];
+          spk |= o.spike ? 1u << e : 0u;
         }
       }
       reinterpret_cast<float4*>(P.V)[q] = make_float4(vout[0], vout[1], vout[2], vout[3]);
       reinterpret_cast<float4*>(P.C)[q] = make_float4(cout[0], cout[1], cout[2], cout[3]);
-      reinterpret_cast<uchar4*>(P.R)[q] = make_uchar4((unsigned char)rout[0], (unsigned char)rout[1],
-                                                      (unsigned char)rout[2], (unsigned char)rout[3]);
+      reinterpret_cast<uint32_t*>(P.R)[q] = rout;
     }
-    body_sync(bar);
-    // places: records grouped by column (E then I) in the body's region; list
-    // entries in each column's part of the step's list (or the compact list)
-    if (P.ccnt != nullptr) {
-      for (int k = tid; k < ncols; k += kUpdateThreads) {
-        const unsigned n = S.tpop[k][0] + S.tpop[k][1];
-        const int c = col0 + k;
-        S.lbase[k] = (long long)c * P.npc +
-                     (n ? (long long)atomicAdd(P.ccnt + (long long)slot * P.ncol + c, n) : 0ll);
-        unsigned d = P.dmin == 1 ? n : 0u;
-        if ((long long)c * P.npc >= first) d += (cin_ ? cin_[c] : 0u) - cout_[c];
-        if (d) {
-          const int v = P.colv != nullptr ? (int)P.colv[c] : c;
-          atomicAdd(P.isum + v, d);
-          atomicAdd(P.gsum + (v >> 5), d);
-        }
-      }
-    }
-    if (tid == 0) {
-      unsigned pos = 0u;
-      for (int k = 0; k < ncols; ++k) {
-        S.tpos[k] = pos;
-        pos += S.tpop[k][0] + S.tpop[k][1];
-      }
-      // the compact list (no per-column lists) takes the tile's spikes at a
-      // shared cursor; per-column lists need none
-      S.cbase = (pos && P.ccnt == nullptr) ? (long long)atomicAdd(P.cnt + slot, pos) : 0ll;
-      S.rbase = S.rc;
-      S.rc += pos;
-      S.spk += pos;
-    }
-    body_sync(bar);
-    const unsigned long long rc = S.rbase;
-    if (P.desc != nullptr) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (__ballot_sync(0xFFFFFFFFu, spk != 0u) == 0u) continue;
+
+    // the chunk's spikes in a row, and their places in the record region
+    unsigned n = 0u;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      if (scol[e] >= 0) {
-        const int k = scol[e];
-        const unsigned r = rank[e] & 0xFFFFu;
-        const unsigned off = (rank[e] & 0x80000000u) ? S.tpop[k][0] + r : r;
-        const uint32_t id = (uint32_t)(i0 + e);
-        const long long pos = P.ccnt != nullptr ? S.lbase[k] + off : S.cbase + S.tpos[k] + off;
-        if (P.desc != nullptr) {
-          // descriptor: id, then the bucket ends of the spiker's row
-          uint4* d = reinterpret_cast<uint4*>(P.desc + ((long long)slot * P.N + pos) * P.desc_words);
-          const unsigned bs = (rank[e] >> 16) & 0xFFu;
-          uint4 a, b;
-          if (bs != 255u) {
-            a = S.bst[bs][0];
-            b = S.bst[bs][1];
-          } else {
-            const uint4* be = reinterpret_cast<const uint4*>(P.bend + (long long)id * kBendStride);
-            a = be[0];
-            b = be[1];
-          }
-          d[0] = make_uint4(id, a.x, a.y, a.z);
-          d[1] = make_uint4(a.w, b.x, b.y, b.z);
-          if (P.desc_words == 16) d[2] = make_uint4(b.w, 0u, 0u, 0u);
+      const unsigned b = __ballot_sync(0xFFFFFFFFu, spk >> e & 1u);
+      if (spk >> e & 1u) S.id[warp][n + __popc(b & ((1u << lane) - 1u))] = 4u * q + (uint32_t)e;
+      n += (unsigned)__popc(b);
+    }
+    unsigned rec = 0u;
+    if (lane == 0) rec = atomicAdd(&S.rc, n);
+    rec = __shfl_sync(0xFFFFFFFFu, rec, 0);
+    __syncwarp();
+    for (unsigned k0 = 0u; k0 < n; k0 += 32u) {
+      const unsigned k = k0 + (unsigned)lane;
+      uint32_t row = 0u;             // the spike's row in bend
+      unsigned long long at = 0ull;  // its place in the lists
+      if (k < n) {
+        const uint32_t id = S.id[warp][k];
+        const uint32_t c = div_by(id, npc, P.npc_m), il = id - c * npc;
+        if (P.ccnt != nullptr) {
+          const uint32_t ct = __ldg(P.ctile + c);
+          row = __ldg(P.colv + c) * npc + il;
+          const size_t ts = (size_t)slot * P.ntile + (ct >> 6);
+          at = ((unsigned long long)slot * P.planes * P.ntile + (ct >> 6)) * P.tcap +
+               next_place(P.ccnt + ts * kCntStride, ct >> 6);
         } else {
-          list[pos] = id;
+          P.ids[next_place(P.cnt + slot, 0u)] = id;
         }
-        syn += P.deg != nullptr ? P.deg[id] : (uint32_t)P.K;
-        const unsigned long long ri = rc + S.tpos[k] + off;
-        const uint32_t gid = SHARD ? gq * 4u + (uint32_t)e : id;
-        if ((long long)ri < P.rec_region) region[ri] = ((unsigned long long)(unsigned)t << 32) | gid;
+        atomicAdd(&P.colcnt[2ull * c + (il < (uint32_t)P.nexc ? 0u : 1u)], 1ull);
+        if (P.deg != nullptr) syn += P.deg[id];
+        uint32_t gid = id;
+        if (SHARD) {
+          const int cy = (int)c / P.W, cx = (int)c - cy * P.W;
+          int gx, gy;
+          shard_global_col(P.sg, cx, cy, &gx, &gy);
+          gid = ((uint32_t)gy * (uint32_t)P.sg.GW + (uint32_t)gx) * npc + il;
+        }
+        const unsigned long long ri = rc0 + rec + k;
+        if ((long long)ri < P.rec_region)
+          P.rec[(long long)vb * P.rec_region + (long long)ri] = ((unsigned long long)(unsigned)t << 32) | gid;
+      }
+      // descriptors: four lanes copy one spike's planes into its list
+      if (P.ccnt != nullptr) {
+        const size_t plane = (size_t)P.ntile * P.tcap;
+        for (unsigned s0 = 0u; s0 < min(n - k0, 32u); s0 += 8u) {
+          const int src = (int)(s0 + ((unsigned)lane >> 2));
+          const uint32_t rs = __shfl_sync(0xFFFFFFFFu, row, src);
+          const unsigned long long as = __shfl_sync(0xFFFFFFFFu, at, src);
+          if (k0 + (unsigned)src < n)
+            for (int p = lane & 3; p < P.planes; p += 4)
+              P.list[as + p * plane] = P.bend[(size_t)rs * P.planes + p];
+        }
       }
     }
-    for (int k = tid; k < ncols; k += kUpdateThreads) {
-      if (S.tpop[k][0]) atomicAdd(&P.colcnt[2 * (col0 + k)], (unsigned long long)S.tpop[k][0]);
-      if (S.tpop[k][1]) atomicAdd(&P.colcnt[2 * (col0 + k) + 1], (unsigned long long)S.tpop[k][1]);
-    }
-    body_sync(bar);
+    __syncwarp();
   }
 
   // external and synaptic events: per-body partial sums, no atomics
@@ -397,22 +415,23 @@ __device__ __forceinline__ void update_body(const StepParams& P, long long t, in
     ksum += __shfl_xor_sync(0xFFFFFFFFu, ksum, o);
     syn += __shfl_xor_sync(0xFFFFFFFFu, syn, o);
   }
-  if ((tid & 31) == 0) {
-    S.ksum[tid >> 5] = ksum;
-    S.synw[tid >> 5] = syn;
+  if (lane == 0) {
+    S.ksum[warp] = ksum;
+    S.syn[warp] = syn;
   }
   body_sync(bar);
   if (tid == 0) {
     unsigned long long tot = 0ull, tsyn = 0ull;
-    for (int w = 0; w < kUpdateThreads / 32; ++w) {
+    for (int w = 0; w < kUpdateWarps; ++w) {
       tot += S.ksum[w];
-      tsyn += S.synw[w];
+      tsyn += S.syn[w];
     }
+    if (S.items) atomicAdd(P.gsum, S.items);
     P.ext_part[vb] += tot;
-    P.spk_part[vb] += S.spk;
-    if (P.syn_part != nullptr) P.syn_part[vb] += tsyn;
-    if ((long long)S.rc > P.rec_region) P.ctl->rec_overflow = 1u;
-    P.rcnt[vb] = S.rc;
+    P.spk_part[vb] += S.rc;
+    if (P.syn_part != nullptr) P.syn_part[vb] += P.deg != nullptr ? tsyn : (unsigned long long)S.rc * (unsigned)P.K;
+    if ((long long)(rc0 + S.rc) > P.rec_region) P.ctl->rec_overflow = 1u;
+    P.rcnt[vb] = rc0 + S.rc;
   }
 }
 
@@ -426,703 +445,437 @@ __global__ void __launch_bounds__(kUpdateThreads, 4) update_kernel(const StepPar
 // Delivery.
 // ---------------------------------------------------------------------------
 
-// Quotient of x by d from m = min(floor(2^32 / d), 2^32 - 1): the estimate
-// is at most one below the quotient, so one correction step finishes it.
-__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t m) {
-  uint32_t q = __umulhi(x, m);
-  if (x - q * d >= d) ++q;
-  return q;
-}
-
-// Tile of virtual column v: tiles of P.tile x P.tile columns in row-major
-// order (those of the last tile row or column may be smaller), columns
-// row-major inside a tile.
-struct TileGeo {
-  int first;   // virtual index of the tile's first column
-  int x0, y0;  // grid position of its first column
-  int tw, th;  // its width and height
-};
-
-__device__ __forceinline__ TileGeo tile_geo(const StepParams& P, int v) {
-  TileGeo g;
-  const int rowcols = P.tile * P.W;  // columns of a full row of tiles
-  const int tr = v / rowcols;
-  g.y0 = tr * P.tile;
-  g.th = min(P.tile, P.H - g.y0);
-  const int rem = v - tr * rowcols;
-  const int tc = rem / (g.th * P.tile);
-  g.x0 = tc * P.tile;
-  g.tw = min(P.tile, P.W - g.x0);
-  g.first = tr * rowcols + tc * g.th * P.tile;
-  return g;
-}
-
-// Shared-memory window of a tile: the ww x wh columns starting at (x0, y0)
-// (periodic; at most the whole grid, so every column appears once).  Slot
-// (rx, ry) holds column ((x0 + rx) mod W, (y0 + ry) mod H).
-struct WinGeo {
-  int x0, y0, ww, wh;
-};
-
-__device__ __forceinline__ WinGeo win_geo(const StepParams& P, const TileGeo& g, bool on) {
-  WinGeo w;
-  w.ww = min(g.tw + 2 * P.ring, P.W);
-  w.wh = min(g.th + 2 * P.ring, P.H);
-  w.x0 = w.ww == P.W ? 0 : wrap(g.x0 - P.ring, P.W);
-  w.y0 = w.wh == P.H ? 0 : wrap(g.y0 - P.ring, P.H);
-  if (!on) w.ww = w.wh = 0;
-  return w;
-}
-
 struct DeliverSmem {
-  unsigned long long wsum[32];    // per-warp sums of block_scan
-  unsigned long long xgp[2];      // items before the group holding lo / hi - 1
-  unsigned long long ipt[2];      // item positions of the block's range ends
-  unsigned long long p0;          // items before virtual column v0
-  int xg[2];                      // group holding lo / hi - 1
-  int v0, v1;                     // first and last virtual column of the block's items
-  int slot[kMaxDelays];           // slot of each bucket's step, -1 before step 0
-  int pe;                         // end (exclusive) of the current part
-  int pwin;                       // the current part uses the window
-  int ccol[kMaxTileCols];         // real column of each column of the current tile part
-  int cx[kMaxTileCols], cy[kMaxTileCols];  // its grid position
-  uint32_t wbase[(kMaxTile + 2) * (kMaxTile + 2)];  // first neuron of each window slot's column
-  unsigned next;                  // next batch of the current tile part
+  unsigned long long wsum[3][32]; // per-warp sums of the range scan
+  int rt[2];                      // tiles holding the ends of the block's range
+  unsigned ri[2];                 // item places of the ends inside them
 };
 
-// Words of the (column, bucket) table and of the F16W neighbour table of a
-// part of `cols` columns.  In the dynamic shared memory of a delivery block
-// the tables of a windowed part (one tile, at most tile^2 columns) come first,
-// then the window; a part without window (at most part_cols columns) keeps
-// its tables at the start of the window area, which it does not use.
-__device__ __forceinline__ int tab_words(const StepParams& P, int cols) {
-  return (cols * P.ndel + 1 + 3) & ~3;
-}
-template <int PREC>
-__device__ __forceinline__ int nb_words(int cols) {
-  return PREC == SNN_EXACT_F16W ? cols * 64 : 0;
-}
-
-// Block-wide exclusive scan of one 64-bit value per thread; *total gets the
-// sum.  Uses S.wsum; contains two barriers.
-__device__ __forceinline__ unsigned long long block_scan(unsigned long long v, DeliverSmem& S,
-                                                         unsigned long long* total) {
+// Sums, over the block's threads, of three 64-bit values, and the exclusive
+// prefix of the first.  Contains one barrier.
+__device__ __forceinline__ void block_scan3(unsigned long long a, unsigned long long b,
+                                            unsigned long long c, DeliverSmem& S,
+                                            unsigned long long* a_excl, unsigned long long* a_total,
+                                            unsigned long long* b_total, unsigned long long* c_total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = (int)(blockDim.x >> 5);
-  unsigned long long incl = v;
+  unsigned long long incl = a;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned long long u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
+    c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
     if (lane >= o) incl += u;
   }
-  if (lane == 31) S.wsum[warp] = incl;
-  __syncthreads();
-  unsigned long long before = 0ull, all = 0ull;
-  for (int w = 0; w < nwarps; ++w) {
-    const unsigned long long s = S.wsum[w];
-    before += w < warp ? s : 0ull;
-    all += s;
+  if (lane == 31) {
+    S.wsum[0][warp] = incl;
+    S.wsum[1][warp] = b;
+    S.wsum[2][warp] = c;
   }
   __syncthreads();
-  *total = all;
-  return before + incl - v;
+  unsigned long long w = lane < nwarps ? S.wsum[0][lane] : 0ull;
+  unsigned long long before = lane < warp ? w : 0ull;
+  b = lane < nwarps ? S.wsum[1][lane] : 0ull;
+  c = lane < nwarps ? S.wsum[2][lane] : 0ull;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    w += __shfl_xor_sync(0xFFFFFFFFu, w, o);
+    before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+    b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
+    c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+  }
+  *a_excl = before + incl - a;
+  *a_total = w;
+  *b_total = b;
+  *c_total = c;
 }
 
-// Neighbour-table entry of F16W record w = half_magnitude(15) << 17 |
-// offset(6) << 11 | l(11): in the row `nbrow` of the spiker's column, the
-// offset's target column -- its shared-window address, or bit 31 set and its
-// first neuron in the accumulator.  The entries of a sector's eight records
-// are loaded before any of them is delivered, so the loads are not ordered
-// behind the shared-memory reductions.  (Measured: one reduction with a
-// generic 64-bit address instead of the two predicated ones made the
-// delivery 2.6-2.8x slower: generic atomics on shared memory are slow.)
-__device__ __forceinline__ uint32_t nb_entry(uint32_t w, uint32_t nbrow) {
-  uint32_t e;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(nbrow + ((w >> 9) & 0xFCu)));
-  return e;
-}
-
-// Deliver F16W record w with its table entry e, as one PTX block: the weight
-// rint(half * 2^16) comes from one rounded multiply-add (x * (+-2^16) +
-// 1.5 * 2^23 lands in [2^23, 2^24), where the float grid is the integers, so
-// the low mantissa bits hold the rounded product); one setp gives both
-// predicates; zero weights (padding records, unused lanes) deliver nothing.
-// No compiler memory barrier: nothing the loop reads aliases the window or
-// the accumulator.
-__device__ __forceinline__ void deliver_f16(uint32_t w, uint32_t e, float wsign,
-                                            const int32_t* acc, uint64_t pol) {
-  asm volatile(
-      "{\n\t"
-      ".reg .u32 t, l, sa, go;\n\t"
-      ".reg .b16 h, hh;\n\t"
-      ".reg .f32 hf, x;\n\t"
-      ".reg .s32 wfx;\n\t"
-      ".reg .u64 ga;\n\t"
-      ".reg .pred pon, pg, ps;\n\t"
-      "and.b32 l, %0, 2047;\n\t"
-      "shr.b32 t, %0, 17;\n\t"
-      "mov.b32 {h, hh}, t;\n\t"
-      "cvt.f32.f16 hf, h;\n\t"
-      "fma.rn.f32 x, hf, %2, 0f4B400000;\n\t"
-      "mov.b32 wfx, x;\n\t"
-      "sub.s32 wfx, wfx, 1262485504;\n\t"
-      "setp.ne.s32 pon, wfx, 0;\n\t"
-      "setp.lt.and.s32 pg|ps, %1, 0, pon;\n\t"
-      "mad.lo.u32 sa, l, 4, %1;\n\t"
-      "@ps red.shared.add.s32 [sa], wfx;\n\t"
-      "add.u32 go, %1, l;\n\t"
-      "and.b32 go, go, 2147483647;\n\t"
-      "mad.wide.u32 ga, go, 4, %3;\n\t"
-      "@pg red.global.add.L2::cache_hint.s32 [ga], wfx, %4;\n\t"
-      "}" ::"r"(w),
-      "r"(e), "f"(wsign), "l"(acc), "l"(pol));
-}
-
-// F32W record {target neuron, round(w * 2^16)}: the target's column is tested
-// against the tile's window; then one setp gives both predicates as above.
-__device__ __forceinline__ void deliver_f32(uint32_t t, int32_t wfx, const WinGeo& wg,
-                                            uint32_t win_s, const StepParams& P, uint64_t pol) {
-  const uint32_t col = div_by(t, (uint32_t)P.npc, P.npc_m);
-  const uint32_t l = t - col * (uint32_t)P.npc;
-  const uint32_t y = div_by(col, (uint32_t)P.W, P.w_m);
-  const uint32_t x = col - y * (uint32_t)P.W;
-  int rx = (int)x - wg.x0;
-  rx += rx < 0 ? P.W : 0;
-  int ry = (int)y - wg.y0;
-  ry += ry < 0 ? P.H : 0;
-  const uint32_t inwin = ((unsigned)rx < (unsigned)wg.ww && (unsigned)ry < (unsigned)wg.wh) ? 1u : 0u;
-  const uint32_t sa = win_s + 4u * (((uint32_t)ry * (uint32_t)wg.ww + (uint32_t)rx) * (uint32_t)P.npc + l);
-  const int32_t* ga = P.acc + t;
-  asm volatile(
-      "{\n\t.reg .pred pon, pg, ps;\n\t"
-      "setp.ne.s32 pon, %2, 0;\n\t"
-      "setp.eq.and.u32 ps|pg, %3, 1, pon;\n\t"
-      "@ps red.shared.add.s32 [%0], %2;\n\t"
-      "@pg red.global.add.L2::cache_hint.s32 [%1], %2, %4;\n\t}" ::"r"(sa),
-      "l"(ga), "r"(wfx), "r"(inwin), "l"(pol));
-}
-
-// A resolved item: the bucket a lane streams.
-struct Item {
-  const uint4* src;  // first 16 bytes of the bucket
-  int units;         // 32-byte sectors
-  uint32_t nbrow;    // F16W: shared address of the neighbour-table row of its column
-  float wsign;       // F16W: +-2^16, the sign of the spiker's population
+// What a warp needs of the part it streams: items a .. b - 1 of a tile.
+struct Part {
+  const unsigned char* syn;  // the tile's first row
+  const uint4* lst;          // lane b: bucket b's descriptors, less its first item's place
+  unsigned pfx;              // lane b: items of the tile before bucket b
+  unsigned a, b;
 };
 
-// Lane's item `item` of a tile part whose (column, bucket) table is
-// tab[0 .. n_entries] (none when item >= hi): item k lies in entry e (column
-// S.ccol[e / ndel], bucket e % ndel) with tab[e] <= k < tab[e + 1].  Its
-// descriptor is read here; the bucket itself is streamed by stream_items.
-template <int PREC>
-__device__ __forceinline__ Item resolve_item(const StepParams& P, unsigned item, unsigned hi,
-                                             const DeliverSmem& S, const unsigned* tab,
-                                             int n_entries, uint32_t nb_s) {
-  Item it;
-  it.src = nullptr;
-  it.units = 0;
-  it.nbrow = 0u;
-  it.wsign = 65536.0f;
-  if (item < hi) {
-    int lo_e = 0, hi_e = n_entries;  // tab[lo_e] <= item < tab[hi_e]
-    while (hi_e - lo_e > 1) {
-      const int mid = (lo_e + hi_e) >> 1;
-      if (tab[mid] <= item)
-        lo_e = mid;
-      else
-        hi_e = mid;
-    }
-    const int k = lo_e / P.ndel;
-    const int b = lo_e - k * P.ndel;
-    const int c = S.ccol[k];
-    const uint32_t* D =
-        P.desc + ((unsigned long long)S.slot[b] * (unsigned long long)P.N +
-                  (unsigned long long)c * (unsigned long long)P.npc + (item - tab[lo_e])) *
-                     (unsigned long long)P.desc_words;
-    // the descriptor: word 0 the spiker, bytes 4.. its bucket ends (units of
-    // 8 slots); bucket b spans ends[b - 1] .. ends[b] (bytes 3 + b and 4 + b)
-    const uint32_t j = D[0];
-    const int w = (3 + b) >> 2, sh = (3 + b) & 3;
-    const uint32_t lo_w = w == 0 ? j : D[w];
-    const uint32_t hi_w = sh == 3 ? D[w + 1] : 0u;
-    const uint32_t ends = __funnelshift_r(lo_w, hi_w, 8 * sh);
-    const int beg = b ? (int)(ends & 0xFFu) : 0;
-    const int end = (int)((ends >> 8) & 0xFFu);
-    // an 8-slot unit is one sector (F16W) or two (F32W)
-    it.units = (end - beg) * (PREC == SNN_EXACT_F16W ? 1 : 2);
-    const unsigned long long slot0 =
-        (unsigned long long)j * (unsigned long long)P.rowcap + (unsigned long long)beg * kSlotUnit;
-    it.src = reinterpret_cast<const uint4*>(static_cast<const char*>(P.syn) +
-                                            slot0 * (PREC == SNN_EXACT_F16W ? 4ull : 8ull));
-    it.nbrow = nb_s + (uint32_t)k * 256u;
-    it.wsign = (int)(j - (uint32_t)c * (uint32_t)P.npc) >= P.nexc ? -65536.0f : 65536.0f;
+// Item `item` of the part: its descriptor's plane and its bucket.  The
+// buckets' prefixes lie in the lanes; a five-step search over them finds the
+// last bucket that starts at or before the item.  Beyond the part: bucket -1.
+__device__ __forceinline__ int load_item(const Part& T, unsigned item, uint4* d) {
+  int lo = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1) {
+    const unsigned v = __shfl_sync(0xFFFFFFFFu, T.pfx, lo + step);
+    if (v <= item) lo += step;
   }
-  return it;
+  const unsigned long long l = __shfl_sync(0xFFFFFFFFu, (unsigned long long)T.lst, lo);
+  if (item >= T.b) return -1;
+  *d = __ldcs(reinterpret_cast<const uint4*>(l) + item);
+  return lo;
 }
 
-// One warp streams the buckets of its lanes' items as one list of 32-byte
-// sectors (F16W: 8 records; F32W: 4), dealt to the lanes in rounds of 32, so
-// no lane idles while another finishes a longer bucket.  The sector of lane L
-// in round g0 belongs to the item holding g0 plus the items that start
-// between g0 and g0 + L (a ballot and an or-reduction over the items' first
-// sectors); the item's fields come by shuffle.  The next round's sectors are
-// requested DEPTH rounds ahead of the ones being delivered.
-template <int PREC, int DEPTH>
-__device__ __forceinline__ void stream_items(const StepParams& P, const Item& it, uint32_t win_s,
-                                             const WinGeo& wg, uint64_t pol) {
-  const int lane = threadIdx.x & 31;
-  // compact the non-empty items to lanes 0 .. nit - 1
-  const unsigned cm = __ballot_sync(0xFFFFFFFFu, it.units > 0);
-  const int nit = __popc(cm);
-  if (nit == 0) return;
-  const int src = lane < nit ? (int)__fns(cm, 0u, lane + 1) : 0;
-  const unsigned long long sp = reinterpret_cast<unsigned long long>(it.src);
-  int units = __shfl_sync(0xFFFFFFFFu, it.units, src);
-  const unsigned slo = __shfl_sync(0xFFFFFFFFu, (unsigned)sp, src);
-  const unsigned shi = __shfl_sync(0xFFFFFFFFu, (unsigned)(sp >> 32), src);
-  const uint32_t nbr = __shfl_sync(0xFFFFFFFFu, it.nbrow, src);
-  const float wsg = __shfl_sync(0xFFFFFFFFu, it.wsign, src);
-  const bool mine = lane < nit;
-  if (!mine) units = 0;
-  int incl = units;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  const int pre = incl - units;  // first sector of compact item `lane`
-  const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-  const unsigned le_mask = lane == 31 ? 0xFFFFFFFFu : ((2u << lane) - 1u);
-  const int32_t* acc = P.acc;
+// Row (bits 0 .. 15) and bucket ends (units): bytes beg, mid, end of an item.
+__device__ __forceinline__ uint2 item_bounds(const uint4& d, int bucket) {
+  if (bucket < 0) return make_uint2(0u, 0u);
+  const int i = bucket % kPlaneBuckets;  // its ends: the i-th halfword of words 1 .. 3
+  const uint32_t w = i < 2 ? d.y : i < 4 ? d.z : d.w;
+  const uint32_t me = i & 1 ? w >> 16 : w & 0xFFFFu;
+  const uint32_t before = i & 1 ? w >> 8 : i == 0 ? d.x >> 16 : i == 2 ? d.y >> 24 : d.z >> 24;
+  return make_uint2(d.x & 0xFFFFu, (before & 0xFFu) | me << 8);
+}
 
-  // sector of round g0 for this lane: its two 16-byte halves and its item's fields
-  auto fetch = [&](int g0, uint4& r0, uint4& r1, uint32_t& nbrow, float& wsign) {
-    r0 = r1 = make_uint4(0u, 0u, 0u, 0u);  // weight 0: nothing delivered
-    nbrow = 0u;
-    wsign = 65536.0f;
-    if (g0 >= total) return;
-    const int ebase = __popc(__ballot_sync(0xFFFFFFFFu, mine && pre <= g0)) - 1;
-    const int pos = pre - g0;
-    const unsigned bit = (mine && pos > 0 && pos < 32) ? (1u << pos) : 0u;
-    const unsigned starts = __reduce_or_sync(0xFFFFFFFFu, bit);
-    const int e = ebase + __popc(starts & le_mask);
-    const unsigned lo = __shfl_sync(0xFFFFFFFFu, slo, e);
-    const unsigned hi = __shfl_sync(0xFFFFFFFFu, shi, e);
-    const int first = __shfl_sync(0xFFFFFFFFu, pre, e);
-    nbrow = __shfl_sync(0xFFFFFFFFu, nbr, e);
-    wsign = __shfl_sync(0xFFFFFFFFu, wsg, e);
-    const int g = g0 + lane;
-    if (g < total) {
-      const uint4* p = reinterpret_cast<const uint4*>((((unsigned long long)hi << 32) | lo)) +
-                       2 * (g - first);
-      r0 = __ldcs(p);
-      r1 = __ldcs(p + 1);
+// Sector-list entries.  F16W: sector (25 bits) | k << 25 | sign of the source
+// << 31; F32W: sector (26 bits) | k << 26.  A sector is counted from the
+// tile's first row: a tile has at most 50 176 rows of at most 255 units of 2
+// (F16W) or 4 (F32W) sectors.
+template <int PREC>
+__device__ constexpr uint32_t sector_bits() {
+  return PREC == SNN_EXACT_F16W ? 25u : 26u;
+}
+
+// One 32-byte sector of the table, read once.  The L2 fetches 64 bytes around
+// it, not the default 128: a bucket (about 270 bytes at a random place) then
+// takes about 300 bytes of DRAM traffic instead of 360 (96x96 FP16 Up state:
+// 745 us a step, 850 us with the default).  The load is predicated, not
+// branched around: a load under a branch is waited for at the branch's end,
+// which leaves one round in flight whatever the depth.
+struct Sector {
+  uint32_t w[8];
+};
+__device__ __forceinline__ void ld_sector(Sector& s, const unsigned char* p, bool on) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %9, 0;\n\t"
+      "@p ld.global.L1::no_allocate.L2::evict_first.L2::64B.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+      : "+r"(s.w[0]), "+r"(s.w[1]), "+r"(s.w[2]), "+r"(s.w[3]), "+r"(s.w[4]), "+r"(s.w[5]),
+        "+r"(s.w[6]), "+r"(s.w[7])
+      : "l"(p), "r"((uint32_t)on));
+}
+
+// Weight of an F16W record, rint(half * 2^16): one rounded multiply-add
+// (x * (+-2^16) + 1.5 * 2^23 lands in [2^23, 2^24), where the float grid is
+// the integers, so the low mantissa bits hold the rounded product).
+__device__ __forceinline__ int32_t half_fx(uint32_t half_bits, float scale) {
+  const float h = __half2float(__ushort_as_half((unsigned short)half_bits));
+  return __float_as_int(__fmaf_rn(h, scale, 12582912.0f)) - 0x4B400000;
+}
+
+// Delivers the records of one in sector: into the window at win_s (WIN), else
+// into the accumulator words of the tile at `acc`.
+template <int PREC, bool WIN>
+__device__ __forceinline__ void deliver_in(const Sector& s, uint32_t win_s, const int32_t* acc) {
+  if (PREC == SNN_EXACT_F16W) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int32_t wfx = half_fx(s.w[q] >> 16, 65536.0f);
+      if (WIN)
+        red_shared(win_s + 4u * (s.w[q] & 0xFFFFu), wfx);
+      else
+        red_add_nz(acc + (s.w[q] & 0xFFFFu), wfx);
     }
-  };
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      const int32_t wfx = (int32_t)s.w[q + 1];
+      if (WIN)
+        red_shared(win_s + 4u * s.w[q], wfx);  // a pad's bit 31 leaves the address
+      else if (wfx != 0)  // a pad's code has bit 31 set
+        red_add_nz(acc + s.w[q], wfx);
+    }
+  }
+}
 
-  // a ring of DEPTH stages: stage s holds the round g0 + 32 s and, once it
-  // has been delivered, is refilled with the round DEPTH stages later
-  uint4 a[DEPTH], b[DEPTH];
-  uint32_t nbs[DEPTH];
-  float wss[DEPTH];
+// Delivers the records of one out sector through the neighbour-table row of
+// the source's column (in shared memory for WIN, else in global memory).
+template <int PREC, bool WIN>
+__device__ __forceinline__ void deliver_out(const Sector& s, float scale, uint32_t nb_s,
+                                            const uint32_t* nb_g, const int32_t* acc) {
+  constexpr int kN = PREC == SNN_EXACT_F16W ? 8 : 4, kW = 8 / kN;
+  uint32_t base[kN];
 #pragma unroll
-  for (int st = 0; st < DEPTH; ++st) fetch(32 * st, a[st], b[st], nbs[st], wss[st]);
-  for (int g0 = 0; g0 < total; g0 += 32 * DEPTH) {
+  for (int q = 0; q < kN; ++q) {
+    const uint32_t code = s.w[kW * q];
+    if (WIN)
+      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(base[q]) : "r"(nb_s + ((code >> 9) & 0xFCu)));
+    else
+      base[q] = __ldg(nb_g + ((code >> 11) & 63u));
+  }
 #pragma unroll
-    for (int st = 0; st < DEPTH; ++st) {
-      if (g0 + 32 * st < total) {
-        if (PREC == SNN_EXACT_F16W) {
-          const uint32_t w8[8] = {a[st].x, a[st].y, a[st].z, a[st].w,
-                                  b[st].x, b[st].y, b[st].z, b[st].w};
-          uint32_t e8[8];
+  for (int q = 0; q < kN; ++q) {
+    const uint32_t code = s.w[kW * q];
+    const int32_t wfx = PREC == SNN_EXACT_F16W ? half_fx(code >> 17, scale) : (int32_t)s.w[kW * q + kW - 1];
+    red_add_nz(acc + (base[q] + (code & 2047u)), wfx);
+  }
+}
+
+// One warp streams its share of a part: batches of bs items, batch q by warp
+// q mod the block's warps (counted from warp `w0`).  WIN: the part's window
+// and neighbour table are in shared memory.
+template <int PREC, int DEPTH, bool WIN>
+__device__ __forceinline__ void stream_part(const StepParams& P, const Part& T, const int32_t* acc_t,
+                                            const uint32_t* nb_g, unsigned bs, int w0, uint32_t win_s,
+                                            uint32_t nb_s, uint32_t* list) {
+  const int lane = threadIdx.x & 31;
+  const unsigned nw = blockDim.x >> 5;
+  const unsigned warp = ((threadIdx.x >> 5) + nw - (unsigned)w0) % nw;
+  constexpr uint32_t kSecMask = (1u << sector_bits<PREC>()) - 1u;
+  static_assert(kListCap % (32 * DEPTH) == 0, "a piece of a batch is whole groups of rounds");
+  const unsigned step = bs * nw;
+  unsigned it0 = T.a + warp * bs;
+  if (it0 >= T.b) return;
+  // this lane's item of the batch at i: none beyond the batch or the part
+  auto item_at = [&](unsigned i, uint4* d) -> int {
+    return load_item(T, (unsigned)lane < bs && i < T.b ? i + lane : 0xFFFFFFFFu, d);
+  };
+  uint4 raw = make_uint4(0u, 0u, 0u, 0u);
+  int nb = item_at(it0, &raw);
+  uint2 cur = item_bounds(raw, nb);
+  for (;;) {
+    // the next batch's descriptors are loaded while this one is streamed
+    nb = item_at(it0 + step, &raw);
+    // sectors of the current batch: the in parts' at 0 .. n_in - 1, the out
+    // parts' from the next multiple of 32
+    const int beg = (int)(cur.y & 0xFFu), mid = (int)(cur.y >> 8 & 0xFFu), end = (int)(cur.y >> 16);
+    const int u_in = (mid - beg) * P.unit_sec, u_out = (end - mid) * P.unit_sec;
+    uint32_t incl = (uint32_t)u_in | (uint32_t)u_out << 16;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) e8[q] = nb_entry(w8[q], nbs[st]);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const int n_in = (int)(tot & 0xFFFFu), n_out = (int)(tot >> 16);
+    const int r_in = (n_in + 31) >> 5, rounds = r_in + ((n_out + 31) >> 5);
+    const int lim_out = r_in * 32 + n_out;
+    for (int c0 = 0; c0 < rounds * 32; c0 += kListCap) {
+      __syncwarp();
+      {
+        // this lane's entries inside [c0, c0 + kListCap)
+        const uint32_t k = div_by(cur.x, (uint32_t)P.npc, P.npc_m), l = cur.x - k * (uint32_t)P.npc;
+        uint32_t tag = cur.x * (uint32_t)P.row_sec + (uint32_t)(beg * P.unit_sec);
+        tag |= k << sector_bits<PREC>();
+        if (PREC == SNN_EXACT_F16W && (int)l >= P.nexc) tag |= 0x80000000u;
+        const int p_in = (int)(incl & 0xFFFFu) - u_in - c0;
+        const int p_out = r_in * 32 + (int)(incl >> 16) - u_out - c0;
+        for (int p = max(p_in, 0); p < min(p_in + u_in, kListCap); ++p)
+          list[p + (p >> 5)] = tag + (uint32_t)(p - p_in);
+        for (int p = max(p_out, 0); p < min(p_out + u_out, kListCap); ++p)
+          list[p + (p >> 5)] = tag + (uint32_t)(u_in + p - p_out);
+      }
+      __syncwarp();
+      const int r0 = c0 >> 5, r1 = min(rounds, r0 + (kListCap >> 5));
+      Sector sec[DEPTH] = {};
+      uint32_t en[DEPTH];
+      auto fetch = [&](int r, Sector& x, uint32_t& e) {
+        const int p = r * 32 + lane;
+        const bool on = r < r1 && p < (r < r_in ? n_in : lim_out);
+        e = on ? list[(r - r0) * 33 + lane] : 0u;
+        ld_sector(x, T.syn + (size_t)(e & kSecMask) * 32u, on);
+      };
 #pragma unroll
-          for (int q = 0; q < 8; ++q) deliver_f16(w8[q], e8[q], wss[st], acc, pol);
-        } else {
+      for (int d = 0; d < DEPTH; ++d) fetch(r0 + d, sec[d], en[d]);
+      for (int r = r0; r < r1; r += DEPTH) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint4 r = h ? b[st] : a[st];
-            deliver_f32(r.x, (int32_t)r.y, wg, win_s, P, pol);
-            deliver_f32(r.z, (int32_t)r.w, wg, win_s, P, pol);
+        for (int d = 0; d < DEPTH; ++d) {
+          const int rr = r + d;
+          if (rr < r_in) {
+            if (rr * 32 + lane < n_in) deliver_in<PREC, WIN>(sec[d], win_s, acc_t);
+          } else if (rr < r1 && rr * 32 + lane < lim_out) {
+            const uint32_t kk = PREC == SNN_EXACT_F16W ? (en[d] >> 25) & 63u : en[d] >> 26;
+            deliver_out<PREC, WIN>(sec[d], __uint_as_float(0x47800000u | (en[d] & 0x80000000u)),
+                                   nb_s + kk * 256u, nb_g + kk * 64u, P.acc);
           }
+          fetch(rr + DEPTH, sec[d], en[d]);
         }
       }
-      fetch(g0 + 32 * (st + DEPTH), a[st], b[st], nbs[st], wss[st]);
     }
+    it0 += step;
+    if (it0 >= T.b || it0 < step) break;
+    cur = item_bounds(raw, nb);
   }
-}
-
-// Adds the window's `slots` columns (n_per_col = npc words each, npc a
-// multiple of 4) into the accumulator with one bulk asynchronous reduction
-// (cp.reduce.async.bulk .add.s32, element-wise atomic in L2) per column,
-// issued by threads 0 .. slots - 1.  The shared-memory writes of every thread
-// are made visible to the bulk copies (async-proxy fence, then a barrier).
-// The copies run while the block sets up its next part; flush_wait (the
-// issuing threads wait until their copies have read the window, then a
-// barrier) must come before anything writes the window area again.
-__device__ __forceinline__ void flush_issue(const DeliverSmem& S, uint32_t win_s, int slots, int npc,
-                                            int32_t* acc, int tid) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-  if (tid < slots) {
-    const uint32_t bytes = (uint32_t)npc * 4u;
-    const uint32_t src = win_s + (uint32_t)tid * bytes;
-    int32_t* dst = acc + S.wbase[tid];
-    asm volatile(
-        "cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;\n\t"
-        "cp.async.bulk.commit_group;" ::"l"(dst),
-        "r"(src), "r"(bytes)
-        : "memory");
-  }
-}
-__device__ __forceinline__ void flush_wait(int tid, int slots) {
-  if (tid < slots) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-  __syncthreads();
 }
 
 // Delivery block vb of vgrid (NT threads) for step t.  The step's items,
-// ordered by (virtual column, delay bucket, spiker), are split into at most
-// vgrid equal contiguous ranges of at least P.min_items items; block vb
-// locates the first and last virtual column of its range from the group and
-// column counts (gsum, isum) and walks the tiles it meets.  For each tile
-// part it tabulates the (column, bucket) counts, builds the F16W neighbour
-// table, lets its warps take batches of kBatchItems items, and flushes the
-// tile's window.  Counts that disagree with the spike lists set the status
-// word instead of being delivered.  `dyn` is the block's dynamic shared
-// memory: table, neighbour table, window.
-template <int PREC, int INFL, int NT>
+// ordered by (tile, delay bucket, spiker), are split into at most vgrid
+// contiguous ranges of equal cost and at least P.min_items items each; block
+// vb locates the tiles and items its range spans from the tiles' counts (isum)
+// and walks the tiles that have items.  A tile's part with at least
+// P.win_items items is delivered through the shared-memory window, a smaller
+// one without any block-wide set-up.  Counts that disagree with the spike
+// lists set the status word; items beyond the lists are not delivered.
+// `dyn` is the block's dynamic shared memory: window, neighbour table, sector
+// lists.
+template <int PREC, int DEPTH, int NT>
 __device__ __forceinline__ void deliver_body(const StepParams& P, long long t, int vb, int vgrid,
                                              DeliverSmem& S, unsigned char* dyn) {
   __syncthreads();  // the shared memory may still be read by a previous body
   const int tid = threadIdx.x;
   const int lane = tid & 31;
-  const int warp = tid >> 5;
-  unsigned* const tab_w = reinterpret_cast<unsigned*>(dyn);  // windowed parts
-  uint32_t* const nb_w = tab_w + tab_words(P, P.tile * P.tile);
-  int32_t* const win = reinterpret_cast<int32_t*>(nb_w + nb_words<PREC>(P.tile * P.tile));
-  unsigned* const tab_s = reinterpret_cast<unsigned*>(win);  // parts without window
-  uint32_t* const nb_s_ = tab_s + tab_words(P, P.part_cols);
-  // the slot that the next update fills holds step t - d_max: no longer read
-  const long long next_slot = (t + 1) % P.nslot;
-  if (vb == 0 && tid == 0) P.cnt[next_slot] = 0u;
-  for (long long c = (long long)vb * NT + tid; c < P.ncol; c += (long long)vgrid * NT)
-    P.ccnt[next_slot * P.ncol + c] = 0u;
-  if (tid < kMaxDelays) {
-    const int b = tid;
-    const long long s = t + 1 - (P.dmin + b);
-    S.slot[b] = (b < P.ndel && s >= 0) ? (int)(s % P.nslot) : -1;
-  }
-  if (tid == 0) {
-    S.v0 = -1;
-    S.v1 = -1;
-    S.xg[0] = S.xg[1] = -1;
-    S.next = 0u;
-  }
+  constexpr int kWarps = NT / 32;
+  int32_t* const win = reinterpret_cast<int32_t*>(dyn);
+  const int win_words = P.tcols * P.npc4;
+  uint32_t* const nbs = reinterpret_cast<uint32_t*>(win + win_words);
+  uint32_t* const list = nbs + P.tcols * 64 + (tid >> 5) * kListWords;
 
-  // the block's item range, from the group counts.  The ranges split the
-  // step's cost evenly: a group of 32 virtual columns costs its items plus a
-  // fixed part (P.cost_win when its items reach the window threshold -- the
-  // set-up and flush of a windowed part -- else P.cost_part when it has
-  // items), laid out before the group's items; a cost point maps to the item
-  // position it falls on (the group's first item while in the fixed part).
-  // The mapping is monotone, so consecutive blocks' ranges tile the items.
-  const int ngrp = (P.ncol + 31) >> 5;
-  const int per = (ngrp + NT - 1) / NT;
+  // The block's item range.  The ranges split the step's cost evenly: a tile
+  // costs its items plus a fixed part (P.cost_win when its items reach the
+  // window threshold -- the set-up and flush of the window -- else
+  // P.cost_part when it has items), laid out before the tile's items; a cost
+  // point maps to the item it falls on (the tile's first item while in the
+  // fixed part).  The mapping is monotone, so consecutive blocks' ranges tile
+  // the items.
+  const int per = (P.ntile + NT - 1) / NT;
   const int g0 = tid * per;
-  auto group_cost = [&](unsigned v) -> unsigned long long {
+  // items of a tile: isum, and with d_min = 1 those of step t
+  const unsigned* const now = P.dmin == 1 ? P.ccnt + (t % P.nslot) * P.ntile * kCntStride : nullptr;
+  auto tile_items = [&](int g) -> unsigned {
+    return P.isum[(long long)g * kCntStride] + (now ? now[(long long)g * kCntStride] : 0u);
+  };
+  auto tile_cost = [&](unsigned v) -> unsigned long long {
     return (unsigned long long)v + (v >= P.win_items ? P.cost_win : (v ? P.cost_part : 0u));
   };
-  unsigned long long mine = 0ull, mcost = 0ull;
-  for (int g = g0; g < g0 + per && g < ngrp; ++g) {
-    const unsigned v = P.gsum[g];
-    mine += v;
-    mcost += group_cost(v);
+  unsigned long long items = 0ull, cost = 0ull, old = 0ull;
+  for (int g = g0; g < g0 + per && g < P.ntile; ++g) {
+    const unsigned v = tile_items(g);
+    items += v;
+    old += P.isum[(long long)g * kCntStride];
+    cost += tile_cost(v);
   }
-  unsigned long long total = 0ull, ctotal = 0ull;
-  const unsigned long long excl = block_scan(mine, S, &total);
-  const unsigned long long cexcl = block_scan(mcost, S, &ctotal);
+  const unsigned want_total = *P.gsum;
+  // lane b: the slot of bucket b's step (-1: before step 0)
+  int slot_l = -1;
+  {
+    const long long s = t + 1 - (P.dmin + lane);
+    if (lane < P.ndel && s >= 0) slot_l = (int)(s % P.nslot);
+  }
+  // the slot that the next update fills holds step t - d_max: no longer read
+  const long long next_slot = (t + 1) % P.nslot;
+  for (long long c = (long long)vb * NT + tid; c < P.ntile; c += (long long)vgrid * NT)
+    P.ccnt[(next_slot * P.ntile + c) * kCntStride] = 0u;
+  unsigned long long cexcl = 0ull, ctotal = 0ull, total = 0ull, old_total = 0ull;
+  block_scan3(cost, items, old, S, &cexcl, &ctotal, &total, &old_total);
+  if (vb == 0 && tid == 0 && (unsigned)old_total != want_total) set_status(P, kStatusCounts);
   const unsigned long long want = (total + P.min_items - 1) / P.min_items;
-  const int nact = (int)(want < (unsigned long long)vgrid ? (want ? want : 1ull) : (unsigned long long)vgrid);
+  const int nact = (int)(want < (unsigned long long)vgrid ? want : (unsigned long long)vgrid);
   if (vb >= nact) return;
+#pragma unroll
   for (int i = 0; i < 2; ++i) {
     const unsigned long long x = ctotal * (unsigned long long)(vb + i) / (unsigned long long)nact;
     if (x >= ctotal) {
-      if (tid == 0) S.ipt[i] = total;
-    } else if (x >= cexcl && x < cexcl + mcost) {
-      unsigned long long rc = cexcl, ri = excl;
-      for (int g = g0; g < g0 + per && g < ngrp; ++g) {
-        const unsigned v = P.gsum[g];
-        const unsigned long long c = group_cost(v);
+      if (tid == 0) {
+        S.rt[i] = P.ntile;
+        S.ri[i] = 0u;
+      }
+    } else if (x >= cexcl && x < cexcl + cost) {
+      unsigned long long rc = cexcl;
+      for (int g = g0; g < g0 + per && g < P.ntile; ++g) {
+        const unsigned v = tile_items(g);
+        const unsigned long long c = tile_cost(v);
         if (x < rc + c) {
+          S.rt[i] = g;
           const unsigned long long fixed = c - v;
-          S.ipt[i] = ri + (x - rc > fixed ? x - rc - fixed : 0ull);
+          S.ri[i] = x - rc > fixed ? (unsigned)(x - rc - fixed) : 0u;
           break;
         }
         rc += c;
-        ri += v;
       }
     }
   }
+  // the window is cleared while the range is found
+  for (int i = tid; i < win_words >> 2; i += NT) reinterpret_cast<int4*>(win)[i] = make_int4(0, 0, 0, 0);
   __syncthreads();
-  const unsigned long long lo = S.ipt[0];
-  const unsigned long long hi = S.ipt[1];
-  if (lo >= hi) return;
-  for (int i = 0; i < 2; ++i) {
-    const unsigned long long x = i == 0 ? lo : hi - 1;
-    if (x >= excl && x < excl + mine) {
-      unsigned long long run = excl;
-      for (int g = g0; g < g0 + per && g < ngrp; ++g) {
-        const unsigned v = P.gsum[g];
-        if (x < run + v) {
-          S.xg[i] = g;
-          S.xgp[i] = run;
-          break;
-        }
-        run += v;
-      }
-    }
-  }
-  __syncthreads();
-  // the virtual columns holding lo and hi - 1, from the column counts of their groups
-  if (warp < 2 && S.xg[warp] >= 0) {
-    const unsigned long long x = warp == 0 ? lo : hi - 1;
-    const int c = S.xg[warp] * 32 + lane;
-    const unsigned v = c < P.ncol ? P.isum[c] : 0u;
-    unsigned incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    const unsigned long long pos = S.xgp[warp] + incl - v;
-    if (c < P.ncol && x >= pos && x < pos + v) {
-      if (warp == 0) {
-        S.v0 = c;
-        S.p0 = pos;
-      } else {
-        S.v1 = c;
-      }
-    }
-  }
-  __syncthreads();
-  const int v0 = S.v0, v1 = S.v1;
-  if (v0 < 0 || v1 < v0) {
-    if (tid == 0) set_status(P, kStatusCounts);
-    return;
-  }
+  const int t0 = S.rt[0], t1 = S.rt[1];
+  const unsigned i0 = S.ri[0], i1 = S.ri[1];
 
-  const uint64_t pol = evict_last_policy();
   const uint32_t win_s = (uint32_t)__cvta_generic_to_shared(win);
-  unsigned long long pbase = S.p0;  // items before the tile part's first column
-  unsigned long long covered = 0ull;  // items of the range found in the spike lists
-  bool win_zero = false;              // the window has been cleared in this body
-  int fl_slots = 0;                   // threads whose window flush may still read the window
-  for (int v = v0; v <= v1;) {
-    // the part's extent: one tile whose items in the range reach the window
-    // threshold (delivered through the window), else a run of consecutive
-    // tiles below it, at most P.part_cols columns (delivered without one)
-    if (warp == 0) {
-      int e = v, tiles = 0;
-      bool wnd = false;
-      unsigned long long pb = pbase;  // items before column e
-      while (e <= v1) {
-        const TileGeo gt = tile_geo(P, e);
-        const int te = min(v1, gt.first + gt.tw * gt.th - 1);
-        if (tiles > 0 && te - v + 1 > P.part_cols) break;
-        unsigned x = 0u;
-        for (int c = e + lane; c <= te; c += 32) x += P.isum[c];
-        x = __reduce_add_sync(0xFFFFFFFFu, x);
-        const unsigned long long lo_in = pb > lo ? pb : lo;
-        const unsigned long long hi_in = pb + x < hi ? pb + x : hi;
-        const unsigned long long in = hi_in > lo_in ? hi_in - lo_in : 0ull;
-        if (P.agg && in >= P.win_items) {
-          if (tiles == 0) {
-            wnd = true;
-            e = te + 1;
-          }
-          break;
-        }
-        pb += x;
-        e = te + 1;
-        ++tiles;
-      }
-      if (lane == 0) {
-        S.pe = e;
-        S.pwin = wnd ? 1 : 0;
-      }
-    }
-    __syncthreads();
-    const int ve = S.pe - 1;
-    const bool windowed = S.pwin != 0;
-    unsigned* const tab = windowed ? tab_w : tab_s;
-    uint32_t* const nb = windowed ? nb_w : nb_s_;
-    const uint32_t nb_s = (uint32_t)__cvta_generic_to_shared(nb);
-    if (!windowed) win_zero = false;  // the tables overwrite the window area
-    const TileGeo g = tile_geo(P, v);
-    const int ncv = ve - v + 1;
-    const int n_entries = ncv * P.ndel;
-    for (int k = tid; k < ncv; k += NT) {
-      const int c = (int)P.vcol[v + k];
-      const int cy = c / P.W;
-      S.ccol[k] = c;
-      S.cx[k] = c - cy * P.W;
-      S.cy[k] = cy;
-    }
-    __syncthreads();
-    // tabulate the tile part: consecutive entries per thread
-    constexpr int kEpt = (kMaxTileCols * kMaxDelays + NT - 1) / NT;
-    const int ept = (n_entries + NT - 1) / NT;
-    unsigned cnt[kEpt];
-    unsigned sum = 0u;
+  const uint32_t nb_s = (uint32_t)__cvta_generic_to_shared(nbs);
+  bool clean = true;      // the window is clear and no flush reads it
+  int rot = 0;            // first warp of the next part without window
+  for (int c0 = t0; c0 <= t1 && c0 < P.ntile; c0 += 32) {
+    const unsigned xs = c0 + lane < P.ntile ? tile_items(c0 + lane) : 0u;
+    unsigned have = __ballot_sync(0xFFFFFFFFu, xs != 0u && c0 + lane <= t1);
+    while (have) {
+      const int m = __ffs(have) - 1;
+      have &= have - 1u;
+      const int tile = c0 + m;
+      const unsigned x = __shfl_sync(0xFFFFFFFFu, xs, m);
+      const unsigned a = tile == t0 ? i0 : 0u;
+      const unsigned b = tile == t1 ? min(i1, x) : x;
+      if (a >= b) continue;
+      // the tile's counts per bucket; a list holds at most tcap spikes
+      const long long ts = (long long)slot_l * P.ntile + tile;
+      const unsigned n = slot_l >= 0 ? min(P.ccnt[ts * kCntStride], (unsigned)P.tcap) : 0u;
+      const uint2 ti = P.tinfo[tile];
+      unsigned incl = n;
 #pragma unroll
-    for (int q = 0; q < kEpt; ++q) {
-      const int e = tid * ept + q;
-      unsigned c = 0u;
-      if (q < ept && e < n_entries) {
-        const int k = e / P.ndel;
-        const int sl = S.slot[e - k * P.ndel];
-        c = sl >= 0 ? P.ccnt[(long long)sl * P.ncol + S.ccol[k]] : 0u;
-        c = min(c, (unsigned)P.npc);  // a column lists at most n_per_col spikes
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += u;
       }
-      cnt[q] = c;
-      sum += c;
-    }
-    unsigned long long ptotal = 0ull;
-    unsigned run = (unsigned)block_scan(sum, S, &ptotal);
-    if (!windowed && fl_slots) {  // this part's tables go into the window area
-      flush_wait(tid, fl_slots);
-      fl_slots = 0;
-    }
-#pragma unroll
-    for (int q = 0; q < kEpt; ++q) {
-      const int e = tid * ept + q;
-      if (q < ept && e < n_entries) tab[e] = run;
-      run += cnt[q];
-    }
-    if (tid == 0) tab[n_entries] = (unsigned)ptotal;
-    // the block's items of this part; a part with few items skips the window
-    // (clearing and flushing it would cost more than it saves)
-    const unsigned a = lo > pbase ? (unsigned)(lo - pbase) : 0u;
-    const unsigned b = hi > pbase ? (unsigned)min(hi - pbase, ptotal) : 0u;
-    covered += b > a ? b - a : 0u;
-    const WinGeo wg = win_geo(P, g, windowed);
-    if (windowed && fl_slots) {
-      flush_wait(tid, fl_slots);
-      fl_slots = 0;
-    }
-    if (windowed && !win_zero) {
-      for (int i = tid; i < (P.win_cap >> 2); i += NT) reinterpret_cast<int4*>(win)[i] = make_int4(0, 0, 0, 0);
-      win_zero = true;
-    }
-    for (int m = tid; m < wg.ww * wg.wh; m += NT) {
-      const int ry = m / wg.ww, rx = m - ry * wg.ww;
-      int x = wg.x0 + rx, y = wg.y0 + ry;
-      x -= x >= P.W ? P.W : 0;
-      y -= y >= P.H ? P.H : 0;
-      S.wbase[m] = ((uint32_t)y * (uint32_t)P.W + (uint32_t)x) * (uint32_t)P.npc;
-    }
-    if (PREC == SNN_EXACT_F16W && b > a) {
-      // the column at each stencil offset of each column of the part: its
-      // shared-window address, or bit 31 set and its first neuron in the
-      // accumulator (offsets with dx + 3 = 7 belong to padding records)
-      for (int m = tid; m < ncv * 64; m += NT) {
-        const int k = m >> 6, off = m & 63;
-        const int tx = wrap(S.cx[k] + (off & 7) - 3, P.W);
-        const int ty = wrap(S.cy[k] + (off >> 3) - 3, P.H);
-        int rx = tx - wg.x0;
-        rx += rx < 0 ? P.W : 0;
-        int ry = ty - wg.y0;
-        ry += ry < 0 ? P.H : 0;
-        nb[m] = (rx < wg.ww && ry < wg.wh)
-                    ? win_s + 4u * (((uint32_t)ry * (uint32_t)wg.ww + (uint32_t)rx) * (uint32_t)P.npc)
-                    : 0x80000000u | (((uint32_t)ty * (uint32_t)P.W + (uint32_t)tx) * (uint32_t)P.npc);
-      }
-    }
-    __syncthreads();
-    // the counts of each column must equal the items the range assumed
-    if (tid < ncv && tab[(tid + 1) * P.ndel] - tab[tid * P.ndel] != P.isum[v + tid])
-      set_status(P, kStatusCounts);
-    // warps claim batches of kBatchItems items; a warp resolves its next
-    // batch (descriptor loads) before it streams the current one
-    if (a < b) {
-      unsigned k0 = 0u;
-      if (lane == 0) k0 = atomicAdd(&S.next, (unsigned)kBatchItems);
-      k0 = a + __shfl_sync(0xFFFFFFFFu, k0, 0);
-      Item cur = resolve_item<PREC>(P, k0 + lane, b, S, tab, n_entries, nb_s);
-      while (k0 < b) {
-        unsigned k1 = 0u;
-        if (lane == 0) k1 = atomicAdd(&S.next, (unsigned)kBatchItems);
-        k1 = a + __shfl_sync(0xFFFFFFFFu, k1, 0);
-        const Item nxt = resolve_item<PREC>(P, k1 + lane, b, S, tab, n_entries, nb_s);
-        stream_items<PREC, INFL>(P, cur, win_s, wg, pol);
-        cur = nxt;
-        k0 = k1;
-      }
-    }
-    const uint32_t wlen = (uint32_t)(wg.ww * wg.wh) * (uint32_t)P.npc;
-    __syncthreads();  // every warp is done with the part
-    if ((P.npc & 3) == 0) {
-      // bulk flush: each window slot (one column, n_per_col words, 16-byte
-      // aligned in both memories) is added into the accumulator by one
-      // asynchronous bulk reduction, which overlaps the next part's set-up;
-      // the window is cleared again before a later part uses it
-      if (windowed) {
-        flush_issue(S, win_s, wg.ww * wg.wh, P.npc, P.acc, tid);
-        fl_slots = wg.ww * wg.wh;
-        win_zero = false;
-      }
-    } else {
-      // flush the window with coalesced reductions, leaving it zeroed: word
-      // m is neuron l of slot s; (s, l) advance with m
-      uint32_t fs = div_by((uint32_t)tid, (uint32_t)P.npc, P.npc_m);
-      uint32_t fl = (uint32_t)tid - fs * (uint32_t)P.npc;
-      for (uint32_t m = tid; m < wlen; m += NT) {
-        const int32_t x = win[m];
-        if (x) {
-          red_add(P.acc + S.wbase[fs] + fl, x, pol);
-          win[m] = 0;
+      const unsigned found = __shfl_sync(0xFFFFFFFFu, incl, 31);
+      if (found != x && tid == 0) set_status(P, kStatusCounts);
+      Part T;
+      T.syn = static_cast<const unsigned char*>(P.syn) + (size_t)ti.x * P.npc * P.row_sec * 32u;
+      T.pfx = lane < P.ndel ? incl - n : 0xFFFFFFFFu;
+      T.lst = P.list + ((((long long)slot_l * P.planes + lane / kPlaneBuckets) * P.ntile + tile) * P.tcap -
+                        (long long)T.pfx);
+      int32_t* const acc_t = P.acc + (size_t)ti.x * P.npc4;
+      const uint32_t* nb_g = P.nbg + (size_t)ti.x * 64;
+      const int cols = (int)ti.y;
+      T.a = a;
+      T.b = min(b, found);
+      if (P.agg && b - a >= P.win_items) {
+        if (!clean) {
+          // the issuing threads' bulk reductions have read the window
+          if (tid < P.tcols) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          __syncthreads();
+          for (int i = tid; i < (cols * P.npc4) >> 2; i += NT)
+            reinterpret_cast<int4*>(win)[i] = make_int4(0, 0, 0, 0);
         }
-        fl += NT;
-        while (fl >= (uint32_t)P.npc) {
-          fl -= (uint32_t)P.npc;
-          ++fs;
+        for (int i = tid; i < cols * 16; i += NT)
+          reinterpret_cast<uint4*>(nbs)[i] = __ldg(reinterpret_cast<const uint4*>(nb_g) + i);
+        __syncthreads();
+        // about four batches per warp, so that none waits long for the last
+        unsigned bs = (b - a) / (4u * kWarps);
+        bs = bs < 4u ? 4u : (bs > 32u ? 32u : bs);
+        stream_part<PREC, DEPTH, true>(P, T, acc_t, nb_g, bs, 0, win_s, nb_s, list);
+        // add the window to the accumulator: one asynchronous bulk reduction
+        // (element-wise atomic in L2) per column, issued once every warp's
+        // reductions are visible to the async proxy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid < cols) {
+          const uint32_t bytes = (uint32_t)P.npc4 * 4u;
+          asm volatile(
+              "cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;\n\t"
+              "cp.async.bulk.commit_group;" ::"l"(acc_t + (size_t)tid * P.npc4),
+              "r"(win_s + (uint32_t)tid * bytes), "r"(bytes)
+              : "memory");
         }
+        clean = false;
+      } else {
+        // few items: every warp takes batches of its own, as many as fill the block
+        const unsigned nit = T.b > T.a ? T.b - T.a : 0u;
+        unsigned bs = (nit + kWarps - 1) / kWarps;
+        bs = bs < 4u ? 4u : (bs > 32u ? 32u : bs);
+        stream_part<PREC, DEPTH, false>(P, T, acc_t, nb_g, bs, rot, win_s, nb_s, list);
+        rot = (int)((rot + (nit + bs - 1) / bs) % kWarps);
       }
     }
-    if (tid == 0) S.next = 0u;
-    pbase += ptotal;
-    v = ve + 1;
-    __syncthreads();
   }
   // the body's bulk reductions must have been performed (not only have read
   // the window) before it ends: the batch kernel's next phase reads the
   // accumulator after a grid barrier
-  if (tid < (kMaxTile + 2) * (kMaxTile + 2)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-  __syncthreads();
-  // every item of the range must have been found in the spike lists
-  if (tid == 0 && covered != hi - lo) set_status(P, kStatusCounts);
+  if (tid < P.tcols) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 template <int PREC>
 __global__ void __launch_bounds__(kDeliverThreads, 1) deliver_kernel(const StepParams P) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ DeliverSmem S;
-  const long long t = P.ctl->t;
-  deliver_body<PREC, PREC == SNN_EXACT_F16W ? kDepthF16 : kDepthF32, kDeliverThreads>(
-      P, t, (int)blockIdx.x, (int)gridDim.x, S, s_dyn);
-
-  // the last block to finish closes the step
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned prev = atomicAdd(&P.ctl->done, 1u);
-    if (prev == gridDim.x - 1) {
-      __threadfence();
-      P.ctl->done = 0u;
-      P.ctl->t = t + 1;
-    }
-  }
+  const long long t = P.ctl->td;
+  if (blockIdx.x == 0 && threadIdx.x == 0) P.ctl->t = t + 1;  // the next update's step
+  deliver_body<PREC, kDepth, kDeliverThreads>(P, t, (int)blockIdx.x, (int)gridDim.x, S, s_dyn);
 }
 
 // ---------------------------------------------------------------------------
@@ -1331,12 +1084,17 @@ __global__ void __launch_bounds__(256) drain_records_kernel(
   }
 }
 
+// Writes the descriptor of neuron l of column c at place `at` of a list
+// (plane 0; the other planes follow at the stride of all tiles' lists).
+__device__ __forceinline__ void list_spike(const StepParams& P, long long at, uint32_t c, uint32_t l) {
+  const uint4* d = P.bend + ((size_t)P.colv[c] * P.npc + l) * P.planes;
+  const long long stride = (long long)P.ntile * P.tcap;
+  for (int p = 0; p < P.planes; ++p) P.list[at + p * stride] = d[p];
+}
+
 // Shard: the received spikes of step t (global indices ids[0 .. n)) that
-// belong to halo columns join the step's per-column lists as the update
-// kernel's own spikes do -- a descriptor {local index, bucket ends} at the
-// next position of the column's list and, with d_min = 1, one more item for
-// the column in this step's delivery (with d_min >= 2 the update kernel of
-// step t + d_min - 1 moves the column's count in).  Indices of the shard's
+// belong to halo columns join the step's lists as the update kernel's own
+// spikes do, at the next place of the tile's list.  Indices of the shard's
 // own columns and of columns outside its local grid are skipped.  An index
 // beyond the global network, or more than n_per_col spikes for one column
 // (a duplicated index), is skipped and sets the status word.
@@ -1360,25 +1118,15 @@ __global__ void __launch_bounds__(256) ingest_kernel(const StepParams P, const u
     if (lx >= P.W || ly >= P.H) continue;  // not in the local grid
     if (lx >= P.sg.tx0 && lx < P.sg.tx0 + P.sg.tw && ly >= P.sg.ty0 && ly < P.sg.ty0 + P.sg.th)
       continue;  // an own column: listed by the update kernel
-    const int c = ly * P.W + lx;
-    const unsigned r = atomicAdd(P.ccnt + slot * P.ncol + c, 1u);
-    if (r >= (unsigned)P.npc) {
+    if (atomicAdd(P.icnt + ly * P.W + lx, 1u) >= (unsigned)P.npc) {
       set_status(P, kStatusIngest);
       continue;
     }
-    const uint32_t id = (uint32_t)c * (uint32_t)P.npc + l;
-    uint4* d = reinterpret_cast<uint4*>(
-        P.desc + ((long long)slot * P.N + (long long)c * P.npc + r) * P.desc_words);
-    const uint4* be = reinterpret_cast<const uint4*>(P.bend + (long long)id * kBendStride);
-    const uint4 a = be[0], b = be[1];
-    d[0] = make_uint4(id, a.x, a.y, a.z);
-    d[1] = make_uint4(a.w, b.x, b.y, b.z);
-    if (P.desc_words == 16) d[2] = make_uint4(b.w, 0u, 0u, 0u);
-    if (P.dmin == 1) {
-      const unsigned v = P.colv[c];
-      atomicAdd(P.isum + v, 1u);
-      atomicAdd(P.gsum + (v >> 5), 1u);
-    }
+    // at most n_per_col spikes of each of its columns: the list has room
+    const uint32_t ct = P.ctile[ly * P.W + lx];
+    const long long tile_slot = slot * P.ntile + (ct >> 6);
+    const unsigned r = next_place(P.ccnt + tile_slot * kCntStride, ct >> 6);
+    list_spike(P, (slot * P.planes * P.ntile + (ct >> 6)) * P.tcap + r, (uint32_t)(ly * P.W + lx), l);
   }
 }
 
@@ -1417,41 +1165,26 @@ cudaError_t launch_ingest(const StepParams& p, const uint32_t* ids, long long n,
   return cudaGetLastError();
 }
 
-size_t deliver_smem(const StepParams& p, int precision) {
-  auto tables = [&](size_t cols) {
-    const size_t tabw = (cols * (size_t)p.ndel + 1 + 3) & ~(size_t)3;
-    return tabw + (precision == SNN_EXACT_F16W ? cols * 64 : 0);
-  };
-  // windowed-part tables, then the window area (which also holds the tables
-  // of a part without window)
-  const size_t area = std::max((size_t)p.win_cap, tables((size_t)p.part_cols));
-  return (tables((size_t)p.tile * p.tile) + area) * 4;
+size_t deliver_smem(int cols, int npc4, bool batch) {
+  const int warps = (batch ? kBatchThreads : kDeliverThreads) / 32;
+  return ((size_t)cols * npc4 + (size_t)cols * 64 + (size_t)warps * kListWords) * 4;
 }
-
-int deliver_threads() { return kDeliverThreads; }
 
 // Delivery grid: one block per SM (a persistent grid).
 int deliver_grid(const StepParams& p, int precision, int num_sms) {
-  const size_t smem = deliver_smem(p, precision);
+  const size_t smem = deliver_smem(p.tcols, p.npc4, false);
+  const void* fn = precision == SNN_EXACT_F16W
+                       ? reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F16W>)
+                       : reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F32W>);
   int per_sm = 0;
-  if (precision == SNN_EXACT_F16W) {
-    if (cudaFuncSetAttribute(deliver_kernel<SNN_EXACT_F16W>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, deliver_kernel<SNN_EXACT_F16W>,
-                                                  kDeliverThreads, smem);
-  } else {
-    if (cudaFuncSetAttribute(deliver_kernel<SNN_EXACT_F32W>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, deliver_kernel<SNN_EXACT_F32W>,
-                                                  kDeliverThreads, smem);
-  }
-  return per_sm * num_sms;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kDeliverThreads, smem);
+  return per_sm > 0 ? num_sms : 0;
 }
 
 cudaError_t launch_deliver(const StepParams& p, int precision, int grid, cudaStream_t st) {
-  const size_t smem = deliver_smem(p, precision);
+  const size_t smem = deliver_smem(p.tcols, p.npc4, false);
   if (precision == SNN_EXACT_F16W)
     deliver_kernel<SNN_EXACT_F16W><<<grid, kDeliverThreads, smem, st>>>(p);
   else
