@@ -230,9 +230,6 @@ int validate(int gw, int gh, const snn_neuron_params* n, const snn_synapse_param
 // each column is flushed once per part) beats a 4x4 tile with a ring of one
 // (88 %, but 36 window columns flushed per 16 columns of spikes) by 13 %, 17 %
 // and 3 %; 5x5 and 4x4 tiles without ring and 3x3 with a ring are slower still.
-constexpr size_t kSmemBudget = 224 * 1024;
-constexpr size_t kBatchSmemBudget = 110 * 1024;
-constexpr size_t kWindowBudget = 196 * 1024;
 // Fewest items a delivery block takes (fewer blocks run when a step has few
 // items).
 constexpr unsigned kMinItems = 64;
@@ -640,6 +637,9 @@ int net_view(snn_net* net, NetView* v) {
   v->ctile = net->ctile;
   v->colv = net->colv;
   v->nbg = net->nbg;
+  v->tinfo = net->tinfo;
+  v->ntile = net->ntile;
+  v->tcols = net->tw * net->th;
   v->nexc = net->nexc;
   v->dmin = net->dmin;
   v->ndel = net->ndel;

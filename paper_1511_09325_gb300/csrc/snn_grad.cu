@@ -22,19 +22,21 @@
 // Forward: grad_deliver_kernel (one warp per source row, pull by delay: the
 // input of step t is every bucket d of every row weighted by s_j(t - d), summed
 // as int64 fixed point in 2^-32 mV, so the sums do not depend on the order;
-// rows whose last d_max spikes are all zero leave after one load)
+// a row whose last d_max spikes are all zero leaves after one load of their bit
+// mask)
 // and grad_update_kernel (one thread per neuron; hard mode is the spiking
 // model's arithmetic, one float rounding per operation).  The state (V, c and
 // the spike history of d_max + 1 steps) is checkpointed every `ckpt` steps.
 // Backward: segment by segment from the end, the forward is recomputed from
 // the segment's checkpoint while a tape of eight values per neuron and step is
 // recorded, then the adjoint recursion runs back through the segment:
-// grad_gather_kernel (one warp per source row: the adjoint of the delayed
-// delivery is a gather over the row's outgoing synapses of the targets' input
-// adjoints at t + d, in a fixed order) and grad_backward_kernel (one thread per
-// neuron: the adjoint of every line above; parameter partials accumulate per
-// neuron in FP64 and are summed on the host in a fixed order).  Every sum has a
-// fixed order, so a run is reproducible bit for bit.
+// grad_gather_kernel (the adjoint of the delayed delivery is a gather over
+// every row's outgoing synapses of the targets' input adjoints at t + d; one
+// block per delay bucket and run of rows, in a fixed order) and
+// grad_backward_kernel (one thread per neuron: the adjoint of every line above;
+// parameter partials accumulate per neuron in FP64 and are summed in a
+// fixed order).  Every sum has a fixed order, so a run is reproducible bit
+// for bit.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -61,6 +63,7 @@ struct GradParams {
   const uint32_t* ctile;      // geometry of the net (see snn_internal.h)
   const uint32_t* colv;
   const uint32_t* nbg;
+  const uint2* tinfo;
   uint32_t seed_lo, seed_hi;
   float beta, theta, vr, dc, pvv, pcc, pvc_e, pvc_i, kappa, J, lam, sqlam;
   float a[4];  // a_EE, a_EI, a_IE, a_II
@@ -71,6 +74,8 @@ struct GradParams {
   float* V;
   float* C;
   float* shist;               // [nslot][N] s of the last nslot steps
+  uint32_t* active;           // [N] bit d - 1: s(t - d) != 0 (t the step due next)
+  uint32_t bucket_mask;       // ndel low bits
   unsigned long long* xe;     // [accw] input sums from E sources, 2^-32 mV, acc order
   unsigned long long* xin;    // [accw] the same from I sources
   float* tape;                // [ckpt][kTape][N]
@@ -80,8 +85,9 @@ struct GradParams {
   float* ibe;                 // [nslot][accw] a[E][p_i] * adjoint of I_i(t), acc order
   float* ibi;                 // [nslot][accw] a[I][p_i] * adjoint of I_i(t)
   float* gb;                  // [3][N] -adjoint of g_i(t) where the gate is open
-  float* sg;                  // [N] gathered adjoint of s_j(t) through its synapses
+  float* part;                // [ndel][N] gathered adjoints of s_j(t) per bucket, rows in table order
   double* gacc;               // [6][N] parameter partials per neuron
+  double* gsum;               // [6] their sums
 };
 
 // Ring position of step s >= 0 (steps are below 2^31: 32-bit remainder).
@@ -106,6 +112,7 @@ __global__ void __launch_bounds__(kThreads) grad_init_kernel(const GradParams P)
   const uint32_t u = (i & 3) == 0 ? x.x : (i & 3) == 1 ? x.y : (i & 3) == 2 ? x.z : x.w;
   P.V[i] = __fmul_rn(P.theta, __fmul_rn(__uint2float_rn(u >> 8), kTwoM24));
   P.C[i] = 0.f;
+  P.active[i] = 0u;
 }
 
 // Word of neuron i in arrays in acc order.
@@ -159,27 +166,25 @@ __device__ __forceinline__ int bucket_of(int k, int end_lane, int ndel) {
 }
 
 // Input of step t: every bucket d of every source row j, weighted by
-// s_j(t - d), into the row's population accumulator.  One warp per row: the
-// lanes first load the row's ndel spike values at once and the warp leaves
-// when all are zero; otherwise it streams the row four records per lane
-// (16-byte loads; a bucket is a whole number of 8-slot units, so the four
-// records of a lane share a bucket).
+// s_j(t - d), into the row's population accumulator.  One warp per row: P.active
+// holds, per neuron, a bit d - 1 for every d with s(t - d) != 0, and the warp
+// leaves after one load when no bucket has a spike; otherwise it streams the
+// row four records per lane (16-byte loads; a bucket part is a whole number of
+// 8-slot units, so the four records of a lane share it).
 __global__ void __launch_bounds__(kThreads) grad_deliver_kernel(const GradParams P, long long t) {
   const long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (j >= P.N) return;
+  const uint32_t act = (P.active[j] >> (P.dmin - 1)) & P.bucket_mask;
+  if (act == 0u) return;
+  const GradRow R = grad_row(P, j);
   float s_lane = 0.f;
   int end_lane = 0x7FFFFFFF, mid_lane = 0;
-  if (lane < P.ndel) {
-    const long long src = t - (P.dmin + lane);
-    s_lane = src >= 0 ? P.shist[ring(src, P.nslot) * P.N + j] : 0.f;
-  }
-  if (__ballot_sync(0xFFFFFFFFu, s_lane != 0.f) == 0u) return;
-  const GradRow R = grad_row(P, j);
   if (lane < P.ndel) {
     const uint32_t e = *reinterpret_cast<const uint16_t*>(R.ends + desc_end(lane));
     mid_lane = (int)(e & 0xFFu) * P.unit;
     end_lane = (int)(e >> 8) * P.unit;
+    if (act >> lane & 1u) s_lane = P.shist[ring(t - (P.dmin + lane), P.nslot) * P.N + j];
   }
   unsigned long long* acc = R.exc ? P.xe : P.xin;
   const int row_end = __shfl_sync(0xFFFFFFFFu, end_lane, P.ndel - 1);
@@ -204,6 +209,16 @@ __global__ void __launch_bounds__(kThreads) grad_deliver_kernel(const GradParams
       }
     }
   }
+}
+
+// Bits of P.active at step t from the spike history (after a checkpoint).
+__global__ void __launch_bounds__(kThreads) grad_active_kernel(const GradParams P, long long t) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P.N) return;
+  uint32_t act = 0u;
+  for (int d = 1; d < P.nslot && d <= t; ++d)
+    act |= P.shist[ring(t - d, P.nslot) * P.N + i] != 0.f ? 1u << (d - 1) : 0u;
+  P.active[i] = act;
 }
 
 // Neuron update of step t; records the tape at slot `slot` (>= 0) and adds
@@ -250,6 +265,7 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
     P.V[i] = __fmaf_rn(cp, pvc, __fmul_rn(Vp, P.pvv));
     P.C[i] = __fmul_rn(cp, P.pcc);
     P.shist[ring(t, P.nslot) * P.N + i] = s;
+    P.active[i] = P.active[i] << 1 | (s != 0.f ? 1u : 0u);
     if (slot >= 0) {
       float* tp = P.tape + (long long)slot * kTape * P.N + i;
       const float vals[kTape] = {V, I, U, g, s, cp, XE, XI};
@@ -281,48 +297,104 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
   }
 }
 
-// Adjoint of s_j(tau) through its outgoing synapses: sum over buckets d with
-// tau + d < T of w * (a[p_j][p_i] * adjoint of I_i(tau + d)).  One warp per
-// row, four records per lane per pass (16-byte loads), a fixed summation
-// order.
-__global__ void __launch_bounds__(kThreads) grad_gather_kernel(const GradParams P, long long tau) {
-  const long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (j >= P.N) return;
-  const GradRow R = grad_row(P, j);
-  const float* ib = R.exc ? P.ibe : P.ibi;
-  long long off_lane = -1;  // ring offset of bucket `lane`'s step, -1 beyond T
-  int end_lane = 0x7FFFFFFF, mid_lane = 0;
-  if (lane < P.ndel) {
-    const long long dst = tau + P.dmin + lane;
-    off_lane = dst < P.T ? ring(dst, P.nslot) * P.accw : -1;
-    const uint32_t e = *reinterpret_cast<const uint16_t*>(R.ends + desc_end(lane));
-    mid_lane = (int)(e & 0xFFu) * P.unit;
-    end_lane = (int)(e >> 8) * P.unit;
-  }
-  const int row_end = __shfl_sync(0xFFFFFFFFu, end_lane, P.ndel - 1);
-  const uint2* row = R.rec;
-  float acc = 0.f;
-#pragma unroll 2
-  for (int k0 = 0; k0 < row_end; k0 += 128) {
-    const int k = k0 + 4 * lane;
-    const int b = bucket_of(k, end_lane, P.ndel);
-    const long long off = __shfl_sync(0xFFFFFFFFu, off_lane, b);
-    const bool in = k < __shfl_sync(0xFFFFFFFFu, mid_lane, b);
-    if (k < row_end && off >= 0) {
-      const uint4 r01 = __ldcs(reinterpret_cast<const uint4*>(row + k));
-      const uint4 r23 = __ldcs(reinterpret_cast<const uint4*>(row + k + 2));
-      const float* ibs = ib + off;
-      const uint32_t tg[4] = {r01.x, r01.z, r23.x, r23.z};
-      const uint32_t wf[4] = {r01.y, r01.w, r23.y, r23.w};
+// Adjoint of s_j(tau) through the synapses of its bucket b, tau + d < T: the
+// sum of w * (a[p_j][p_i] * adjoint of I_i(tau + d)), to part[b].  A block
+// takes bucket b of a run of rows of one population in one delivery tile.  It
+// first copies the tile's adjoints at tau + d to shared memory, where the four
+// fifths of the row's targets that lie in the tile are looked up (in parts);
+// the others come from L2.  Eight lanes share a row: a lane takes every eighth
+// 32-byte sector of the bucket (four records), and the lanes' sums are added
+// in a fixed order.
+// What bounds it: each record needs one scattered 4-byte read of an adjoint.
+// As L2 reads (one warp per row, all buckets) they took 75 us a step on the
+// 4x4 network, whose table is 197 MB (DRAM floor 31 us); looked up in shared
+// memory, 54 us.  Loading a row's sectors one row ahead (384 threads, more
+// registers) took 68 us.
+constexpr int kGatherThreads = 512;
+constexpr int kGatherDepth = 3;  // sectors in flight per lane
+
+__global__ void __launch_bounds__(kGatherThreads, 2)
+    grad_gather_kernel(const GradParams P, long long tau, int rows_e, int rows_i, int blocks_e,
+                       int blocks_i) {
+  extern __shared__ __align__(16) float s_ib[];
+  const int b = (int)blockIdx.y;
+  const long long dst = tau + P.dmin + b;
+  if (dst >= P.T) return;
+  const int per_tile = blocks_e + blocks_i;
+  const int tile = (int)blockIdx.x / per_tile;
+  int part = (int)blockIdx.x - tile * per_tile;
+  const bool exc = part < blocks_e;
+  part -= exc ? 0 : blocks_e;
+  const uint2 ti = P.tinfo[tile];
+  const uint32_t npop = (uint32_t)(exc ? P.nexc : P.npc - P.nexc);  // rows of a column
+  const uint32_t rows = npop * ti.y;
+  const uint32_t per_block = (uint32_t)(exc ? rows_e : rows_i);
+  const uint32_t r0 = (uint32_t)part * per_block;
+  if (r0 >= rows) return;
+  const uint32_t r1 = min(rows, r0 + per_block);
+  const float* ib = (exc ? P.ibe : P.ibi) + ring(dst, P.nslot) * P.accw;
+  const float* own = ib + (size_t)ti.x * P.npc4;
+  for (uint32_t i = threadIdx.x; i < ti.y * (uint32_t)P.npc4 / 4u; i += kGatherThreads)
+    reinterpret_cast<float4*>(s_ib)[i] = __ldg(reinterpret_cast<const float4*>(own) + i);
+  __syncthreads();
+  const uint32_t lane8 = threadIdx.x & 7u;
+  const int beg_at = b % kPlaneBuckets ? desc_end(b) - 1 : desc_start(b);
+  const uint32_t us = (uint32_t)P.unit / 4u;  // sectors of a unit
+  // row r of the population: its place in the table; its bucket ends are
+  // loaded one row ahead
+  auto row_of = [&](uint32_t r) -> size_t {
+    const uint32_t k = r / npop;
+    return (size_t)(ti.x + k) * P.npc + (exc ? 0u : (uint32_t)P.nexc) + (r - k * npop);
+  };
+  uint32_t beg_n = 0u, me_n = 0u;
+  auto load_ends = [&](uint32_t r) {
+    if (r >= r1) return;
+    const uint8_t* d = P.bend + row_of(r) * (size_t)(P.planes * 16);
+    beg_n = d[beg_at];
+    me_n = *reinterpret_cast<const uint16_t*>(d + desc_end(b));
+  };
+  load_ends(r0 + threadIdx.x / 8u);
+  // every lane takes part in the row loop (its sums are shuffled)
+  for (uint32_t rb = r0; rb < r1; rb += kGatherThreads / 8) {
+    const uint32_t r = rb + threadIdx.x / 8u;
+    float acc = 0.f;
+    size_t jv = 0;
+    const uint32_t beg = beg_n, me = me_n;
+    load_ends(r + kGatherThreads / 8);
+    if (r < r1) {
+      const uint32_t k = r / npop;
+      jv = row_of(r);
+      const uint32_t n_in = ((me & 0xFFu) - beg) * us, n = ((me >> 8) - beg) * us;
+      const uint4* sec = reinterpret_cast<const uint4*>(P.syn + jv * (size_t)P.rowcap + beg * (uint32_t)P.unit);
+      const uint32_t* nb = P.nbg + (size_t)(ti.x + k) * 64;
+      for (uint32_t s0 = lane8; s0 < n; s0 += 8u * kGatherDepth) {
+        uint4 x[kGatherDepth], y[kGatherDepth];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (!(tg[q] & kPad)) acc = __fmaf_rn((float)(int32_t)wf[q], ibs[target_word(R, in, tg[q])], acc);
+        for (int q = 0; q < kGatherDepth; ++q) {
+          const uint32_t s = min(s0 + 8u * q, n - 1u);
+          x[q] = __ldcs(sec + 2u * s);
+          y[q] = __ldcs(sec + 2u * s + 1u);
+        }
+#pragma unroll
+        for (int q = 0; q < kGatherDepth; ++q) {
+          const uint32_t s = s0 + 8u * q;
+          if (s >= n) continue;
+          const uint32_t c[4] = {x[q].x, x[q].z, y[q].x, y[q].z};
+          const uint32_t w[4] = {x[q].y, x[q].w, y[q].y, y[q].w};
+          const bool in = s < n_in;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            if (c[m] & kPad) continue;
+            const float v = in ? s_ib[c[m]] : __ldg(ib + (__ldg(nb + ((c[m] >> 11) & 63u)) + (c[m] & 2047u)));
+            acc = __fmaf_rn((float)(int32_t)w[m], v, acc);
+          }
+        }
+      }
     }
-  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-  if (lane == 0) P.sg[j] = __fmul_rn(acc, kTwoM16);
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if (r < r1 && lane8 == 0u) P.part[(size_t)b * P.N + jv] = acc;
+  }
 }
 
 // One step of the adjoint recursion for step tau (tape slot `slot`): takes the
@@ -335,7 +407,15 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   const float* tp = P.tape + (long long)slot * kTape * P.N + i;
   const float V = tp[0], I = tp[P.N], U = tp[2 * P.N], g = tp[3 * P.N], s = tp[4 * P.N];
   const float cp = tp[5 * P.N], XE = tp[6 * P.N], XI = tp[7 * P.N];
-  float sbar = (exc ? P.dlds_e : P.dlds_i) + P.sg[i] + P.gb[ring(tau + 1, 3) * P.N + i] +
+  // the adjoint of s(tau) through the synapses: the buckets that end before T
+  const uint32_t c = (uint32_t)i / (uint32_t)P.npc, l = (uint32_t)i - c * (uint32_t)P.npc;
+  const uint32_t v = P.colv[c];
+  const float* part = P.part + (size_t)v * P.npc + l;
+  float sg = 0.f;
+  const int nb = (int)min((long long)P.ndel, max(0ll, P.T - tau - P.dmin));
+#pragma unroll 8
+  for (int b = 0; b < nb; ++b) sg += part[(size_t)b * P.N];
+  float sbar = (exc ? P.dlds_e : P.dlds_i) + __fmul_rn(sg, kTwoM16) + P.gb[ring(tau + 1, 3) * P.N + i] +
                P.gb[ring(tau + 2, 3) * P.N + i];
   const float vb1 = P.vbar[i], cb1 = P.cbar[i];
   const float pvc = exc ? P.pvc_e : P.pvc_i;
@@ -363,7 +443,7 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   P.gb[ring(tau, 3) * P.N + i] = g > 0.f ? -ubar * (V + I - P.vr) : 0.f;
   const float aE = exc ? P.a[0] : P.a[1];
   const float aI = exc ? P.a[2] : P.a[3];
-  const long long iw = ring(tau, P.nslot) * P.accw + acc_word(P, i);
+  const long long iw = ring(tau, P.nslot) * P.accw + (long long)v * P.npc4 + l;
   P.ibe[iw] = aE * ib;
   P.ibi[iw] = aI * ib;
   // I = a[E][p] X_E + a[I][p] X_I + J (lam + sqrt(lam) xi),  h = 1 ms
@@ -373,12 +453,30 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   ga[5 * P.N] += (double)ib * (double)P.J * (1.0 + (double)xi / (2.0 * (double)P.sqlam));
 }
 
+// Sums of the six parameters' partials over the neurons, one block per
+// parameter, in a fixed order.
+constexpr int kSumThreads = 1024;
+__global__ void __launch_bounds__(kSumThreads) grad_sum_kernel(const GradParams P) {
+  __shared__ double s_sum[kSumThreads];
+  const double* p = P.gacc + (size_t)blockIdx.x * P.N;
+  double sum = 0.0;
+#pragma unroll 4
+  for (long long i = threadIdx.x; i < P.N; i += kSumThreads) sum += p[i];
+  s_sum[threadIdx.x] = sum;
+  for (int o = kSumThreads / 2; o > 0; o >>= 1) {
+    __syncthreads();
+    if ((int)threadIdx.x < o) s_sum[threadIdx.x] += s_sum[threadIdx.x + o];
+  }
+  if (threadIdx.x == 0) P.gsum[blockIdx.x] = s_sum[0];
+}
+
 }  // namespace
 
 struct snn_grad {
   NetView v{};
   long long T = 0;
   int ckpt = 0, nseg = 0, hard = 1, nslot = 0, ublocks = 0, wblocks = 0;
+  size_t gather_smem = 0;
   float beta = 5.f;
   double targets[2] = {3.0, 8.0};
   double kappa = 0.0, pvv = 0.0, pcc = 0.0;
@@ -424,6 +522,25 @@ void grad_release(snn_grad* g) {
   g->bufs.clear();
 }
 
+// Gather of step tau: the buckets that end before T, their blocks in one wave
+// (a block copies its tile's adjoints first, so few and long ones: with 340
+// blocks for 304 places the 4x4 network took 63 us a step, with 300 it takes
+// 54) but at least kGatherMinRows rows each, shared between E and I rows.
+constexpr int kGatherMinRows = 128;
+void launch_gather(snn_grad* g, long long tau) {
+  const NetView& v = g->v;
+  const int nb = (int)std::min<long long>(v.ndel, g->T - tau - v.dmin);
+  if (nb <= 0) return;
+  const int slots = v.num_sms * (2 * (g->gather_smem + 2048) <= kSmemBudget ? 2 : 1);
+  const long long re = (long long)v.tcols * v.nexc, ri = (long long)v.tcols * (v.npc - v.nexc);
+  const int most = (int)std::max<long long>(
+      2, std::min<long long>(slots / (nb * v.ntile), (re + ri) / kGatherMinRows));
+  const int be = re ? std::max(1, (int)(most * re / (re + ri))) : 0;
+  const int bi = ri ? std::max(1, most - be) : 0;
+  grad_gather_kernel<<<dim3(v.ntile * (be + bi), nb), kGatherThreads, g->gather_smem, v.stream>>>(
+      g->P, tau, be ? (int)((re + be - 1) / be) : 0, bi ? (int)((ri + bi - 1) / bi) : 0, be, bi);
+}
+
 cudaError_t launch_forward_step(snn_grad* g, long long t, int slot, int rates) {
   const GradParams& P = g->P;
   cudaStream_t st = g->v.stream;
@@ -466,6 +583,12 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   const long long N = v.N;
   g->ublocks = (int)((N + kThreads - 1) / kThreads);
   g->wblocks = (int)((N * 32 + kThreads - 1) / kThreads);
+  g->gather_smem = (size_t)v.tcols * v.npc4 * 4;
+  if (cudaFuncSetAttribute(grad_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kSmemBudget) != cudaSuccess) {
+    delete g;
+    return fail_global(SNN_ECUDA, "the gather kernel does not fit on the device");
+  }
   // propagators in FP64 as the spiking tables compute them (h = 1 ms)
   const double tm = v.neuron.tau_m, tc = v.neuron.tau_c;
   g->pvv = std::exp(-1.0 / tm);
@@ -482,9 +605,11 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   P.ctile = v.ctile;
   P.colv = v.colv;
   P.nbg = v.nbg;
+  P.tinfo = v.tinfo;
   P.nexc = v.nexc;
   P.dmin = v.dmin;
   P.ndel = v.ndel;
+  P.bucket_mask = v.ndel == 32 ? 0xFFFFFFFFu : (1u << v.ndel) - 1u;
   P.nslot = g->nslot;
   P.rowcap = v.rowcap;
   P.hard = g->hard;
@@ -508,6 +633,8 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   if (!rc) rc = galloc(g, &P.V, n);
   if (!rc) rc = galloc(g, &P.C, n);
   if (!rc) rc = galloc(g, &P.shist, n * g->nslot);
+  if (!rc) rc = galloc(g, &P.active, n);
+  if (!rc) rc = galloc(g, &P.gsum, 6);
   if (!rc) rc = galloc(g, &P.xe, accw);
   if (!rc) rc = galloc(g, &P.xin, accw);
   if (!rc) rc = galloc(g, &P.tape, n * kTape * g->ckpt);
@@ -517,7 +644,7 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   if (!rc) rc = galloc(g, &P.ibe, accw * g->nslot);
   if (!rc) rc = galloc(g, &P.ibi, accw * g->nslot);
   if (!rc) rc = galloc(g, &P.gb, n * 3);
-  if (!rc) rc = galloc(g, &P.sg, n);
+  if (!rc) rc = galloc(g, &P.part, n * v.ndel);
   if (!rc) rc = galloc(g, &P.gacc, n * 6);
   if (!rc) rc = galloc(g, &g->ck, n * (2 + g->nslot) * g->nseg);
   if (rc) {
@@ -611,21 +738,18 @@ int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, 
     SNN_GCUDA(g, cudaMemcpyAsync(P.C, ck + n, n * 4, cudaMemcpyDeviceToDevice, st));
     SNN_GCUDA(g, cudaMemcpyAsync(P.shist, ck + 2 * n, n * g->nslot * 4, cudaMemcpyDeviceToDevice,
                                  st));
+    grad_active_kernel<<<g->ublocks, kThreads, 0, st>>>(P, t0);
     for (long long t = t0; t < t1; ++t) SNN_GCUDA(g, launch_forward_step(g, t, (int)(t - t0), 0));
     for (long long tau = t1 - 1; tau >= t0; --tau) {
-      grad_gather_kernel<<<g->wblocks, kThreads, 0, st>>>(P, tau);
+      launch_gather(g, tau);
       grad_backward_kernel<<<g->ublocks, kThreads, 0, st>>>(P, tau, (int)(tau - t0));
     }
     SNN_GCUDA(g, cudaGetLastError());
   }
-  std::vector<double> acc(n * 6);
-  SNN_GCUDA(g, cudaMemcpyAsync(acc.data(), P.gacc, acc.size() * 8, cudaMemcpyDeviceToHost, st));
+  grad_sum_kernel<<<6, kSumThreads, 0, st>>>(P);
+  SNN_GCUDA(g, cudaGetLastError());
+  SNN_GCUDA(g, cudaMemcpyAsync(grad, P.gsum, 6 * sizeof(double), cudaMemcpyDeviceToHost, st));
   SNN_GCUDA(g, cudaStreamSynchronize(st));
-  for (int k = 0; k < 6; ++k) {
-    double sum = 0.0;
-    for (size_t i = 0; i < n; ++i) sum += acc[(size_t)k * n + i];
-    grad[k] = sum;
-  }
   return SNN_OK;
 }
 

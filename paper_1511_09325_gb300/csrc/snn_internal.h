@@ -82,6 +82,12 @@ constexpr int kMaxGridSide = 16383;     // columns per grid side (14-bit coordin
 constexpr int kMaxTile = 8;             // delivery tile side, columns
 constexpr int kMaxTileCols = kMaxTile * kMaxTile;
 constexpr int kCntStride = 8;           // words from one tile counter to the next
+// Shared memory of a delivery block: of a net of its own (one block per SM) and
+// of the batch kernel (two per SM); the window alone takes at most
+// kWindowBudget.
+constexpr size_t kSmemBudget = 224 * 1024;
+constexpr size_t kBatchSmemBudget = 110 * 1024;
+constexpr size_t kWindowBudget = 196 * 1024;
 // Words of a tile's window per item of the fewest that make a part use the
 // window, and per item of its fixed cost in the range split (set-up and
 // flush); the fixed cost, in items, of a tile with fewer but some items.
@@ -284,6 +290,8 @@ struct NetView {
   const uint32_t* ctile;
   const uint32_t* colv;
   const uint32_t* nbg;
+  const uint2* tinfo;
+  int ntile, tcols;
   uint64_t seed;
   snn_neuron_params neuron;
   cudaStream_t stream;

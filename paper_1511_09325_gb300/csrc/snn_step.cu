@@ -1177,7 +1177,9 @@ int deliver_grid(const StepParams& p, int precision, int num_sms) {
                        ? reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F16W>)
                        : reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F32W>);
   int per_sm = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  // the attribute belongs to the kernel, not to the net: always the budget
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)std::max(smem, kSmemBudget)) != cudaSuccess)
     return 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kDeliverThreads, smem);
   return per_sm > 0 ? num_sms : 0;
@@ -1222,7 +1224,8 @@ size_t batch_smem(size_t max_deliver_smem) {
 
 int batch_grid(int precision, int infl, int num_sms, size_t smem) {
   void* fn = batch_kernel_ptr(precision, infl);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)std::max(smem, kBatchSmemBudget)) != cudaSuccess)
     return 0;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBatchThreads, smem);
