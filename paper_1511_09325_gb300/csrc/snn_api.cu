@@ -327,8 +327,10 @@ int capture(snn_net* net, int steps, cudaGraphExec_t* out) {
   SNN_CUDA(net, cudaStreamBeginCapture(net->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t le = cudaSuccess;
   for (int s = 0; s < steps && le == cudaSuccess; ++s) {
-    le = launch_update(net->sp, net->update_grid, net->stream);
-    if (le == cudaSuccess) le = launch_deliver(net->sp, net->precision, net->deliver_grid, net->stream);
+    // the graph's first kernel follows whatever the stream holds: a plain launch
+    le = launch_update(net->sp, net->update_grid, s > 0, net->stream);
+    if (le == cudaSuccess)
+      le = launch_deliver(net->sp, net->precision, net->deliver_grid, true, net->stream);
   }
   cudaError_t ee = cudaStreamEndCapture(net->stream, &g);
   if (le != cudaSuccess) {
@@ -791,7 +793,7 @@ int snn_shard_update(snn_net* net) {
   if (net->shard_phase != 0) return fail(net, SNN_ESTATE, "snn_shard_deliver is due first");
   int rc = check_status(net);
   if (rc) return rc;
-  SNN_CUDA(net, launch_update(net->sp, net->update_grid, net->stream));
+  SNN_CUDA(net, launch_update(net->sp, net->update_grid, false, net->stream));
   net->shard_phase = 1;
   return SNN_OK;
 }
@@ -826,7 +828,7 @@ int snn_shard_deliver(snn_net* net, const int32_t* ids, int64_t n, int32_t ids_o
   }
   SNN_CUDA(net, launch_ingest(net->sp, src, n, net->stream));
   if (staged) SNN_CUDA(net, cudaEventRecord(net->ingest_ev, net->stream));
-  SNN_CUDA(net, launch_deliver(net->sp, net->precision, net->deliver_grid, net->stream));
+  SNN_CUDA(net, launch_deliver(net->sp, net->precision, net->deliver_grid, false, net->stream));
   net->shard_phase = 0;
   return SNN_OK;
 }
@@ -879,10 +881,10 @@ int snn_step_profiled(snn_net* net, int64_t n_steps, double* ms, double* bytes) 
   if (e == cudaSuccess) e = launch_sum_parts(net->spk_part, net->update_grid, dspk, net->stream);
   for (int64_t s = 0; s < n_steps && e == cudaSuccess; ++s) {
     e = cudaEventRecord(ev[3 * s], net->stream);
-    if (e == cudaSuccess) e = launch_update(net->sp, net->update_grid, net->stream);
+    if (e == cudaSuccess) e = launch_update(net->sp, net->update_grid, false, net->stream);
     if (e == cudaSuccess) e = cudaEventRecord(ev[3 * s + 1], net->stream);
     if (e == cudaSuccess)
-      e = launch_deliver(net->sp, net->precision, net->deliver_grid, net->stream);
+      e = launch_deliver(net->sp, net->precision, net->deliver_grid, false, net->stream);
     if (e == cudaSuccess) e = cudaEventRecord(ev[3 * s + 2], net->stream);
     if (e == cudaSuccess)
       e = launch_sum_parts(net->spk_part, net->update_grid, dspk + s + 1, net->stream);

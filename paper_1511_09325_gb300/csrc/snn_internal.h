@@ -319,7 +319,9 @@ cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
 // Readback of rows in the order they were drawn, within a row by delay.
 cudaError_t launch_read_rows(const BuildParams& bp, int precision, bool paper, cudaStream_t st);
 cudaError_t launch_init_state(const StepParams& p, cudaStream_t st);
-cudaError_t launch_update(const StepParams& p, int grid, cudaStream_t st);
+// `overlap`: programmatic dependent launch (step graphs, where update and
+// delivery alternate); else a plain launch.
+cudaError_t launch_update(const StepParams& p, int grid, bool overlap, cudaStream_t st);
 int update_grid(long long N, int num_sms);
 // Delivery: dynamic shared memory of one block of a net's own kernel or of
 // the batch kernel (window, neighbour table, the warps' sector lists) for
@@ -327,7 +329,7 @@ int update_grid(long long N, int num_sms);
 // does not fit).
 size_t deliver_smem(int cols, int npc4, bool batch);
 int deliver_grid(const StepParams& p, int precision, int num_sms);
-cudaError_t launch_deliver(const StepParams& p, int precision, int grid, cudaStream_t st);
+cudaError_t launch_deliver(const StepParams& p, int precision, int grid, bool overlap, cudaStream_t st);
 // Compact the per-block record regions into id and step arrays and reset
 // them; header = {records kept, 1 if records were dropped, first step, last
 // step}, written to header and to the mapped host header map_hdr.  The arrays

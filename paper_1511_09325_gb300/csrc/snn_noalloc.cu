@@ -141,7 +141,7 @@ extern "C" int snn_update_noalloc(int grid_w, int grid_h, const snn_neuron_param
   e = cudaMemsetAsync(base, 0, kOffCol + 16 * (size_t)ncol, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(base + kOffCtl + offsetof(Ctl, t), &t, sizeof(t), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_update(p, grid, st);
+  if (e == cudaSuccess) e = launch_update(p, grid, false, st);
   if (e == cudaSuccess)
     e = launch_sum_parts(p.ext_part, grid, reinterpret_cast<unsigned long long*>(base + kOffExtSum), st);
   unsigned n = 0u;
