@@ -574,7 +574,7 @@ def _batched_form(snn, torch, stream, steps=2000, n_nets=64):
     out["tuned_choice"] = choice
     out["tuned_schedule"] = {"sector_rounds_in_flight": [2, 2, 1, 1][choice % 4],
                              "windows": choice % 2 == 0,
-                             "delivery_blocks_per_column": [8, 4, 2, 1][choice // 4]}
+                             "min_items_per_delivery_block": [64, 128, 256, 512][choice // 4]}
     tuned_steps = 2 * 2 * 4 * 25  # two stages of two rounds of four candidates
     r0 = [m.stats()[0] for m in b.members]
     ev0 = torch.cuda.Event(enable_timing=True)

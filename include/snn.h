@@ -381,8 +381,8 @@ snn_net* snn_batch_net(snn_batch* batch, int k);
  * snn_batch_tune -- pick the fastest delivery schedule for this batch (rounds
  * of 32-byte sectors in flight per lane: 2 or 1, i.e. 4 or 2 chunks of 16
  * bytes; shared-memory windows: on or off), then
- * the fastest delivery density (8, 4, 2 or 1 virtual delivery blocks per
- * member column, at most the member's standalone grid), each by timing two
+ * the fastest delivery density (at least 64, 128, 256 or 512 delivery items per
+ * block), each by timing two
  * interleaved rounds of steps_per_trial steps of every candidate (16 trials
  * in all).  The trial steps advance the simulation (every candidate computes
  * identical sums).  *choice (may be NULL) receives the pick, schedule (0..3)

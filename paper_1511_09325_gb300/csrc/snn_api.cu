@@ -25,7 +25,7 @@ struct snn_net {
   bool batch_member = false;          // windows sized for the batch kernel's blocks
   unsigned min_items = 256;  // fewest items a delivery block takes
   unsigned win_items = 0;  // fewest items of a windowed tile part
-  unsigned cost_win = 0, cost_part = kCostPart;  // range split's fixed costs
+  unsigned cost_win = 0;     // range split's fixed cost of a tile with a window
   long long N = 0, Npad = 0, ncol = 0;
   uint64_t seed = 0;
   snn_neuron_params neuron{};
@@ -367,7 +367,6 @@ void fill_step_params(snn_net* net) {
   p.min_items = net->min_items;
   p.win_items = net->win_items;
   p.cost_win = net->cost_win;
-  p.cost_part = net->cost_part;
   p.npc_m = recip32((uint32_t)net->npc);
   p.seed_lo = (uint32_t)(net->seed & 0xFFFFFFFFu);
   p.seed_hi = (uint32_t)(net->seed >> 32);
@@ -1245,13 +1244,14 @@ struct snn_batch {
   int precision = 0, num_sms = 0, max_npc = 0;
   int infl = 4;            // 16-byte chunks in flight in the delivery loop
   int agg = 1;             // block windows for the local half of the synapses
-  int dens8 = 64;          // delivery virtual blocks per 8 member columns
+  unsigned min_items = kBatchMinItems;  // fewest items a delivery block takes
   int choice = -1;         // autotuner's pick (-1: not tuned)
-  std::vector<int> first;  // host copy of d_first
+  std::vector<int> first;  // [2][n + 1]: first update virtual blocks, first tiles
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   StepParams* d_nets = nullptr;
-  int* d_first = nullptr;  // [2][n + 1]: update, delivery virtual blocks
+  int* d_first = nullptr;  // first, on the device
+  BatchTile* d_tiles = nullptr;
   unsigned* d_bar = nullptr;
   long long t = 0;
   long long spin_limit = 1LL << 25;
@@ -1281,39 +1281,36 @@ void batch_release(snn_batch* b) {
   b->nets.clear();
   if (b->d_nets) cudaFree(b->d_nets);
   if (b->d_first) cudaFree(b->d_first);
+  if (b->d_tiles) cudaFree(b->d_tiles);
   if (b->d_bar) cudaFree(b->d_bar);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
-}
-
-// Delivery virtual blocks of member k: dens8 per 8 columns (at least one, at
-// most its standalone grid).  Any count gives the same sums (the items are
-// split into that many equal ranges).
-void batch_delivery_firsts(snn_batch* b) {
-  const size_t n = b->nets.size();
-  for (size_t k = 0; k < n; ++k) {
-    const snn_net* net = b->nets[k];
-    const long long dg =
-        std::min<long long>(net->deliver_grid, std::max<long long>(1, (long long)b->dens8 * net->ncol / 8));
-    b->first[(n + 1) + k + 1] = b->first[(n + 1) + k] + (int)dg;
-  }
-}
-
-// Upload the virtual-block tables (host copy in b->first).
-int batch_upload_firsts(snn_batch* b) {
-  SNN_BCUDA(b, cudaMemcpyAsync(b->d_first, b->first.data(), b->first.size() * sizeof(int),
-                               cudaMemcpyHostToDevice, b->stream));
-  SNN_BCUDA(b, cudaStreamSynchronize(b->stream));
-  return SNN_OK;
 }
 
 // Upload the members' step parameters with the batch's window setting.
 int batch_upload(snn_batch* b) {
   std::vector<StepParams> ps(b->nets.size());
+  std::vector<BatchTile> tiles;
   for (size_t k = 0; k < b->nets.size(); ++k) {
     b->nets[k]->agg = b->agg != 0;
     fill_step_params(b->nets[k]);
     ps[k] = b->nets[k]->sp;
+    const StepParams& p = ps[k];
+    for (int m = 0; m < p.ntile; ++m) {
+      BatchTile bt{};
+      bt.isum = p.isum + (size_t)m * kCntStride;
+      bt.ccnt = p.ccnt + (size_t)m * kCntStride;
+      bt.stride = (uint32_t)(p.ntile * kCntStride);
+      bt.nslot = p.nslot;
+      bt.dmin = p.dmin;
+      bt.net = (int)k;
+      bt.tile = m;
+      bt.win_items = p.win_items;
+      bt.cost_win = p.cost_win;
+      tiles.push_back(bt);
+    }
   }
+  SNN_BCUDA(b, cudaMemcpyAsync(b->d_tiles, tiles.data(), tiles.size() * sizeof(BatchTile),
+                               cudaMemcpyHostToDevice, b->stream));
   SNN_BCUDA(b, cudaMemcpyAsync(b->d_nets, ps.data(), ps.size() * sizeof(StepParams),
                                cudaMemcpyHostToDevice, b->stream));
   SNN_BCUDA(b, cudaStreamSynchronize(b->stream));
@@ -1329,16 +1326,21 @@ int batch_run(snn_batch* b, long long n_steps) {
   BatchParams bp{};
   bp.nets = b->d_nets;
   bp.u_first = b->d_first;
-  bp.d_first = b->d_first + (n + 1);
+  bp.t_first = b->d_first + (n + 1);
+  bp.tiles = b->d_tiles;
   bp.n_nets = n;
+  bp.n_tiles = b->first.back();
+  bp.min_items = b->min_items;
   bp.t0 = b->t;
   bp.n_steps = n_steps;
   bp.bar = b->d_bar;
   bp.spin_limit = b->spin_limit;
   bp.extra_arrivals = b->extra_arrivals;
-  size_t dsm = 0;
-  for (const snn_net* net : b->nets) dsm = std::max(dsm, deliver_smem(net->sp.tcols, net->sp.npc4, true));
-  const size_t smem = batch_smem(dsm);
+  for (const snn_net* net : b->nets) {
+    bp.win_words = std::max(bp.win_words, net->sp.tcols * net->sp.npc4);
+    bp.max_cols = std::max(bp.max_cols, net->sp.tcols);
+  }
+  const size_t smem = batch_smem(bp.win_words, bp.max_cols);
   const int grid = batch_grid(b->precision, b->infl, b->num_sms, smem);
   if (grid < 1) return bfail(b, SNN_ECUDA, "batch kernel does not fit on the device");
   SNN_BCUDA(b, cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream));
@@ -1394,6 +1396,7 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
     b->num_sms = net->num_sms;
     // update: the net's own grid (its partial sums and record regions)
     b->first[k + 1] = b->first[k] + net->update_grid;
+    b->first[(n_nets + 1) + k + 1] = b->first[(n_nets + 1) + k] + net->ntile;
   }
   if (rc != SNN_OK) {
     const std::string why = g_err;
@@ -1401,9 +1404,9 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
     delete b;
     return bfail(nullptr, rc, why);
   }
-  batch_delivery_firsts(b);
   cudaError_t e = cudaMalloc(&b->d_nets, sizeof(StepParams) * (size_t)n_nets);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_first, b->first.size() * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, (size_t)b->first.back() * sizeof(BatchTile));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_bar, 4 * sizeof(unsigned));
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_first, b->first.data(), b->first.size() * sizeof(int),
@@ -1441,10 +1444,10 @@ int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) {
   if (!b || steps_per_trial < 1) return bfail(b, SNN_EINVAL, "bad argument");
   // every variant computes the same sums, so the trials simply advance the
   // simulation; two interleaved rounds even out changes in activity.  Stage
-  // 0 times the four delivery schedules, stage 1 the delivery densities with
-  // the schedule that won.
+  // 0 times the four delivery schedules, stage 1 the delivery densities (the
+  // fewest items a block takes) with the schedule that won.
   const int infl[4] = {4, 4, 2, 2}, agg[4] = {1, 0, 1, 0};
-  const int dens8[4] = {64, 32, 16, 8};  // 8, 4, 2 and 1 blocks per column
+  const unsigned min_items[4] = {64, 128, 256, 512};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t ce = cudaEventCreate(&e0);
   if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
@@ -1463,9 +1466,7 @@ int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) {
           b->agg = agg[v];
           rc = batch_upload(b);
         } else {
-          b->dens8 = dens8[v];
-          batch_delivery_firsts(b);
-          rc = batch_upload_firsts(b);
+          b->min_items = min_items[v];
         }
         if (rc) break;
         cudaError_t e = cudaEventRecord(e0, b->stream);
@@ -1495,10 +1496,7 @@ int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != SNN_OK) return rc;
-  b->dens8 = dens8[pick[1]];
-  batch_delivery_firsts(b);
-  rc = batch_upload_firsts(b);
-  if (rc) return rc;
+  b->min_items = min_items[pick[1]];
   b->choice = pick[0] + 4 * pick[1];
   if (choice) *choice = b->choice;
   return SNN_OK;

@@ -190,7 +190,7 @@ struct StepParams {
   int agg;                 // shared-memory windows over the delivery tiles
   unsigned min_items;      // fewest items a delivery block takes (fewer blocks run)
   unsigned win_items;      // fewest items of a part that uses the window
-  unsigned cost_win, cost_part;  // fixed cost (in items) of a windowed / other tile
+  unsigned cost_win;       // fixed cost (in items) of a tile with a window
   uint32_t npc_m;          // floor(2^32 / n_per_col) (capped)
   uint32_t seed_lo, seed_hi;
   float theta, vr, dc, pvv, pcc, pvc_e, pvc_i;
@@ -231,11 +231,21 @@ struct StepParams {
 
 // A batch of nets advanced by one persistent launch (snn_batch_*).
 constexpr int kMaxBatch = 256;
+struct BatchTile {          // a tile of a member
+  const unsigned* isum;
+  unsigned* ccnt;           // its counter in slot 0
+  uint32_t stride;          // words from one slot's counters to the next
+  int nslot, dmin, net, tile;
+  unsigned win_items, cost_win;
+};
 struct BatchParams {
   StepParams* nets;         // [n_nets], device
   const int* u_first;       // [n_nets + 1] first update virtual block of each net
-  const int* d_first;       // [n_nets + 1] first delivery virtual block of each net
-  int n_nets;
+  const int* t_first;       // [n_nets + 1] first tile of each net
+  const BatchTile* tiles;   // [n_tiles], device
+  int n_nets, n_tiles;
+  int win_words, max_cols;  // largest window and tile of the members
+  unsigned min_items;       // fewest items a delivery block takes
   long long t0, n_steps;
   unsigned* bar;            // grid barrier: arrivals, generation, error flag
   long long spin_limit;     // polls before a barrier wait gives up
@@ -340,9 +350,9 @@ cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_
                                  uint32_t* stage_steps, unsigned long long* header,
                                  unsigned long long* map_hdr, uint32_t* map_ids,
                                  uint32_t* map_steps, long long map_cap, cudaStream_t st);
-// Batch kernel: dynamic shared memory for members whose largest delivery
-// layout is max_deliver_smem, its grid (0 if it does not fit), its launch.
-size_t batch_smem(size_t max_deliver_smem);
+// Batch kernel: dynamic shared memory for members whose largest window has
+// win_words words and whose largest tile has max_cols columns, its grid (0 if it does not fit), its launch.
+size_t batch_smem(int win_words, int max_cols);
 int batch_grid(int precision, int infl, int num_sms, size_t smem);
 cudaError_t launch_batch(const BatchParams& b, int precision, int infl, int grid, size_t smem,
                          cudaStream_t st);
