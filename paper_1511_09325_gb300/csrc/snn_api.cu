@@ -90,6 +90,7 @@ struct snn_net {
   uint32_t* hingest = nullptr;
   long long ingest_cap = 0;
   cudaEvent_t ingest_ev = nullptr;
+  cudaEvent_t copy_ev[2] = {nullptr, nullptr};  // halves of the pinned copies out
   std::string err;
 };
 
@@ -172,6 +173,8 @@ void release(snn_net* net) {
   if (net->ingest) cudaFree(net->ingest);
   if (net->hingest) cudaFreeHost(net->hingest);
   if (net->ingest_ev) cudaEventDestroy(net->ingest_ev);
+  for (cudaEvent_t ev : net->copy_ev)
+    if (ev) cudaEventDestroy(ev);
   void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->ctile,
                   net->colv, net->tinfo, net->nbg, net->icnt, net->ccnt, net->deg, net->syn_part,
                   net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage, net->dhdr,
@@ -613,6 +616,38 @@ int sync(snn_net* net) {
   return SNN_OK;
 }
 
+// Copies `bytes` of device memory to pageable host memory `dst`.  A larger
+// copy goes through the two halves of the pinned record buffer (which no call
+// leaves in use), one half filled by the GPU while the other is copied out:
+// a pageable copy into fresh heap memory ran at 1.4 GB/s (state of 48x48
+// columns, 25.8 MB: 18 ms; staged: 2.6 ms).  Arrays of 32 MB and more, which the
+// allocator maps by large pages, are faster copied directly (96x96, 103 MB: 6.4
+// ms direct, 9.8 ms staged).
+int copy_out(snn_net* net, void* dst, const void* src, size_t bytes) {
+  const size_t half = (size_t)net->hmap_cap * 4 / 4096 * 4096;
+  if (bytes <= 65536 || bytes >= (32u << 20) || half == 0) {
+    SNN_CUDA(net, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, net->stream));
+    return SNN_OK;
+  }
+  for (cudaEvent_t& ev : net->copy_ev)
+    if (!ev) SNN_CUDA(net, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  char* const buf = reinterpret_cast<char*>(net->hmap);
+  const size_t parts = (bytes + half - 1) / half;
+  for (size_t k = 0; k <= parts; ++k) {
+    if (k < parts) {
+      SNN_CUDA(net, cudaMemcpyAsync(buf + (k & 1) * half, static_cast<const char*>(src) + k * half,
+                                    std::min(half, bytes - k * half), cudaMemcpyDeviceToHost, net->stream));
+      SNN_CUDA(net, cudaEventRecord(net->copy_ev[k & 1], net->stream));
+    }
+    if (k > 0) {
+      SNN_CUDA(net, cudaEventSynchronize(net->copy_ev[(k - 1) & 1]));
+      std::memcpy(static_cast<char*>(dst) + (k - 1) * half, buf + ((k - 1) & 1) * half,
+                  std::min(half, bytes - (k - 1) * half));
+    }
+  }
+  return SNN_OK;
+}
+
 Ctl read_ctl(snn_net* net, cudaError_t* e) {
   Ctl c{};
   *e = cudaMemcpyAsync(&c, net->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, net->stream);
@@ -921,25 +956,6 @@ int snn_step_profiled(snn_net* net, int64_t n_steps, double* ms, double* bytes) 
 
 namespace {
 
-// Records per region since the last drain, and the number kept.
-int record_counts(snn_net* net, std::vector<unsigned long long>* cnt, long long* kept,
-                  bool* lost) {
-  cnt->assign((size_t)net->update_grid, 0ull);
-  Ctl c{};
-  SNN_CUDA(net, cudaMemcpyAsync(cnt->data(), net->rcnt, cnt->size() * 8, cudaMemcpyDeviceToHost,
-                                net->stream));
-  SNN_CUDA(net, cudaMemcpyAsync(&c, net->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, net->stream));
-  SNN_CUDA(net, cudaStreamSynchronize(net->stream));
-  *kept = 0;
-  *lost = c.rec_overflow != 0u;
-  for (unsigned long long v : *cnt) {
-    const long long k = (long long)v < net->rec_region ? (long long)v : net->rec_region;
-    *kept += k;
-    if ((long long)v > net->rec_region) *lost = true;
-  }
-  return SNN_OK;
-}
-
 int reset_records(snn_net* net) {
   const unsigned zero32 = 0u;
   SNN_CUDA(net, cudaMemsetAsync(net->rcnt, 0, (size_t)net->update_grid * 8, net->stream));
@@ -953,12 +969,9 @@ int reset_records(snn_net* net) {
 
 int snn_pending_spikes(snn_net* net, int64_t* n_out) {
   if (!net || !n_out) return fail(net, SNN_EINVAL, "null argument");
-  std::vector<unsigned long long> cnt;
-  long long kept = 0;
-  bool lost = false;
-  int rc = record_counts(net, &cnt, &kept, &lost);
-  if (rc) return rc;
-  *n_out = kept;
+  SNN_CUDA(net, launch_count_records(net->sp, net->update_grid, net->hhdr_dev, net->stream));
+  SNN_CUDA(net, cudaStreamSynchronize(net->stream));
+  *n_out = (int64_t)net->hhdr[0];
   return SNN_OK;
 }
 
@@ -1114,11 +1127,11 @@ int snn_stats(snn_net* net, double* recurrent_events, double* external_events, i
 int snn_get_state(snn_net* net, float* v, float* c, uint8_t* refractory) {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
   const size_t N = (size_t)net->N;
-  if (v) SNN_CUDA(net, cudaMemcpyAsync(v, net->V, N * 4, cudaMemcpyDeviceToHost, net->stream));
-  if (c) SNN_CUDA(net, cudaMemcpyAsync(c, net->C, N * 4, cudaMemcpyDeviceToHost, net->stream));
-  if (refractory)
-    SNN_CUDA(net, cudaMemcpyAsync(refractory, net->R, N, cudaMemcpyDeviceToHost, net->stream));
-  return sync(net);
+  int rc = SNN_OK;
+  if (v) rc = copy_out(net, v, net->V, N * 4);
+  if (c && !rc) rc = copy_out(net, c, net->C, N * 4);
+  if (refractory && !rc) rc = copy_out(net, refractory, net->R, N);
+  return rc ? rc : sync(net);
 }
 
 int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int32_t* delay,

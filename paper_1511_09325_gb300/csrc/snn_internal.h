@@ -350,6 +350,10 @@ cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_
                                  uint32_t* stage_steps, unsigned long long* header,
                                  unsigned long long* map_hdr, uint32_t* map_ids,
                                  uint32_t* map_steps, long long map_cap, cudaStream_t st);
+// Counts the records a drain would return: {kept, 1 if records were dropped}
+// to the mapped host header.
+cudaError_t launch_count_records(const StepParams& p, int nreg, unsigned long long* map_hdr,
+                                 cudaStream_t st);
 // Batch kernel: dynamic shared memory for members whose largest window has
 // win_words words and whose largest tile has max_cols columns, its grid (0 if it does not fit), its launch.
 size_t batch_smem(int win_words, int max_cols);

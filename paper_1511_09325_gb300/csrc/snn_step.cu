@@ -144,15 +144,6 @@ __device__ __forceinline__ int slot_of(const StepParams& P, long long s) {
   return (s >> 32) == 0 ? (int)((uint32_t)s % (uint32_t)P.nslot) : (int)(s % P.nslot);
 }
 
-// The step graph launches each kernel while the one before it still runs
-// (programmatic dependent launch): what comes before grid_wait reads only what
-// no step writes; grid_wait returns when the kernel before has finished and
-// its writes are visible; grid_go lets the next kernel's blocks be launched.
-// Both are no-ops in a plain launch.  1000 steps: 14.2 -> 13.7 ms at 2x2, 58.6 ->
-// 54.4 ms at 24x24 FP32.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Records the first inconsistency a kernel finds; the host turns it into
 // SNN_ESTATE.
 __device__ __forceinline__ void set_status(const StepParams& P, unsigned code) {
@@ -209,44 +200,62 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
   const uint32_t npc = (uint32_t)P.npc;
   const uint32_t quads = (uint32_t)((P.N + 3) / 4);  // below 2^29
   const uint32_t stride = (uint32_t)vgrid * (uint32_t)(kUpdateWarps * 32);  // quads
-  // whole: a quad lies in one column; else (in a net) its input is read word
-  // by word
+  // A quad's input: one 16-byte access where columns are whole quads (or acc
+  // is indexed by the neuron); else word by word, in its first neuron's column
+  // and the next one (columns of 2 or 3 neurons: see below).
   const bool whole = (npc & 3u) == 0u;
   const bool direct = P.colv == nullptr || whole;
+  const bool split = !direct && npc >= 4u;
 
   // The state of the warp's next chunk is requested before the current chunk
-  // is processed, and the virtual index of the column of the one after it
+  // is processed, and the virtual index of the column(s) of the one after it
   // (which its input's address needs), so their latency overlaps the work.
-  // q0: quad of the current chunk's lane 0; a: quad of the input; l: place of
-  // the quad's first neuron in its column.
+  // l: place of the quad's first neuron in its column; a: quad of its input, or
+  // word of the first neuron's input with a2 the word that neuron would have
+  // in front of the next column.
   float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), pc = pv;
   uint32_t pr = 0u;
   int4 pa = make_int4(0, 0, 0, 0);
-  auto place = [&](uint32_t q, uint32_t* l, uint32_t* v) {
+  auto place = [&](uint32_t q, uint32_t* l, uint32_t* v, uint32_t* v2) {
     const uint32_t c = div_by(4u * q, npc, P.npc_m);
     *l = 4u * q - c * npc;
     *v = P.colv != nullptr && q < quads ? __ldg(P.colv + c) : 0u;
+    *v2 = split && q < quads && c + 1u < (uint32_t)P.ncol ? __ldg(P.colv + c + 1u) : 0u;
   };
-  auto input_quad = [&](uint32_t q, uint32_t l, uint32_t v) -> uint32_t {
-    return P.colv == nullptr ? q : (uint32_t)(((unsigned long long)v * (uint32_t)P.npc4 + l) >> 2);
+  auto input = [&](uint32_t q, uint32_t l, uint32_t v, uint32_t v2, uint32_t* a, uint32_t* a2) {
+    const unsigned long long w = (unsigned long long)v * (uint32_t)P.npc4 + l;
+    *a = P.colv == nullptr ? q : whole ? (uint32_t)(w >> 2) : (uint32_t)w;
+    *a2 = v2 * (uint32_t)P.npc4 + l - npc;
   };
-  auto load = [&](uint32_t q, uint32_t a) {
+  // word of neuron 4 q + e's input (split)
+  auto word = [&](uint32_t l, uint32_t a, uint32_t a2, uint32_t e) -> int32_t* {
+    return P.acc + (size_t)(uint32_t)((l + e < npc ? a : a2) + e);
+  };
+  auto load = [&](uint32_t q, uint32_t l, uint32_t a, uint32_t a2) {
     if (q < quads) {
       pv = ld_stream(reinterpret_cast<const float4*>(P.V) + q);
       pc = ld_stream(reinterpret_cast<const float4*>(P.C) + q);
       pr = ld_stream(reinterpret_cast<const uint32_t*>(P.R) + q);
-      if (direct) pa = ld_stream(reinterpret_cast<const int4*>(P.acc) + a);
+      if (direct) {
+        pa = ld_stream(reinterpret_cast<const int4*>(P.acc) + a);
+      } else if (split) {
+        const uint32_t n = (uint32_t)min(4ll, P.N - 4ll * q);
+        pa.x = *word(l, a, a2, 0u);
+        pa.y = n > 1u ? *word(l, a, a2, 1u) : 0;
+        pa.z = n > 2u ? *word(l, a, a2, 2u) : 0;
+        pa.w = n > 3u ? *word(l, a, a2, 3u) : 0;
+      }
     }
   };
   uint32_t q = (uint32_t)vb * (uint32_t)(kUpdateWarps * 32) + (uint32_t)tid;
-  uint32_t l, l_nxt, v, v_nxt;
-  place(q, &l, &v);
-  place(q + stride, &l_nxt, &v_nxt);
-  uint32_t a = input_quad(q, l, v);
+  uint32_t l, l_nxt, v, v2, v_nxt, v2_nxt, a, a2;
+  place(q, &l, &v, &v2);
+  place(q + stride, &l_nxt, &v_nxt, &v2_nxt);
+  input(q, l, v, v2, &a, &a2);
   body_sync(bar);  // the shared memory may still be read by a previous body
   S.pois[tid] = poisson_entry(P, tid);
   const long long t = t_of();
-  load(q, a);
+  load(q, l, a, a2);
   const int slot = slot_of(P, t);
   if (tid == 0) {
     S.rc = 0u;
@@ -284,11 +293,11 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
     const float4 v4 = pv, c4 = pc;
     const uint32_t r4 = pr;
     int4 a4 = pa;
-    const uint32_t a_own = a, l_own = l;
+    const uint32_t a_own = a, a2_own = a2, l_own = l;
     l = l_nxt;
-    a = input_quad(q + stride, l, v_nxt);
-    load(q + stride, a);
-    place(q + 2u * stride, &l_nxt, &v_nxt);
+    input(q + stride, l, v_nxt, v2_nxt, &a, &a2);
+    load(q + stride, l, a, a2);
+    place(q + 2u * stride, &l_nxt, &v_nxt, &v2_nxt);
 
     uint32_t gq = q;  // global quad of the four neurons
     bool own = q < quads;
@@ -305,6 +314,10 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
       const uint4 x = philox4x32_10(make_uint4(gq, (uint32_t)t, kTagExt, 0u), P.seed_lo, P.seed_hi);
       if (direct) {
         reinterpret_cast<int4*>(P.acc)[a_own] = make_int4(0, 0, 0, 0);
+      } else if (split) {
+#pragma unroll
+        for (uint32_t e = 0; e < 4u; ++e)
+          if (4ll * q + e < P.N) *word(l_own, a_own, a2_own, e) = 0;
       } else {
         int32_t in[4];
 #pragma unroll
@@ -1237,6 +1250,31 @@ __device__ __forceinline__ void list_spike(const StepParams& P, long long at, ui
   for (int p = 0; p < P.planes; ++p) P.list[at + p * stride] = d[p];
 }
 
+// Counts the records a drain would return: header {records kept, 1 if any were
+// dropped} to mapped host memory (one block).
+__global__ void __launch_bounds__(1024) count_records_kernel(const unsigned long long* rcnt, int nreg,
+                                                             long long region, const Ctl* ctl,
+                                                             unsigned long long* map_hdr) {
+  __shared__ unsigned long long s_kept[32];
+  unsigned long long kept = 0ull;
+  unsigned lost = ctl->rec_overflow;
+  for (int r = threadIdx.x; r < nreg; r += blockDim.x) {
+    const unsigned long long v = rcnt[r];
+    kept += (long long)v < region ? v : (unsigned long long)region;
+    lost |= (long long)v > region ? 1u : 0u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xFFFFFFFFu, kept, o);
+  if ((threadIdx.x & 31) == 0) s_kept[threadIdx.x >> 5] = kept;
+  const int any = __syncthreads_or((int)lost);
+  if (threadIdx.x == 0) {
+    kept = 0ull;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) kept += s_kept[w];
+    map_hdr[0] = kept;
+    map_hdr[1] = any ? 1ull : 0ull;
+  }
+}
+
 // Shard: the received spikes of step t (global indices ids[0 .. n)) that
 // belong to halo columns join the step's lists as the update kernel's own
 // spikes do, at the next place of the tile's list.  Indices of the shard's
@@ -1296,23 +1334,6 @@ int update_grid(long long N, int num_sms) {
 }
 
 namespace {
-// Launches kernel fn(p); `overlap`: while the kernel before it on the stream
-// still runs (see grid_wait).
-cudaError_t launch_step(const void* fn, const StepParams& p, int grid, int threads, size_t smem,
-                        bool overlap, cudaStream_t st) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1u : 0u;
-  void* args[] = {const_cast<StepParams*>(&p)};
-  return cudaLaunchKernelExC(&cfg, fn, args);
-}
 const void* deliver_fn(int precision) {
   return precision == SNN_EXACT_F16W ? reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F16W>)
                                      : reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F32W>);
@@ -1322,7 +1343,8 @@ const void* deliver_fn(int precision) {
 cudaError_t launch_update(const StepParams& p, int grid, bool overlap, cudaStream_t st) {
   const void* fn = p.sg.on ? reinterpret_cast<const void*>(update_kernel<true>)
                            : reinterpret_cast<const void*>(update_kernel<false>);
-  return launch_step(fn, p, grid, kUpdateThreads, 0, overlap, st);
+  void* args[] = {const_cast<StepParams*>(&p)};
+  return launch_overlapped(fn, dim3((unsigned)grid), kUpdateThreads, 0, args, overlap, st);
 }
 
 cudaError_t launch_ingest(const StepParams& p, const uint32_t* ids, long long n, cudaStream_t st) {
@@ -1351,8 +1373,9 @@ int deliver_grid(const StepParams& p, int precision, int num_sms) {
 }
 
 cudaError_t launch_deliver(const StepParams& p, int precision, int grid, bool overlap, cudaStream_t st) {
-  return launch_step(deliver_fn(precision), p, grid, kDeliverThreads,
-                     deliver_smem(p.tcols, p.npc4, false), overlap, st);
+  void* args[] = {const_cast<StepParams*>(&p)};
+  return launch_overlapped(deliver_fn(precision), dim3((unsigned)grid), kDeliverThreads,
+                           deliver_smem(p.tcols, p.npc4, false), args, overlap, st);
 }
 
 cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_ids,
@@ -1362,6 +1385,12 @@ cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_
   drain_records_kernel<<<nreg, 256, 0, st>>>(p.rcnt, nreg, p.rec_region, p.rec, p.ctl, header,
                                              map_hdr, stage_ids, stage_steps, map_ids, map_steps,
                                              map_cap);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_count_records(const StepParams& p, int nreg, unsigned long long* map_hdr,
+                                 cudaStream_t st) {
+  count_records_kernel<<<1, 1024, 0, st>>>(p.rcnt, nreg, p.rec_region, p.ctl, map_hdr);
   return cudaGetLastError();
 }
 
