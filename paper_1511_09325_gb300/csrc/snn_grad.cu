@@ -172,6 +172,8 @@ __device__ __forceinline__ int bucket_of(int k, int end_lane, int ndel) {
 // row four records per lane (16-byte loads; a bucket part is a whole number of
 // 8-slot units, so the four records of a lane share it).
 __global__ void __launch_bounds__(kThreads) grad_deliver_kernel(const GradParams P, long long t) {
+  grid_wait();
+  grid_go();
   const long long j = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (j >= P.N) return;
@@ -226,6 +228,8 @@ __global__ void __launch_bounds__(kThreads) grad_active_kernel(const GradParams 
 // `rates` is set.
 __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams P, long long t,
                                                               int slot, int rates) {
+  grid_wait();
+  grid_go();
   __shared__ float s_sum[kThreads / 32][2];
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   float s = 0.f;
@@ -310,10 +314,10 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
 // 4x4 network, whose table is 197 MB (DRAM floor 31 us); looked up in shared
 // memory, 54 us.  Loading a row's sectors one row ahead (384 threads, more
 // registers) took 68 us.
-constexpr int kGatherThreads = 512;
+constexpr int kGatherThreads = 1024;  // per SM: one block, or two of half as many
 constexpr int kGatherDepth = 3;  // sectors in flight per lane
 
-__global__ void __launch_bounds__(kGatherThreads, 2)
+__global__ void __launch_bounds__(kGatherThreads, 1)
     grad_gather_kernel(const GradParams P, long long tau, int rows_e, int rows_i, int blocks_e,
                        int blocks_i) {
   extern __shared__ __align__(16) float s_ib[];
@@ -334,7 +338,7 @@ __global__ void __launch_bounds__(kGatherThreads, 2)
   const uint32_t r1 = min(rows, r0 + per_block);
   const float* ib = (exc ? P.ibe : P.ibi) + ring(dst, P.nslot) * P.accw;
   const float* own = ib + (size_t)ti.x * P.npc4;
-  for (uint32_t i = threadIdx.x; i < ti.y * (uint32_t)P.npc4 / 4u; i += kGatherThreads)
+  for (uint32_t i = threadIdx.x; i < ti.y * (uint32_t)P.npc4 / 4u; i += blockDim.x)
     reinterpret_cast<float4*>(s_ib)[i] = __ldg(reinterpret_cast<const float4*>(own) + i);
   __syncthreads();
   const uint32_t lane8 = threadIdx.x & 7u;
@@ -355,12 +359,12 @@ __global__ void __launch_bounds__(kGatherThreads, 2)
   };
   load_ends(r0 + threadIdx.x / 8u);
   // every lane takes part in the row loop (its sums are shuffled)
-  for (uint32_t rb = r0; rb < r1; rb += kGatherThreads / 8) {
+  for (uint32_t rb = r0; rb < r1; rb += blockDim.x / 8u) {
     const uint32_t r = rb + threadIdx.x / 8u;
     float acc = 0.f;
     size_t jv = 0;
     const uint32_t beg = beg_n, me = me_n;
-    load_ends(r + kGatherThreads / 8);
+    load_ends(r + blockDim.x / 8u);
     if (r < r1) {
       const uint32_t k = r / npop;
       jv = row_of(r);
@@ -401,6 +405,8 @@ __global__ void __launch_bounds__(kGatherThreads, 2)
 // adjoints of V(tau+1), c(tau+1) and leaves those of V(tau), c(tau).
 __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParams P, long long tau,
                                                                 int slot) {
+  grid_wait();
+  grid_go();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P.N) return;
   const bool exc = (int)((uint32_t)i % (uint32_t)P.npc) < P.nexc;
@@ -525,28 +531,40 @@ void grad_release(snn_grad* g) {
 // Gather of step tau: the buckets that end before T, their blocks in one wave
 // (a block copies its tile's adjoints first, so few and long ones: with 340
 // blocks for 304 places the 4x4 network took 63 us a step, with 300 it takes
-// 54) but at least kGatherMinRows rows each, shared between E and I rows.
+// 54) but at least kGatherMinRows rows each, shared between E and I rows.  A
+// plain launch: launched while the backward kernel still holds registers, its
+// blocks would not fit in one wave; nor does it let the backward kernel be
+// launched early (4x4, 500 steps: 45 ms, 52 ms with either).
 constexpr int kGatherMinRows = 128;
-void launch_gather(snn_grad* g, long long tau) {
+cudaError_t launch_gather(snn_grad* g, long long tau) {
   const NetView& v = g->v;
   const int nb = (int)std::min<long long>(v.ndel, g->T - tau - v.dmin);
-  if (nb <= 0) return;
-  const int slots = v.num_sms * (2 * (g->gather_smem + 2048) <= kSmemBudget ? 2 : 1);
+  if (nb <= 0) return cudaSuccess;
+  const int per_sm = 2 * (g->gather_smem + 2048) <= kSmemBudget ? 2 : 1;
+  const int slots = v.num_sms * per_sm;
   const long long re = (long long)v.tcols * v.nexc, ri = (long long)v.tcols * (v.npc - v.nexc);
   const int most = (int)std::max<long long>(
       2, std::min<long long>(slots / (nb * v.ntile), (re + ri) / kGatherMinRows));
   const int be = re ? std::max(1, (int)(most * re / (re + ri))) : 0;
   const int bi = ri ? std::max(1, most - be) : 0;
-  grad_gather_kernel<<<dim3(v.ntile * (be + bi), nb), kGatherThreads, g->gather_smem, v.stream>>>(
-      g->P, tau, be ? (int)((re + be - 1) / be) : 0, bi ? (int)((ri + bi - 1) / bi) : 0, be, bi);
+  int rows_e = be ? (int)((re + be - 1) / be) : 0, rows_i = bi ? (int)((ri + bi - 1) / bi) : 0;
+  int blocks_e = be, blocks_i = bi;
+  void* args[] = {&g->P, &tau, &rows_e, &rows_i, &blocks_e, &blocks_i};
+  return launch_overlapped(reinterpret_cast<const void*>(grad_gather_kernel),
+                           dim3((unsigned)(v.ntile * (be + bi)), (unsigned)nb), kGatherThreads / per_sm,
+                           g->gather_smem, args, false, v.stream);
 }
 
 cudaError_t launch_forward_step(snn_grad* g, long long t, int slot, int rates) {
   const GradParams& P = g->P;
   cudaStream_t st = g->v.stream;
-  grad_deliver_kernel<<<g->wblocks, kThreads, 0, st>>>(P, t);
-  grad_update_kernel<<<g->ublocks, kThreads, 0, st>>>(P, t, slot, rates);
-  return cudaGetLastError();
+  void* dargs[] = {const_cast<GradParams*>(&P), &t};
+  void* uargs[] = {const_cast<GradParams*>(&P), &t, &slot, &rates};
+  const cudaError_t e = launch_overlapped(reinterpret_cast<const void*>(grad_deliver_kernel),
+                                          dim3((unsigned)g->wblocks), kThreads, 0, dargs, true, st);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(reinterpret_cast<const void*>(grad_update_kernel), dim3((unsigned)g->ublocks),
+                           kThreads, 0, uargs, true, st);
 }
 
 }  // namespace
@@ -741,8 +759,11 @@ int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, 
     grad_active_kernel<<<g->ublocks, kThreads, 0, st>>>(P, t0);
     for (long long t = t0; t < t1; ++t) SNN_GCUDA(g, launch_forward_step(g, t, (int)(t - t0), 0));
     for (long long tau = t1 - 1; tau >= t0; --tau) {
-      launch_gather(g, tau);
-      grad_backward_kernel<<<g->ublocks, kThreads, 0, st>>>(P, tau, (int)(tau - t0));
+      SNN_GCUDA(g, launch_gather(g, tau));
+      int slot = (int)(tau - t0);
+      void* args[] = {&P, &tau, &slot};
+      SNN_GCUDA(g, launch_overlapped(reinterpret_cast<const void*>(grad_backward_kernel),
+                                     dim3((unsigned)g->ublocks), kThreads, 0, args, true, st));
     }
     SNN_GCUDA(g, cudaGetLastError());
   }
