@@ -9,10 +9,12 @@
 // scratch (step counter, spike-list cursor, per-block partial sums and the
 // per-column spike counters) lives in one file-scope device array below, of a
 // fixed size, which every GPU that loads the library holds until exit.
+#include <algorithm>
 #include <cstddef>
 #include <mutex>
 #include <string>
 
+#include "snn_device.cuh"
 #include "snn_internal.h"
 
 using namespace snn;
@@ -26,7 +28,7 @@ constexpr int kMaxDevices = 64;
 // Byte offsets inside the scratch array.
 constexpr size_t kOffCtl = 0;                                       // Ctl
 constexpr size_t kOffCnt = 256;                                     // u32 spike count
-constexpr size_t kOffExtSum = 264;                                  // u64 sum of ext_part
+constexpr size_t kOffOut = 264;                                     // u64 spikes, sum of ext_part
 constexpr size_t kOffExt = 512;                                     // u64[blocks]
 constexpr size_t kOffSpk = kOffExt + 8 * (size_t)kNoAllocMaxBlocks;  // u64[blocks]
 constexpr size_t kOffRc = kOffSpk + 8 * (size_t)kNoAllocMaxBlocks;   // u64[blocks]
@@ -36,6 +38,36 @@ constexpr size_t kScratchBytes = kOffCol + 16 * (size_t)kNoAllocMaxCols;  // 311
 static_assert(sizeof(Ctl) <= kOffCnt, "control block overlaps the counters");
 
 __device__ __align__(256) unsigned char g_update_scratch[kScratchBytes];
+
+// Clears the first `words` 8-byte words of the scratch, with the step index in
+// the control block.
+constexpr int kThreads = 1024;
+__global__ void __launch_bounds__(kThreads) begin_kernel(unsigned long long* scratch, int words,
+                                                         long long t) {
+  grid_go();
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < words; i += gridDim.x * kThreads)
+    scratch[i] = i == (int)(offsetof(Ctl, t) / 8) ? (unsigned long long)t : 0ull;
+}
+
+// Results after the update: the spike count and the external events, side by
+// side, and a copy of the column counts when wanted.
+__global__ void __launch_bounds__(kThreads) end_kernel(const unsigned* cnt, const unsigned long long* ext_part,
+                                                       int nparts, unsigned long long* out,
+                                                       const unsigned long long* colcnt,
+                                                       unsigned long long* col_counts, int ncounts) {
+  grid_wait();
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < ncounts; i += gridDim.x * kThreads)
+    col_counts[i] = colcnt[i];
+  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+  unsigned long long s = 0ull;
+  for (int i = threadIdx.x; i < nparts; i += 32) s += ext_part[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if (threadIdx.x == 0) {
+    out[0] = *cnt;
+    out[1] = s;
+  }
+}
 
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
@@ -135,26 +167,32 @@ extern "C" int snn_update_noalloc(int grid_w, int grid_h, const snn_neuron_param
   p.rec_region = 0;
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // everything the kernel accumulates into starts at zero; the step index
-  // goes into the control block
-  const long long t = step;
-  e = cudaMemsetAsync(base, 0, kOffCol + 16 * (size_t)ncol, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(base + kOffCtl + offsetof(Ctl, t), &t, sizeof(t), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_update(p, grid, false, st);
-  if (e == cudaSuccess)
-    e = launch_sum_parts(p.ext_part, grid, reinterpret_cast<unsigned long long*>(base + kOffExtSum), st);
-  unsigned n = 0u;
-  unsigned long long ext = 0ull;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&n, base + kOffCnt, sizeof(n), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&ext, base + kOffExtSum, sizeof(ext), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && col_counts)
-    e = cudaMemcpyAsync(col_counts, base + kOffCol, 16 * (size_t)ncol, cudaMemcpyDeviceToDevice, st);
+  // Three kernels and one copy back: everything the update accumulates into
+  // starts at zero, and the step index goes into the control block; then the
+  // results.  (A memset, a copy in, the update, a sum and three copies before:
+  // each of the copies to or from pageable memory waited for the stream.)
+  const int words = (int)((kOffCol + 16 * (size_t)ncol) / 8), ncounts = col_counts ? 2 * (int)ncol : 0;
+  begin_kernel<<<std::min(num_sms, (words + kThreads - 1) / kThreads), kThreads, 0, st>>>(
+      reinterpret_cast<unsigned long long*>(base), words, step);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_update(p, grid, true, st);
+  unsigned long long* d_out = reinterpret_cast<unsigned long long*>(base + kOffOut);
+  unsigned long long out[2] = {0ull, 0ull};
+  if (e == cudaSuccess) {
+    const unsigned* cnt = p.cnt;
+    const unsigned long long* ext = p.ext_part;
+    const unsigned long long* col = p.colcnt;
+    int nparts = grid, nc = ncounts;
+    void* args[] = {&cnt, &ext, &nparts, &d_out, &col, &col_counts, &nc};
+    e = launch_overlapped(reinterpret_cast<const void*>(end_kernel),
+                          dim3((unsigned)std::max(1, std::min(num_sms, (ncounts + kThreads - 1) / kThreads))),
+                          kThreads, 0, args, true, st);
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, sizeof(out), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess)
     return fail_global(SNN_ECUDA, std::string("snn_update_noalloc: ") + cudaGetErrorString(e));
-  *n_spikes = (int64_t)n;
-  if (ext_events) *ext_events = (int64_t)ext;
+  *n_spikes = (int64_t)out[0];
+  if (ext_events) *ext_events = (int64_t)out[1];
   return SNN_OK;
 }
