@@ -373,6 +373,7 @@ void fill_step_params(snn_net* net) {
   p.npc_m = recip32((uint32_t)net->npc);
   p.seed_lo = (uint32_t)(net->seed & 0xFFFFFFFFu);
   p.seed_hi = (uint32_t)(net->seed >> 32);
+  philox_keys(&p);
   p.pvv = t.pvv;
   p.pcc = t.pcc;
   p.pvc_e = t.pvc[0];

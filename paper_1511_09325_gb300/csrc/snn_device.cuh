@@ -11,18 +11,25 @@ namespace snn {
 // two round constants, xors the high halves into the other words and the key,
 // and permutes; the key advances by the Weyl constants after every round.
 // Counter = (a, b, stream tag, 0), key = 64-bit seed.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0,
-                                               uint32_t k1) {
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1) {
+  const unsigned long long p0 = (unsigned long long)0xD2511F53u * c.x;
+  const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * c.z;
+  return make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1,
+                    (uint32_t)p0);
+}
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c.x;
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-    c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+    c = philox_round(c, k0, k1);
     k0 += 0x9E3779B9u;
     k1 += 0xBB67AE85u;
   }
+  return c;
+}
+// The same with the rounds' keys laid out in turn (key[2 r], key[2 r + 1]).
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const uint32_t* key) {
+#pragma unroll
+  for (int r = 0; r < 10; ++r) c = philox_round(c, key[2 * r], key[2 * r + 1]);
   return c;
 }
 

@@ -193,6 +193,7 @@ struct StepParams {
   unsigned cost_win;       // fixed cost (in items) of a tile with a window
   uint32_t npc_m;          // floor(2^32 / n_per_col) (capped)
   uint32_t seed_lo, seed_hi;
+  uint32_t key[20];        // the seed's Philox keys of the ten rounds
   float theta, vr, dc, pvv, pcc, pvc_e, pvc_i;
   int32_t jx;
   int nref;
@@ -312,6 +313,14 @@ int net_view(snn_net* net, NetView* v);
 inline uint32_t recip32(uint32_t d) {
   const unsigned long long m = (1ull << 32) / (unsigned long long)d;
   return m > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)m;
+}
+
+// The seed's Philox round keys (Weyl sequences of the two key words).
+inline void philox_keys(StepParams* p) {
+  for (uint32_t r = 0; r < 10; ++r) {
+    p->key[2 * r] = p->seed_lo + r * 0x9E3779B9u;
+    p->key[2 * r + 1] = p->seed_hi + r * 0xBB67AE85u;
+  }
 }
 
 // Shared host helpers (snn_api.cu).

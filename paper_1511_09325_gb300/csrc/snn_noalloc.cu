@@ -140,6 +140,7 @@ extern "C" int snn_update_noalloc(int grid_w, int grid_h, const snn_neuron_param
   p.ncol = (int)ncol;
   p.seed_lo = (uint32_t)(seed & 0xFFFFFFFFu);
   p.seed_hi = (uint32_t)(seed >> 32);
+  philox_keys(&p);
   p.theta = neuron->theta;
   p.vr = neuron->v_reset;
   p.dc = neuron->dc;

@@ -58,27 +58,21 @@ struct NeuronOut {
   bool spike;
 };
 
-// One neuron, one step; every float operation rounded as written.
+// One neuron, one step; every float operation rounded as written.  Selects, no
+// branches: a refractory neuron (r > 0) discards its input and is clamped to
+// V_reset.
 __device__ __forceinline__ NeuronOut neuron_step(float v, float c, uint32_t r,
                                                  int32_t I, float pvc,
                                                  const StepParams& P) {
   NeuronOut o;
-  o.spike = false;
-  if (r > 0u) {
-    r -= 1u;
-    v = P.vr;
-  } else {
-    v = __fadd_rn(v, __fmul_rn(__int2float_rn(I), 1.52587890625e-05f));
-    if (v >= P.theta) {
-      o.spike = true;
-      v = P.vr;
-      r = (uint32_t)P.nref;
-      c = __fadd_rn(c, P.dc);
-    }
-  }
-  o.v = __fmaf_rn(c, pvc, __fmul_rn(v, P.pvv));
-  o.c = __fmul_rn(c, P.pcc);
-  o.r = r;
+  const float u = __fadd_rn(v, __fmul_rn(__int2float_rn(I), 1.52587890625e-05f));
+  const bool active = r == 0u;
+  o.spike = active && u >= P.theta;
+  const float w = active && !o.spike ? u : P.vr;
+  const float ca = o.spike ? __fadd_rn(c, P.dc) : c;
+  o.r = active ? (o.spike ? (uint32_t)P.nref : 0u) : r - 1u;
+  o.v = __fmaf_rn(ca, pvc, __fmul_rn(w, P.pvv));
+  o.c = __fmul_rn(ca, P.pcc);
   return o;
 }
 
@@ -311,7 +305,7 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
     }
     unsigned spk = 0u;  // bit e: neuron 4 q + e fired
     if (own) {
-      const uint4 x = philox4x32_10(make_uint4(gq, (uint32_t)t, kTagExt, 0u), P.seed_lo, P.seed_hi);
+      const uint4 x = philox4x32_10(make_uint4(gq, (uint32_t)t, kTagExt, 0u), P.key);
       if (direct) {
         reinterpret_cast<int4*>(P.acc)[a_own] = make_int4(0, 0, 0, 0);
       } else if (split) {
@@ -352,7 +346,6 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
             kp[e] = k;
           }
       }
-      const bool tail = 4ll * q + 4 > P.N;  // the last quad may end early
       float vout[4], cout[4];
       uint32_t rout = 0u;
 #pragma unroll
@@ -363,16 +356,21 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
           le -= le >= npc ? npc : 0u;
         }
         const int32_t I = ain[e] + kp[e] * P.jx;
-        const NeuronOut o = neuron_step(vin[e], cin[e], r4 >> (8 * e) & 0xFFu, I,
-                                        le < (uint32_t)P.nexc ? P.pvc_e : P.pvc_i, P);
+        const uint32_t r = r4 >> (8 * e) & 0xFFu;
+        const NeuronOut o = neuron_step(vin[e], cin[e], r, I, le < (uint32_t)P.nexc ? P.pvc_e : P.pvc_i, P);
         vout[e] = o.v;
         cout[e] = o.c;
-        rout |= (o.r & 0xFFu) << (8 * e);
-        if (!tail || 4ll * q + e < P.N) {
-          ksum += (unsigned)kp[e];
-          spk |= o.spike ? 1u << e : 0u;
-        }
+        rout |= o.r << (8 * e);
+        spk |= o.spike ? 1u << e : 0u;
       }
+      if (q == quads - 1u && (P.N & 3)) {  // the last quad ends early
+        const int live = (int)(P.N & 3);
+        spk &= (1u << live) - 1u;
+#pragma unroll
+        for (int e = 1; e < 4; ++e)
+          if (e >= live) kp[e] = 0;
+      }
+      ksum += (unsigned)(kp[0] + kp[1] + kp[2] + kp[3]);
       reinterpret_cast<float4*>(P.V)[q] = make_float4(vout[0], vout[1], vout[2], vout[3]);
       reinterpret_cast<float4*>(P.C)[q] = make_float4(cout[0], cout[1], cout[2], cout[3]);
       reinterpret_cast<uint32_t*>(P.R)[q] = rout;
