@@ -234,8 +234,9 @@ int validate(int gw, int gh, const snn_neuron_params* n, const snn_synapse_param
 // (88 %, but 36 window columns flushed per 16 columns of spikes) by 13 %, 17 %
 // and 3 %; 5x5 and 4x4 tiles without ring and 3x3 with a ring are slower still.
 // Fewest items a delivery block takes (fewer blocks run when a step has few
-// items).
-constexpr unsigned kMinItems = 64;
+// items).  Measured (us per delivery, mean state) with 128, 64, 32 and 16: 2x2
+// FP32 12.1, 11.2, 10.8, 10.6; 8x8 FP16 18.4, 16.8, 15.2, 15.1.
+constexpr unsigned kMinItems = 16;
 constexpr unsigned kBatchMinItems = 256;
 
 void choose_tiles(snn_net* net) {
