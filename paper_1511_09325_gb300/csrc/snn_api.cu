@@ -39,6 +39,8 @@ struct snn_net {
   uint8_t* R = nullptr;
   int32_t* acc = nullptr;
   uint4* list = nullptr;                  // spike lists
+  uint16_t* rlist = nullptr;              // or lists of rows
+  bool lean = false;                      // keep lists of rows in any case
   uint32_t* ctile = nullptr;              // geometry tables (see snn_internal.h)
   uint32_t* colv = nullptr;
   uint2* tinfo = nullptr;
@@ -175,7 +177,7 @@ void release(snn_net* net) {
   if (net->ingest_ev) cudaEventDestroy(net->ingest_ev);
   for (cudaEvent_t ev : net->copy_ev)
     if (ev) cudaEventDestroy(ev);
-  void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->ctile,
+  void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->rlist, net->ctile,
                   net->colv, net->tinfo, net->nbg, net->icnt, net->ccnt, net->deg, net->syn_part,
                   net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage, net->dhdr,
                   net->colcnt, net->ext_part, net->spk_part};
@@ -390,6 +392,7 @@ void fill_step_params(snn_net* net) {
   p.acc = net->acc;
   p.ids = nullptr;
   p.list = net->list;
+  p.rlist = net->rlist;
   p.planes = net->planes;
   p.ctile = net->ctile;
   p.colv = net->colv;
@@ -503,6 +506,16 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->bend, (size_t)net->N * net->planes * 16))) return rc;
   net->total_syn = net->N * (long long)net->K;
   if (net->sg.on && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
+  // the longest row (bp.max_units), read back by a count pass
+  unsigned max_units[2] = {0u, 0u};
+  auto longest_row = [&](auto&& count) -> cudaError_t {
+    cudaError_t ce = cudaMemsetAsync(bp.max_units, 0, 8, net->stream);
+    if (ce == cudaSuccess) ce = count(bp, net->num_sms, net->stream);
+    if (ce == cudaSuccess)
+      ce = cudaMemcpyAsync(max_units, bp.max_units, 8, cudaMemcpyDeviceToHost, net->stream);
+    return ce == cudaSuccess ? cudaStreamSynchronize(net->stream) : ce;
+  };
+  bp.bend = net->bend;
   if (net->connectivity == SNN_CONN_PAPER) {
     // count pass: bucket ends, out-degrees and the longest row, which sets
     // the row stride of the table
@@ -510,18 +523,12 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
     if ((rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
     if ((rc = dalloc(net, &dmax, 8))) return rc;
     net->device_bytes -= 8;
-    unsigned max_units[2] = {0u, 0u};
-    bp.bend = net->bend;
     bp.deg = net->deg;
     bp.max_units = dmax;
     cudaError_t ce = cudaSuccess;
     for (net->unit = kSlotUnit; ce == cudaSuccess; net->unit *= 2) {
       bp.unit = net->unit;
-      ce = cudaMemsetAsync(dmax, 0, 8, net->stream);
-      if (ce == cudaSuccess) ce = launch_paper_count(bp, net->num_sms, net->stream);
-      if (ce == cudaSuccess)
-        ce = cudaMemcpyAsync(max_units, dmax, 8, cudaMemcpyDeviceToHost, net->stream);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(net->stream);
+      ce = longest_row(launch_paper_count);
       if (max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
     }
     cudaFree(dmax);
@@ -536,6 +543,24 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
     net->total_syn = 0;
     for (uint32_t d : deg) net->total_syn += d;
   }
+  // Lists of descriptors take planes x 16 bytes per neuron and step.  Where
+  // they do not fit the device beside the table, lists of rows take their place
+  // and the table's rows get the longest row's length, not the longest possible.
+  const size_t tcap = (size_t)net->tw * net->th * net->npc;
+  const size_t list_len = (size_t)net->nslot * net->ntile * tcap;
+  const size_t rest = (size_t)net->Npad * 17 + (size_t)net->rec_region * net->update_grid * 16 + (64u << 20);
+  size_t free_bytes = 0, all_bytes = 0;
+  SNN_CUDA(net, cudaMemGetInfo(&free_bytes, &all_bytes));
+  const bool rows = net->lean || (size_t)net->N * net->rowcap * net->rec_size +
+                                         list_len * net->planes * 16 + rest > free_bytes;
+  if (rows && net->connectivity != SNN_CONN_PAPER) {
+    if ((rc = dalloc(net, &bp.max_units, 8))) return rc;
+    net->device_bytes -= 8;
+    const cudaError_t ce = longest_row(launch_row_lengths);
+    cudaFree(bp.max_units);
+    if (ce != cudaSuccess) return cuda_fail(net, ce, "row-length pass");
+    net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
+  }
   bp.rowcap = net->rowcap;
   const size_t syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
   if ((rc = dalloc(net, &net->syn, syn_bytes))) return rc;
@@ -546,9 +571,11 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   const size_t ccnt_bytes = (size_t)net->nslot * net->ntile * kCntStride * 4;
   const size_t isum_bytes = (size_t)net->ntile * kCntStride * 4;
   if ((rc = dalloc(net, &net->acc, acc_bytes))) return rc;
-  const size_t tcap = (size_t)net->tw * net->th * net->npc;
-  if ((rc = dalloc(net, &net->list, (size_t)net->nslot * net->planes * net->ntile * tcap * 16)))
+  if (rows) {
+    if ((rc = dalloc(net, &net->rlist, list_len * 2))) return rc;
+  } else if ((rc = dalloc(net, &net->list, list_len * net->planes * 16))) {
     return rc;
+  }
   if ((rc = dalloc(net, &net->ccnt, ccnt_bytes))) return rc;
   if ((rc = dalloc(net, &net->isum, isum_bytes))) return rc;
   if ((rc = dalloc(net, &net->gsum, 4))) return rc;
@@ -597,6 +624,8 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
                                             : launch_build(bp, precision, net->num_sms, net->stream);
   }
   fill_step_params(net);
+  if (rows && deliver_grid(net->sp, precision, net->num_sms) < 1)
+    return fail(net, SNN_ECUDA, "delivery kernel does not fit on the device");
   if (e == cudaSuccess) e = launch_init_state(net->sp, net->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
   cudaFree(wtab);
@@ -701,7 +730,7 @@ namespace {
 int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
               const snn_synapse_params* synapse, uint64_t seed, int precision,
               void* cuda_stream, bool batch_member, snn_net** out,
-              const ShardGeo* shard = nullptr) {
+              const ShardGeo* shard = nullptr, bool lean = false) {
   if (!out) return fail(nullptr, SNN_EINVAL, "out is NULL");
   *out = nullptr;
   std::string why;
@@ -710,6 +739,7 @@ int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
   snn_net* net = new (std::nothrow) snn_net();
   if (!net) return fail(nullptr, SNN_ENOMEM, "host allocation failed");
   net->batch_member = batch_member;
+  net->lean = lean;
   net->min_items = batch_member ? kBatchMinItems : kMinItems;
   if (shard) net->sg = *shard;
   if (cuda_stream) {
@@ -1356,10 +1386,12 @@ int batch_run(snn_batch* b, long long n_steps) {
     bp.max_cols = std::max(bp.max_cols, net->sp.tcols);
   }
   const size_t smem = batch_smem(bp.win_words, bp.max_cols);
-  const int grid = batch_grid(b->precision, b->infl, b->num_sms, smem);
+  bool rows = false;
+  for (const snn_net* net : b->nets) rows = rows || net->rlist != nullptr;
+  const int grid = batch_grid(b->precision, b->infl, rows, b->num_sms, smem);
   if (grid < 1) return bfail(b, SNN_ECUDA, "batch kernel does not fit on the device");
   SNN_BCUDA(b, cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream));
-  SNN_BCUDA(b, launch_batch(bp, b->precision, b->infl, grid, smem, b->stream));
+  SNN_BCUDA(b, launch_batch(bp, b->precision, b->infl, rows, grid, smem, b->stream));
   unsigned flags[3] = {0u, 0u, 0u};
   SNN_BCUDA(b, cudaMemcpyAsync(flags, b->d_bar, sizeof(flags), cudaMemcpyDeviceToHost, b->stream));
   SNN_BCUDA(b, cudaStreamSynchronize(b->stream));
@@ -1400,10 +1432,20 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
   }
   int rc = SNN_OK;
   b->first.assign(2 * (size_t)(n_nets + 1), 0);
+  bool lean = false;
   for (int k = 0; k < n_nets && rc == SNN_OK; ++k) {
     snn_net* net = nullptr;
     rc = build_net(grid_w[k], grid_h[k], neuron + k, synapse + k, seeds[k], precision, b->stream,
-                   true, &net);
+                   true, &net, nullptr, lean);
+    if (rc == SNN_ENOMEM && !lean) {
+      // the members before took more memory than they need: once more, all lean
+      for (snn_net* n : b->nets) snn_destroy(n);
+      b->nets.clear();
+      lean = true;
+      rc = SNN_OK;
+      k = -1;
+      continue;
+    }
     if (rc != SNN_OK) break;
     net->in_batch = true;
     b->nets.push_back(net);

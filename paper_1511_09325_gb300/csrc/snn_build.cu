@@ -242,7 +242,7 @@ __device__ __forceinline__ void pad_parts(const BuildParams& P, RowSmem& S, cons
 }
 
 // Rows of the fixed law, one warp per row; MODE fill builds them, read writes
-// rows j0 .. j0 + n_rows - 1 to the rd_* arrays.
+// rows j0 .. j0 + n_rows - 1 to the rd_* arrays, count finds the longest.
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const BuildParams P) {
   __shared__ RowSmem S;
@@ -275,7 +275,11 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const Buil
       if (lane == 0) P.deg[j] = nkept;
     }
     __syncwarp();
-    open_parts<MODE>(P, S, r);
+    const unsigned units = open_parts<MODE>(P, S, r);
+    if (MODE == kModeCount) {
+      if (lane == 0) atomicMax(P.max_units, units);
+      continue;
+    }
 
     const uint32_t* wt = P.wtab + (r.lj < P.nexc ? 0 : 65536);
     const long long out0 = MODE == kModeRead ? P.rd_off[i] : 0;
@@ -443,6 +447,11 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
 }
 
 }  // namespace
+
+cudaError_t launch_row_lengths(const BuildParams& bp, int num_sms, cudaStream_t st) {
+  build_rows_kernel<SNN_EXACT_F32W, kModeCount><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st) {
   paper_rows_kernel<SNN_EXACT_F32W, kModeCount><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);

@@ -34,6 +34,8 @@
 //          spikes of the last d_max + 1 steps (slot t % (d_max + 1)) per tile,
 //          in no fixed order; ccnt[slot][tile] of them (one counter per 32
 //          bytes).  The items of a bucket read one plane of one list in order.
+//   rlist  u16[d_max + 1][ntile][tcap]: the spikers' rows in their tiles, in
+//          place of `list` where the device has no room for it.
 //   isum   u32[ntile] (bucket, spiker) items of each tile over the steps that
 //          the delivery of step t reads, less step t itself (one counter per 32
 //          bytes); gsum: their sum.
@@ -206,6 +208,7 @@ struct StepParams {
   int32_t* acc;
   uint32_t* ids;   // compact spike-id list (noalloc form only)
   uint4* list;     // spike lists per slot, plane and tile (with ccnt)
+  uint16_t* rlist; // lists of rows instead (list is null then)
   const uint32_t* ctile;
   const uint32_t* colv;   // null: acc is indexed by the real neuron index
   const uint2* tinfo;
@@ -330,6 +333,8 @@ int validate_neuron_params(const snn_neuron_params* n, std::string* why);
 // Kernel launchers (snn_build.cu / snn_step.cu).
 cudaError_t launch_build(const BuildParams& bp, int precision, int num_sms,
                          cudaStream_t st);
+// Longest row in units of the fixed law's rows (to max_units[0]).
+cudaError_t launch_row_lengths(const BuildParams& bp, int num_sms, cudaStream_t st);
 // Paper connectivity law: the count pass writes bend, deg and max_units; the
 // fill pass (same draws) writes the rows.
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st);
@@ -366,8 +371,9 @@ cudaError_t launch_count_records(const StepParams& p, int nreg, unsigned long lo
 // Batch kernel: dynamic shared memory for members whose largest window has
 // win_words words and whose largest tile has max_cols columns, its grid (0 if it does not fit), its launch.
 size_t batch_smem(int win_words, int max_cols);
-int batch_grid(int precision, int infl, int num_sms, size_t smem);
-cudaError_t launch_batch(const BatchParams& b, int precision, int infl, int grid, size_t smem,
+// `rows`: some member keeps lists of rows.
+int batch_grid(int precision, int infl, bool rows, int num_sms, size_t smem);
+cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, int grid, size_t smem,
                          cudaStream_t st);
 // Shard: list the received spikes (global indices ids[0 .. n)) of the halo
 // columns in the step's lists, as the update kernel lists its own.

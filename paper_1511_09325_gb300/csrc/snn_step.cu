@@ -400,8 +400,9 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
           const uint32_t ct = __ldg(P.ctile + c);
           row = __ldg(P.colv + c) * npc + il;
           const size_t ts = (size_t)slot * P.ntile + (ct >> 6);
-          at = ((unsigned long long)slot * P.planes * P.ntile + (ct >> 6)) * P.tcap +
-               next_place(P.ccnt + ts * kCntStride, ct >> 6);
+          const unsigned place = next_place(P.ccnt + ts * kCntStride, ct >> 6);
+          at = ((unsigned long long)slot * P.planes * P.ntile + (ct >> 6)) * P.tcap + place;
+          if (P.rlist != nullptr) P.rlist[ts * P.tcap + place] = (uint16_t)((ct & 63u) * npc + il);
         } else {
           P.ids[next_place(P.cnt + slot, 0u)] = id;
         }
@@ -419,7 +420,7 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
           P.rec[(long long)vb * P.rec_region + (long long)ri] = ((unsigned long long)(unsigned)t << 32) | gid;
       }
       // descriptors: four lanes copy one spike's planes into its list
-      if (P.ccnt != nullptr) {
+      if (P.list != nullptr) {
         const size_t plane = (size_t)P.ntile * P.tcap;
         for (unsigned s0 = 0u; s0 < min(n - k0, 32u); s0 += 8u) {
           const int src = (int)(s0 + ((unsigned)lane >> 2));
@@ -527,7 +528,10 @@ __device__ __forceinline__ void block_scan3(unsigned long long a, unsigned long 
 // What a warp needs of the part it streams: items a .. b - 1 of a tile.
 struct Part {
   const unsigned char* syn;  // the tile's first row
-  const uint4* lst;          // lane b: bucket b's descriptors, less its first item's place
+  const uint4* lst;          // lane b: bucket b's descriptors (lists of rows: its
+                             // u16 rows), less its first item's place
+  const uint4* bend;         // lists of rows: the tile's first descriptor, else null
+  int planes;
   unsigned pfx;              // lane b: items of the tile before bucket b
   unsigned a, b;
 };
@@ -535,6 +539,8 @@ struct Part {
 // Item `item` of the part: its descriptor's plane and its bucket.  The
 // buckets' prefixes lie in the lanes; a five-step search over them finds the
 // last bucket that starts at or before the item.  Beyond the part: bucket -1.
+// ROWS: the net may keep lists of rows.
+template <bool ROWS>
 __device__ __forceinline__ int load_item(const Part& T, unsigned item, uint4* d) {
   int lo = 0;
 #pragma unroll
@@ -544,7 +550,12 @@ __device__ __forceinline__ int load_item(const Part& T, unsigned item, uint4* d)
   }
   const unsigned long long l = __shfl_sync(0xFFFFFFFFu, (unsigned long long)T.lst, lo);
   if (item >= T.b) return -1;
-  *d = __ldcs(reinterpret_cast<const uint4*>(l) + item);
+  if (ROWS && T.bend != nullptr) {
+    const uint32_t row = __ldcs(reinterpret_cast<const uint16_t*>(l) + item);
+    *d = __ldg(T.bend + (size_t)row * T.planes + lo / kPlaneBuckets);
+  } else {
+    *d = __ldcs(reinterpret_cast<const uint4*>(l) + item);
+  }
   return lo;
 }
 
@@ -645,7 +656,7 @@ __device__ __forceinline__ void deliver_out(const Sector& s, float scale, uint32
 // One warp streams its share of a part: batches of bs items, batch q by warp
 // q mod the block's warps (counted from warp `w0`).  WIN: the part's window
 // and neighbour table are in shared memory.
-template <int PREC, int DEPTH, bool WIN>
+template <int PREC, int DEPTH, bool ROWS, bool WIN>
 __device__ __forceinline__ void stream_part(const StepParams& P, const Part& T, const int32_t* acc_t,
                                             const uint32_t* nb_g, unsigned bs, int w0, uint32_t win_s,
                                             uint32_t nb_s, uint32_t* list) {
@@ -659,7 +670,7 @@ __device__ __forceinline__ void stream_part(const StepParams& P, const Part& T, 
   if (it0 >= T.b) return;
   // this lane's item of the batch at i: none beyond the batch or the part
   auto item_at = [&](unsigned i, uint4* d) -> int {
-    return load_item(T, (unsigned)lane < bs && i < T.b ? i + lane : 0xFFFFFFFFu, d);
+    return load_item<ROWS>(T, (unsigned)lane < bs && i < T.b ? i + lane : 0xFFFFFFFFu, d);
   };
   uint4 raw = make_uint4(0u, 0u, 0u, 0u);
   int nb = item_at(it0, &raw);
@@ -795,7 +806,7 @@ struct NetTiles {
 // block's dynamic shared memory: window, neighbour table, sector lists (for
 // windows of at most win_words words and max_cols columns).  The step is
 // t_of(), called when the lists may be read.
-template <int PREC, int DEPTH, int NT, class Tiles, class F>
+template <int PREC, int DEPTH, int NT, bool ROWS, class Tiles, class F>
 __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, int vgrid, int win_words,
                                                int max_cols, DeliverSmem& S, unsigned char* dyn) {
   const int tid = threadIdx.x;
@@ -925,6 +936,13 @@ __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, i
       T.pfx = lane < P.ndel ? incl - n : 0xFFFFFFFFu;
       T.lst = P.list + ((((long long)slot_l * P.planes + lane / kPlaneBuckets) * P.ntile + tile) * P.tcap -
                         (long long)T.pfx);
+      T.bend = nullptr;
+      T.planes = 0;
+      if (ROWS && P.rlist != nullptr) {
+        T.lst = reinterpret_cast<const uint4*>(P.rlist + (ts * P.tcap - (long long)T.pfx));
+        T.bend = P.bend + (size_t)ti.x * P.npc * P.planes;
+        T.planes = P.planes;
+      }
       int32_t* const acc_t = P.acc + (size_t)ti.x * P.npc4;
       const uint32_t* nb_g = P.nbg + (size_t)ti.x * 64;
       const int cols = (int)ti.y;
@@ -946,7 +964,7 @@ __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, i
         // warp's items rounded down, 45.2 rounded up, 43.8 so)
         const unsigned per_warp = (b - a + 32u * kWarps - 1u) / (32u * kWarps);
         const unsigned bs = max(2u, (b - a + per_warp * kWarps - 1u) / (per_warp * kWarps));
-        stream_part<PREC, DEPTH, true>(P, T, acc_t, nb_g, bs, 0, win_s, nb_s, list);
+        stream_part<PREC, DEPTH, ROWS, true>(P, T, acc_t, nb_g, bs, 0, win_s, nb_s, list);
         // add the window to the accumulator: one asynchronous bulk reduction
         // (element-wise atomic in L2) per column, issued once every warp's
         // reductions are visible to the async proxy
@@ -966,7 +984,7 @@ __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, i
         const unsigned nit = T.b > T.a ? T.b - T.a : 0u;
         unsigned bs = (nit + kWarps - 1) / kWarps;
         bs = bs < 2u ? 2u : (bs > 32u ? 32u : bs);
-        stream_part<PREC, DEPTH, false>(P, T, acc_t, nb_g, bs, rot, win_s, nb_s, list);
+        stream_part<PREC, DEPTH, ROWS, false>(P, T, acc_t, nb_g, bs, rot, win_s, nb_s, list);
         rot = (int)((rot + (nit + bs - 1) / bs) % kWarps);
       }
     }
@@ -977,12 +995,17 @@ __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, i
   if (tid < kMaxTileCols) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-template <int PREC>
+// ROWS: for nets with lists of rows.  Those take 42 bytes per neuron instead of
+// 1344 (20 delays), but an item's descriptor is then 16 bytes at a random place
+// instead of the next 16 bytes of a list, which is slower (96x96 FP16, an early
+// form of this kernel: 1077 against 892 us a step in an Up state, 132 against
+// 118 in a Down state), so they are kept only where the others do not fit.
+template <int PREC, bool ROWS>
 __global__ void __launch_bounds__(kDeliverThreads, 1) deliver_kernel(const StepParams P) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ DeliverSmem S;
   NetTiles tiles(P);
-  deliver_blocks<PREC, kDepth, kDeliverThreads>(
+  deliver_blocks<PREC, kDepth, kDeliverThreads, ROWS>(
       tiles,
       [&]() -> long long {
         grid_wait();
@@ -1101,7 +1124,7 @@ __device__ __forceinline__ int net_of(const int* first, int n, int g) {
   return lo;
 }
 
-template <int PREC, int INFL>
+template <int PREC, int INFL, bool ROWS>
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchParams B) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ StepParams s_p[kUpdateSubs];  // the nets of the current virtual bodies
@@ -1129,8 +1152,8 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchPara
     }
     if (!grid_barrier(B, &s_ok)) return;
     BatchTiles tiles(B, s_p[0]);
-    deliver_blocks<PREC, INFL, kBatchThreads>(tiles, [&]() -> long long { return t; }, (int)blockIdx.x,
-                                              (int)gridDim.x, B.win_words, B.max_cols, SD, s_dyn);
+    deliver_blocks<PREC, INFL, kBatchThreads, ROWS>(tiles, [&]() -> long long { return t; }, (int)blockIdx.x,
+                                                    (int)gridDim.x, B.win_words, B.max_cols, SD, s_dyn);
     // each net's tiles must sum to its own total
     for (int k = (int)blockIdx.x * (kBatchThreads / 32) + (int)(threadIdx.x >> 5); k < n;
          k += (int)gridDim.x * (kBatchThreads / 32)) {
@@ -1242,9 +1265,16 @@ __global__ void __launch_bounds__(256) drain_records_kernel(
   }
 }
 
-// Writes the descriptor of neuron l of column c at place `at` of a list
-// (plane 0; the other planes follow at the stride of all tiles' lists).
-__device__ __forceinline__ void list_spike(const StepParams& P, long long at, uint32_t c, uint32_t l) {
+// Lists neuron l of column c at place r of its tile's list of the step: its row,
+// or its descriptor (plane 0; the other planes follow at the stride of all
+// tiles' lists).
+__device__ __forceinline__ void list_spike(const StepParams& P, long long slot, uint32_t ct, unsigned r,
+                                           uint32_t c, uint32_t l) {
+  if (P.rlist != nullptr) {
+    P.rlist[(slot * P.ntile + (ct >> 6)) * P.tcap + r] = (uint16_t)((ct & 63u) * (uint32_t)P.npc + l);
+    return;
+  }
+  const long long at = (slot * P.planes * P.ntile + (ct >> 6)) * P.tcap + r;
   const uint4* d = P.bend + ((size_t)P.colv[c] * P.npc + l) * P.planes;
   const long long stride = (long long)P.ntile * P.tcap;
   for (int p = 0; p < P.planes; ++p) P.list[at + p * stride] = d[p];
@@ -1309,7 +1339,7 @@ __global__ void __launch_bounds__(256) ingest_kernel(const StepParams P, const u
     const uint32_t ct = P.ctile[ly * P.W + lx];
     const long long tile_slot = slot * P.ntile + (ct >> 6);
     const unsigned r = next_place(P.ccnt + tile_slot * kCntStride, ct >> 6);
-    list_spike(P, (slot * P.planes * P.ntile + (ct >> 6)) * P.tcap + r, (uint32_t)(ly * P.W + lx), l);
+    list_spike(P, slot, ct, r, (uint32_t)(ly * P.W + lx), l);
   }
 }
 
@@ -1334,9 +1364,14 @@ int update_grid(long long N, int num_sms) {
 }
 
 namespace {
-const void* deliver_fn(int precision) {
-  return precision == SNN_EXACT_F16W ? reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F16W>)
-                                     : reinterpret_cast<const void*>(deliver_kernel<SNN_EXACT_F32W>);
+template <int PREC>
+const void* deliver_fn(bool rows) {
+  return rows ? reinterpret_cast<const void*>(deliver_kernel<PREC, true>)
+              : reinterpret_cast<const void*>(deliver_kernel<PREC, false>);
+}
+const void* deliver_fn(const StepParams& p, int precision) {
+  const bool rows = p.rlist != nullptr;
+  return precision == SNN_EXACT_F16W ? deliver_fn<SNN_EXACT_F16W>(rows) : deliver_fn<SNN_EXACT_F32W>(rows);
 }
 }  // namespace
 
@@ -1362,7 +1397,7 @@ size_t deliver_smem(int cols, int npc4, bool batch) {
 // Delivery grid: one block per SM (a persistent grid).
 int deliver_grid(const StepParams& p, int precision, int num_sms) {
   const size_t smem = deliver_smem(p.tcols, p.npc4, false);
-  const void* fn = deliver_fn(precision);
+  const void* fn = deliver_fn(p, precision);
   int per_sm = 0;
   // the attribute belongs to the kernel, not to the net: always the budget
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1374,7 +1409,7 @@ int deliver_grid(const StepParams& p, int precision, int num_sms) {
 
 cudaError_t launch_deliver(const StepParams& p, int precision, int grid, bool overlap, cudaStream_t st) {
   void* args[] = {const_cast<StepParams*>(&p)};
-  return launch_overlapped(deliver_fn(precision), dim3((unsigned)grid), kDeliverThreads,
+  return launch_overlapped(deliver_fn(p, precision), dim3((unsigned)grid), kDeliverThreads,
                            deliver_smem(p.tcols, p.npc4, false), args, overlap, st);
 }
 
@@ -1395,15 +1430,16 @@ cudaError_t launch_count_records(const StepParams& p, int nreg, unsigned long lo
 }
 
 namespace {
-template <int PREC, int INFL>
+template <int PREC, int INFL, bool ROWS>
 void* batch_fn() {
-  return reinterpret_cast<void*>(batch_kernel<PREC, INFL>);
+  return reinterpret_cast<void*>(batch_kernel<PREC, INFL, ROWS>);
 }
 // The batch tuner's schedule `infl` (2 or 4) selects 1 or 2 rounds of
-// sectors in flight per lane.
-void* batch_kernel_ptr(int precision, int infl) {
-  if (precision == SNN_EXACT_F16W) return infl == 2 ? batch_fn<1, 1>() : batch_fn<1, 2>();
-  return infl == 2 ? batch_fn<0, 1>() : batch_fn<0, 2>();
+// sectors in flight per lane (always 1 for lists of rows).
+void* batch_kernel_ptr(int precision, int infl, bool rows) {
+  if (rows) return precision == SNN_EXACT_F16W ? batch_fn<1, 1, true>() : batch_fn<0, 1, true>();
+  if (precision == SNN_EXACT_F16W) return infl == 2 ? batch_fn<1, 1, false>() : batch_fn<1, 2, false>();
+  return infl == 2 ? batch_fn<0, 1, false>() : batch_fn<0, 2, false>();
 }
 }  // namespace
 
@@ -1412,8 +1448,8 @@ size_t batch_smem(int win_words, int max_cols) {
                   ((size_t)win_words + (size_t)max_cols * 64 + (size_t)(kBatchThreads / 32) * kListWords) * 4);
 }
 
-int batch_grid(int precision, int infl, int num_sms, size_t smem) {
-  void* fn = batch_kernel_ptr(precision, infl);
+int batch_grid(int precision, int infl, bool rows, int num_sms, size_t smem) {
+  void* fn = batch_kernel_ptr(precision, infl, rows);
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)std::max(smem, kBatchSmemBudget)) != cudaSuccess)
     return 0;
@@ -1422,10 +1458,10 @@ int batch_grid(int precision, int infl, int num_sms, size_t smem) {
   return per_sm * num_sms;
 }
 
-cudaError_t launch_batch(const BatchParams& b, int precision, int infl, int grid, size_t smem,
+cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, int grid, size_t smem,
                          cudaStream_t st) {
   void* args[] = {const_cast<BatchParams*>(&b)};
-  return cudaLaunchCooperativeKernel(batch_kernel_ptr(precision, infl), dim3(grid),
+  return cudaLaunchCooperativeKernel(batch_kernel_ptr(precision, infl, rows), dim3(grid),
                                      dim3(kBatchThreads), args, smem, st);
 }
 
