@@ -365,7 +365,7 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
 /*
  * snn_batch_step -- advance every member n_steps steps in one cooperative
  * launch: each step runs all members' update blocks, a grid barrier, all
- * members' delivery blocks and a second barrier.  Barrier waits are bounded;
+ * members' deliveries and a second barrier.  Barrier waits are bounded;
  * a wait that gives up ends the launch and the call returns SNN_ETIMEOUT (the
  * members' state is then undefined).  Synchronises the batch's stream.
  */

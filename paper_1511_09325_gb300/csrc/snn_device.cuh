@@ -54,8 +54,8 @@ __device__ __forceinline__ int wrap(int v, int n) {
 // before still runs (programmatic dependent launch): what comes before
 // grid_wait reads only what no step writes; grid_wait returns when the kernel
 // before has finished and its writes are visible; grid_go lets the next
-// kernel's blocks be launched.  Both are no-ops in a plain launch.  1000 steps: 14.2 -> 13.7 ms at 2x2, 58.6 ->
-// 54.4 ms at 24x24 FP32.
+// kernel's blocks be launched.  Both are no-ops in a plain launch.  1000 steps:
+// 14.2 -> 13.7 ms at 2x2, 58.6 -> 54.4 ms at 24x24 FP32.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

