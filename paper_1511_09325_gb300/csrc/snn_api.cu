@@ -1175,9 +1175,14 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   int rc = snn_row_lengths(net, j0, n, len.data());
   if (rc) return rc;
   // the device walks each row's draws again and decodes the records in that
-  // order, a bounded number of rows at a time
-  constexpr int64_t kRows = 4096;
-  const int64_t m = std::min(n, kRows);
+  // order, a bounded number of rows at a time: in the drain's stage, which is
+  // idle between reads, or where that is too small in a buffer of its own
+  constexpr int64_t kRows = 4096, kFewRows = 32;
+  int32_t longest = 0;
+  for (int32_t l : len) longest = std::max(longest, l);
+  const int64_t in_stage = net->rec_region * net->update_grid / (1 + 2 * (int64_t)longest);
+  const bool staged = in_stage >= std::min(n, kFewRows);
+  const int64_t m = std::min(n, staged ? std::min(in_stage, kRows) : kRows);
   size_t most = 0;
   std::vector<long long> off;
   for (int64_t r0 = 0; r0 < n; r0 += m) {
@@ -1185,11 +1190,13 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
     for (int64_t r = r0; r < std::min(n, r0 + m); ++r) k += (size_t)len[r];
     most = std::max(most, k);
   }
-  unsigned char* buf = nullptr;  // offsets, targets, delays, weights
+  unsigned char* buf = reinterpret_cast<unsigned char*>(net->stage);  // offsets, targets, delays, weights
   const size_t off_bytes = (size_t)m * 8, b8 = most * 8, b4 = most * 4;
-  rc = dalloc(net, &buf, off_bytes + b8 + 2 * b4);
-  if (rc) return rc;
-  net->device_bytes -= off_bytes + b8 + 2 * b4;
+  if (!staged) {
+    rc = dalloc(net, &buf, off_bytes + b8 + 2 * b4);
+    if (rc) return rc;
+    net->device_bytes -= off_bytes + b8 + 2 * b4;
+  }
   BuildParams bp = net->bp;
   bp.syn = net->syn;
   bp.bend = net->bend;
@@ -1223,7 +1230,7 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
     if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
     at += k;
   }
-  cudaFree(buf);
+  if (!staged) cudaFree(buf);
   if (e != cudaSuccess) return cuda_fail(net, e, "synapse readback");
   return SNN_OK;
 }

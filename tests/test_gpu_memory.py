@@ -110,3 +110,17 @@ def test_same_results_without_room_for_descriptors(name):
     assert len(got) == len(want)
     for g, w in zip(got, want):
         assert np.array_equal(g, w)
+
+
+@pytest.mark.parametrize("records", [1, 2000, 1 << 14, 1 << 20])
+def test_synapse_readback_in_the_drain_stage(records):
+    # 4 x 3 columns of 50 neurons, rows of 60: the stage holds no row, 16
+    # (a buffer of its own is taken below 32), 135, or all 600
+    n, s = W.neuron_params(n_per_col=50, n_exc=40), W.synapse_params(k_out=60)
+    with snn.Net(4, 3, n, s, SEED, "f32w") as net:
+        want = net.synapses(0, net.n)
+        net.set_record_capacity(records)
+        for got, w in zip(net.synapses(0, net.n), want):
+            assert np.array_equal(got, w)
+        net.step(5)
+        assert net.synapses(0, 1)[0].shape == (1, 60)
