@@ -21,6 +21,7 @@ struct snn_net {
   int deliver_grid = 0;
   int npc4 = 0, unit = kSlotUnit;     // words of a column in acc; slots of a bucket unit
   int planes = 1;                     // planes of a spike descriptor
+  int ord_units = 0;                  // 8-slot units of the longest row, one part per bucket
   int tw = 1, th = 1, ntile = 1;      // delivery tiles
   bool batch_member = false;          // windows sized for the batch kernel's blocks
   unsigned min_items = 256;  // fewest items a delivery block takes
@@ -442,6 +443,7 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   net->rec_size = precision == SNN_EXACT_F16W ? 4 : 8;
   net->planes = (net->ndel + kPlaneBuckets - 1) / kPlaneBuckets;
   choose_unit(net, sp->k_out);
+  net->ord_units = (sp->k_out + (kSlotUnit - 1) * std::min(sp->k_out, net->ndel) + kSlotUnit - 1) / kSlotUnit;
   net->rec_cap = 1LL << 24;
   rc = make_host_tables(*np, *sp, precision, &net->tables, &why);
   if (rc != SNN_OK) return fail(net, rc, why);
@@ -536,6 +538,7 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
     if (max_units[1] > 255u || max_units[0] > 255u)
       return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
     net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
+    net->ord_units = (int)std::max(1u, max_units[1]);
     std::vector<uint32_t> deg((size_t)net->N);
     SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
                                   net->stream));
@@ -707,6 +710,11 @@ int net_view(snn_net* net, NetView* v) {
   v->tinfo = net->tinfo;
   v->ntile = net->ntile;
   v->tcols = net->tw * net->th;
+  v->ord_units = net->ord_units;
+  v->build = net->bp;
+  v->build.unit = net->unit;
+  v->build.rowcap = net->rowcap;
+  v->paper = net->connectivity == SNN_CONN_PAPER;
   v->nexc = net->nexc;
   v->dmin = net->dmin;
   v->ndel = net->ndel;

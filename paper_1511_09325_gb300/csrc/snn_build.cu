@@ -30,13 +30,15 @@ namespace {
 constexpr int kBuildWarps = 8;
 constexpr int kDropped = 0xFE;  // offset class: not kept by the shard
 constexpr int kOut = 0xFF;      // offset class: another tile
-constexpr int kModeCount = 0, kModeFill = 1, kModeRead = 2;
+constexpr int kModeCount = 0, kModeFill = 1, kModeRead = 2, kModeOrder = 3;
 
 // Shared tables of a block and its warps' rows.
 struct RowSmem {
   unsigned cnt[kBuildWarps][64];       // synapses per bucket part (2 b, 2 b + 1)
   unsigned cur[kBuildWarps][64];       // next slot of each part
-  unsigned rd[kBuildWarps][32];        // readback: next entry of each delay
+  unsigned rd[kBuildWarps][32];        // readback: next entry of each delay; draw
+                                       // order: next place of each bucket
+  uint32_t mask[kBuildWarps][64];      // draw order: bit p: place p is an in record
   uint8_t cls[kBuildWarps][kMaxOff + 1];  // target's place in the tile per offset
   uint32_t thr[kMaxOff];
   uint8_t guide[256];                  // offsets whose threshold is <= (b << 24)
@@ -110,6 +112,23 @@ __device__ __forceinline__ int offset_of(const BuildParams& P, const RowSmem& S,
   return m;
 }
 
+// A bucket in draw order: its synapses, of both parts, from place 8 * first on,
+// in 8-place units first .. end - 1 (the calling lane's bucket).
+struct DrawBucket {
+  unsigned first, end;
+};
+__device__ __forceinline__ DrawBucket draw_bucket(const BuildParams& P, unsigned ci, unsigned co) {
+  const unsigned lane = threadIdx.x & 31u;
+  const unsigned u = (ci + co + 7u) / 8u;
+  unsigned incl = u;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= (unsigned)o) incl += v;
+  }
+  return DrawBucket{incl - u, incl};
+}
+
 // Parts' sizes (S.cnt) to bucket ends and first slots; lane b holds bucket b.
 // Returns the row's units.
 template <int MODE>
@@ -134,6 +153,12 @@ __device__ __forceinline__ unsigned open_parts(const BuildParams& P, RowSmem& S,
   S.cur[w][2 * lane + 1] = (excl + ui) * unit;
   if (MODE == kModeRead) {
     S.rd[w][lane] = icnt - ci - co;
+  } else if (MODE == kModeOrder) {
+    const DrawBucket d = draw_bucket(P, ci, co);
+    S.rd[w][lane] = 8u * d.first;
+    S.mask[w][lane] = 0u;
+    S.mask[w][lane + 32] = 0u;
+    if (lane < P.ndel) P.ord_end[r.at * P.ndel + lane] = (uint8_t)d.end;
   } else {
     uint8_t* d = P.bend + r.at * P.planes * 16;
     if (lane < P.planes * kPlaneBuckets)
@@ -160,7 +185,7 @@ __device__ __forceinline__ void place(const BuildParams& P, RowSmem& S, const Ro
   const unsigned rank = __popc(peers & lt);
   const unsigned pos = S.cur[w][bb & 63] + rank;
   unsigned dpeers = 0u, dpos = 0u;
-  if (MODE == kModeRead) {
+  if (MODE == kModeRead || MODE == kModeOrder) {
     dpeers = __match_any_sync(0xFFFFFFFFu, bb >> 1);
     dpos = S.rd[w][(bb >> 1) & 31] + __popc(dpeers & lt);
   }
@@ -180,6 +205,8 @@ __device__ __forceinline__ void place(const BuildParams& P, RowSmem& S, const Ro
         const int32_t wfx = __float2int_rn(__fmul_rn(__uint_as_float(wbits), 65536.0f));
         static_cast<uint2*>(P.syn)[s] = make_uint2(code, (uint32_t)wfx);
       }
+    } else if (MODE == kModeOrder) {
+      if (!out) atomicOr(&S.mask[w][dpos >> 5 & 63u], 1u << (dpos & 31u));
     } else {
       uint32_t code;
       int32_t wfx;
@@ -212,7 +239,8 @@ __device__ __forceinline__ void place(const BuildParams& P, RowSmem& S, const Ro
       P.rd_wfx[o] = wfx;
     }
     if (rank == 0) S.cur[w][bb] += __popc(peers);
-    if (MODE == kModeRead && (dpeers & lt) == 0u) S.rd[w][bb >> 1] += __popc(dpeers);
+    if ((MODE == kModeRead || MODE == kModeOrder) && (dpeers & lt) == 0u)
+      S.rd[w][bb >> 1] += __popc(dpeers);
   }
   __syncwarp();
 }
@@ -241,8 +269,61 @@ __device__ __forceinline__ void pad_parts(const BuildParams& P, RowSmem& S, cons
   __syncwarp();
 }
 
+// Writes the row's draw order: a word per unit of 8 places in draw order, bits
+// 0-7: which places hold in records, bits 8-19 and 20-31: the slots of the
+// first in and out records at or after the unit's start.
+__device__ __forceinline__ void write_order(const BuildParams& P, RowSmem& S, const Row& r) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned unit = (unsigned)P.unit;
+  const unsigned ci = lane < P.ndel ? S.cnt[w][2 * lane] : 0u;
+  const unsigned co = lane < P.ndel ? S.cnt[w][2 * lane + 1] : 0u;
+  const DrawBucket d = draw_bucket(P, ci, co);
+  // lane b: bucket b's in records before it in the row, and its parts' first units
+  const unsigned ui = (ci + unit - 1u) / unit, uo = (co + unit - 1u) / unit;
+  unsigned uincl = ui + uo, cincl = ci;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned u = __shfl_up_sync(0xFFFFFFFFu, uincl, o);
+    const unsigned c = __shfl_up_sync(0xFFFFFFFFu, cincl, o);
+    if (lane >= o) {
+      uincl += u;
+      cincl += c;
+    }
+  }
+  const unsigned in0 = (uincl - ui - uo) * unit, out0 = (uincl - uo) * unit;
+  const unsigned units = __shfl_sync(0xFFFFFFFFu, d.end, 31);
+  unsigned before = 0u;  // in records of the units before
+  for (unsigned u0 = 0u; u0 < units; u0 += 32u) {
+    const unsigned u = u0 + (unsigned)lane;
+    const uint32_t m = u < units ? S.mask[w][u >> 2 & 63u] >> (8u * (u & 3u)) & 0xFFu : 0u;
+    unsigned incl = (unsigned)__popc(m);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    // the unit's bucket: the first with end > u
+    int b = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const unsigned e = __shfl_sync(0xFFFFFFFFu, d.end, b + step - 1);
+      if (e <= u) b += step;
+    }
+    b = min(b, 31);
+    const unsigned n_in = before + incl - (unsigned)__popc(m) -
+                          __shfl_sync(0xFFFFFFFFu, cincl - ci, b);  // of the bucket, before u
+    const unsigned f = __shfl_sync(0xFFFFFFFFu, d.first, b);
+    const unsigned i0 = __shfl_sync(0xFFFFFFFFu, in0, b), o0 = __shfl_sync(0xFFFFFFFFu, out0, b);
+    if (u < units && u < (unsigned)P.ord_units)
+      P.ord[r.at * (size_t)P.ord_units + u] = m | (i0 + n_in) << 8 | (o0 + 8u * (u - f) - n_in) << 20;
+    before += __shfl_sync(0xFFFFFFFFu, incl, 31);
+  }
+  __syncwarp();
+}
+
 // Rows of the fixed law, one warp per row; MODE fill builds them, read writes
-// rows j0 .. j0 + n_rows - 1 to the rd_* arrays, count finds the longest.
+// rows j0 .. j0 + n_rows - 1 to the rd_* arrays, count finds the longest, order
+// writes the rows' draw order.
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const BuildParams P) {
   __shared__ RowSmem S;
@@ -301,6 +382,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const Buil
       place<PREC, MODE>(P, S, r, bb, m, l, MODE == kModeFill ? wt[x.w >> 16] : 0u, out0);
     }
     if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
+    if (MODE == kModeOrder) write_order(P, S, r);
   }
 }
 
@@ -342,7 +424,7 @@ __global__ void __launch_bounds__(256) init_state_kernel(const StepParams P) {
 // scan of the lanes' kept counts ranks them.  The count pass writes the
 // bucket ends, the out-degree and the largest row; the fill pass makes the
 // same draws and places every synapse, then pads the parts; the read pass
-// counts and then reads back.
+// counts and then reads back, and the order pass likewise.
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const BuildParams P) {
   __shared__ RowSmem S;
@@ -443,6 +525,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
     }
     if (MODE != kModeCount) walk(true);
     if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
+    if (MODE == kModeOrder) write_order(P, S, r);
   }
 }
 
@@ -488,6 +571,14 @@ cudaError_t launch_read_rows(const BuildParams& bp, int precision, bool paper, c
     build_rows_kernel<SNN_EXACT_F16W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
   else
     build_rows_kernel<SNN_EXACT_F32W, kModeRead><<<grid, kBuildWarps * 32, 0, st>>>(bp);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_draw_order(const BuildParams& bp, bool paper, int num_sms, cudaStream_t st) {
+  if (paper)
+    paper_rows_kernel<SNN_EXACT_F32W, kModeOrder><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
+  else
+    build_rows_kernel<SNN_EXACT_F32W, kModeOrder><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
   return cudaGetLastError();
 }
 

@@ -30,9 +30,9 @@
 // Backward: segment by segment from the end, the forward is recomputed from
 // the segment's checkpoint while a tape of eight values per neuron and step is
 // recorded, then the adjoint recursion runs back through the segment:
-// grad_gather_kernel (the adjoint of the delayed delivery is a gather over
-// every row's outgoing synapses of the targets' input adjoints at t + d; one
-// block per delay bucket and run of rows, in a fixed order) and
+// grad_gather_kernel (one warp per source row: the adjoint of the delayed
+// delivery is a gather over the row's outgoing synapses of the targets' input
+// adjoints at t + d, summed in the order in which they were drawn) and
 // grad_backward_kernel (one thread per neuron: the adjoint of every line above;
 // parameter partials accumulate per neuron in FP64 and are summed in a
 // fixed order).  Every sum has a fixed order, so a run is reproducible bit
@@ -59,11 +59,14 @@ constexpr float kTwoM24 = 5.9604644775390625e-08f;  // 2^-24
 
 struct GradParams {
   long long N, accw;          // neurons; words of an array in acc order
-  int npc, npc4, nexc, dmin, ndel, nslot, rowcap, unit, planes, hard, T;
+  int npc, npc4, nexc, ncol, dmin, ndel, nslot, rowcap, unit, planes, hard, T;
   const uint32_t* ctile;      // geometry of the net (see snn_internal.h)
   const uint32_t* colv;
   const uint32_t* nbg;
-  const uint2* tinfo;
+  uint32_t* vtile;            // [ncol] first word of each virtual column's tile
+  uint32_t* ord;              // the rows' draw order (see BuildParams), null: as stored
+  uint8_t* ord_end;
+  int ord_units;
   uint32_t seed_lo, seed_hi;
   float beta, theta, vr, dc, pvv, pcc, pvc_e, pvc_i, kappa, J, lam, sqlam;
   float a[4];  // a_EE, a_EI, a_IE, a_II
@@ -85,7 +88,7 @@ struct GradParams {
   float* ibe;                 // [nslot][accw] a[E][p_i] * adjoint of I_i(t), acc order
   float* ibi;                 // [nslot][accw] a[I][p_i] * adjoint of I_i(t)
   float* gb;                  // [3][N] -adjoint of g_i(t) where the gate is open
-  float* part;                // [ndel][N] gathered adjoints of s_j(t) per bucket, rows in table order
+  float* sg;                  // [N] gathered adjoints of s_j(t), rows in table order
   double* gacc;               // [6][N] parameter partials per neuron
   double* gsum;               // [6] their sums
 };
@@ -301,103 +304,198 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
   }
 }
 
-// Adjoint of s_j(tau) through the synapses of its bucket b, tau + d < T: the
-// sum of w * (a[p_j][p_i] * adjoint of I_i(tau + d)), to part[b].  A block
-// takes bucket b of a run of rows of one population in one delivery tile.  It
-// first copies the tile's adjoints at tau + d to shared memory, where the four
-// fifths of the row's targets that lie in the tile are looked up (in parts);
-// the others come from L2.  Eight lanes share a row: a lane takes every eighth
-// 32-byte sector of the bucket (four records), and the lanes' sums are added
-// in a fixed order.
-// What bounds it: each record needs one scattered 4-byte read of an adjoint.
-// As L2 reads (one warp per row, all buckets) they took 75 us a step on the
-// 4x4 network, whose table is 197 MB (DRAM floor 31 us); looked up in shared
-// memory, 54 us.  Loading a row's sectors one row ahead (384 threads, more
-// registers) took 68 us.
-constexpr int kGatherThreads = 1024;  // per SM: one block, or two of half as many
-constexpr int kGatherDepth = 3;  // sectors in flight per lane
+// Adjoint of s_j(tau) through its outgoing synapses: the sum over the buckets d
+// with tau + d < T of w * (a[p_j][p_i] * adjoint of I_i(tau + d)).
+// The order of the FP32 sum is part of the result: the row's synapses, bucket by
+// bucket, in the order in which they were drawn, each bucket padded to 8 places;
+// lane e of the row's warp adds places 4 e .. 4 e + 3 of every run of 128, and the
+// lanes' sums are added as a tree.  Where no synapse leaves its tile (a net of one
+// tile, units of 8 slots) the table itself lies in that order; else P.ord gives
+// the slots of each unit of 8 places (see write_order in snn_build.cu).
 
-__global__ void __launch_bounds__(kGatherThreads, 1)
-    grad_gather_kernel(const GradParams P, long long tau, int rows_e, int rows_i, int blocks_e,
-                       int blocks_i) {
-  extern __shared__ __align__(16) float s_ib[];
-  const int b = (int)blockIdx.y;
-  const long long dst = tau + P.dmin + b;
-  if (dst >= P.T) return;
-  const int per_tile = blocks_e + blocks_i;
-  const int tile = (int)blockIdx.x / per_tile;
-  int part = (int)blockIdx.x - tile * per_tile;
-  const bool exc = part < blocks_e;
-  part -= exc ? 0 : blocks_e;
-  const uint2 ti = P.tinfo[tile];
-  const uint32_t npop = (uint32_t)(exc ? P.nexc : P.npc - P.nexc);  // rows of a column
-  const uint32_t rows = npop * ti.y;
-  const uint32_t per_block = (uint32_t)(exc ? rows_e : rows_i);
-  const uint32_t r0 = (uint32_t)part * per_block;
-  if (r0 >= rows) return;
-  const uint32_t r1 = min(rows, r0 + per_block);
-  const float* ib = (exc ? P.ibe : P.ibi) + ring(dst, P.nslot) * P.accw;
-  const float* own = ib + (size_t)ti.x * P.npc4;
-  for (uint32_t i = threadIdx.x; i < ti.y * (uint32_t)P.npc4 / 4u; i += blockDim.x)
-    reinterpret_cast<float4*>(s_ib)[i] = __ldg(reinterpret_cast<const float4*>(own) + i);
-  __syncthreads();
-  const uint32_t lane8 = threadIdx.x & 7u;
-  const int beg_at = b % kPlaneBuckets ? desc_end(b) - 1 : desc_start(b);
-  const uint32_t us = (uint32_t)P.unit / 4u;  // sectors of a unit
-  // row r of the population: its place in the table; its bucket ends are
-  // loaded one row ahead
-  auto row_of = [&](uint32_t r) -> size_t {
-    const uint32_t k = r / npop;
-    return (size_t)(ti.x + k) * P.npc + (exc ? 0u : (uint32_t)P.nexc) + (r - k * npop);
-  };
-  uint32_t beg_n = 0u, me_n = 0u;
-  auto load_ends = [&](uint32_t r) {
-    if (r >= r1) return;
-    const uint8_t* d = P.bend + row_of(r) * (size_t)(P.planes * 16);
-    beg_n = d[beg_at];
-    me_n = *reinterpret_cast<const uint16_t*>(d + desc_end(b));
-  };
-  load_ends(r0 + threadIdx.x / 8u);
-  // every lane takes part in the row loop (its sums are shuffled)
-  for (uint32_t rb = r0; rb < r1; rb += blockDim.x / 8u) {
-    const uint32_t r = rb + threadIdx.x / 8u;
-    float acc = 0.f;
-    size_t jv = 0;
-    const uint32_t beg = beg_n, me = me_n;
-    load_ends(r + blockDim.x / 8u);
-    if (r < r1) {
-      const uint32_t k = r / npop;
-      jv = row_of(r);
-      const uint32_t n_in = ((me & 0xFFu) - beg) * us, n = ((me >> 8) - beg) * us;
-      const uint4* sec = reinterpret_cast<const uint4*>(P.syn + jv * (size_t)P.rowcap + beg * (uint32_t)P.unit);
-      const uint32_t* nb = P.nbg + (size_t)(ti.x + k) * 64;
-      for (uint32_t s0 = lane8; s0 < n; s0 += 8u * kGatherDepth) {
-        uint4 x[kGatherDepth], y[kGatherDepth];
+// One warp per row, the targets' adjoints read from L2 (MAP: the rows' order is
+// P.ord's, its words loaded a run ahead).  Each record needs one scattered 4-byte
+// read of an adjoint, a 32-byte sector of the L2, which bounds it.  MAP on 12x12
+// columns, 60 steps forward and backward: 57.5 ms with six blocks per SM, 59.5
+// with five, 66.4 with four.
+template <bool MAP>
+__global__ void __launch_bounds__(kThreads, MAP ? 6 : 1)
+    grad_gather_kernel(const GradParams P, long long tau) {
+  const long long at = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // row of the table
+  const int lane = threadIdx.x & 31;
+  if (at >= P.N) return;
+  const uint32_t v = (uint32_t)at / (uint32_t)P.npc;
+  const bool exc = (int)((uint32_t)at - v * (uint32_t)P.npc) < P.nexc;
+  const float* ib = exc ? P.ibe : P.ibi;
+  const uint32_t* nb = P.nbg + (size_t)v * 64;
+  const uint32_t tile = P.vtile[v];
+  long long off_lane = -1;    // ring offset of bucket `lane`'s step, -1 beyond T
+  int end_lane = 0x7FFFFFFF;  // end of bucket `lane` in places
+  int slot_lane = 0;          // its end in slots (MAP)
+  if (lane < P.ndel) {
+    const long long dst = tau + P.dmin + lane;
+    off_lane = dst < P.T ? ring(dst, P.nslot) * P.accw : -1;
+    slot_lane = (int)P.bend[at * (P.planes * 16) + desc_end(lane) + 1] * P.unit;
+    end_lane = MAP ? (int)P.ord_end[at * P.ndel + lane] * 8 : slot_lane;
+  }
+  const int row_end = __shfl_sync(0xFFFFFFFFu, end_lane, P.ndel - 1);
+  const uint2* row = P.syn + at * (long long)P.rowcap;
+  const uint32_t* ord = MAP ? P.ord + at * (long long)P.ord_units : nullptr;
+  float acc = 0.f;
+  uint32_t u_next = MAP && 4 * lane < row_end ? __ldg(ord + (lane >> 1)) : 0u;  // a run ahead
+#pragma unroll (MAP ? 1 : 2)
+  for (int k0 = 0; k0 < row_end; k0 += 128) {
+    const int k = k0 + 4 * lane;
+    const int b = bucket_of(k, end_lane, P.ndel);
+    const long long off = __shfl_sync(0xFFFFFFFFu, off_lane, b);
+    const int slot_end = MAP ? __shfl_sync(0xFFFFFFFFu, slot_lane, b) : 0;
+    const uint32_t u = u_next;
+    if (MAP && k + 128 < row_end) u_next = __ldg(ord + ((k + 128) >> 3));
+    if (k < row_end && off >= 0) {
+      const float* ibs = ib + off;
+      uint32_t code[4], w[4] = {0u, 0u, 0u, 0u};
+      uint32_t in = 0xFu;  // bit q: record q is an in record
+      if (MAP) {
+        const uint32_t h = (uint32_t)k & 4u;
+        in = u >> h & 0xFu;
+        const uint32_t before = __popc(u & ((1u << h) - 1u));  // in records of the unit's first half
+        uint32_t ip = (u >> 8 & 0xFFFu) + before, op = (u >> 20) + h - before;
 #pragma unroll
-        for (int q = 0; q < kGatherDepth; ++q) {
-          const uint32_t s = min(s0 + 8u * q, n - 1u);
-          x[q] = __ldcs(sec + 2u * s);
-          y[q] = __ldcs(sec + 2u * s + 1u);
-        }
-#pragma unroll
-        for (int q = 0; q < kGatherDepth; ++q) {
-          const uint32_t s = s0 + 8u * q;
-          if (s >= n) continue;
-          const uint32_t c[4] = {x[q].x, x[q].z, y[q].x, y[q].z};
-          const uint32_t w[4] = {x[q].y, x[q].w, y[q].y, y[q].w};
-          const bool in = s < n_in;
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            if (c[m] & kPad) continue;
-            const float v = in ? s_ib[c[m]] : __ldg(ib + (__ldg(nb + ((c[m] >> 11) & 63u)) + (c[m] & 2047u)));
-            acc = __fmaf_rn((float)(int32_t)w[m], v, acc);
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t s = in >> q & 1u ? ip++ : op++;
+          code[q] = kPad;  // places beyond the bucket's synapses: pads, or beyond its slots
+          if ((int)s < slot_end) {
+            const uint2 x = __ldg(row + s);
+            code[q] = x.x;
+            w[q] = x.y;
           }
         }
+      } else {
+        const uint4 x = __ldcs(reinterpret_cast<const uint4*>(row + k));
+        const uint4 y = __ldcs(reinterpret_cast<const uint4*>(row + k + 2));
+        code[0] = x.x; code[1] = x.z; code[2] = y.x; code[3] = y.z;
+        w[0] = x.y; w[1] = x.w; w[2] = y.y; w[3] = y.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (code[q] & kPad) continue;
+        const uint32_t t =
+            in >> q & 1u ? tile + code[q] : __ldg(nb + (code[q] >> 11 & 63u)) + (code[q] & 2047u);
+        acc = __fmaf_rn((float)(int32_t)w[q], ibs[t], acc);
       }
     }
+  }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    if (r < r1 && lane8 == 0u) P.part[(size_t)b * P.N + jv] = acc;
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+  if (lane == 0) P.sg[at] = __fmul_rn(acc, kTwoM16);
+}
+
+// The same for a net of one tile whose adjoints of a step fit shared memory twice:
+// a block takes a run of rows of one population, up to kGatherRows per warp, and
+// goes through the buckets; the adjoints at tau + d are copied to shared memory
+// while the bucket before is summed, and each row's records of a bucket are
+// loaded while the bucket before is summed.  The lanes' sums of all rows stay in
+// registers.
+// The adjoints come from shared memory instead of L2; what is left is the table
+// (4x4: 197 MB, 31 us of DRAM time) and a barrier per bucket, with 17 of 32 lanes
+// at work on a bucket of 62 synapses.  4x4, 500 steps forward and backward: 44.6
+// ms, by the warps of grad_gather_kernel 57.9 ms; 4x3 (200 steps) 16.9 and 19.9 ms;
+// 3x3 13.9 and 15.1 ms.  2x2 and smaller nets have too few rows to hide the
+// barriers (300 steps of 2x2: 15.3 and 14.1 ms).
+constexpr int kGatherThreads = 512;  // one block per SM
+constexpr int kGatherWarps = kGatherThreads / 32;
+constexpr int kGatherRows = 9;       // rows per warp, at most
+constexpr int kGatherBufs = 4;       // windows in shared memory, at most
+
+template <int ROWS>
+__global__ void __launch_bounds__(kGatherThreads, 1)
+    grad_gather_tile_kernel(const GradParams P, long long tau, int nb, int bufs, int per_block, int blocks_e) {
+  extern __shared__ __align__(16) float s_ib[];  // [bufs][accw]
+  const bool exc = (int)blockIdx.x < blocks_e;
+  const uint32_t npop = (uint32_t)(exc ? P.nexc : P.npc - P.nexc);  // rows of a column
+  const uint32_t r0 = (uint32_t)(exc ? blockIdx.x : blockIdx.x - blocks_e) * (uint32_t)per_block;
+  const uint32_t rows = npop * (uint32_t)P.ncol;
+  const uint32_t r1 = min(rows, r0 + (uint32_t)per_block);
+  const float* ib = exc ? P.ibe : P.ibi;
+  const int lane = threadIdx.x & 31;
+  const uint32_t words = (uint32_t)P.accw;
+  auto window = [&](int b, int buf) {  // bucket b's adjoints on their way to buffer `buf`
+    if (b < nb) {
+      const float* src = ib + ring(tau + P.dmin + b, P.nslot) * P.accw;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_ib + buf * words);
+      for (uint32_t i = threadIdx.x * 4u; i < words; i += kGatherThreads * 4u)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 4u), "l"(src + i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int b = 0; b + 1 < bufs; ++b) window(b, b);
+  float acc[ROWS];
+  int end_lane[ROWS];  // lane b: end of bucket b of each row, in slots
+  uint32_t row[ROWS];  // rows of the table
+  uint4 x[ROWS], y[ROWS];
+  const uint32_t rw = r0 + (threadIdx.x >> 5);
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    const uint32_t r = min(rw + (uint32_t)(i * kGatherWarps), rows - 1u);
+    const uint32_t c = r / npop;
+    row[i] = c * (uint32_t)P.npc + (exc ? 0u : (uint32_t)P.nexc) + (r - c * npop);
+    end_lane[i] = 0;
+    if (rw + (uint32_t)(i * kGatherWarps) < r1 && lane < P.ndel)
+      end_lane[i] = (int)P.bend[(size_t)row[i] * (uint32_t)(P.planes * 16) + desc_end(lane) + 1] * kSlotUnit;
+    acc[i] = 0.f;
+  }
+  // the lane's place in the bucket of slots beg .. end - 1 (beyond it if k >= end)
+  auto place = [&](int beg) { return beg + 4 * ((lane - (beg >> 2)) & 31); };
+  auto load = [&](int i, int beg, int end) {  // lanes beyond the bucket repeat its last group
+    const int k = max(0, min(place(beg), end - 4));
+    const uint4* p = reinterpret_cast<const uint4*>(P.syn + (size_t)row[i] * (uint32_t)P.rowcap + k);
+    x[i] = __ldcs(p);
+    y[i] = __ldcs(p + 1);
+  };
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) load(i, 0, __shfl_sync(0xFFFFFFFFu, end_lane[i], 0));
+  int buf = 0;  // bucket b's buffer
+  for (int b = 0; b < nb; ++b) {
+    // all but the last bufs - 2 windows have arrived
+    if (bufs == 2)
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    else if (bufs == 3)
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else
+      asm volatile("cp.async.wait_group 2;" ::: "memory");
+    __syncthreads();
+    window(b + bufs - 1, buf ? buf - 1 : bufs - 1);
+    const float* win = s_ib + buf * words;
+    buf = buf + 1 < bufs ? buf + 1 : 0;
+    auto add = [&](float a, const uint4& p, const uint4& q, bool on) {
+      const uint32_t code[4] = {p.x, p.z, q.x, q.z}, w[4] = {p.y, p.w, q.y, q.w};
+      float v[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) v[m] = on && !(code[m] & kPad) ? win[code[m]] : 0.f;
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (on && !(code[m] & kPad)) a = __fmaf_rn((float)(int32_t)w[m], v[m], a);
+      return a;
+    };
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const int beg = b ? __shfl_sync(0xFFFFFFFFu, end_lane[i], b - 1) : 0;
+      const int end = __shfl_sync(0xFFFFFFFFu, end_lane[i], b);
+      const int nxt = b + 1 < nb ? __shfl_sync(0xFFFFFFFFu, end_lane[i], b + 1) : end;
+      acc[i] = add(acc[i], x[i], y[i], place(beg) < end);
+      load(i, end, nxt);
+      for (int k = place(beg) + 128; k < end; k += 128) {
+        const uint4* p = reinterpret_cast<const uint4*>(P.syn + (size_t)row[i] * (uint32_t)P.rowcap + k);
+        acc[i] = add(acc[i], __ldcs(p), __ldcs(p + 1), true);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    float a = acc[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
+    if (lane == 0 && rw + (uint32_t)(i * kGatherWarps) < r1) P.sg[row[i]] = __fmul_rn(a, kTwoM16);
   }
 }
 
@@ -413,15 +511,11 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   const float* tp = P.tape + (long long)slot * kTape * P.N + i;
   const float V = tp[0], I = tp[P.N], U = tp[2 * P.N], g = tp[3 * P.N], s = tp[4 * P.N];
   const float cp = tp[5 * P.N], XE = tp[6 * P.N], XI = tp[7 * P.N];
-  // the adjoint of s(tau) through the synapses: the buckets that end before T
   const uint32_t c = (uint32_t)i / (uint32_t)P.npc, l = (uint32_t)i - c * (uint32_t)P.npc;
   const uint32_t v = P.colv[c];
-  const float* part = P.part + (size_t)v * P.npc + l;
-  float sg = 0.f;
-  const int nb = (int)min((long long)P.ndel, max(0ll, P.T - tau - P.dmin));
-#pragma unroll 8
-  for (int b = 0; b < nb; ++b) sg += part[(size_t)b * P.N];
-  float sbar = (exc ? P.dlds_e : P.dlds_i) + __fmul_rn(sg, kTwoM16) + P.gb[ring(tau + 1, 3) * P.N + i] +
+  // the adjoint of s(tau) through the synapses (none that ends before T: 0)
+  const float sg = tau + P.dmin < P.T ? P.sg[(size_t)v * P.npc + l] : 0.f;
+  float sbar = (exc ? P.dlds_e : P.dlds_i) + sg + P.gb[ring(tau + 1, 3) * P.N + i] +
                P.gb[ring(tau + 2, 3) * P.N + i];
   const float vb1 = P.vbar[i], cb1 = P.cbar[i];
   const float pvc = exc ? P.pvc_e : P.pvc_i;
@@ -459,6 +553,12 @@ __global__ void __launch_bounds__(kThreads) grad_backward_kernel(const GradParam
   ga[5 * P.N] += (double)ib * (double)P.J * (1.0 + (double)xi / (2.0 * (double)P.sqlam));
 }
 
+// First word of the tile of every virtual column, one block per tile.
+__global__ void __launch_bounds__(kThreads) grad_tile_words_kernel(const GradParams P, const uint2* tinfo) {
+  const uint2 ti = tinfo[blockIdx.x];
+  for (uint32_t k = threadIdx.x; k < ti.y; k += blockDim.x) P.vtile[ti.x + k] = ti.x * (uint32_t)P.npc4;
+}
+
 // Sums of the six parameters' partials over the neurons, one block per
 // parameter, in a fixed order.
 constexpr int kSumThreads = 1024;
@@ -482,7 +582,6 @@ struct snn_grad {
   NetView v{};
   long long T = 0;
   int ckpt = 0, nseg = 0, hard = 1, nslot = 0, ublocks = 0, wblocks = 0;
-  size_t gather_smem = 0;
   float beta = 5.f;
   double targets[2] = {3.0, 8.0};
   double kappa = 0.0, pvv = 0.0, pcc = 0.0;
@@ -528,31 +627,40 @@ void grad_release(snn_grad* g) {
   g->bufs.clear();
 }
 
-// Gather of step tau: the buckets that end before T, their blocks in one wave
-// (a block copies its tile's adjoints first, so few and long ones: with 340
-// blocks for 304 places the 4x4 network took 63 us a step, with 300 it takes
-// 54) but at least kGatherMinRows rows each, shared between E and I rows.  A
-// plain launch: launched while the backward kernel still holds registers, its
-// blocks would not fit in one wave; nor does it let the backward kernel be
-// launched early (4x4, 500 steps: 45 ms, 52 ms with either).
-constexpr int kGatherMinRows = 128;
+// The tile kernel for `per` rows per block.
+const void* gather_tile_fn(long long per) {
+  return per <= 5 * kGatherWarps   ? reinterpret_cast<const void*>(grad_gather_tile_kernel<5>)
+         : per <= 7 * kGatherWarps ? reinterpret_cast<const void*>(grad_gather_tile_kernel<7>)
+                                   : reinterpret_cast<const void*>(grad_gather_tile_kernel<kGatherRows>);
+}
+
+// Gather of step tau, by the tile kernel where the rows lie in draw order, two
+// steps' adjoints fit a block's shared memory and there are more than three rows
+// per warp of a full wave.  Its blocks: one wave, as few rows per block as that
+// allows.  A plain launch: launched while the backward kernel
+// still holds registers, its blocks would not fit in one wave.
 cudaError_t launch_gather(snn_grad* g, long long tau) {
   const NetView& v = g->v;
-  const int nb = (int)std::min<long long>(v.ndel, g->T - tau - v.dmin);
+  int nb = (int)std::min<long long>(v.ndel, g->T - tau - v.dmin);
   if (nb <= 0) return cudaSuccess;
-  const int per_sm = 2 * (g->gather_smem + 2048) <= kSmemBudget ? 2 : 1;
-  const int slots = v.num_sms * per_sm;
-  const long long re = (long long)v.tcols * v.nexc, ri = (long long)v.tcols * (v.npc - v.nexc);
-  const int most = (int)std::max<long long>(
-      2, std::min<long long>(slots / (nb * v.ntile), (re + ri) / kGatherMinRows));
-  const int be = re ? std::max(1, (int)(most * re / (re + ri))) : 0;
-  const int bi = ri ? std::max(1, most - be) : 0;
-  int rows_e = be ? (int)((re + be - 1) / be) : 0, rows_i = bi ? (int)((ri + bi - 1) / bi) : 0;
-  int blocks_e = be, blocks_i = bi;
-  void* args[] = {&g->P, &tau, &rows_e, &rows_i, &blocks_e, &blocks_i};
-  return launch_overlapped(reinterpret_cast<const void*>(grad_gather_kernel),
-                           dim3((unsigned)(v.ntile * (be + bi)), (unsigned)nb), kGatherThreads / per_sm,
-                           g->gather_smem, args, false, v.stream);
+  const size_t win = (size_t)v.acc_words * 4;
+  if (g->P.ord || 2 * win > kSmemBudget || v.N <= 3 * kGatherWarps * v.num_sms) {
+    void* args[] = {&g->P, &tau};
+    return launch_overlapped(g->P.ord ? reinterpret_cast<const void*>(grad_gather_kernel<true>)
+                                      : reinterpret_cast<const void*>(grad_gather_kernel<false>),
+                             dim3((unsigned)g->wblocks), kThreads, 0, args, false, v.stream);
+  }
+  const long long ncol = v.N / v.npc;
+  const long long re = ncol * v.nexc, ri = v.N - re;
+  const long long most = kGatherWarps * kGatherRows;
+  long long per = std::min(most, (v.N + v.num_sms - 1) / v.num_sms);
+  while (per < most && (re + per - 1) / per + (ri + per - 1) / per > v.num_sms) ++per;
+  int per_block = (int)per, blocks_e = (int)((re + per - 1) / per);
+  const int blocks = blocks_e + (int)((ri + per - 1) / per);
+  int bufs = (int)std::min<size_t>(kGatherBufs, kSmemBudget / win);
+  void* args[] = {&g->P, &tau, &nb, &bufs, &per_block, &blocks_e};
+  return launch_overlapped(gather_tile_fn(per), dim3((unsigned)blocks), kGatherThreads, bufs * win, args, false,
+                           v.stream);
 }
 
 cudaError_t launch_forward_step(snn_grad* g, long long t, int slot, int rates) {
@@ -601,12 +709,12 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   const long long N = v.N;
   g->ublocks = (int)((N + kThreads - 1) / kThreads);
   g->wblocks = (int)((N * 32 + kThreads - 1) / kThreads);
-  g->gather_smem = (size_t)v.tcols * v.npc4 * 4;
-  if (cudaFuncSetAttribute(grad_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kSmemBudget) != cudaSuccess) {
-    delete g;
-    return fail_global(SNN_ECUDA, "the gather kernel does not fit on the device");
-  }
+  for (int rows : {5, 7, kGatherRows})
+    if (cudaFuncSetAttribute(gather_tile_fn(rows * kGatherWarps), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kSmemBudget) != cudaSuccess) {
+      delete g;
+      return fail_global(SNN_ECUDA, "the gather kernel does not fit on the device");
+    }
   // propagators in FP64 as the spiking tables compute them (h = 1 ms)
   const double tm = v.neuron.tau_m, tc = v.neuron.tau_c;
   g->pvv = std::exp(-1.0 / tm);
@@ -618,12 +726,12 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   P.accw = v.acc_words;
   P.npc = v.npc;
   P.npc4 = v.npc4;
+  P.ncol = (int)(N / v.npc);
   P.unit = v.unit;
   P.planes = v.planes;
   P.ctile = v.ctile;
   P.colv = v.colv;
   P.nbg = v.nbg;
-  P.tinfo = v.tinfo;
   P.nexc = v.nexc;
   P.dmin = v.dmin;
   P.ndel = v.ndel;
@@ -662,9 +770,15 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   if (!rc) rc = galloc(g, &P.ibe, accw * g->nslot);
   if (!rc) rc = galloc(g, &P.ibi, accw * g->nslot);
   if (!rc) rc = galloc(g, &P.gb, n * 3);
-  if (!rc) rc = galloc(g, &P.part, n * v.ndel);
+  if (!rc) rc = galloc(g, &P.sg, n);
   if (!rc) rc = galloc(g, &P.gacc, n * 6);
   if (!rc) rc = galloc(g, &g->ck, n * (2 + g->nslot) * g->nseg);
+  if (!rc) rc = galloc(g, &P.vtile, (size_t)(N / v.npc));
+  // rows whose synapses lie in another order than they were drawn in
+  const bool map = v.ntile > 1 || v.unit != kSlotUnit;
+  P.ord_units = v.ord_units;
+  if (!rc && map) rc = galloc(g, &P.ord, n * v.ord_units);
+  if (!rc && map) rc = galloc(g, &P.ord_end, n * v.ndel);
   if (rc) {
     const std::string why = g->err;
     grad_release(g);
@@ -676,11 +790,22 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   std::vector<float> qf(qd.size());
   for (size_t k = 0; k < qd.size(); ++k) qf[k] = (float)qd[k];
   cudaError_t e = cudaMemcpyAsync(g->q, qf.data(), qf.size() * 4, cudaMemcpyHostToDevice, v.stream);
+  if (e == cudaSuccess) {
+    grad_tile_words_kernel<<<(unsigned)v.ntile, kThreads, 0, v.stream>>>(P, v.tinfo);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && map) {
+    BuildParams bp = v.build;
+    bp.ord = P.ord;
+    bp.ord_end = P.ord_end;
+    bp.ord_units = P.ord_units;
+    e = launch_draw_order(bp, v.paper, v.num_sms, v.stream);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(v.stream);
   if (e != cudaSuccess) {
     grad_release(g);
     delete g;
-    return fail_global(SNN_ECUDA, std::string("quantile table: ") + cudaGetErrorString(e));
+    return fail_global(SNN_ECUDA, std::string("gradient tables: ") + cudaGetErrorString(e));
   }
   *out = g;
   return SNN_OK;

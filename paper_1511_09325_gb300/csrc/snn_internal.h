@@ -286,6 +286,11 @@ struct BuildParams {
   long long* rd_target;
   int32_t* rd_delay;
   int32_t* rd_wfx;
+  // draw order of the rows (the differentiable form's sums; see snn_grad.cu):
+  // a word per 8 places of a row, and the ends of its buckets in such units
+  uint32_t* ord;          // [ncol * npc][ord_units], rows in the order of syn
+  uint8_t* ord_end;       // [ncol * npc][ndel]
+  int ord_units;
 };
 
 // Byte of a descriptor that holds the end of the in part of bucket b (the end
@@ -306,6 +311,9 @@ struct NetView {
   const uint32_t* nbg;
   const uint2* tinfo;
   int ntile, tcols;
+  int ord_units;       // units of the longest row in draw order
+  BuildParams build;   // the construction's draws
+  bool paper;
   uint64_t seed;
   snn_neuron_params neuron;
   cudaStream_t stream;
@@ -342,6 +350,8 @@ cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
                               cudaStream_t st);
 // Readback of rows in the order they were drawn, within a row by delay.
 cudaError_t launch_read_rows(const BuildParams& bp, int precision, bool paper, cudaStream_t st);
+// The rows' draw order (bp.ord, bp.ord_end), drawn again.
+cudaError_t launch_draw_order(const BuildParams& bp, bool paper, int num_sms, cudaStream_t st);
 cudaError_t launch_init_state(const StepParams& p, cudaStream_t st);
 // `overlap`: programmatic dependent launch (step graphs, where update and
 // delivery alternate); else a plain launch.
