@@ -17,6 +17,7 @@ struct snn_net {
   // configuration
   int W = 0, H = 0, npc = 0, nexc = 0, K = 0, dmin = 0, ndel = 0, nslot = 0;
   int precision = 0, rowcap = 0, rec_size = 0, num_sms = 0, update_grid = 0;
+  bool wide = false;  // F16W with a weight of 64 mV or more
   bool agg = true;
   int deliver_grid = 0;
   int npc4 = 0, unit = kSlotUnit;     // words of a column in acc; slots of a bucket unit
@@ -366,6 +367,7 @@ void fill_step_params(snn_net* net) {
   p.row_sec = net->rowcap * net->rec_size / 32;
   p.unit_sec = net->unit * net->rec_size / 32;
   p.ncol = (int)net->ncol;
+  p.wide = net->wide ? 1 : 0;
   p.agg = net->agg ? 1 : 0;
   p.npc4 = net->npc4;
   p.ntile = net->ntile;
@@ -447,6 +449,9 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   net->rec_cap = 1LL << 24;
   rc = make_host_tables(*np, *sp, precision, &net->tables, &why);
   if (rc != SNN_OK) return fail(net, rc, why);
+  constexpr uint32_t kHalf64 = 0x5400u;  // 64 as a half
+  if (precision == SNN_EXACT_F16W)
+    for (uint32_t w : net->tables.wtab) net->wide = net->wide || w >= kHalf64;
   net->sp.theta = np->theta;
   net->sp.vr = np->v_reset;
   net->sp.dc = np->dc;
@@ -1401,12 +1406,15 @@ int batch_run(snn_batch* b, long long n_steps) {
     bp.max_cols = std::max(bp.max_cols, net->sp.tcols);
   }
   const size_t smem = batch_smem(bp.win_words, bp.max_cols);
-  bool rows = false;
-  for (const snn_net* net : b->nets) rows = rows || net->rlist != nullptr;
-  const int grid = batch_grid(b->precision, b->infl, rows, b->num_sms, smem);
+  bool rows = false, wide = false;
+  for (const snn_net* net : b->nets) {
+    rows = rows || net->rlist != nullptr;
+    wide = wide || net->wide;
+  }
+  const int grid = batch_grid(b->precision, b->infl, rows, wide, b->num_sms, smem);
   if (grid < 1) return bfail(b, SNN_ECUDA, "batch kernel does not fit on the device");
   SNN_BCUDA(b, cudaMemsetAsync(b->d_bar, 0, 3 * sizeof(unsigned), b->stream));
-  SNN_BCUDA(b, launch_batch(bp, b->precision, b->infl, rows, grid, smem, b->stream));
+  SNN_BCUDA(b, launch_batch(bp, b->precision, b->infl, rows, wide, grid, smem, b->stream));
   unsigned flags[3] = {0u, 0u, 0u};
   SNN_BCUDA(b, cudaMemcpyAsync(flags, b->d_bar, sizeof(flags), cudaMemcpyDeviceToHost, b->stream));
   SNN_BCUDA(b, cudaStreamSynchronize(b->stream));

@@ -189,6 +189,7 @@ struct StepParams {
   int tcols;               // columns of the largest tile
   int planes;              // 16-byte planes of a spike descriptor
   int row_sec, unit_sec;   // 32-byte sectors of a row and of a bucket unit
+  int wide;                // F16W: some weight is 64 mV or more
   int agg;                 // shared-memory windows over the delivery tiles
   unsigned min_items;      // fewest items a delivery block takes (fewer blocks run)
   unsigned win_items;      // fewest items of a part that uses the window
@@ -381,10 +382,10 @@ cudaError_t launch_count_records(const StepParams& p, int nreg, unsigned long lo
 // Batch kernel: dynamic shared memory for members whose largest window has
 // win_words words and whose largest tile has max_cols columns, its grid (0 if it does not fit), its launch.
 size_t batch_smem(int win_words, int max_cols);
-// `rows`: some member keeps lists of rows.
-int batch_grid(int precision, int infl, bool rows, int num_sms, size_t smem);
-cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, int grid, size_t smem,
-                         cudaStream_t st);
+// `rows`: some member keeps lists of rows; `wide`: some member has wide weights.
+int batch_grid(int precision, int infl, bool rows, bool wide, int num_sms, size_t smem);
+cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, bool wide, int grid,
+                         size_t smem, cudaStream_t st);
 // Shard: list the received spikes (global indices ids[0 .. n)) of the halo
 // columns in the step's lists, as the update kernel lists its own.
 cudaError_t launch_ingest(const StepParams& p, const uint32_t* ids, long long n, cudaStream_t st);

@@ -55,6 +55,13 @@ constexpr int kUpdateThreads = 256;
 constexpr int kDeliverThreads = 768;   // one delivery block per SM (24 warps, 2 rounds in flight)
 constexpr int kBatchThreads = 512;     // batch kernel: 2 update sub-blocks or one delivery block
 constexpr int kUpdateSubs = kBatchThreads / kUpdateThreads;
+// Precision of a kernel: SNN_EXACT_F32W, SNN_EXACT_F16W, or F16W with a weight of
+// 64 mV or more (see half_fx).
+constexpr int kF16Wide = 2;
+template <int PREC>
+__device__ constexpr bool f16() {
+  return PREC != SNN_EXACT_F32W;
+}
 constexpr int kDepth = 2;        // rounds of 32-byte sectors in flight per lane
 constexpr int kUpdateWarps = kUpdateThreads / 32;
 constexpr int kChunk = 128;      // neurons of a warp's chunk (four per lane)
@@ -588,7 +595,7 @@ __device__ __forceinline__ uint2 item_bounds(const uint4& d, int bucket) {
 // (F16W) or 4 (F32W) sectors.
 template <int PREC>
 __device__ constexpr uint32_t sector_bits() {
-  return PREC == SNN_EXACT_F16W ? 25u : 26u;
+  return f16<PREC>() ? 25u : 26u;
 }
 
 // One 32-byte sector of the table, read once.  The L2 fetches 64 bytes around
@@ -610,11 +617,14 @@ __device__ __forceinline__ void ld_sector(Sector& s, const unsigned char* p, boo
       : "l"(p), "r"((uint32_t)on));
 }
 
-// Weight of an F16W record, rint(half * 2^16): one rounded multiply-add
-// (x * (+-2^16) + 1.5 * 2^23 lands in [2^23, 2^24), where the float grid is
-// the integers, so the low mantissa bits hold the rounded product).
+// Weight of an F16W record, rint(half * 2^16) with the scale's sign.  One rounded
+// multiply-add: x * (+-2^16) + 1.5 * 2^23 lands in [2^23, 2^24), where the float
+// grid is the integers, so the low mantissa bits hold the rounded product.  That
+// holds for weights below 64 mV; nets with larger ones (kF16Wide) convert.
+template <int PREC>
 __device__ __forceinline__ int32_t half_fx(uint32_t half_bits, float scale) {
   const float h = __half2float(__ushort_as_half((unsigned short)half_bits));
+  if (PREC == kF16Wide) return __float2int_rn(__fmul_rn(h, scale));
   return __float_as_int(__fmaf_rn(h, scale, 12582912.0f)) - 0x4B400000;
 }
 
@@ -622,10 +632,10 @@ __device__ __forceinline__ int32_t half_fx(uint32_t half_bits, float scale) {
 // into the accumulator words of the tile at `acc`.
 template <int PREC, bool WIN>
 __device__ __forceinline__ void deliver_in(const Sector& s, uint32_t win_s, const int32_t* acc) {
-  if (PREC == SNN_EXACT_F16W) {
+  if (f16<PREC>()) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int32_t wfx = half_fx(s.w[q] >> 16, 65536.0f);
+      const int32_t wfx = half_fx<PREC>(s.w[q] >> 16, 65536.0f);
       if (WIN)
         red_shared(win_s + 4u * (s.w[q] & 0xFFFFu), wfx);
       else
@@ -648,7 +658,7 @@ __device__ __forceinline__ void deliver_in(const Sector& s, uint32_t win_s, cons
 template <int PREC, bool WIN>
 __device__ __forceinline__ void deliver_out(const Sector& s, float scale, uint32_t nb_s,
                                             const uint32_t* nb_g, const int32_t* acc) {
-  constexpr int kN = PREC == SNN_EXACT_F16W ? 8 : 4, kW = 8 / kN;
+  constexpr int kN = f16<PREC>() ? 8 : 4, kW = 8 / kN;
   uint32_t base[kN];
 #pragma unroll
   for (int q = 0; q < kN; ++q) {
@@ -661,7 +671,7 @@ __device__ __forceinline__ void deliver_out(const Sector& s, float scale, uint32
 #pragma unroll
   for (int q = 0; q < kN; ++q) {
     const uint32_t code = s.w[kW * q];
-    const int32_t wfx = PREC == SNN_EXACT_F16W ? half_fx(code >> 17, scale) : (int32_t)s.w[kW * q + kW - 1];
+    const int32_t wfx = f16<PREC>() ? half_fx<PREC>(code >> 17, scale) : (int32_t)s.w[kW * q + kW - 1];
     red_add_nz(acc + (base[q] + (code & 2047u)), wfx);
   }
 }
@@ -712,7 +722,7 @@ __device__ __forceinline__ void stream_part(const StepParams& P, const Part& T, 
         const uint32_t k = div_by(cur.x, (uint32_t)P.npc, P.npc_m), l = cur.x - k * (uint32_t)P.npc;
         uint32_t tag = cur.x * (uint32_t)P.row_sec + (uint32_t)(beg * P.unit_sec);
         tag |= k << sector_bits<PREC>();
-        if (PREC == SNN_EXACT_F16W && (int)l >= P.nexc) tag |= 0x80000000u;
+        if (f16<PREC>() && (int)l >= P.nexc) tag |= 0x80000000u;
         const int p_in = (int)(incl & 0xFFFFu) - u_in - c0;
         const int p_out = r_in * 32 + (int)(incl >> 16) - u_out - c0;
         for (int p = max(p_in, 0); p < min(p_in + u_in, kListCap); ++p)
@@ -739,7 +749,7 @@ __device__ __forceinline__ void stream_part(const StepParams& P, const Part& T, 
           if (rr < r_in) {
             if (rr * 32 + lane < n_in) deliver_in<PREC, WIN>(sec[d], win_s, acc_t);
           } else if (rr < r1 && rr * 32 + lane < lim_out) {
-            const uint32_t kk = PREC == SNN_EXACT_F16W ? (en[d] >> 25) & 63u : en[d] >> 26;
+            const uint32_t kk = f16<PREC>() ? (en[d] >> 25) & 63u : en[d] >> 26;
             deliver_out<PREC, WIN>(sec[d], __uint_as_float(0x47800000u | (en[d] & 0x80000000u)),
                                    nb_s + kk * 256u, nb_g + kk * 64u, P.acc);
           }
@@ -1384,6 +1394,7 @@ const void* deliver_fn(bool rows) {
 }
 const void* deliver_fn(const StepParams& p, int precision) {
   const bool rows = p.rlist != nullptr;
+  if (p.wide) return deliver_fn<kF16Wide>(rows);
   return precision == SNN_EXACT_F16W ? deliver_fn<SNN_EXACT_F16W>(rows) : deliver_fn<SNN_EXACT_F32W>(rows);
 }
 }  // namespace
@@ -1448,8 +1459,9 @@ void* batch_fn() {
   return reinterpret_cast<void*>(batch_kernel<PREC, INFL, ROWS>);
 }
 // The batch tuner's schedule `infl` (2 or 4) selects 1 or 2 rounds of
-// sectors in flight per lane (always 1 for lists of rows).
-void* batch_kernel_ptr(int precision, int infl, bool rows) {
+// sectors in flight per lane (always 1 for lists of rows and wide weights).
+void* batch_kernel_ptr(int precision, int infl, bool rows, bool wide) {
+  if (wide) return batch_fn<kF16Wide, 1, true>();
   if (rows) return precision == SNN_EXACT_F16W ? batch_fn<1, 1, true>() : batch_fn<0, 1, true>();
   if (precision == SNN_EXACT_F16W) return infl == 2 ? batch_fn<1, 1, false>() : batch_fn<1, 2, false>();
   return infl == 2 ? batch_fn<0, 1, false>() : batch_fn<0, 2, false>();
@@ -1461,8 +1473,8 @@ size_t batch_smem(int win_words, int max_cols) {
                   ((size_t)win_words + (size_t)max_cols * 64 + (size_t)(kBatchThreads / 32) * kListWords) * 4);
 }
 
-int batch_grid(int precision, int infl, bool rows, int num_sms, size_t smem) {
-  void* fn = batch_kernel_ptr(precision, infl, rows);
+int batch_grid(int precision, int infl, bool rows, bool wide, int num_sms, size_t smem) {
+  void* fn = batch_kernel_ptr(precision, infl, rows, wide);
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)std::max(smem, kBatchSmemBudget)) != cudaSuccess)
     return 0;
@@ -1471,10 +1483,10 @@ int batch_grid(int precision, int infl, bool rows, int num_sms, size_t smem) {
   return per_sm * num_sms;
 }
 
-cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, int grid, size_t smem,
-                         cudaStream_t st) {
+cudaError_t launch_batch(const BatchParams& b, int precision, int infl, bool rows, bool wide, int grid,
+                         size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<BatchParams*>(&b)};
-  return cudaLaunchCooperativeKernel(batch_kernel_ptr(precision, infl, rows), dim3(grid),
+  return cudaLaunchCooperativeKernel(batch_kernel_ptr(precision, infl, rows, wide), dim3(grid),
                                      dim3(kBatchThreads), args, smem, st);
 }
 
