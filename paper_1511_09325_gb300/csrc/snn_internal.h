@@ -84,11 +84,13 @@ constexpr int kMaxGridSide = 16383;     // columns per grid side (14-bit coordin
 constexpr int kMaxTile = 8;             // delivery tile side, columns
 constexpr int kMaxTileCols = kMaxTile * kMaxTile;
 constexpr int kCntStride = 8;           // words from one tile counter to the next
-// Shared memory of a delivery block: of a net of its own (one block per SM) and
-// of the batch kernel (two per SM); the window alone takes at most
+// Dynamic shared memory of a delivery block: of a net of its own (one block per
+// SM) and of the batch kernel (two per SM, with their static part and the 1 KB
+// that the system keeps of each block in the SM's 228 KB: with 110 KB, tiles of
+// more than 111 376 bytes left one block per SM); the window alone takes at most
 // kWindowBudget.
 constexpr size_t kSmemBudget = 224 * 1024;
-constexpr size_t kBatchSmemBudget = 110 * 1024;
+constexpr size_t kBatchSmemBudget = 108 * 1024;
 constexpr size_t kWindowBudget = 196 * 1024;
 // Words of a tile's window per item of the fewest that make a part use the
 // window, and per item of its fixed cost in the range split (set-up and

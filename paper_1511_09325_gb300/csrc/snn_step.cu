@@ -1468,6 +1468,10 @@ void* batch_kernel_ptr(int precision, int infl, bool rows, bool wide) {
 }
 }  // namespace
 
+static_assert(2 * (kBatchSmemBudget + kUpdateSubs * sizeof(StepParams) + sizeof(DeliverSmem) +
+                   (kMaxBatch + 1) * sizeof(int) + 64 + 1024) <= 228 * 1024,
+              "two blocks of the batch kernel fit an SM");
+
 size_t batch_smem(int win_words, int max_cols) {
   return std::max(kUpdateSubs * sizeof(UpdateSmem),
                   ((size_t)win_words + (size_t)max_cols * 64 + (size_t)(kBatchThreads / 32) * kListWords) * 4);
