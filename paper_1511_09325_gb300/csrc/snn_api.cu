@@ -368,13 +368,12 @@ void fill_step_params(snn_net* net) {
   p.unit_sec = net->unit * net->rec_size / 32;
   p.ncol = (int)net->ncol;
   p.wide = net->wide ? 1 : 0;
-  p.agg = net->agg ? 1 : 0;
   p.npc4 = net->npc4;
   p.ntile = net->ntile;
   p.tcols = net->tw * net->th;
   p.tcap = p.tcols * net->npc;
   p.min_items = net->min_items;
-  p.win_items = net->win_items;
+  p.win_items = net->agg ? net->win_items : 0xFFFFFFFFu;  // no windows: none is paid for either
   p.cost_win = net->cost_win;
   p.npc_m = recip32((uint32_t)net->npc);
   p.seed_lo = (uint32_t)(net->seed & 0xFFFFFFFFu);

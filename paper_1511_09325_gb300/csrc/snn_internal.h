@@ -192,9 +192,8 @@ struct StepParams {
   int planes;              // 16-byte planes of a spike descriptor
   int row_sec, unit_sec;   // 32-byte sectors of a row and of a bucket unit
   int wide;                // F16W: some weight is 64 mV or more
-  int agg;                 // shared-memory windows over the delivery tiles
   unsigned min_items;      // fewest items a delivery block takes (fewer blocks run)
-  unsigned win_items;      // fewest items of a part that uses the window
+  unsigned win_items;      // fewest items of a part that uses the window (2^32 - 1: none does)
   unsigned cost_win;       // fixed cost (in items) of a tile with a window
   uint32_t npc_m;          // floor(2^32 / n_per_col) (capped)
   uint32_t seed_lo, seed_hi;

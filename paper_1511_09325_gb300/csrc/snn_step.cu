@@ -971,7 +971,7 @@ __device__ __forceinline__ void deliver_blocks(Tiles& tiles, F&& t_of, int vb, i
       const int cols = (int)ti.y;
       T.a = a;
       T.b = min(b, found);
-      if (P.agg && b - a >= P.win_items) {
+      if (b - a >= P.win_items) {
         if (!clean) {
           // the issuing threads' bulk reductions have read the window
           if (tid < kMaxTileCols) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
