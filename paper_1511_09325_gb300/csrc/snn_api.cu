@@ -42,7 +42,7 @@ struct snn_net {
   int32_t* acc = nullptr;
   uint4* list = nullptr;                  // spike lists
   uint16_t* rlist = nullptr;              // or lists of rows
-  bool lean = false;                      // keep lists of rows in any case
+  bool lean = false;                      // lists of rows
   uint32_t* ctile = nullptr;              // geometry tables (see snn_internal.h)
   uint32_t* colv = nullptr;
   uint2* tinfo = nullptr;
@@ -422,6 +422,21 @@ void fill_step_params(snn_net* net) {
   p.spk_part = net->spk_part;
 }
 
+// Whether a net whose arrays still to be allocated take `small` bytes with lists
+// of rows and `large` with lists of descriptors (`had`: allocated already), on a
+// device with `free` bytes, takes the descriptors: only where they leave room for a
+// second net of this size if there is room for two without them, and half as much
+// in any case (for a differentiable view, or the caller's own arrays).
+// Descriptors are about 1300 of an FP16 net's 7200 or an FP32 net's 13 100 bytes
+// per neuron; lists of rows cost time: 1000 steps of 96x96 FP16 451 instead of 408
+// ms, of 48x48 FP32 149 instead of 140 ms.
+bool roomy_lists(size_t free, size_t had, size_t small, size_t large) {
+  constexpr size_t kSlack = 48u << 20;  // rounding of two dozen allocations
+  const size_t other = had + small;     // the second net, without descriptors
+  if (large + kSlack + other / 2 > free) return false;
+  return large + kSlack + other <= free || small + kSlack + other > free;
+}
+
 int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
                const snn_synapse_params* sp, uint64_t seed, int precision) {
   std::string why;
@@ -512,37 +527,34 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->bend, (size_t)net->N * net->planes * 16))) return rc;
   net->total_syn = net->N * (long long)net->K;
   if (net->sg.on && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
-  // the longest row (bp.max_units), read back by a count pass
+  // count pass: bucket ends, out-degrees and the longest row (max_units), which
+  // sets the row stride of the table
+  const bool paper = net->connectivity == SNN_CONN_PAPER;
   unsigned max_units[2] = {0u, 0u};
-  auto longest_row = [&](auto&& count) -> cudaError_t {
-    cudaError_t ce = cudaMemsetAsync(bp.max_units, 0, 8, net->stream);
-    if (ce == cudaSuccess) ce = count(bp, net->num_sms, net->stream);
+  if (paper && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
+  if ((rc = dalloc(net, &bp.max_units, 8))) return rc;
+  net->device_bytes -= 8;
+  bp.bend = net->bend;
+  bp.deg = net->deg;
+  cudaError_t ce = cudaSuccess;
+  if (paper) net->unit = kSlotUnit;  // 16 slots only where a row needs them
+  for (;; net->unit *= 2) {
+    bp.unit = net->unit;
+    ce = cudaMemsetAsync(bp.max_units, 0, 8, net->stream);
+    if (ce == cudaSuccess)
+      ce = paper ? launch_paper_count(bp, net->num_sms, net->stream) : launch_build_count(bp, net->num_sms, net->stream);
     if (ce == cudaSuccess)
       ce = cudaMemcpyAsync(max_units, bp.max_units, 8, cudaMemcpyDeviceToHost, net->stream);
-    return ce == cudaSuccess ? cudaStreamSynchronize(net->stream) : ce;
-  };
-  bp.bend = net->bend;
-  if (net->connectivity == SNN_CONN_PAPER) {
-    // count pass: bucket ends, out-degrees and the longest row, which sets
-    // the row stride of the table
-    unsigned* dmax = nullptr;
-    if ((rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
-    if ((rc = dalloc(net, &dmax, 8))) return rc;
-    net->device_bytes -= 8;
-    bp.deg = net->deg;
-    bp.max_units = dmax;
-    cudaError_t ce = cudaSuccess;
-    for (net->unit = kSlotUnit; ce == cudaSuccess; net->unit *= 2) {
-      bp.unit = net->unit;
-      ce = longest_row(launch_paper_count);
-      if (max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
-    }
-    cudaFree(dmax);
-    if (ce != cudaSuccess) return cuda_fail(net, ce, "connectivity count pass");
-    if (max_units[1] > 255u || max_units[0] > 255u)
-      return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
-    net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
-    net->ord_units = (int)std::max(1u, max_units[1]);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(net->stream);
+    if (ce != cudaSuccess || max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
+  }
+  cudaFree(bp.max_units);
+  if (ce != cudaSuccess) return cuda_fail(net, ce, "connectivity count pass");
+  if (max_units[1] > 255u || max_units[0] > 255u)
+    return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
+  net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
+  if (paper) net->ord_units = (int)std::max(1u, max_units[1]);
+  if (net->deg) {
     std::vector<uint32_t> deg((size_t)net->N);
     SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
                                   net->stream));
@@ -550,33 +562,31 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
     net->total_syn = 0;
     for (uint32_t d : deg) net->total_syn += d;
   }
-  // Lists of descriptors take planes x 16 bytes per neuron and step.  Where
-  // they do not fit the device beside the table, lists of rows take their place
-  // and the table's rows get the longest row's length, not the longest possible.
+  // Spike lists: of descriptors (planes x 16 bytes per neuron and step) or, where
+  // the device has little room, of rows (2 bytes).
   const size_t tcap = (size_t)net->tw * net->th * net->npc;
   const size_t list_len = (size_t)net->nslot * net->ntile * tcap;
-  const size_t rest = (size_t)net->Npad * 17 + (size_t)net->rec_region * net->update_grid * 16 + (64u << 20);
+  const size_t syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
+  const size_t acc_bytes = (size_t)net->ncol * net->npc4 * 4;
+  const size_t ccnt_bytes = (size_t)net->nslot * net->ntile * kCntStride * 4;
+  const size_t isum_bytes = (size_t)net->ntile * kCntStride * 4;
+  const size_t icnt_bytes = net->sg.on ? (size_t)net->ncol * 4 : 0;
+  const size_t rec_bytes = (size_t)net->rec_region * net->update_grid * 8;
+  const size_t col_bytes = (size_t)net->ncol * 2 * 8;
+  const size_t wtab_bytes = net->tables.wtab.size() * 4;
+  const size_t rest = (size_t)net->Npad * 9 + acc_bytes + ccnt_bytes + isum_bytes + icnt_bytes +
+                      2 * rec_bytes + col_bytes + wtab_bytes;
   size_t free_bytes = 0, all_bytes = 0;
   SNN_CUDA(net, cudaMemGetInfo(&free_bytes, &all_bytes));
-  const bool rows = net->lean || (size_t)net->N * net->rowcap * net->rec_size +
-                                         list_len * net->planes * 16 + rest > free_bytes;
-  if (rows && net->connectivity != SNN_CONN_PAPER) {
-    if ((rc = dalloc(net, &bp.max_units, 8))) return rc;
-    net->device_bytes -= 8;
-    const cudaError_t ce = longest_row(launch_row_lengths);
-    cudaFree(bp.max_units);
-    if (ce != cudaSuccess) return cuda_fail(net, ce, "row-length pass");
-    net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
-  }
+  if (!roomy_lists(free_bytes, net->device_bytes, syn_bytes + rest + list_len * 2,
+                   syn_bytes + rest + list_len * net->planes * 16))
+    net->lean = true;
+  const bool rows = net->lean;
   bp.rowcap = net->rowcap;
-  const size_t syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
   if ((rc = dalloc(net, &net->syn, syn_bytes))) return rc;
   if ((rc = dalloc(net, &net->V, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->C, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->R, (size_t)net->Npad))) return rc;
-  const size_t acc_bytes = (size_t)net->ncol * net->npc4 * 4;
-  const size_t ccnt_bytes = (size_t)net->nslot * net->ntile * kCntStride * 4;
-  const size_t isum_bytes = (size_t)net->ntile * kCntStride * 4;
   if ((rc = dalloc(net, &net->acc, acc_bytes))) return rc;
   if (rows) {
     if ((rc = dalloc(net, &net->rlist, list_len * 2))) return rc;
@@ -586,11 +596,11 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->ccnt, ccnt_bytes))) return rc;
   if ((rc = dalloc(net, &net->isum, isum_bytes))) return rc;
   if ((rc = dalloc(net, &net->gsum, 4))) return rc;
-  if (net->sg.on && (rc = dalloc(net, &net->icnt, (size_t)net->ncol * 4))) return rc;
+  if (icnt_bytes && (rc = dalloc(net, &net->icnt, icnt_bytes))) return rc;
   if ((rc = dalloc(net, &net->ctl, sizeof(Ctl)))) return rc;
-  if ((rc = dalloc(net, &net->rec, (size_t)net->rec_region * net->update_grid * 8))) return rc;
+  if ((rc = dalloc(net, &net->rec, rec_bytes))) return rc;
   if ((rc = dalloc(net, &net->rcnt, (size_t)net->update_grid * 8))) return rc;
-  if ((rc = dalloc(net, &net->stage, (size_t)net->rec_region * net->update_grid * 8))) return rc;
+  if ((rc = dalloc(net, &net->stage, rec_bytes))) return rc;
   if ((rc = dalloc(net, &net->dhdr, 32))) return rc;
   SNN_CUDA(net, cudaHostAlloc(&net->hstatus, 16, cudaHostAllocMapped));
   SNN_CUDA(net, cudaHostGetDevicePointer(&net->hstatus_dev, net->hstatus, 0));
@@ -600,16 +610,16 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   net->hmap_cap = std::min<long long>(net->rec_region * net->update_grid, kMappedRecords);
   SNN_CUDA(net, cudaHostAlloc(&net->hmap, (size_t)net->hmap_cap * 8, cudaHostAllocMapped));
   SNN_CUDA(net, cudaHostGetDevicePointer(&net->hmap_dev, net->hmap, 0));
-  if ((rc = dalloc(net, &net->colcnt, (size_t)net->ncol * 2 * 8))) return rc;
+  if ((rc = dalloc(net, &net->colcnt, col_bytes))) return rc;
   if ((rc = dalloc(net, &net->ext_part, (size_t)net->update_grid * 8))) return rc;
   if ((rc = dalloc(net, &net->spk_part, (size_t)net->update_grid * 8))) return rc;
   if ((rc = dalloc(net, &net->syn_part, (size_t)net->update_grid * 8))) return rc;
   uint32_t* wtab = nullptr;
-  if ((rc = dalloc(net, &wtab, net->tables.wtab.size() * 4))) return rc;
-  net->device_bytes -= net->tables.wtab.size() * 4;
+  if ((rc = dalloc(net, &wtab, wtab_bytes))) return rc;
+  net->device_bytes -= wtab_bytes;
 
-  cudaError_t e = cudaMemcpyAsync(wtab, net->tables.wtab.data(), net->tables.wtab.size() * 4,
-                                  cudaMemcpyHostToDevice, net->stream);
+  cudaError_t e = cudaMemcpyAsync(wtab, net->tables.wtab.data(), wtab_bytes, cudaMemcpyHostToDevice,
+                                  net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->ctl, 0, sizeof(Ctl), net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->acc, 0, acc_bytes, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->ccnt, 0, ccnt_bytes, net->stream);
@@ -625,8 +635,6 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if (e == cudaSuccess) {
     bp.wtab = wtab;
     bp.syn = net->syn;
-    bp.bend = net->bend;
-    bp.deg = net->deg;
     e = net->connectivity == SNN_CONN_PAPER ? launch_paper_fill(bp, precision, net->num_sms, net->stream)
                                             : launch_build(bp, precision, net->num_sms, net->stream);
   }
@@ -637,15 +645,6 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
   cudaFree(wtab);
   if (e != cudaSuccess) return cuda_fail(net, e, "network construction");
-  if (net->sg.on) {
-    // synapses kept by the shard: those into its own columns
-    std::vector<uint32_t> deg((size_t)net->N);
-    SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
-                                  net->stream));
-    SNN_CUDA(net, cudaStreamSynchronize(net->stream));
-    net->total_syn = 0;
-    for (uint32_t d : deg) net->total_syn += d;
-  }
   return SNN_OK;
 }
 
@@ -766,9 +765,14 @@ int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
   }
   int rc = build_impl(net, grid_w, grid_h, neuron, synapse, seed, precision);
   if (rc != SNN_OK) {
+    const bool smaller = rc == SNN_ENOMEM && !net->lean;
     g_err = net->err;
     release(net);
     delete net;
+    // the room went to others meanwhile: once more with the smaller lists
+    if (smaller)
+      return build_net(grid_w, grid_h, neuron, synapse, seed, precision, cuda_stream, batch_member, out, shard,
+                       true);
     return rc;
   }
   *out = net;

@@ -10,11 +10,12 @@
 // A delay bucket has two parts (see snn_internal.h): the synapses that end in
 // the source's own delivery tile, stored as words of the tile's window, and
 // the others, stored as a stencil offset and an index.
-// One warp owns one row: a first pass counts the synapses of every bucket
-// part, a second pass regenerates them and stores each into its part in k
-// order (warp match + popc rank), then the parts' tails are padded.  Rows are
-// stored, and walked, in virtual column order.  The same walk reads rows back
-// in the order in which they were drawn.
+// One warp owns one row: a count pass counts the synapses of every bucket part
+// and writes the bucket ends and the longest row, which sets the rows' stride; a
+// fill pass regenerates them and stores each into its part in k order (warp match
+// + popc rank), then the parts' tails are padded.  Rows are stored, and walked, in
+// virtual column order.  The same walk reads rows back in the order in which they
+// were drawn.
 // A shard (see ShardGeo) draws every synapse with the neuron's global index
 // and keeps only those whose target column is one of its own (local and
 // global stencil arithmetic agree for such targets: the halo is as wide as
@@ -173,6 +174,18 @@ __device__ __forceinline__ unsigned open_parts(const BuildParams& P, RowSmem& S,
   return __shfl_sync(0xFFFFFFFFu, incl, 31);
 }
 
+// First slots of the parts from the stored bucket ends (S.cur; lane b: bucket b).
+__device__ __forceinline__ void stored_parts(const BuildParams& P, RowSmem& S, const Row& r) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane < P.ndel) {
+    const uint8_t* d = P.bend + r.at * P.planes * 16;
+    const int at = lane % kPlaneBuckets ? desc_end(lane) - 1 : desc_start(lane);
+    S.cur[w][2 * lane] = (unsigned)d[at] * (unsigned)P.unit;
+    S.cur[w][2 * lane + 1] = (unsigned)d[desc_end(lane)] * (unsigned)P.unit;
+  }
+  __syncwarp();
+}
+
 // Places (or reads back) one synapse per lane: part bb = 2 bucket + (0 in,
 // 1 out) or 64 for none.
 template <int PREC, int MODE>
@@ -321,9 +334,9 @@ __device__ __forceinline__ void write_order(const BuildParams& P, RowSmem& S, co
   __syncwarp();
 }
 
-// Rows of the fixed law, one warp per row; MODE fill builds them, read writes
-// rows j0 .. j0 + n_rows - 1 to the rd_* arrays, count finds the longest, order
-// writes the rows' draw order.
+// Rows of the fixed law, one warp per row; MODE count writes their bucket ends
+// and the longest row, fill builds them, read writes rows j0 .. j0 + n_rows - 1 to
+// the rd_* arrays, order writes the rows' draw order.
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const BuildParams P) {
   __shared__ RowSmem S;
@@ -338,28 +351,32 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const Buil
     const uint32_t j = (uint32_t)(MODE == kModeRead ? P.j0 + i : i);
     const int c = (int)(j / (uint32_t)P.npc);
     const Row r = open_row<false>(P, S, c, (int)(j - (uint32_t)c * (uint32_t)P.npc));
-    S.cnt[w][lane] = 0u;
-    S.cnt[w][lane + 32] = 0u;
-    __syncwarp();
-    // pass 1: synapses per bucket part
-    unsigned nkept = 0u;
-    for (int k = lane; k < P.K; k += 32) {
-      const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
-      const int cl = S.cls[w][k < P.k_local ? kMaxOff : offset_of(P, S, x.y)];
-      if (cl != kDropped) {
-        atomicAdd(&S.cnt[w][2 * below(x.z, ndel) + (cl == kOut ? 1 : 0)], 1u);
-        ++nkept;
+    if (MODE == kModeFill) {
+      stored_parts(P, S, r);
+    } else {
+      S.cnt[w][lane] = 0u;
+      S.cnt[w][lane + 32] = 0u;
+      __syncwarp();
+      // pass 1: synapses per bucket part
+      unsigned nkept = 0u;
+      for (int k = lane; k < P.K; k += 32) {
+        const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
+        const int cl = S.cls[w][k < P.k_local ? kMaxOff : offset_of(P, S, x.y)];
+        if (cl != kDropped) {
+          atomicAdd(&S.cnt[w][2 * below(x.z, ndel) + (cl == kOut ? 1 : 0)], 1u);
+          ++nkept;
+        }
       }
-    }
-    if (MODE == kModeFill && P.deg != nullptr) {
-      nkept = __reduce_add_sync(0xFFFFFFFFu, nkept);
-      if (lane == 0) P.deg[j] = nkept;
-    }
-    __syncwarp();
-    const unsigned units = open_parts<MODE>(P, S, r);
-    if (MODE == kModeCount) {
-      if (lane == 0) atomicMax(P.max_units, units);
-      continue;
+      __syncwarp();
+      const unsigned units = open_parts<MODE>(P, S, r);
+      if (MODE == kModeCount) {
+        nkept = __reduce_add_sync(0xFFFFFFFFu, nkept);
+        if (lane == 0) {
+          atomicMax(P.max_units, units);
+          if (P.deg != nullptr) P.deg[j] = nkept;
+        }
+        continue;
+      }
     }
 
     const uint32_t* wt = P.wtab + (r.lj < P.nexc ? 0 : 65536);
@@ -445,12 +462,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
     const long long out0 = MODE == kModeRead ? P.rd_off[i] : 0;
     S.cnt[w][lane] = 0u;
     S.cnt[w][lane + 32] = 0u;
-    if (MODE == kModeFill && lane < P.ndel) {
-      const uint8_t* d = P.bend + r.at * P.planes * 16;
-      const int at = lane % kPlaneBuckets ? desc_end(lane) - 1 : desc_start(lane);
-      S.cur[w][2 * lane] = (unsigned)d[at] * (unsigned)P.unit;
-      S.cur[w][2 * lane + 1] = (unsigned)d[desc_end(lane)] * (unsigned)P.unit;
-    }
+    if (MODE == kModeFill) stored_parts(P, S, r);
     __syncwarp();
     // one walk over the candidates; `placing`: place them, else count them
     auto walk = [&](bool placing) -> unsigned {
@@ -531,7 +543,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
 
 }  // namespace
 
-cudaError_t launch_row_lengths(const BuildParams& bp, int num_sms, cudaStream_t st) {
+cudaError_t launch_build_count(const BuildParams& bp, int num_sms, cudaStream_t st) {
   build_rows_kernel<SNN_EXACT_F32W, kModeCount><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);
   return cudaGetLastError();
 }

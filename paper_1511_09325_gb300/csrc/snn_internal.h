@@ -341,12 +341,12 @@ int fail_global(int code, const std::string& msg);
 int validate_neuron_params(const snn_neuron_params* n, std::string* why);
 
 // Kernel launchers (snn_build.cu / snn_step.cu).
+// Fixed law: the count pass writes bend, deg (shards) and max_units[0]; the fill
+// pass (same draws) writes the rows.
+cudaError_t launch_build_count(const BuildParams& bp, int num_sms, cudaStream_t st);
 cudaError_t launch_build(const BuildParams& bp, int precision, int num_sms,
                          cudaStream_t st);
-// Longest row in units of the fixed law's rows (to max_units[0]).
-cudaError_t launch_row_lengths(const BuildParams& bp, int num_sms, cudaStream_t st);
-// Paper connectivity law: the count pass writes bend, deg and max_units; the
-// fill pass (same draws) writes the rows.
+// Paper connectivity law: the same two passes (deg and max_units[1] in any case).
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st);
 cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
                               cudaStream_t st);
