@@ -173,11 +173,12 @@ __device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t m) {
   return q;
 }
 
-// The next place at *count for each active lane: one atomic for the lanes of
-// the same `key` (mostly one; the lanes of a key have the same counter).
-__device__ __forceinline__ unsigned next_place(unsigned* count, uint32_t key) {
+// The next place at *count for each lane of `live`, all of which make this call:
+// one atomic for the lanes of the same `key` (mostly one; the lanes of a key have
+// the same counter).
+__device__ __forceinline__ unsigned next_place(unsigned live, unsigned* count, uint32_t key) {
   const unsigned lane = threadIdx.x & 31u;
-  const unsigned peers = __match_any_sync(__activemask(), key);
+  const unsigned peers = __match_any_sync(live, key);
   const int lead = __ffs(peers) - 1;
   unsigned pos = 0u;
   if ((int)lane == lead) pos = atomicAdd(count, (unsigned)__popc(peers));
@@ -413,6 +414,7 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
       const unsigned k = k0 + (unsigned)lane;
       uint32_t row = 0u;             // the spike's row in bend
       unsigned long long at = 0ull;  // its place in the lists
+      const unsigned live = n - k0 < 32u ? (1u << (n - k0)) - 1u : 0xFFFFFFFFu;  // lanes with k < n
       if (k < n) {
         const uint32_t id = S.id[warp][k];
         const uint32_t c = div_by(id, npc, P.npc_m), il = id - c * npc;
@@ -420,11 +422,11 @@ __device__ __forceinline__ void update_body(const StepParams& P, F&& t_of, int v
           const uint32_t ct = __ldg(P.ctile + c);
           row = __ldg(P.colv + c) * npc + il;
           const size_t ts = (size_t)slot * P.ntile + (ct >> 6);
-          const unsigned place = next_place(P.ccnt + ts * kCntStride, ct >> 6);
+          const unsigned place = next_place(live, P.ccnt + ts * kCntStride, ct >> 6);
           at = ((unsigned long long)slot * P.planes * P.ntile + (ct >> 6)) * P.tcap + place;
           if (P.rlist != nullptr) P.rlist[ts * P.tcap + place] = (uint16_t)((ct & 63u) * npc + il);
         } else {
-          P.ids[next_place(P.cnt + slot, 0u)] = id;
+          P.ids[next_place(live, P.cnt + slot, 0u)] = id;
         }
         atomicAdd(&P.colcnt[2ull * c + (il < (uint32_t)P.nexc ? 0u : 1u)], 1ull);
         if (P.deg != nullptr) syn += P.deg[id];
@@ -1340,29 +1342,39 @@ __global__ void __launch_bounds__(256) ingest_kernel(const StepParams P, const u
   const long long slot = t % P.nslot;
   const unsigned long long ng = (unsigned long long)P.sg.GW * (unsigned long long)P.sg.GH *
                                 (unsigned long long)P.npc;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+  const int lane = threadIdx.x & 31;
+  // (whole warps: the lanes that list a spike take their places together)
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k - lane < n;
        k += (long long)gridDim.x * blockDim.x) {
-    const uint32_t g = ids[k];
-    if ((unsigned long long)g >= ng) {
-      set_status(P, kStatusIngest);
-      continue;
+    uint32_t c = 0u, l = 0u;  // local column and place in it
+    bool halo = false;
+    if (k < n) {
+      const uint32_t g = ids[k];
+      if ((unsigned long long)g >= ng) {
+        set_status(P, kStatusIngest);
+      } else {
+        const uint32_t gc = g / (uint32_t)P.npc;
+        l = g - gc * (uint32_t)P.npc;
+        const int gy = (int)(gc / (uint32_t)P.sg.GW), gx = (int)gc - gy * P.sg.GW;
+        const int lx = wrap(gx - P.sg.ex0, P.sg.GW), ly = wrap(gy - P.sg.ey0, P.sg.GH);
+        const bool own = lx >= P.sg.tx0 && lx < P.sg.tx0 + P.sg.tw && ly >= P.sg.ty0 &&
+                         ly < P.sg.ty0 + P.sg.th;  // listed by the update kernel
+        halo = lx < P.W && ly < P.H && !own;
+        c = (uint32_t)(ly * P.W + lx);
+        if (halo && atomicAdd(P.icnt + c, 1u) >= (unsigned)P.npc) {
+          set_status(P, kStatusIngest);
+          halo = false;
+        }
+      }
     }
-    const uint32_t gc = g / (uint32_t)P.npc;
-    const uint32_t l = g - gc * (uint32_t)P.npc;
-    const int gy = (int)(gc / (uint32_t)P.sg.GW), gx = (int)gc - gy * P.sg.GW;
-    const int lx = wrap(gx - P.sg.ex0, P.sg.GW), ly = wrap(gy - P.sg.ey0, P.sg.GH);
-    if (lx >= P.W || ly >= P.H) continue;  // not in the local grid
-    if (lx >= P.sg.tx0 && lx < P.sg.tx0 + P.sg.tw && ly >= P.sg.ty0 && ly < P.sg.ty0 + P.sg.th)
-      continue;  // an own column: listed by the update kernel
-    if (atomicAdd(P.icnt + ly * P.W + lx, 1u) >= (unsigned)P.npc) {
-      set_status(P, kStatusIngest);
-      continue;
+    const unsigned live = __ballot_sync(0xFFFFFFFFu, halo);
+    if (halo) {
+      // at most n_per_col spikes of each of its columns: the list has room
+      const uint32_t ct = P.ctile[c];
+      const long long tile_slot = slot * P.ntile + (ct >> 6);
+      const unsigned r = next_place(live, P.ccnt + tile_slot * kCntStride, ct >> 6);
+      list_spike(P, slot, ct, r, c, l);
     }
-    // at most n_per_col spikes of each of its columns: the list has room
-    const uint32_t ct = P.ctile[ly * P.W + lx];
-    const long long tile_slot = slot * P.ntile + (ct >> 6);
-    const unsigned r = next_place(P.ccnt + tile_slot * kCntStride, ct >> 6);
-    list_spike(P, slot, ct, r, (uint32_t)(ly * P.W + lx), l);
   }
 }
 
