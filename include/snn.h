@@ -179,7 +179,8 @@ int snn_get_state(snn_net* net, float* v, float* c, uint8_t* refractory);
  * the device table into host arrays, grouped by neuron (neuron j0's first),
  * within a neuron by delay: target neuron, delay (steps), weight in 2^-16 mV.
  * The arrays hold the sum of the rows' lengths (snn_row_lengths): n * k_out
- * entries under SNN_CONN_FIXED.
+ * entries under SNN_CONN_FIXED.  SNN_ESTATE when a stored row does not hold as
+ * many synapses in each delay bucket as the seed draws for it.
  */
 int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target,
                       int32_t* delay, int32_t* wfx);
@@ -198,6 +199,16 @@ int snn_row_lengths(snn_net* net, int64_t j0, int64_t n, int32_t* counts);
  * column out of range.
  */
 int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t group_only);
+
+/*
+ * snn_debug_flip_byte -- testing aid with no counterpart in the paper: xors mask
+ * into one byte of `neuron`'s row of the synapse table (in_table nonzero) or of
+ * its descriptor (bucket ends), as a memory fault would, so that
+ * snn_read_synapses must report it.  The same call undoes it, which it must
+ * before the net is stepped again.  Synchronises the net's stream.  SNN_EINVAL
+ * for a neuron or byte out of range.
+ */
+int snn_debug_flip_byte(snn_net* net, int64_t neuron, int64_t byte, int32_t mask, int32_t in_table);
 
 /*
  * snn_info -- sizes of the net: info[0] = N neurons, [1] = synapses,

@@ -1196,7 +1196,7 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   constexpr int64_t kRows = 4096, kFewRows = 32;
   int32_t longest = 0;
   for (int32_t l : len) longest = std::max(longest, l);
-  const int64_t in_stage = net->rec_region * net->update_grid / (1 + 2 * (int64_t)longest);
+  const int64_t in_stage = (net->rec_region * net->update_grid - 1) / (1 + 2 * (int64_t)longest);
   const bool staged = in_stage >= std::min(n, kFewRows);
   const int64_t m = std::min(n, staged ? std::min(in_stage, kRows) : kRows);
   size_t most = 0;
@@ -1206,8 +1206,9 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
     for (int64_t r = r0; r < std::min(n, r0 + m); ++r) k += (size_t)len[r];
     most = std::max(most, k);
   }
-  unsigned char* buf = reinterpret_cast<unsigned char*>(net->stage);  // offsets, targets, delays, weights
-  const size_t off_bytes = (size_t)m * 8, b8 = most * 8, b4 = most * 4;
+  // error word, offsets, targets, delays, weights
+  unsigned char* buf = reinterpret_cast<unsigned char*>(net->stage);
+  const size_t off_bytes = 8 + (size_t)m * 8, b8 = most * 8, b4 = most * 4;
   if (!staged) {
     rc = dalloc(net, &buf, off_bytes + b8 + 2 * b4);
     if (rc) return rc;
@@ -1218,11 +1219,13 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   bp.bend = net->bend;
   bp.unit = net->unit;
   bp.rowcap = net->rowcap;
-  bp.rd_off = reinterpret_cast<long long*>(buf);
+  bp.rd_bad = reinterpret_cast<unsigned*>(buf);
+  bp.rd_off = reinterpret_cast<long long*>(buf + 8);
   bp.rd_target = reinterpret_cast<long long*>(buf + off_bytes);
   bp.rd_delay = reinterpret_cast<int32_t*>(buf + off_bytes + b8);
   bp.rd_wfx = reinterpret_cast<int32_t*>(buf + off_bytes + b8 + b4);
-  cudaError_t e = cudaSuccess;
+  unsigned bad = 0u;
+  cudaError_t e = cudaMemsetAsync(bp.rd_bad, 0, 4, net->stream);
   size_t at = 0;
   for (int64_t r0 = 0; r0 < n && e == cudaSuccess; r0 += m) {
     bp.j0 = j0 + r0;
@@ -1233,7 +1236,7 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
       off[(size_t)r] = (long long)k;
       k += (size_t)len[r0 + r];
     }
-    e = cudaMemcpyAsync(buf, off.data(), off.size() * 8, cudaMemcpyHostToDevice, net->stream);
+    e = cudaMemcpyAsync(buf + 8, off.data(), off.size() * 8, cudaMemcpyHostToDevice, net->stream);
     if (e == cudaSuccess)
       e = launch_read_rows(bp, net->precision, net->connectivity == SNN_CONN_PAPER, net->stream);
     if (e == cudaSuccess && k > 0) {
@@ -1246,8 +1249,11 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
     if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
     at += k;
   }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, bp.rd_bad, 4, cudaMemcpyDeviceToHost, net->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
   if (!staged) cudaFree(buf);
   if (e != cudaSuccess) return cuda_fail(net, e, "synapse readback");
+  if (bad) return fail(net, SNN_ESTATE, "a row of the table does not hold the synapses drawn for it");
   return SNN_OK;
 }
 
@@ -1292,6 +1298,26 @@ int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t 
   SNN_CUDA(net, cudaMemcpy(&word, net->gsum, 4, cudaMemcpyDeviceToHost));
   word += (unsigned)delta;
   SNN_CUDA(net, cudaMemcpy(net->gsum, &word, 4, cudaMemcpyHostToDevice));
+  return SNN_OK;
+}
+
+int snn_debug_flip_byte(snn_net* net, int64_t neuron, int64_t byte, int32_t mask, int32_t in_table) {
+  if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
+  const int64_t row_bytes = in_table ? (int64_t)net->rowcap * net->rec_size : (int64_t)net->planes * 16;
+  if (neuron < 0 || neuron >= net->N || byte < 0 || byte >= row_bytes)
+    return fail(net, SNN_EINVAL, "neuron or byte out of range");
+  int rc = sync(net);
+  if (rc) return rc;
+  const int64_t col = neuron / net->npc;
+  const uint32_t ct = net->h_ctile[(size_t)col];
+  uint2 ti;
+  SNN_CUDA(net, cudaMemcpy(&ti, net->tinfo + (ct >> 6), sizeof(ti), cudaMemcpyDeviceToHost));
+  const int64_t row = (int64_t)(ti.x + (ct & 63u)) * net->npc + neuron % net->npc;
+  uint8_t* const at = (in_table ? static_cast<uint8_t*>(net->syn) : net->bend) + row * row_bytes + byte;
+  uint8_t v = 0;
+  SNN_CUDA(net, cudaMemcpy(&v, at, 1, cudaMemcpyDeviceToHost));
+  v = (uint8_t)(v ^ (uint8_t)mask);
+  SNN_CUDA(net, cudaMemcpy(at, &v, 1, cudaMemcpyHostToDevice));
   return SNN_OK;
 }
 

@@ -15,7 +15,8 @@
 // fill pass regenerates them and stores each into its part in k order (warp match
 // + popc rank), then the parts' tails are padded.  Rows are stored, and walked, in
 // virtual column order.  The same walk reads rows back in the order in which they
-// were drawn.
+// were drawn, and checks that the stored ends, records and padding are where the
+// draws say.
 // A shard (see ShardGeo) draws every synapse with the neuron's global index
 // and keeps only those whose target column is one of its own (local and
 // global stencil arithmetic agree for such targets: the halo is as wide as
@@ -152,8 +153,15 @@ __device__ __forceinline__ unsigned open_parts(const BuildParams& P, RowSmem& S,
   const unsigned excl = incl - ui - uo;
   S.cur[w][2 * lane] = excl * unit;
   S.cur[w][2 * lane + 1] = (excl + ui) * unit;
+  const uint32_t row = (uint32_t)((r.cy - r.y0) * r.tw + (r.cx - r.x0)) * (uint32_t)P.npc + (uint32_t)r.lj;
   if (MODE == kModeRead) {
     S.rd[w][lane] = icnt - ci - co;
+    // the stored descriptor says the same
+    const uint8_t* d = P.bend + r.at * P.planes * 16;
+    bool bad = lane < P.ndel && *reinterpret_cast<const uint16_t*>(d + desc_end(lane)) != (excl + ui | incl << 8);
+    if (lane < P.ndel && lane % kPlaneBuckets == 0)
+      bad = bad || *reinterpret_cast<const uint32_t*>(d + desc_start(lane) - 2) != (row | excl << 16);
+    if (bad) atomicOr(P.rd_bad, 1u);
   } else if (MODE == kModeOrder) {
     const DrawBucket d = draw_bucket(P, ci, co);
     S.rd[w][lane] = 8u * d.first;
@@ -165,10 +173,8 @@ __device__ __forceinline__ unsigned open_parts(const BuildParams& P, RowSmem& S,
     if (lane < P.planes * kPlaneBuckets)
       *reinterpret_cast<uint16_t*>(d + desc_end(lane)) =
           (uint16_t)(min(excl + ui, 255u) | min(incl, 255u) << 8);
-    if (lane < P.planes * kPlaneBuckets && lane % kPlaneBuckets == 0) {
-      const uint32_t row = (uint32_t)((r.cy - r.y0) * r.tw + (r.cx - r.x0)) * (uint32_t)P.npc + (uint32_t)r.lj;
+    if (lane < P.planes * kPlaneBuckets && lane % kPlaneBuckets == 0)
       *reinterpret_cast<uint32_t*>(d + desc_start(lane) - 2) = row | min(excl, 255u) << 16;
-    }
   }
   __syncwarp();
   return __shfl_sync(0xFFFFFFFFu, incl, 31);
@@ -183,6 +189,29 @@ __device__ __forceinline__ void stored_parts(const BuildParams& P, RowSmem& S, c
     S.cur[w][2 * lane] = (unsigned)d[at] * (unsigned)P.unit;
     S.cur[w][2 * lane + 1] = (unsigned)d[desc_end(lane)] * (unsigned)P.unit;
   }
+  __syncwarp();
+}
+
+// Whether a stored record is padding.
+template <int PREC>
+__device__ __forceinline__ bool is_pad(const BuildParams& P, size_t s, bool out) {
+  if (PREC != SNN_EXACT_F16W) return static_cast<const uint2*>(P.syn)[s].x & kPad;
+  const uint32_t rec = static_cast<const uint32_t*>(P.syn)[s];
+  return out ? (rec & 0x3800u) == kPadF16 : (rec >> 16 & 0x7FFFu) == kPadHalf;
+}
+
+// Readback: the slots behind a part's last synapse must be padding.
+template <int PREC>
+__device__ __forceinline__ void check_pads(const BuildParams& P, RowSmem& S, const Row& r) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned unit = (unsigned)P.unit;
+  bool bad = false;
+  for (int part = 0; lane < P.ndel && part < 2; ++part) {
+    const unsigned at = S.cur[w][2 * lane + part];
+    const unsigned end = (at + unit - 1u) / unit * unit;
+    for (unsigned s = at; s < end; ++s) bad = bad || !is_pad<PREC>(P, r.at * (size_t)P.rowcap + s, part == 1);
+  }
+  if (bad) atomicOr(P.rd_bad, 1u);
   __syncwarp();
 }
 
@@ -223,6 +252,7 @@ __device__ __forceinline__ void place(const BuildParams& P, RowSmem& S, const Ro
     } else {
       uint32_t code;
       int32_t wfx;
+      if (is_pad<PREC>(P, s, out)) atomicOr(P.rd_bad, 1u);
       if (PREC == SNN_EXACT_F16W) {
         const uint32_t rec = static_cast<const uint32_t*>(P.syn)[s];
         code = out ? rec & 0x1FFFFu : rec & 0xFFFFu;
@@ -399,6 +429,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const Buil
       place<PREC, MODE>(P, S, r, bb, m, l, MODE == kModeFill ? wt[x.w >> 16] : 0u, out0);
     }
     if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
+    if (MODE == kModeRead) check_pads<PREC>(P, S, r);
     if (MODE == kModeOrder) write_order(P, S, r);
   }
 }
@@ -537,6 +568,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
     }
     if (MODE != kModeCount) walk(true);
     if (MODE == kModeFill) pad_parts<PREC>(P, S, r);
+    if (MODE == kModeRead) check_pads<PREC>(P, S, r);
     if (MODE == kModeOrder) write_order(P, S, r);
   }
 }

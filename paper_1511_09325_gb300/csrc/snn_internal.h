@@ -288,6 +288,7 @@ struct BuildParams {
   long long* rd_target;
   int32_t* rd_delay;
   int32_t* rd_wfx;
+  unsigned* rd_bad;       // set if a row does not hold what its draws say
   // draw order of the rows (the differentiable form's sums; see snn_grad.cu):
   // a word per 8 places of a row, and the ends of its buckets in such units
   uint32_t* ord;          // [ncol * npc][ord_units], rows in the order of syn

@@ -22,7 +22,7 @@ PRECISIONS = {"f32w": SNN_EXACT_F32W, "f16w": SNN_EXACT_F16W}
 EXPORTS = ("snn_build", "snn_step", "snn_read_spikes", "snn_pending_spikes",
            "snn_set_record_capacity", "snn_read_rates", "snn_stats", "snn_get_state",
            "snn_read_synapses", "snn_row_lengths", "snn_info", "snn_step_profiled", "snn_update_noalloc",
-           "snn_debug_offset_count",
+           "snn_debug_offset_count", "snn_debug_flip_byte",
            "snn_build_shard", "snn_shard_update", "snn_shard_deliver", "snn_shard_info",
            "snn_shard_geometry",
            "snn_batch_build", "snn_batch_step", "snn_batch_net", "snn_batch_tune",
@@ -90,6 +90,7 @@ def load(path=LIB_PATH):
     L.snn_info.argtypes = [vp, vp, i32]
     L.snn_step_profiled.argtypes = [vp, i64, vp, vp]
     L.snn_debug_offset_count.argtypes = [vp, i64, ctypes.c_int32, ctypes.c_int32]
+    L.snn_debug_flip_byte.argtypes = [vp, i64, i64, ctypes.c_int32, ctypes.c_int32]
     L.snn_update_noalloc.argtypes = [i32, i32, P(NeuronParams), ctypes.c_uint64, i64,
                                      vp, vp, vp, vp, vp, P(i64), P(i64), vp, vp]
     L.snn_batch_build.argtypes = [i32, vp, vp, vp, vp, vp, i32, vp, P(vp)]
@@ -330,6 +331,11 @@ def snn_debug_offset_count(handle, column, delta, group_only=False):
     """Testing aid: offset one column's delivery item count (see snn.h)."""
     _check(load().snn_debug_offset_count(handle, int(column), int(delta), 1 if group_only else 0),
            handle)
+
+
+def snn_debug_flip_byte(handle, neuron, byte, mask, in_table=False):
+    """Testing aid: xor a byte of a neuron's table row or descriptor (see snn.h)."""
+    _check(load().snn_debug_flip_byte(handle, int(neuron), int(byte), int(mask), 1 if in_table else 0), handle)
 
 
 def snn_step_profiled(handle, n_steps):
