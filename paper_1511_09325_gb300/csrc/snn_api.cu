@@ -47,7 +47,6 @@ struct snn_net {
   uint32_t* colv = nullptr;
   uint2* tinfo = nullptr;
   uint32_t* nbg = nullptr;
-  std::vector<uint32_t> h_ctile;
   unsigned* icnt = nullptr;
   BuildParams bp{};                       // the construction's draws, for readback
   unsigned* hstatus = nullptr;            // status word (pinned, mapped)
@@ -265,45 +264,6 @@ void choose_tiles(snn_net* net) {
   net->ntile = ((net->W + net->tw - 1) / net->tw) * ((net->H + net->th - 1) / net->th);
 }
 
-// Geometry tables (see snn_internal.h): the tile, place and virtual index of
-// every column, every tile's first virtual column and columns, and the first
-// word in acc of the column at each stencil offset of each virtual column.
-struct Geometry {
-  std::vector<uint32_t> ctile, colv, nbg;
-  std::vector<uint2> tinfo;
-};
-
-void geometry_tables(const snn_net* net, Geometry* g) {
-  const int W = net->W, H = net->H;
-  g->ctile.assign((size_t)net->ncol, 0u);
-  g->colv.assign((size_t)net->ncol, 0u);
-  g->nbg.assign((size_t)net->ncol * 64, 0u);
-  uint32_t v = 0u;
-  for (int y0 = 0; y0 < H; y0 += net->th)
-    for (int x0 = 0; x0 < W; x0 += net->tw) {
-      const int w = std::min(net->tw, W - x0), h = std::min(net->th, H - y0);
-      uint2 ti;
-      ti.x = v;
-      ti.y = (unsigned)(w * h);
-      for (int y = y0; y < y0 + h; ++y)
-        for (int x = x0; x < x0 + w; ++x, ++v) {
-          const size_t c = (size_t)y * W + x;
-          g->ctile[c] = (uint32_t)g->tinfo.size() << 6 | (v - ti.x);
-          g->colv[c] = v;
-        }
-      g->tinfo.push_back(ti);
-    }
-  for (int y = 0; y < H; ++y)
-    for (int x = 0; x < W; ++x) {
-      uint32_t* row = g->nbg.data() + (size_t)g->colv[(size_t)y * W + x] * 64;
-      for (int dy = -3; dy <= 3; ++dy)
-        for (int dx = -3; dx <= 3; ++dx) {
-          const int tx = ((x + dx) % W + W) % W, ty = ((y + dy) % H + H) % H;
-          row[(dy + 3) << 3 | (dx + 3)] = g->colv[(size_t)ty * W + tx] * (uint32_t)net->npc4;
-        }
-    }
-}
-
 // Slots of a bucket unit and of a row for rows of at most K synapses in
 // `parts` bucket parts: units of 8 slots, or of 16 where a row could exceed
 // the 255 units that its bucket ends count.
@@ -509,20 +469,12 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   bp.th = net->th;
   bp.unit = net->unit;
   bp.planes = net->planes;
-  Geometry geo;
-  geometry_tables(net, &geo);
-  net->h_ctile = geo.ctile;
-  auto upload = [&](auto** dst, const auto& src) -> int {
-    const size_t bytes = src.size() * sizeof(src[0]);
-    if (int arc = dalloc(net, dst, bytes)) return arc;
-    SNN_CUDA(net, cudaMemcpyAsync(*dst, src.data(), bytes, cudaMemcpyHostToDevice, net->stream));
-    return SNN_OK;
-  };
-  if ((rc = upload(&net->ctile, geo.ctile))) return rc;
-  if ((rc = upload(&net->colv, geo.colv))) return rc;
-  if ((rc = upload(&net->tinfo, geo.tinfo))) return rc;
-  if ((rc = upload(&net->nbg, geo.nbg))) return rc;
-  SNN_CUDA(net, cudaStreamSynchronize(net->stream));
+  if ((rc = dalloc(net, &net->ctile, (size_t)net->ncol * 4))) return rc;
+  if ((rc = dalloc(net, &net->colv, (size_t)net->ncol * 4))) return rc;
+  if ((rc = dalloc(net, &net->tinfo, (size_t)net->ntile * sizeof(uint2)))) return rc;
+  if ((rc = dalloc(net, &net->nbg, (size_t)net->ncol * 64 * 4))) return rc;
+  SNN_CUDA(net, launch_geometry(gw, gh, net->tw, net->th, net->npc4, net->ctile, net->colv, net->tinfo, net->nbg,
+                                net->stream));
   bp.colv = net->colv;
   if ((rc = dalloc(net, &net->bend, (size_t)net->N * net->planes * 16))) return rc;
   net->total_syn = net->N * (long long)net->K;
@@ -1283,12 +1235,16 @@ const char* snn_last_error(const snn_net* net) {
   return net ? net->err.c_str() : g_err.c_str();
 }
 
+static TilePlace place_of(const snn_net* net, int64_t column) {
+  return tile_place(net->W, net->H, net->tw, net->th, (int)(column % net->W), (int)(column / net->W));
+}
+
 int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t group_only) {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
   if (column < 0 || column >= net->ncol) return fail(net, SNN_EINVAL, "column out of range");
   int rc = sync(net);
   if (rc) return rc;
-  unsigned* const tile = net->isum + (size_t)(net->h_ctile[(size_t)column] >> 6) * kCntStride;
+  unsigned* const tile = net->isum + (size_t)place_of(net, column).tile * kCntStride;
   unsigned word = 0u;
   if (!group_only) {
     SNN_CUDA(net, cudaMemcpy(&word, tile, 4, cudaMemcpyDeviceToHost));
@@ -1308,11 +1264,7 @@ int snn_debug_flip_byte(snn_net* net, int64_t neuron, int64_t byte, int32_t mask
     return fail(net, SNN_EINVAL, "neuron or byte out of range");
   int rc = sync(net);
   if (rc) return rc;
-  const int64_t col = neuron / net->npc;
-  const uint32_t ct = net->h_ctile[(size_t)col];
-  uint2 ti;
-  SNN_CUDA(net, cudaMemcpy(&ti, net->tinfo + (ct >> 6), sizeof(ti), cudaMemcpyDeviceToHost));
-  const int64_t row = (int64_t)(ti.x + (ct & 63u)) * net->npc + neuron % net->npc;
+  const int64_t row = (int64_t)place_of(net, neuron / net->npc).v * net->npc + neuron % net->npc;
   uint8_t* const at = (in_table ? static_cast<uint8_t*>(net->syn) : net->bend) + row * row_bytes + byte;
   uint8_t v = 0;
   SNN_CUDA(net, cudaMemcpy(&v, at, 1, cudaMemcpyDeviceToHost));

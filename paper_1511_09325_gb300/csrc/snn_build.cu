@@ -573,7 +573,36 @@ __global__ void __launch_bounds__(kBuildWarps * 32) paper_rows_kernel(const Buil
   }
 }
 
+// Geometry tables, one thread per column and stencil offset (offset fields of 7
+// name no column).
+__global__ void __launch_bounds__(256) geometry_kernel(int W, int H, int tw, int th, int npc4, uint32_t* ctile,
+                                                       uint32_t* colv, uint2* tinfo, uint32_t* nbg) {
+  const long long n = (long long)W * H * 64;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int c = (int)(i >> 6), off = (int)(i & 63);
+    const int y = c / W, x = c - y * W;
+    const TilePlace p = tile_place(W, H, tw, th, x, y);
+    const int dx = (off & 7) - 3, dy = (off >> 3) - 3;
+    nbg[(size_t)p.v * 64 + off] =
+        dx > 3 || dy > 3 ? 0u
+                         : tile_place(W, H, tw, th, wrap(x + dx, W), wrap(y + dy, H)).v * (uint32_t)npc4;
+    if (off) continue;
+    ctile[c] = p.tile << 6 | p.k;
+    colv[c] = p.v;
+    if (p.k == 0u) tinfo[p.tile] = make_uint2(p.v, (unsigned)(p.w * p.h));
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_geometry(int W, int H, int tw, int th, int npc4, uint32_t* ctile, uint32_t* colv,
+                            uint2* tinfo, uint32_t* nbg, cudaStream_t st) {
+  const long long blocks = ((long long)W * H * 64 + 255) / 256;
+  geometry_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, st>>>(W, H, tw, th, npc4, ctile, colv,
+                                                                               tinfo, nbg);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_build_count(const BuildParams& bp, int num_sms, cudaStream_t st) {
   build_rows_kernel<SNN_EXACT_F32W, kModeCount><<<num_sms * 8, kBuildWarps * 32, 0, st>>>(bp);

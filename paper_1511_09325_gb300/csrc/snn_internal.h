@@ -182,6 +182,24 @@ __host__ __device__ inline bool shard_owns_global(const ShardGeo& g, int W, int 
   return lx < W && ly < H && lx >= g.tx0 && lx < g.tx0 + g.tw && ly >= g.ty0 && ly < g.ty0 + g.th;
 }
 
+// The delivery tile of column (x, y) of a W x H grid, its place in the tile and
+// its virtual index: tiles of tw x th columns (narrower at the right and lower
+// edges), row by row.
+struct TilePlace {
+  uint32_t tile, k, v;
+  int w, h;  // the tile's size
+};
+__host__ __device__ inline TilePlace tile_place(int W, int H, int tw, int th, int x, int y) {
+  const int tx = x / tw, ty = y / th, x0 = tx * tw, y0 = ty * th;
+  TilePlace p;
+  p.w = W - x0 < tw ? W - x0 : tw;
+  p.h = H - y0 < th ? H - y0 : th;
+  p.tile = (uint32_t)ty * (uint32_t)((W + tw - 1) / tw) + (uint32_t)tx;
+  p.k = (uint32_t)((y - y0) * p.w + x - x0);
+  p.v = (uint32_t)y0 * (uint32_t)W + (uint32_t)(x0 * p.h) + p.k;
+  return p;
+}
+
 // Everything a step kernel needs, passed by value (constant bank).
 struct StepParams {
   long long N;
@@ -342,6 +360,11 @@ int fail_global(int code, const std::string& msg);
 int validate_neuron_params(const snn_neuron_params* n, std::string* why);
 
 // Kernel launchers (snn_build.cu / snn_step.cu).
+// Geometry tables (see above): the tile, place and virtual index of every column,
+// every tile's first virtual column and columns, and the first word in acc of the
+// column at each stencil offset of each virtual column.
+cudaError_t launch_geometry(int W, int H, int tw, int th, int npc4, uint32_t* ctile, uint32_t* colv,
+                            uint2* tinfo, uint32_t* nbg, cudaStream_t st);
 // Fixed law: the count pass writes bend, deg (shards) and max_units[0]; the fill
 // pass (same draws) writes the rows.
 cudaError_t launch_build_count(const BuildParams& bp, int num_sms, cudaStream_t st);
