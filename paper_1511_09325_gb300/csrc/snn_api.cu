@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -715,7 +716,12 @@ int build_net(int grid_w, int grid_h, const snn_neuron_params* neuron,
     }
     net->own_stream = true;
   }
-  int rc = build_impl(net, grid_w, grid_h, neuron, synapse, seed, precision);
+  int rc = SNN_OK;
+  try {
+    rc = build_impl(net, grid_w, grid_h, neuron, synapse, seed, precision);
+  } catch (...) {
+    rc = fail(net, SNN_ENOMEM, kNoHostMemory);
+  }
   if (rc != SNN_OK) {
     const bool smaller = rc == SNN_ENOMEM && !net->lean;
     g_err = net->err;
@@ -896,18 +902,19 @@ int snn_step(snn_net* net, int64_t n_steps) {
   return SNN_OK;
 }
 
-int snn_step_profiled(snn_net* net, int64_t n_steps, double* ms, double* bytes) {
+int snn_step_profiled(snn_net* net, int64_t n_steps, double* ms, double* bytes) try {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
   if (net->in_batch) return fail(net, SNN_ESTATE, "net belongs to a batch: use snn_batch_step");
   if (net->sg.on)
     return fail(net, SNN_ESTATE, "a shard steps by snn_shard_update and snn_shard_deliver");
   if (n_steps < 0) return fail(net, SNN_EINVAL, "n_steps must be >= 0");
+  if (n_steps >= 1LL << 40) return fail(net, SNN_ENOMEM, kNoHostMemory);  // three events a step
   std::vector<cudaEvent_t> ev((size_t)n_steps * 3 + 1);
+  std::vector<unsigned long long> hspk((size_t)n_steps + 1, 0ull);
   unsigned long long* dspk = nullptr;  // spikes so far, after each step
   int rc = dalloc(net, &dspk, ((size_t)n_steps + 1) * 8);
   if (rc) return rc;
   net->device_bytes -= ((size_t)n_steps + 1) * 8;
-  std::vector<unsigned long long> hspk((size_t)n_steps + 1, 0ull);
   size_t made = 0;
   cudaError_t e = cudaSuccess;
   for (; made < ev.size() && e == cudaSuccess; ++made) e = cudaEventCreate(&ev[made]);
@@ -953,6 +960,7 @@ int snn_step_profiled(snn_net* net, int64_t n_steps, double* ms, double* bytes) 
   }
   return rc;
 }
+SNN_CATCH(fail(net, SNN_ENOMEM, kNoHostMemory))
 
 namespace {
 
@@ -975,7 +983,7 @@ int snn_pending_spikes(snn_net* net, int64_t* n_out) {
   return SNN_OK;
 }
 
-int snn_read_spikes(snn_net* net, int32_t* steps, int32_t* ids, int64_t cap, int64_t* n_out) {
+int snn_read_spikes(snn_net* net, int32_t* steps, int32_t* ids, int64_t cap, int64_t* n_out) try {
   if (!net || !n_out || cap < 0 || (cap > 0 && (!steps || !ids)))
     return fail(net, SNN_EINVAL, "bad argument");
   *n_out = 0;
@@ -1034,6 +1042,7 @@ int snn_read_spikes(snn_net* net, int32_t* steps, int32_t* ids, int64_t cap, int
   if (lost) return fail(net, SNN_EOVERFLOW, "spike records dropped (buffer or cap too small)");
   return SNN_OK;
 }
+SNN_CATCH(fail(net, SNN_ENOMEM, kNoHostMemory))
 
 int snn_set_record_capacity(snn_net* net, int64_t capacity) {
   if (!net || capacity < 1) return fail(net, SNN_EINVAL, "bad argument");
@@ -1066,7 +1075,7 @@ int snn_set_record_capacity(snn_net* net, int64_t capacity) {
   return reset_records(net);
 }
 
-int snn_read_rates(snn_net* net, float* hz, int64_t n, float* pop_hz) {
+int snn_read_rates(snn_net* net, float* hz, int64_t n, float* pop_hz) try {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
   if (hz && n < 2 * net->ncol) return fail(net, SNN_EINVAL, "hz array too small");
   cudaError_t e;
@@ -1099,8 +1108,9 @@ int snn_read_rates(snn_net* net, float* hz, int64_t n, float* pop_hz) {
   }
   return SNN_OK;
 }
+SNN_CATCH(fail(net, SNN_ENOMEM, kNoHostMemory))
 
-int snn_stats(snn_net* net, double* recurrent_events, double* external_events, int64_t* steps) {
+int snn_stats(snn_net* net, double* recurrent_events, double* external_events, int64_t* steps) try {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
   cudaError_t e;
   Ctl c = read_ctl(net, &e);
@@ -1123,6 +1133,7 @@ int snn_stats(snn_net* net, double* recurrent_events, double* external_events, i
   if (steps) *steps = (int64_t)c.t;
   return SNN_OK;
 }
+SNN_CATCH(fail(net, SNN_ENOMEM, kNoHostMemory))
 
 int snn_get_state(snn_net* net, float* v, float* c, uint8_t* refractory) {
   if (!net) return fail(nullptr, SNN_EINVAL, "net is NULL");
@@ -1135,7 +1146,7 @@ int snn_get_state(snn_net* net, float* v, float* c, uint8_t* refractory) {
 }
 
 int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int32_t* delay,
-                      int32_t* wfx) {
+                      int32_t* wfx) try {
   if (!net || j0 < 0 || n < 0 || j0 + n > net->N || (n > 0 && (!target || !delay || !wfx)))
     return fail(net, SNN_EINVAL, "bad argument");
   if (n == 0) return SNN_OK;
@@ -1153,6 +1164,7 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   const int64_t m = std::min(n, staged ? std::min(in_stage, kRows) : kRows);
   size_t most = 0;
   std::vector<long long> off;
+  off.reserve((size_t)m);
   for (int64_t r0 = 0; r0 < n; r0 += m) {
     size_t k = 0;
     for (int64_t r = r0; r < std::min(n, r0 + m); ++r) k += (size_t)len[r];
@@ -1208,6 +1220,7 @@ int snn_read_synapses(snn_net* net, int64_t j0, int64_t n, int64_t* target, int3
   if (bad) return fail(net, SNN_ESTATE, "a row of the table does not hold the synapses drawn for it");
   return SNN_OK;
 }
+SNN_CATCH(fail(net, SNN_ENOMEM, kNoHostMemory))
 
 int snn_row_lengths(snn_net* net, int64_t j0, int64_t n, int32_t* counts) {
   if (!net || j0 < 0 || n < 0 || j0 + n > net->N || (n > 0 && !counts))
@@ -1410,7 +1423,7 @@ extern "C" {
 
 int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
                     const snn_neuron_params* neuron, const snn_synapse_params* synapse,
-                    const uint64_t* seeds, int precision, void* cuda_stream, snn_batch** out) {
+                    const uint64_t* seeds, int precision, void* cuda_stream, snn_batch** out) try {
   if (!out) return bfail(nullptr, SNN_EINVAL, "out is NULL");
   *out = nullptr;
   if (n_nets < 1 || n_nets > kMaxBatch) return bfail(nullptr, SNN_EINVAL, "n_nets must be in 1..256");
@@ -1421,21 +1434,26 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
     const int rc = validate(grid_w[k], grid_h[k], neuron + k, synapse + k, precision, &why);
     if (rc != SNN_OK) return bfail(nullptr, rc, "net " + std::to_string(k) + ": " + why);
   }
-  snn_batch* b = new (std::nothrow) snn_batch();
+  struct Release {
+    void operator()(snn_batch* b) const {
+      batch_release(b);
+      delete b;
+    }
+  };
+  std::unique_ptr<snn_batch, Release> b(new (std::nothrow) snn_batch());
   if (!b) return bfail(nullptr, SNN_ENOMEM, "host allocation failed");
   b->precision = precision;
   if (cuda_stream) {
     b->stream = static_cast<cudaStream_t>(cuda_stream);
   } else {
     cudaError_t e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-      delete b;
+    if (e != cudaSuccess)
       return bfail(nullptr, SNN_ECUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e));
-    }
     b->own_stream = true;
   }
   int rc = SNN_OK;
   b->first.assign(2 * (size_t)(n_nets + 1), 0);
+  b->nets.reserve((size_t)n_nets);
   bool lean = false;
   for (int k = 0; k < n_nets && rc == SNN_OK; ++k) {
     snn_net* net = nullptr;
@@ -1459,12 +1477,7 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
     b->first[k + 1] = b->first[k] + net->update_grid;
     b->first[(n_nets + 1) + k + 1] = b->first[(n_nets + 1) + k] + net->ntile;
   }
-  if (rc != SNN_OK) {
-    const std::string why = g_err;
-    batch_release(b);
-    delete b;
-    return bfail(nullptr, rc, why);
-  }
+  if (rc != SNN_OK) return rc;  // with the member's message
   cudaError_t e = cudaMalloc(&b->d_nets, sizeof(StepParams) * (size_t)n_nets);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_first, b->first.size() * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, (size_t)b->first.back() * sizeof(BatchTile));
@@ -1474,34 +1487,29 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
                         cudaMemcpyHostToDevice, b->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    batch_release(b);
-    delete b;
     return bfail(nullptr, e == cudaErrorMemoryAllocation ? SNN_ENOMEM : SNN_ECUDA,
                  std::string("batch buffers: ") + cudaGetErrorString(e));
   }
-  rc = batch_upload(b);
-  if (rc != SNN_OK) {
-    const std::string why = b->err;
-    batch_release(b);
-    delete b;
-    return bfail(nullptr, rc, why);
-  }
-  *out = b;
+  rc = batch_upload(b.get());
+  if (rc != SNN_OK) return bfail(nullptr, rc, b->err);
+  *out = b.release();
   return SNN_OK;
 }
+SNN_CATCH(bfail(nullptr, SNN_ENOMEM, kNoHostMemory))
 
-int snn_batch_step(snn_batch* b, int64_t n_steps) {
+int snn_batch_step(snn_batch* b, int64_t n_steps) try {
   if (!b) return bfail(nullptr, SNN_EINVAL, "batch is NULL");
   if (n_steps < 0) return bfail(b, SNN_EINVAL, "n_steps must be >= 0");
   return batch_run(b, n_steps);
 }
+SNN_CATCH(bfail(b, SNN_ENOMEM, kNoHostMemory))
 
 snn_net* snn_batch_net(snn_batch* b, int k) {
   if (!b || k < 0 || k >= (int)b->nets.size()) return nullptr;
   return b->nets[k];
 }
 
-int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) {
+int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) try {
   if (!b || steps_per_trial < 1) return bfail(b, SNN_EINVAL, "bad argument");
   // every variant computes the same sums, so the trials simply advance the
   // simulation; two interleaved rounds even out changes in activity.  Stage
@@ -1562,6 +1570,7 @@ int snn_batch_tune(snn_batch* b, int64_t steps_per_trial, int32_t* choice) {
   if (choice) *choice = b->choice;
   return SNN_OK;
 }
+SNN_CATCH(bfail(b, SNN_ENOMEM, kNoHostMemory))
 
 int snn_batch_set_wait(snn_batch* b, int64_t spin_limit, int32_t extra_arrivals) {
   if (!b || spin_limit < 1 || extra_arrivals < 0) return bfail(b, SNN_EINVAL, "bad argument");

@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -680,7 +681,7 @@ cudaError_t launch_forward_step(snn_grad* g, long long t, int slot, int rates) {
 extern "C" {
 
 int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int32_t hard,
-                   float beta, const double* target_rates, snn_grad** out) {
+                   float beta, const double* target_rates, snn_grad** out) try {
   if (!out) return fail_global(SNN_EINVAL, "out is NULL");
   *out = nullptr;
   NetView v{};
@@ -693,8 +694,16 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   if (!(beta > 0.f) || !std::isfinite(beta)) return fail_global(SNN_EINVAL, "beta must be > 0");
   if (v.neuron.tau_c == v.neuron.tau_m)
     return fail_global(SNN_EINVAL, "tau_c must differ from tau_m");
-  snn_grad* g = new (std::nothrow) snn_grad();
+  struct Release {
+    void operator()(snn_grad* g) const {
+      grad_release(g);
+      delete g;
+    }
+  };
+  std::unique_ptr<snn_grad, Release> own(new (std::nothrow) snn_grad());
+  snn_grad* const g = own.get();
   if (!g) return fail_global(SNN_ENOMEM, "host allocation failed");
+  g->bufs.reserve(32);
   g->v = v;
   g->T = n_steps;
   g->ckpt = (int)std::min<long long>(checkpoint_every, n_steps);
@@ -711,10 +720,8 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   g->wblocks = (int)((N * 32 + kThreads - 1) / kThreads);
   for (int rows : {5, 7, kGatherRows})
     if (cudaFuncSetAttribute(gather_tile_fn(rows * kGatherWarps), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmemBudget) != cudaSuccess) {
-      delete g;
+                             (int)kSmemBudget) != cudaSuccess)
       return fail_global(SNN_ECUDA, "the gather kernel does not fit on the device");
-    }
   // propagators in FP64 as the spiking tables compute them (h = 1 ms)
   const double tm = v.neuron.tau_m, tc = v.neuron.tau_c;
   g->pvv = std::exp(-1.0 / tm);
@@ -779,12 +786,7 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
   P.ord_units = v.ord_units;
   if (!rc && map) rc = galloc(g, &P.ord, n * v.ord_units);
   if (!rc && map) rc = galloc(g, &P.ord_end, n * v.ndel);
-  if (rc) {
-    const std::string why = g->err;
-    grad_release(g);
-    delete g;
-    return fail_global(rc, why);
-  }
+  if (rc) return fail_global(rc, g->err);
   P.q = g->q;
   const std::vector<double>& qd = quantile_table();
   std::vector<float> qf(qd.size());
@@ -802,16 +804,14 @@ int snn_grad_build(snn_net* net, int64_t n_steps, int32_t checkpoint_every, int3
     e = launch_draw_order(bp, v.paper, v.num_sms, v.stream);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(v.stream);
-  if (e != cudaSuccess) {
-    grad_release(g);
-    delete g;
+  if (e != cudaSuccess)
     return fail_global(SNN_ECUDA, std::string("gradient tables: ") + cudaGetErrorString(e));
-  }
-  *out = g;
+  *out = own.release();
   return SNN_OK;
 }
+SNN_CATCH(fail_global(SNN_ENOMEM, kNoHostMemory))
 
-int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, double* grad) {
+int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, double* grad) try {
   if (!g || !theta || !loss) return gfail(g, SNN_EINVAL, "null argument");
   for (int k = 0; k < 6; ++k)
     if (!std::isfinite(theta[k])) return gfail(g, SNN_EINVAL, "parameters must be finite");
@@ -898,6 +898,7 @@ int snn_grad_run(snn_grad* g, const double* theta, double* loss, double* rates, 
   SNN_GCUDA(g, cudaStreamSynchronize(st));
   return SNN_OK;
 }
+SNN_CATCH(gfail(g, SNN_ENOMEM, kNoHostMemory))
 
 const char* snn_grad_last_error(const snn_grad* g) { return g ? g->err.c_str() : ""; }
 

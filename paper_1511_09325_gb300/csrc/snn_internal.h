@@ -357,6 +357,13 @@ inline void philox_keys(StepParams* p) {
 
 // Shared host helpers (snn_api.cu).
 int fail_global(int code, const std::string& msg);
+// End of the function-try block of a C entry: what a host allocation throws
+// becomes SNN_ENOMEM.  (The message fits a string without an allocation.)
+#define SNN_CATCH(fail_call) \
+  catch (...) {              \
+    return fail_call;        \
+  }
+constexpr const char* kNoHostMemory = "no host memory";
 int validate_neuron_params(const snn_neuron_params* n, std::string* why);
 
 // Kernel launchers (snn_build.cu / snn_step.cu).
