@@ -384,7 +384,7 @@ def _kernel_roofline(snn, torch, cfg, seed, stream, lead, P, workload, window):
                             "deliver": kbytes[1] / (kms[1] * 1e-3) / 1e9 / hbm},
             "algorithmic_bytes_per_launch": {"update": kbytes[0] / P, "deliver": kbytes[1] / P},
             "bytes_model": "update 26 B per neuron + 12 B per spike; deliver per spike k_out x "
-                           "record bytes (4 B FP16 record: 15-bit weight + 17-bit target; 8 B "
+                           "record bytes (4 B FP16 record: weight and target in one word; 8 B "
                            "FP32 record) + 6 B per delay bucket (descriptor id and bucket end)"}
 
 

@@ -116,6 +116,10 @@ enum {
  * On success *out receives the net (destroy with snn_destroy).  Returns
  * SNN_EINVAL for parameters outside the stated ranges, SNN_ENOMEM when the
  * synapse table does not fit, SNN_ECUDA on a CUDA error.
+ * A net keeps its last spikes in lists of about 1300 bytes per neuron (delays of
+ * 1..20 ms), or of 42 bytes, which are slower to deliver from (7 to 10 %): the
+ * larger ones only where a second net of the same size still fits the device if
+ * it would without them, and half as much in any case.
  */
 int snn_build(int grid_w, int grid_h, const snn_neuron_params* neuron,
               const snn_synapse_params* synapse, uint64_t seed, int precision,
@@ -193,10 +197,10 @@ int snn_row_lengths(snn_net* net, int64_t j0, int64_t n, int32_t* counts);
  * delta to the number of delivery items the library has counted for the group
  * of columns (delivery tile) that holds `column` (0 <= column < grid_w *
  * grid_h) and to the count of all groups, or to the latter only when
- * group_only is nonzero, as a bookkeeping fault would.  The spike lists are left as they are, so the next
- * delivery finds counts that disagree with them and must set the net's status
- * word (see snn_step).  Synchronises the net's stream.  SNN_EINVAL for a
- * column out of range.
+ * group_only is nonzero, as a bookkeeping fault would.  The spike lists are
+ * left as they are, so the next delivery finds counts that disagree with them
+ * and must set the net's status word (see snn_step).  Synchronises the net's
+ * stream.  SNN_EINVAL for a column out of range.
  */
 int snn_debug_offset_count(snn_net* net, int64_t column, int32_t delta, int32_t group_only);
 

@@ -65,7 +65,6 @@ struct snn_net {
   long long rec_region = 0;  // records per update block
   unsigned long long* rcnt = nullptr;
   unsigned long long* stage = nullptr;   // large drains on the device: ids then steps (u32)
-  unsigned long long* dhdr = nullptr;    // drain header (device, 4 words)
   unsigned long long* hhdr = nullptr;    // drain header (pinned, mapped)
   unsigned long long* hhdr_dev = nullptr;
   uint32_t* hmap = nullptr;              // small drains: ids then steps (pinned, mapped)
@@ -181,7 +180,7 @@ void release(snn_net* net) {
     if (ev) cudaEventDestroy(ev);
   void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->rlist, net->ctile,
                   net->colv, net->tinfo, net->nbg, net->icnt, net->ccnt, net->deg, net->syn_part,
-                  net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage, net->dhdr,
+                  net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage,
                   net->colcnt, net->ext_part, net->spk_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -228,21 +227,20 @@ int validate(int gw, int gh, const snn_neuron_params* n, const snn_synapse_param
   return SNN_OK;
 }
 
-// Delivery tiles: the largest square tile (side <= kMaxTile) whose window,
-// neighbour table and the warps' sector lists fit the shared memory of a
-// delivery block -- one block per SM for a net of its own, two per SM in the
-// batch kernel -- then evened out over the grid's sides (24 columns make four
-// tiles of 6, 8 make two of 4).  Measured at 96x96 (FP16, Down, middle and Up
-// states): a 6x6 tile without ring (80 % of the synapses land in the window,
-// each column is flushed once per part) beats a 4x4 tile with a ring of one
-// (88 %, but 36 window columns flushed per 16 columns of spikes) by 13 %, 17 %
-// and 3 %; 5x5 and 4x4 tiles without ring and 3x3 with a ring are slower still.
 // Fewest items a delivery block takes (fewer blocks run when a step has few
 // items).  Measured (us per delivery, mean state) with 128, 64, 32 and 16: 2x2
 // FP32 12.1, 11.2, 10.8, 10.6; 8x8 FP16 18.4, 16.8, 15.2, 15.1.
 constexpr unsigned kMinItems = 16;
 constexpr unsigned kBatchMinItems = 256;
 
+// Delivery tiles: the largest square tile (side <= kMaxTile) whose window,
+// neighbour table and the warps' sector lists fit the shared memory of a
+// delivery block -- one block per SM for a net of its own, two per SM in the
+// batch kernel -- then evened out over the grid's sides (24 columns make four
+// tiles of 6, 8 make two of 4).  The largest tile keeps most synapses in the
+// window (6x6: 80 %).  Measured at 96x96 (FP16, us per delivery in Down and Up
+// states): 6x6 tiles 101 and 746; 5x5 187 and 792; 4x4 with a window of the 20
+// most-hit columns around each 168 and 701.
 void choose_tiles(snn_net* net) {
   net->npc4 = (net->npc + 3) / 4 * 4;
   const size_t budget = net->batch_member ? kBatchSmemBudget : kSmemBudget;
@@ -554,7 +552,6 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->rec, rec_bytes))) return rc;
   if ((rc = dalloc(net, &net->rcnt, (size_t)net->update_grid * 8))) return rc;
   if ((rc = dalloc(net, &net->stage, rec_bytes))) return rc;
-  if ((rc = dalloc(net, &net->dhdr, 32))) return rc;
   SNN_CUDA(net, cudaHostAlloc(&net->hstatus, 16, cudaHostAllocMapped));
   SNN_CUDA(net, cudaHostGetDevicePointer(&net->hstatus_dev, net->hstatus, 0));
   *net->hstatus = 0u;
@@ -684,10 +681,6 @@ int net_view(snn_net* net, NetView* v) {
 }
 
 }  // namespace snn
-
-extern "C" {
-
-}  // extern "C"
 
 namespace {
 
@@ -993,7 +986,7 @@ int snn_read_spikes(snn_net* net, int32_t* steps, int32_t* ids, int64_t cap, int
   const long long stage_cap = net->rec_region * net->update_grid;
   uint32_t* stage_ids = reinterpret_cast<uint32_t*>(net->stage);
   SNN_CUDA(net, launch_drain_records(net->sp, net->update_grid, stage_ids, stage_ids + stage_cap,
-                                     net->dhdr, net->hhdr_dev, net->hmap_dev,
+                                     net->hhdr_dev, net->hmap_dev,
                                      net->hmap_dev + net->hmap_cap, net->hmap_cap, net->stream));
   SNN_CUDA(net, cudaStreamSynchronize(net->stream));
   if (int src = check_status(net)) return src;
@@ -1300,7 +1293,7 @@ void snn_destroy(snn_net* net) {
 // ---------------------------------------------------------------------------
 struct snn_batch {
   std::vector<snn_net*> nets;
-  int precision = 0, num_sms = 0, max_npc = 0;
+  int precision = 0, num_sms = 0;
   int infl = 4;            // 16-byte chunks in flight in the delivery loop
   int agg = 1;             // block windows for the local half of the synapses
   unsigned min_items = kBatchMinItems;  // fewest items a delivery block takes
@@ -1471,7 +1464,6 @@ int snn_batch_build(int n_nets, const int32_t* grid_w, const int32_t* grid_h,
     if (rc != SNN_OK) break;
     net->in_batch = true;
     b->nets.push_back(net);
-    b->max_npc = std::max(b->max_npc, net->npc);
     b->num_sms = net->num_sms;
     // update: the net's own grid (its partial sums and record regions)
     b->first[k + 1] = b->first[k] + net->update_grid;

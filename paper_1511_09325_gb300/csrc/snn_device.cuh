@@ -38,12 +38,6 @@ __device__ __forceinline__ uint32_t below(uint32_t x, uint32_t n) {
   return __umulhi(x, n);
 }
 
-__device__ __forceinline__ uint32_t lane_id() {
-  uint32_t l;
-  asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
-  return l;
-}
-
 // Periodic wrap of a coordinate that may lie several periods outside [0, n).
 __device__ __forceinline__ int wrap(int v, int n) {
   int r = v % n;

@@ -79,7 +79,6 @@ constexpr int kMaxOff = 48;      // remote stencil offsets (radius <= 3)
 constexpr uint32_t kPad = 0x80000000u;
 constexpr uint32_t kPadHalf = 1u;
 constexpr uint32_t kPadF16 = 7u << 11;
-constexpr int kCenterCode = (3 << 3) | 3;
 constexpr int kMaxGridSide = 16383;     // columns per grid side (14-bit coordinates)
 constexpr int kMaxTile = 8;             // delivery tile side, columns
 constexpr int kMaxTileCols = kMaxTile * kMaxTile;
@@ -97,11 +96,12 @@ constexpr size_t kWindowBudget = 196 * 1024;
 // flush); the fixed cost, in items, of a tile with fewer but some items.
 // Without a window each of an item's ~62 synapses is an L2 reduction (about
 // 1.3 per ns and SM), with one the window's words are cleared and added once
-// (about 7.5 words per ns and SM).  Measured (us per delivery, mean state): a
-// window from 1 item per 87, 175 and 350 words on gives 18.9, 18.2 and 18.1 at
-// 8x8 FP16, 45.1, 43.4 and 43.5 at 24x24 FP16, the same at 96x96; a cost of 1
-// item per 30, 44 and 88 words gives 44.4, 43.4 and 43.2 at 24x24 FP16, and
-// 368, 365 and 372 at 96x96.
+// (about 7.5 words per ns and SM).  Measured (us per delivery over 1000 steps from
+// step 600 on: 8x8 FP16, 24x24 FP16, 24x24 FP32, 96x96 FP16): a window from 1 item
+// per 87 words on 15.9, 37.5, 42.4, 417; 175: 15.4, 33.9, 39.8, 416; 250: 15.2,
+// 33.6, 39.5, 417; 350: 15.1, 33.6, 39.5, 417.  A cost of 1 item per 30 words 15.5,
+// 34.4, 40.5, 422; 44: 15.3, 33.8, 39.9, 417; 60: 15.2, 33.6, 39.5, 417; 88: 15.0,
+// 33.5, 39.2, 417.
 constexpr int kWinWordsPerItem = 250;
 constexpr int kCostWordsPerItem = 60;
 constexpr unsigned kCostPart = 32;
@@ -399,13 +399,11 @@ int deliver_grid(const StepParams& p, int precision, int num_sms);
 cudaError_t launch_deliver(const StepParams& p, int precision, int grid, bool overlap, cudaStream_t st);
 // Compact the per-block record regions into id and step arrays and reset
 // them; header = {records kept, 1 if records were dropped, first step, last
-// step}, written to header and to the mapped host header map_hdr.  The arrays
-// go to the mapped host buffers when they hold at most map_cap records, else
-// to the device stage.
+// step}, written to the mapped host header map_hdr.  The arrays go to the mapped
+// host buffers when they hold at most map_cap records, else to the device stage.
 constexpr long long kMappedRecords = 1LL << 18;  // mapped host records per net
 cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_ids,
-                                 uint32_t* stage_steps, unsigned long long* header,
-                                 unsigned long long* map_hdr, uint32_t* map_ids,
+                                 uint32_t* stage_steps, unsigned long long* map_hdr, uint32_t* map_ids,
                                  uint32_t* map_steps, long long map_cap, cudaStream_t st);
 // Counts the records a drain would return: {kept, 1 if records were dropped}
 // to the mapped host header.

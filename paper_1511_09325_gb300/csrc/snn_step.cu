@@ -1198,13 +1198,13 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchPara
 // and step arrays, starting at the number of records kept in the regions
 // before b, to the mapped host buffers when all kept records fit them
 // (map_cap) and to the device stage otherwise.  Block 0 writes the header
-// {records kept, 1 if any were dropped, first step, last step} to device and
-// mapped host memory (each region is in step order, so its first and last
+// {records kept, 1 if any were dropped, first step, last step} to mapped host
+// memory (each region is in step order, so its first and last
 // records bound its steps).  The last block to finish resets the region
 // counters and the overflow flag.
 __global__ void __launch_bounds__(256) drain_records_kernel(
     unsigned long long* rcnt, int nreg, long long region, const unsigned long long* rec,
-    Ctl* ctl, unsigned long long* header, unsigned long long* map_hdr, uint32_t* stage_ids,
+    Ctl* ctl, unsigned long long* map_hdr, uint32_t* stage_ids,
     uint32_t* stage_steps, uint32_t* map_ids, uint32_t* map_steps, long long map_cap) {
   __shared__ unsigned long long s_pre[8], s_tot[8];
   __shared__ unsigned s_tmin[8], s_tmax[8], s_lost[8];
@@ -1257,10 +1257,7 @@ __global__ void __launch_bounds__(256) drain_records_kernel(
   if (b == 0 && threadIdx.x == 0) {
     const unsigned long long h[4] = {tot, (lost || ctl->rec_overflow) ? 1ull : 0ull,
                                      (unsigned long long)tmin, (unsigned long long)tmax};
-    for (int k = 0; k < 4; ++k) {
-      header[k] = h[k];
-      map_hdr[k] = h[k];
-    }
+    for (int k = 0; k < 4; ++k) map_hdr[k] = h[k];
   }
   const bool to_map = (long long)tot <= map_cap;
   uint32_t* ids = (to_map ? map_ids : stage_ids) + pre;
@@ -1450,10 +1447,9 @@ cudaError_t launch_deliver(const StepParams& p, int precision, int grid, bool ov
 }
 
 cudaError_t launch_drain_records(const StepParams& p, int nreg, uint32_t* stage_ids,
-                                 uint32_t* stage_steps, unsigned long long* header,
-                                 unsigned long long* map_hdr, uint32_t* map_ids,
+                                 uint32_t* stage_steps, unsigned long long* map_hdr, uint32_t* map_ids,
                                  uint32_t* map_steps, long long map_cap, cudaStream_t st) {
-  drain_records_kernel<<<nreg, 256, 0, st>>>(p.rcnt, nreg, p.rec_region, p.rec, p.ctl, header,
+  drain_records_kernel<<<nreg, 256, 0, st>>>(p.rcnt, nreg, p.rec_region, p.rec, p.ctl,
                                              map_hdr, stage_ids, stage_steps, map_ids, map_steps,
                                              map_cap);
   return cudaGetLastError();
