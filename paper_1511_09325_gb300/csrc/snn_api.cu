@@ -59,6 +59,7 @@ struct snn_net {
   int connectivity = SNN_CONN_FIXED;
   unsigned* isum = nullptr;
   unsigned* gsum = nullptr;
+  unsigned* max_units = nullptr;           // the construction's longest row
   Ctl* ctl = nullptr;
   unsigned long long* rec = nullptr;
   long long rec_cap = 0;     // requested total record capacity
@@ -180,7 +181,7 @@ void release(snn_net* net) {
     if (ev) cudaEventDestroy(ev);
   void* ptrs[] = {net->syn, net->bend, net->V, net->C, net->R, net->acc, net->list, net->rlist, net->ctile,
                   net->colv, net->tinfo, net->nbg, net->icnt, net->ccnt, net->deg, net->syn_part,
-                  net->isum, net->gsum, net->ctl, net->rec, net->rcnt, net->stage,
+                  net->isum, net->gsum, net->max_units, net->ctl, net->rec, net->rcnt, net->stage,
                   net->colcnt, net->ext_part, net->spk_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -263,16 +264,23 @@ void choose_tiles(snn_net* net) {
   net->ntile = ((net->W + net->tw - 1) / net->tw) * ((net->H + net->th - 1) / net->th);
 }
 
-// Slots of a bucket unit and of a row for rows of at most K synapses in
-// `parts` bucket parts: units of 8 slots, or of 16 where a row could exceed
-// the 255 units that its bucket ends count.
+// Slots of a bucket unit and of a row for rows of at most K synapses: units of 8
+// slots, or of 16 where a row could exceed the 255 units that its bucket ends
+// count; a row's slots as estimated for the longest row of the fixed law -- a part's
+// padding is 0 .. unit - 1 slots, about equally often, so the sum over the parts
+// stays within six standard deviations of its mean in nets of any size that fits
+// (1240 synapses in 40 parts: 1472; the longest of 96x96 columns has 1448) unless
+// the parts are short; then the longest row is counted.
 void choose_unit(snn_net* net, int K) {
-  const int parts = 2 * net->ndel;
+  const int n = std::min(K, 2 * net->ndel);  // parts that hold a synapse
+  int most = 0;                              // slots of the longest row possible
   for (net->unit = kSlotUnit;; net->unit *= 2) {
-    const int n = std::min(K, parts);  // parts that hold a synapse
-    net->rowcap = (K + (net->unit - 1) * n + net->unit - 1) / net->unit * net->unit;
-    if (net->rowcap / net->unit <= 255 || net->unit == 2 * kSlotUnit) break;
+    most = (K + (net->unit - 1) * n + net->unit - 1) / net->unit * net->unit;
+    if (most / net->unit <= 255 || net->unit == 2 * kSlotUnit) break;
   }
+  const double u = net->unit;
+  const double slots = K + n * (u - 1.0) / 2.0 + 6.0 * std::sqrt(n * (u * u - 1.0) / 12.0);
+  net->rowcap = std::min(most, ((int)slots / net->unit + 1) * net->unit);
 }
 
 // A kernel found inconsistent counts: the net's stepping is no longer exact.
@@ -386,7 +394,7 @@ void fill_step_params(snn_net* net) {
 // device with `free` bytes, takes the descriptors: only where they leave room for a
 // second net of this size if there is room for two without them, and half as much
 // in any case (for a differentiable view, or the caller's own arrays).
-// Descriptors are about 1300 of an FP16 net's 7200 or an FP32 net's 13 100 bytes
+// Descriptors are about 1300 of an FP16 net's 7300 or an FP32 net's 13 200 bytes
 // per neuron; lists of rows cost time: 1000 steps of 96x96 FP16 451 instead of 408
 // ms, of 48x48 FP32 149 instead of 140 ms.
 bool roomy_lists(size_t free, size_t had, size_t small, size_t large) {
@@ -478,46 +486,47 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if ((rc = dalloc(net, &net->bend, (size_t)net->N * net->planes * 16))) return rc;
   net->total_syn = net->N * (long long)net->K;
   if (net->sg.on && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
-  // count pass: bucket ends, out-degrees and the longest row (max_units), which
-  // sets the row stride of the table
   const bool paper = net->connectivity == SNN_CONN_PAPER;
-  unsigned max_units[2] = {0u, 0u};
   if (paper && (rc = dalloc(net, &net->deg, (size_t)net->N * 4))) return rc;
-  if ((rc = dalloc(net, &bp.max_units, 8))) return rc;
-  net->device_bytes -= 8;
+  unsigned max_units[2] = {0u, 0u};
+  if ((rc = dalloc(net, &net->max_units, 8))) return rc;
+  bp.max_units = net->max_units;
   bp.bend = net->bend;
   bp.deg = net->deg;
-  cudaError_t ce = cudaSuccess;
-  if (paper) net->unit = kSlotUnit;  // 16 slots only where a row needs them
-  for (;; net->unit *= 2) {
-    bp.unit = net->unit;
-    ce = cudaMemsetAsync(bp.max_units, 0, 8, net->stream);
-    if (ce == cudaSuccess)
-      ce = paper ? launch_paper_count(bp, net->num_sms, net->stream) : launch_build_count(bp, net->num_sms, net->stream);
+  // runs a pass over the rows and reads max_units back
+  auto pass = [&](auto&& launch) -> cudaError_t {
+    cudaError_t ce = cudaMemsetAsync(bp.max_units, 0, 8, net->stream);
+    if (ce == cudaSuccess) ce = launch();
     if (ce == cudaSuccess)
       ce = cudaMemcpyAsync(max_units, bp.max_units, 8, cudaMemcpyDeviceToHost, net->stream);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(net->stream);
-    if (ce != cudaSuccess || max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
-  }
-  cudaFree(bp.max_units);
-  if (ce != cudaSuccess) return cuda_fail(net, ce, "connectivity count pass");
-  if (max_units[1] > 255u || max_units[0] > 255u)
-    return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
-  net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
-  if (paper) net->ord_units = (int)std::max(1u, max_units[1]);
-  if (net->deg) {
-    std::vector<uint32_t> deg((size_t)net->N);
-    SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
-                                  net->stream));
-    SNN_CUDA(net, cudaStreamSynchronize(net->stream));
-    net->total_syn = 0;
-    for (uint32_t d : deg) net->total_syn += d;
+    return ce == cudaSuccess ? cudaStreamSynchronize(net->stream) : ce;
+  };
+  // the longest row sets the row stride of the table
+  auto count_rows = [&]() -> int {
+    const cudaError_t ce = pass([&] {
+      return paper ? launch_paper_count(bp, net->num_sms, net->stream)
+                   : launch_build_count(bp, net->num_sms, net->stream);
+    });
+    if (ce != cudaSuccess) return cuda_fail(net, ce, "connectivity count pass");
+    net->rowcap = (int)std::max(1u, max_units[0]) * net->unit;
+    return SNN_OK;
+  };
+  if (paper) {
+    // bucket ends, out-degrees and the longest row; 16 slots only where a row needs them
+    for (net->unit = kSlotUnit;; net->unit *= 2) {
+      bp.unit = net->unit;
+      if ((rc = count_rows())) return rc;
+      if (max_units[0] <= 255u || net->unit == 2 * kSlotUnit) break;
+    }
+    if (max_units[1] > 255u || max_units[0] > 255u)
+      return fail(net, SNN_EINVAL, "a row of the paper law needs more than 2040 slots");
+    net->ord_units = (int)std::max(1u, max_units[1]);
   }
   // Spike lists: of descriptors (planes x 16 bytes per neuron and step) or, where
   // the device has little room, of rows (2 bytes).
   const size_t tcap = (size_t)net->tw * net->th * net->npc;
   const size_t list_len = (size_t)net->nslot * net->ntile * tcap;
-  const size_t syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
+  size_t syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
   const size_t acc_bytes = (size_t)net->ncol * net->npc4 * 4;
   const size_t ccnt_bytes = (size_t)net->nslot * net->ntile * kCntStride * 4;
   const size_t isum_bytes = (size_t)net->ntile * kCntStride * 4;
@@ -533,8 +542,15 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
                    syn_bytes + rest + list_len * net->planes * 16))
     net->lean = true;
   const bool rows = net->lean;
-  bp.rowcap = net->rowcap;
-  if ((rc = dalloc(net, &net->syn, syn_bytes))) return rc;
+  if (rows && !paper && (rc = count_rows())) return rc;
+  auto alloc_table = [&]() -> int {
+    bp.rowcap = net->rowcap;
+    syn_bytes = (size_t)net->N * net->rowcap * net->rec_size;
+    const int arc = dalloc(net, &net->syn, syn_bytes);
+    bp.syn = net->syn;
+    return arc;
+  };
+  if ((rc = alloc_table())) return rc;
   if ((rc = dalloc(net, &net->V, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->C, (size_t)net->Npad * 4))) return rc;
   if ((rc = dalloc(net, &net->R, (size_t)net->Npad))) return rc;
@@ -582,19 +598,38 @@ int build_impl(snn_net* net, int gw, int gh, const snn_neuron_params* np,
   if (e == cudaSuccess) e = cudaMemsetAsync(net->spk_part, 0, (size_t)net->update_grid * 8, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->syn_part, 0, (size_t)net->update_grid * 8, net->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(net->rcnt, 0, (size_t)net->update_grid * 8, net->stream);
-  if (e == cudaSuccess) {
-    bp.wtab = wtab;
-    bp.syn = net->syn;
-    e = net->connectivity == SNN_CONN_PAPER ? launch_paper_fill(bp, precision, net->num_sms, net->stream)
-                                            : launch_build(bp, precision, net->num_sms, net->stream);
+  bp.wtab = wtab;
+  auto fill = [&] {
+    return paper ? launch_paper_fill(bp, precision, net->num_sms, net->stream)
+                 : launch_build(bp, precision, net->num_sms, net->stream);
+  };
+  if (e == cudaSuccess) e = pass(fill);
+  if (e == cudaSuccess && !paper && max_units[0] > 0u) {
+    // a row is longer than estimated: the table again, by the rows' count
+    cudaFree(net->syn);
+    net->syn = nullptr;
+    net->device_bytes -= syn_bytes;
+    rc = count_rows();
+    if (!rc) rc = alloc_table();
+    if (!rc) e = pass(fill);
   }
+  cudaFree(wtab);
+  if (rc) return rc;
   fill_step_params(net);
   if (rows && deliver_grid(net->sp, precision, net->num_sms) < 1)
     return fail(net, SNN_ECUDA, "delivery kernel does not fit on the device");
   if (e == cudaSuccess) e = launch_init_state(net->sp, net->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
-  cudaFree(wtab);
   if (e != cudaSuccess) return cuda_fail(net, e, "network construction");
+  if (net->deg) {
+    // paper law: the rows' out-degrees; shard: the synapses into its own columns
+    std::vector<uint32_t> deg((size_t)net->N);
+    SNN_CUDA(net, cudaMemcpyAsync(deg.data(), net->deg, deg.size() * 4, cudaMemcpyDeviceToHost,
+                                  net->stream));
+    SNN_CUDA(net, cudaStreamSynchronize(net->stream));
+    net->total_syn = 0;
+    for (uint32_t d : deg) net->total_syn += d;
+  }
   return SNN_OK;
 }
 

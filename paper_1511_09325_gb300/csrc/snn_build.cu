@@ -10,11 +10,13 @@
 // A delay bucket has two parts (see snn_internal.h): the synapses that end in
 // the source's own delivery tile, stored as words of the tile's window, and
 // the others, stored as a stencil offset and an index.
-// One warp owns one row: a count pass counts the synapses of every bucket part
-// and writes the bucket ends and the longest row, which sets the rows' stride; a
-// fill pass regenerates them and stores each into its part in k order (warp match
-// + popc rank), then the parts' tails are padded.  Rows are stored, and walked, in
-// virtual column order.  The same walk reads rows back in the order in which they
+// One warp owns one row: a first pass counts the synapses of every bucket part, a
+// second pass regenerates them and stores each into its part in k order (warp
+// match + popc rank), then the parts' tails are padded.  Both run in one kernel,
+// where the counting hides behind the stores (96x96: 126 ms, 178 ms as two
+// kernels), with the rows' stride estimated; a row that is longer is reported and
+// left out, and the build counts all rows first then, as it does where memory is
+// short.  Rows are stored, and walked, in virtual column order.  The same walk reads rows back in the order in which they
 // were drawn, and checks that the stored ends, records and padding are where the
 // draws say.
 // A shard (see ShardGeo) draws every synapse with the neuron's global index
@@ -364,9 +366,10 @@ __device__ __forceinline__ void write_order(const BuildParams& P, RowSmem& S, co
   __syncwarp();
 }
 
-// Rows of the fixed law, one warp per row; MODE count writes their bucket ends
-// and the longest row, fill builds them, read writes rows j0 .. j0 + n_rows - 1 to
-// the rd_* arrays, order writes the rows' draw order.
+// Rows of the fixed law, one warp per row; MODE fill builds them (max_units[0]: the
+// longest row beyond the stride, else untouched), read writes rows j0 .. j0 +
+// n_rows - 1 to the rd_* arrays, count finds the longest, order writes the rows'
+// draw order.
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const BuildParams P) {
   __shared__ RowSmem S;
@@ -381,32 +384,28 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_rows_kernel(const Buil
     const uint32_t j = (uint32_t)(MODE == kModeRead ? P.j0 + i : i);
     const int c = (int)(j / (uint32_t)P.npc);
     const Row r = open_row<false>(P, S, c, (int)(j - (uint32_t)c * (uint32_t)P.npc));
-    if (MODE == kModeFill) {
-      stored_parts(P, S, r);
-    } else {
-      S.cnt[w][lane] = 0u;
-      S.cnt[w][lane + 32] = 0u;
-      __syncwarp();
-      // pass 1: synapses per bucket part
-      unsigned nkept = 0u;
-      for (int k = lane; k < P.K; k += 32) {
-        const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
-        const int cl = S.cls[w][k < P.k_local ? kMaxOff : offset_of(P, S, x.y)];
-        if (cl != kDropped) {
-          atomicAdd(&S.cnt[w][2 * below(x.z, ndel) + (cl == kOut ? 1 : 0)], 1u);
-          ++nkept;
-        }
+    S.cnt[w][lane] = 0u;
+    S.cnt[w][lane + 32] = 0u;
+    __syncwarp();
+    // pass 1: synapses per bucket part
+    unsigned nkept = 0u;
+    for (int k = lane; k < P.K; k += 32) {
+      const uint4 x = philox4x32_10(make_uint4(r.jj, (uint32_t)k, kTagConn, 0u), P.seed_lo, P.seed_hi);
+      const int cl = S.cls[w][k < P.k_local ? kMaxOff : offset_of(P, S, x.y)];
+      if (cl != kDropped) {
+        atomicAdd(&S.cnt[w][2 * below(x.z, ndel) + (cl == kOut ? 1 : 0)], 1u);
+        ++nkept;
       }
-      __syncwarp();
-      const unsigned units = open_parts<MODE>(P, S, r);
-      if (MODE == kModeCount) {
-        nkept = __reduce_add_sync(0xFFFFFFFFu, nkept);
-        if (lane == 0) {
-          atomicMax(P.max_units, units);
-          if (P.deg != nullptr) P.deg[j] = nkept;
-        }
-        continue;
-      }
+    }
+    if (MODE == kModeFill && P.deg != nullptr) {
+      nkept = __reduce_add_sync(0xFFFFFFFFu, nkept);
+      if (lane == 0) P.deg[j] = nkept;
+    }
+    __syncwarp();
+    const unsigned units = open_parts<MODE>(P, S, r);
+    if (MODE == kModeCount || (MODE == kModeFill && (int)units * P.unit > P.rowcap)) {
+      if (lane == 0) atomicMax(P.max_units, units);
+      continue;
     }
 
     const uint32_t* wt = P.wtab + (r.lj < P.nexc ? 0 : 65536);

@@ -372,12 +372,14 @@ int validate_neuron_params(const snn_neuron_params* n, std::string* why);
 // column at each stencil offset of each virtual column.
 cudaError_t launch_geometry(int W, int H, int tw, int th, int npc4, uint32_t* ctile, uint32_t* colv,
                             uint2* tinfo, uint32_t* nbg, cudaStream_t st);
-// Fixed law: the count pass writes bend, deg (shards) and max_units[0]; the fill
-// pass (same draws) writes the rows.
+// Fixed law: the fill pass writes bend, deg (shards), the rows of at most rowcap
+// slots, and the longest of the others to max_units[0]; the count pass writes the
+// longest row.
 cudaError_t launch_build_count(const BuildParams& bp, int num_sms, cudaStream_t st);
 cudaError_t launch_build(const BuildParams& bp, int precision, int num_sms,
                          cudaStream_t st);
-// Paper connectivity law: the same two passes (deg and max_units[1] in any case).
+// Paper connectivity law: the count pass writes bend, deg and max_units; the
+// fill pass (same draws) writes the rows.
 cudaError_t launch_paper_count(const BuildParams& bp, int num_sms, cudaStream_t st);
 cudaError_t launch_paper_fill(const BuildParams& bp, int precision, int num_sms,
                               cudaStream_t st);

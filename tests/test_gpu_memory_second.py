@@ -1,7 +1,12 @@
-"""A net takes the larger spike lists only where that leaves room for what fits the
+"""Table strides and spike lists.
+
+A net takes the larger spike lists only where that leaves room for what fits the
 device beside it without them: a second net, a pair of shards, a differentiable
 view.  And a net of very small columns, whose counters weigh as much as its
 neurons, builds where only the smaller lists fit.
+
+The rows' stride is an estimate of the longest row; where a row is longer, the
+longest one's length.
 """
 import contextlib
 
@@ -9,6 +14,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1511_09325_gb300 import build as B
 from paper_1511_09325_gb300 import snn
 from paper_1511_09325_gb300 import workloads as W
@@ -106,3 +112,29 @@ def test_small_columns_where_only_the_smaller_lists_fit():
             net.step(4)
             got = net.state()
     assert all(np.array_equal(x, y) for x, y in zip(got, want))
+
+
+@pytest.mark.parametrize("prec", ["f32w", "f16w"])
+def test_rows_longer_than_estimated(prec):
+    # 20 synapses over 40 bucket parts of equal weight (all remote, a flat stencil, half
+    # of it in the own 6 x 6 tile): the estimate is 152 slots, a row whose synapses all
+    # lie in parts of their own takes 160
+    oracle.build()
+    n = W.neuron_params(n_per_col=200, n_exc=160, nu_ext_kHz=3.0)
+    s = W.synapse_params(k_out=20, frac_local=0.0, lambda_cols=1e6)
+    p = oracle.make_params(*GRID, n, s, SEED)
+    with snn.Net(*GRID, n, s, SEED, prec) as net:
+        assert net.info()["row_capacity"] == 160
+        for j0 in (0, 12345, net.n - 200):
+            got = net.synapses(j0, 200)
+            o = oracle.synapses(p, prec, j0, 200)
+            by_delay = np.argsort(o["delay"], axis=1, kind="stable")
+            for g, k in zip(got, ("target", "delay", "wfx")):
+                assert np.array_equal(g, np.take_along_axis(o[k], by_delay, 1))
+        net.step(STEPS)
+        st, ids, over = net.spikes()
+        v = net.state()[0]
+    o = oracle.run(p, prec, STEPS)
+    key = lambda t, i: np.sort(np.asarray(t, np.int64) << 32 | np.asarray(i, np.int64))
+    assert not over and len(ids) > 0
+    assert np.array_equal(key(st, ids), key(o["t"], o["i"])) and np.array_equal(v.astype(np.float64), o["v"])
