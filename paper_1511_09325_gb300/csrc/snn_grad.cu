@@ -317,10 +317,10 @@ __global__ void __launch_bounds__(kThreads) grad_update_kernel(const GradParams 
 // One warp per row, the targets' adjoints read from L2 (MAP: the rows' order is
 // P.ord's, its words loaded a run ahead).  Each record needs one scattered 4-byte
 // read of an adjoint, a 32-byte sector of the L2, which bounds it.  MAP on 12x12
-// columns, 60 steps forward and backward: 57.5 ms with six blocks per SM, 59.5
-// with five, 66.4 with four.
+// columns, 60 steps forward and backward: 54.5 ms with five blocks per SM, 56.1 with
+// six, 56.5 with eight.
 template <bool MAP>
-__global__ void __launch_bounds__(kThreads, MAP ? 6 : 1)
+__global__ void __launch_bounds__(kThreads, MAP ? 5 : 1)
     grad_gather_kernel(const GradParams P, long long tau) {
   const long long at = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // row of the table
   const int lane = threadIdx.x & 31;
@@ -363,13 +363,11 @@ __global__ void __launch_bounds__(kThreads, MAP ? 6 : 1)
         uint32_t ip = (u >> 8 & 0xFFFu) + before, op = (u >> 20) + h - before;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const uint32_t s = in >> q & 1u ? ip++ : op++;
-          code[q] = kPad;  // places beyond the bucket's synapses: pads, or beyond its slots
-          if ((int)s < slot_end) {
-            const uint2 x = __ldg(row + s);
-            code[q] = x.x;
-            w[q] = x.y;
-          }
+          // places beyond the bucket's synapses: pads, or beyond its slots
+          const int s = (int)(in >> q & 1u ? ip++ : op++);
+          const uint2 x = __ldg(row + min(s, slot_end - 1));
+          code[q] = s < slot_end ? x.x : kPad;
+          w[q] = x.y;
         }
       } else {
         const uint4 x = __ldcs(reinterpret_cast<const uint4*>(row + k));
@@ -377,12 +375,20 @@ __global__ void __launch_bounds__(kThreads, MAP ? 6 : 1)
         code[0] = x.x; code[1] = x.z; code[2] = y.x; code[3] = y.z;
         w[0] = x.y; w[1] = x.w; w[2] = y.y; w[3] = y.w;
       }
+      if (MAP) {  // (no load under a branch, where it would be waited for)
+        float v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (code[q] & kPad) continue;
-        const uint32_t t =
-            in >> q & 1u ? tile + code[q] : __ldg(nb + (code[q] >> 11 & 63u)) + (code[q] & 2047u);
-        acc = __fmaf_rn((float)(int32_t)w[q], ibs[t], acc);
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t out = __ldg(nb + (code[q] >> 11 & 63u)) + (code[q] & 2047u);
+          v[q] = __ldg(ibs + (code[q] & kPad ? 0u : in >> q & 1u ? tile + code[q] : out));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (!(code[q] & kPad)) acc = __fmaf_rn((float)(int32_t)w[q], v[q], acc);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (!(code[q] & kPad)) acc = __fmaf_rn((float)(int32_t)w[q], ibs[tile + code[q]], acc);
       }
     }
   }
